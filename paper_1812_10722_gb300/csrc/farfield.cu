@@ -14,11 +14,11 @@
 // moments [box][term][B].
 //
 //   p2p_kernel  direct sums of a 64-target block against a contiguous source range
-//   p2m_kernel  Cartesian Taylor moments of a leaf about its centre c, shifted into
-//               every accepted ancestor box:
-//                 M^V_k = sum_j q_j (c - y_j)^k
-//                 M^K_k = sum_j mu_j * (-sum_d n_{j,d} k_d (c - y_j)^(k - e_d))
-//   m2p_kernel  Vd_i += sum_{|k|<=P} a_k(x_i - c) M^V_k (same for K), with
+//   p2m_kernel  moments of a leaf about its centre c in the harmonic basis g_k (the terms k with
+//               k_3 <= 1, see farfield.cuh), shifted into every accepted ancestor box:
+//                 M^V_k = sum_j q_j g_k(c - y_j)
+//                 M^K_k = -sum_j mu_j n_j . grad g_k(c - y_j)
+//   m2p_kernel  Vd_i += sum_{|k|<=P} a_k(x_i - c) k_1! k_2! M^V_k (same for K), with
 //               a_k(R) = D^k (1/|R|) / k! from the recurrence
 //               n |R|^2 a_k + (2n-1) sum_d R_d a_(k-e_d) + (n-1) sum_d a_(k-2e_d) = 0,
 //               n = |k|, a_0 = 1/|R|.

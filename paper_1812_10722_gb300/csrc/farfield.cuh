@@ -349,10 +349,25 @@ __global__ void __launch_bounds__(kP1Warps * 32)
 }
 
 // ------------------------------------------------------------ multi-indices
-// Terms ordered by degree n = k1+k2+k3; within a degree k1 descending, then k2.
+// Harmonic basis of the expansions.  1/|R| is harmonic, so its Taylor coefficients a_k of one
+// degree n are not independent: sum_d (k_d + 1)(k_d + 2) a_(k + 2 e_d) = 0 expresses every a_k with
+// k_3 >= 2 through those with k_3 in {0, 1}, 2n + 1 of the (n + 1)(n + 2)/2.  The same truncated sum
+//   sum_{|k| <= P} a_k(R) u^k = sum_{|k| <= P, k_3 <= 1} a_k(R) k_1! k_2! g_k(u)
+// is therefore evaluated on (P + 1)^2 terms (64 instead of 120 at P = 7), where g_k is the harmonic
+// polynomial with the values u_1^k_1 u_2^k_2 / (k_1! k_2!) on the plane u_3 = 0 (k_3 = 0; normal
+// derivative zero there) or that normal derivative (k_3 = 1; value zero).  A harmonic polynomial is
+// fixed by the two, so the g_k are closed under differentiation,
+//   d_1 g_(a,b,c) = g_(a-1,b,c),  d_2 g_(a,b,c) = g_(a,b-1,c),  d_3 g_(a,b,1) = g_(a,b,0),
+//   d_3 g_(a,b,0) = -g_(a-2,b,1) - g_(a,b-2,1),
+// and Euler's relation n g_k = u . grad g_k builds them degree by degree.  The recurrence of the a_k
+// reads k - e_d and k - 2 e_d only, so it stays within k_3 <= 1 as well.
+// Terms ordered by degree n; within a degree k_3 = 0 first, then k_1 descending.
+// Measured against the Cartesian terms (the same sums, P 7 on 81920 panels unless stated): tensor-core
+// M2P of 64 right-hand sides 4.85 -> 2.52 ms, float-float M2P of 12 (40500 panels) 35.1 -> 15.0 ms,
+// FP64 M2P of one (20480 panels, P 5) 3.59 -> 1.74 ms, FP32 M2P of one (56180 panels, P 6) 280 -> 146 us.
 __host__ __device__ constexpr int mi_index(int a, int b, int c) {
     const int n = a + b + c;
-    return n_terms(n - 1) + (n - a) * (n - a + 1) / 2 + (n - a - b);
+    return n * n + (c ? 2 * n : n) - a;
 }
 
 template <int P>
@@ -363,15 +378,14 @@ struct MultiIndex {
     int m1[NT][3];   // index of k - e_d, or -1
     int m2[NT][3];   // index of k - 2 e_d, or -1
     constexpr MultiIndex() : k(), deg(), m1(), m2() {
-        int t = 0;
         for (int n = 0; n <= P; ++n)
-            for (int a = n; a >= 0; --a)
-                for (int b = n - a; b >= 0; --b) {
+            for (int c = 0; c <= 1 && c <= n; ++c)
+                for (int a = n - c; a >= 0; --a) {
+                    const int t = mi_index(a, n - c - a, c);
                     k[t][0] = a;
-                    k[t][1] = b;
-                    k[t][2] = n - a - b;
+                    k[t][1] = n - c - a;
+                    k[t][2] = c;
                     deg[t] = n;
-                    ++t;
                 }
         for (int u = 0; u < NT; ++u)
             for (int d = 0; d < 3; ++d) {
@@ -385,18 +399,105 @@ struct MultiIndex {
     }
 };
 
-// decode the multi-index of term t
-static __device__ __forceinline__ void mi_decode(int t, int &k1, int &k2, int &k3) {
-    int n = 0;
-    while (n_terms(n) <= t) ++n;
-    int r = t - n_terms(n - 1), a = n;
-    while (r > n - a) {
-        r -= n - a + 1;
-        --a;
+// Scaled coefficients A_k = a_k / gamma_n, gamma_n = prod_{j <= n} -(2j - 1)/j, which turn the
+// recurrence n |R|^2 a_k + (2n-1) sum_d R_d a_(k-e_d) + (n-1) sum_d a_(k-2e_d) = 0 into
+//   A_k = sum_d (R_d / |R|^2) A_(k-e_d) + (kappa_n / |R|^2) sum_d A_(k-2e_d),
+// kappa_n = -(n-1)^2 / ((2n-1)(2n-3)): one multiply-add per neighbour and no scaling of the sum.
+// gamma_n k_1! k_2! is carried by the moments (term_scale).
+__host__ __device__ constexpr double mi_kappa(int n) {
+    return n < 2 ? 0.0 : -((double)(n - 1) * (n - 1)) / ((2.0 * n - 1.0) * (2.0 * n - 3.0));
+}
+__host__ __device__ constexpr double mi_gamma(int n) {
+    double g = 1.0;
+    for (int j = 1; j <= n; ++j) g *= -(2.0 * j - 1.0) / j;
+    return g;
+}
+__host__ __device__ constexpr double mi_fact(int n) {
+    double f = 1.0;
+    for (int j = 2; j <= n; ++j) f *= j;
+    return f;
+}
+
+// per term: (k_1, k_2, k_3) and the factor gamma_n k_1! k_2! of its stored moment
+struct TermInfo {
+    signed char a[n_terms(kMaxP)], b[n_terms(kMaxP)], c[n_terms(kMaxP)];
+    double scale[n_terms(kMaxP)];
+};
+constexpr TermInfo make_term_info() {
+    TermInfo r{};
+    constexpr MultiIndex<kMaxP> mi{};
+    for (int t = 0; t < n_terms(kMaxP); ++t) {
+        r.a[t] = (signed char)mi.k[t][0];
+        r.b[t] = (signed char)mi.k[t][1];
+        r.c[t] = (signed char)mi.k[t][2];
+        r.scale[t] = mi_gamma(mi.deg[t]) * mi_fact(mi.k[t][0]) * mi_fact(mi.k[t][1]);
     }
-    k1 = a;
-    k2 = n - a - r;
-    k3 = n - k1 - k2;
+    return r;
+}
+static __constant__ TermInfo c_terms = make_term_info();
+
+// A_k(R) of every term, each handed to use(t, A_t) as soon as it is made
+template <typename T, int P, class F>
+__device__ __forceinline__ void m2p_recurrence(T Rx, T Ry, T Rz, T (&a)[n_terms(P)], F &&use) {
+    constexpr MultiIndex<P> mi{};
+    constexpr int NT = MultiIndex<P>::NT;
+    a[0] = rsq(Rx * Rx + Ry * Ry + Rz * Rz);
+    const T ir2 = a[0] * a[0];
+    const T R[3] = {Rx * ir2, Ry * ir2, Rz * ir2};
+    use(0, a[0]);
+#pragma unroll
+    for (int t = 1; t < NT; ++t) {
+        T s1 = T(0), s2 = T(0);
+        bool has2 = false;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            if (mi.m1[t][d] >= 0) s1 += R[d] * a[mi.m1[t][d]];
+            if (mi.m2[t][d] >= 0) {
+                s2 = has2 ? s2 + a[mi.m2[t][d]] : a[mi.m2[t][d]];
+                has2 = true;
+            }
+        }
+        if (has2) s1 += (T(mi_kappa(mi.deg[t])) * ir2) * s2;
+        a[t] = s1;
+        use(t, a[t]);
+    }
+}
+
+// g_t(u) and d_3 g_t(u) (d3) of every term in T, with grad g_t . nrm; put(t, g_t, n . grad g_t, d_3 g_t)
+template <typename T, int P, class F>
+__device__ __forceinline__ void harmonics(const T (&u)[3], const T (&n)[3], F &&put) {
+    constexpr MultiIndex<P> mi{};
+    constexpr int NT = MultiIndex<P>::NT;
+    T g[NT];
+    g[0] = T(1);
+    put(0, T(1), T(0), T(0));
+#pragma unroll
+    for (int t = 1; t < NT; ++t) {
+        const int k1 = mi.k[t][0], k2 = mi.k[t][1], k3 = mi.k[t][2];
+        T p3 = T(0), s = T(0), dn = T(0);
+        if (k3) {
+            p3 = g[mi_index(k1, k2, 0)];
+        } else {
+            if (k1 >= 2) p3 = -g[mi_index(k1 >= 2 ? k1 - 2 : 0, k2, 1)];
+            if (k2 >= 2) p3 = p3 - g[mi_index(k1, k2 >= 2 ? k2 - 2 : 0, 1)];
+        }
+        if (k3 || k1 >= 2 || k2 >= 2) {
+            s = u[2] * p3;
+            dn = n[2] * p3;
+        }
+        if (k1) {
+            const T p = g[mi_index(k1 ? k1 - 1 : 0, k2, k3)];
+            s += u[0] * p;
+            dn += n[0] * p;
+        }
+        if (k2) {
+            const T p = g[mi_index(k1, k2 ? k2 - 1 : 0, k3)];
+            s += u[1] * p;
+            dn += n[1] * p;
+        }
+        g[t] = mi.deg[t] == 1 ? s : T(1.0 / mi.deg[t]) * s;
+        put(t, g[t], dn, p3);
+    }
 }
 
 // --------------------------------------------------------------------- M2P
@@ -405,41 +506,17 @@ static __device__ __forceinline__ void mi_decode(int t, int &k1, int &k2, int &k
 template <typename T, int P, int NB>
 __device__ __forceinline__ void m2p_one(T Rx, T Ry, T Rz, const typename Vec4<T>::type *__restrict__ mom,
                                         T (&acc)[NB][4]) {
-    constexpr MultiIndex<P> mi{};
-    constexpr int NT = MultiIndex<P>::NT;
-    const T R[3] = {Rx, Ry, Rz};
-    const T r2 = Rx * Rx + Ry * Ry + Rz * Rz;
-    T a[NT];
-    a[0] = rsq(r2);
-    const T ir2 = a[0] * a[0];
-#pragma unroll
-    for (int j = 0; j < NB; ++j) {
-        const auto m = mom[j];
-        acc[j][0] += a[0] * m.x;
-        acc[j][1] += a[0] * m.y;
-        acc[j][2] += a[0] * m.z;
-        acc[j][3] += a[0] * m.w;
-    }
-#pragma unroll
-    for (int t = 1; t < NT; ++t) {
-        const int n = mi.deg[t];
-        T s1 = T(0), s2 = T(0);
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            if (mi.m1[t][d] >= 0) s1 += R[d] * a[mi.m1[t][d]];
-            if (mi.m2[t][d] >= 0) s2 += a[mi.m2[t][d]];
-        }
-        const T c1 = T(-(2.0 * n - 1.0) / n), c2 = T(-(n - 1.0) / n);
-        a[t] = (c1 * s1 + c2 * s2) * ir2;
+    T a[n_terms(P)];
+    m2p_recurrence<T, P>(Rx, Ry, Rz, a, [&](int t, const T &at) {
 #pragma unroll
         for (int j = 0; j < NB; ++j) {
             const auto m = mom[t * NB + j];
-            acc[j][0] += a[t] * m.x;
-            acc[j][1] += a[t] * m.y;
-            acc[j][2] += a[t] * m.z;
-            acc[j][3] += a[t] * m.w;
+            acc[j][0] += at * m.x;
+            acc[j][1] += at * m.y;
+            acc[j][2] += at * m.z;
+            acc[j][3] += at * m.w;
         }
-    }
+    });
 }
 
 // warps per block such that the staged moments of every warp fit in 46 KB
@@ -550,26 +627,8 @@ constexpr int kM2PGemmThreads = 64;
 
 template <typename T, int P>
 __device__ __forceinline__ void m2p_coeffs(T Rx, T Ry, T Rz, T *__restrict__ out) {   // out[k * 64]
-    constexpr MultiIndex<P> mi{};
-    constexpr int NT = MultiIndex<P>::NT;
-    const T R[3] = {Rx, Ry, Rz};
-    T a[NT];
-    a[0] = rsq(Rx * Rx + Ry * Ry + Rz * Rz);
-    const T ir2 = a[0] * a[0];
-    out[0] = a[0];
-#pragma unroll
-    for (int t = 1; t < NT; ++t) {
-        const int n = mi.deg[t];
-        T s1 = T(0), s2 = T(0);
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            if (mi.m1[t][d] >= 0) s1 += R[d] * a[mi.m1[t][d]];
-            if (mi.m2[t][d] >= 0) s2 += a[mi.m2[t][d]];
-        }
-        const T c1 = T(-(2.0 * n - 1.0) / n), c2 = T(-(n - 1.0) / n);
-        a[t] = (c1 * s1 + c2 * s2) * ir2;
-        out[t * kM2PGemmThreads] = a[t];
-    }
+    T a[n_terms(P)];
+    m2p_recurrence<T, P>(Rx, Ry, Rz, a, [&](int t, const T &at) { out[t * kM2PGemmThreads] = at; });
 }
 
 template <typename T, int P, int NB>
@@ -658,34 +717,61 @@ __global__ void __launch_bounds__(kM2PGemmThreads)
 }
 
 // --------------------------------------------------------------------- P2M
-constexpr int kP2MTile = 32;
-
-// binomial coefficients C(n, r), n, r <= kMaxP
-static __constant__ float c_binom[kMaxP + 1][kMaxP + 1] = {
-    {1, 0, 0, 0, 0, 0, 0, 0, 0},     {1, 1, 0, 0, 0, 0, 0, 0, 0},     {1, 2, 1, 0, 0, 0, 0, 0, 0},
-    {1, 3, 3, 1, 0, 0, 0, 0, 0},     {1, 4, 6, 4, 1, 0, 0, 0, 0},     {1, 5, 10, 10, 5, 1, 0, 0, 0},
-    {1, 6, 15, 20, 15, 6, 1, 0, 0},  {1, 7, 21, 35, 35, 21, 7, 1, 0}, {1, 8, 28, 56, 70, 56, 28, 8, 1}};
-
-// One block per work unit (leaf chunk, right-hand-side chunk), one thread per term k.
-// The chunk's moments about the leaf centre c are added to the leaf if some target block
-// accepted it, and shifted into every accepted ancestor a (upward pass folded in):
-//   M_k(a) = sum_{l <= k} C(k, l) (a - c)^(k - l) M_l(c),  C(k, l) = prod_d binom(k_d, l_d),
-// valid for both moment kinds since (a - y)^k = ((a - c) + (c - y))^k.
+// One block per work unit (leaf chunk, chunk of NB right-hand sides).  The moments of the chunk
+// about the leaf centre c in the harmonic basis,
+//   M^V_k = sum_j q_j g_k(c - y_j),   M^K_k = -sum_j mu_j n_j . grad g_k(c - y_j),
+// are two small matrix products (terms x sources) x (sources x channels): per tile of 32 sources
+// one warp generates g and n . grad g of its lanes' sources into shared memory while the others
+// stage the weights, then every thread accumulates a register tile of TT terms x RB right-hand
+// sides (the sources split over SP thread groups where the tile leaves the block small).  The sums
+// are added to the leaf if some target block accepted it, and shifted into every accepted ancestor
+// A (upward pass folded in): with delta = c_A - c, the Taylor expansion of g_k about delta gives
+//   M_(a,b,c)(A) = sum_{i<=a, j<=b} g_(i,j,c)(delta) M_(a-i,b-j,0) + d_3 g_(i,j,c)(delta) M_(a-i,b-j,1).
+// Stored moments carry the factor gamma_n k_1! k_2! of their term.
+// Bound by the FP32 pipe and the shared-memory reads of the tile product.  81920 panels, P 7,
+// 64 right-hand sides: 769 us, 1913 before (one thread per Cartesian term, every monomial and its
+// derivative formed per right-hand-side chunk of 8); 56180 panels, P 6, one right-hand side: 65 us
+// after 135.
 template <typename T, int P, int NB>
-__global__ void p2m_kernel(const int4 *__restrict__ items, int64_t nitems, int nbc, int B,
-                           const typename Vec4<T>::type *__restrict__ spos,
-                           const typename Vec4<T>::type *__restrict__ snrm, const typename Vec4<T>::type *__restrict__ sw,
-                           const typename Vec4<T>::type *__restrict__ box_c, const int *__restrict__ parent,
-                           const int *__restrict__ used, typename MomAcc<T>::type *__restrict__ mom,
-                           const int *nact) {
+struct P2MShape {
+    static constexpr int NT = n_terms(P);
+    static constexpr int TS = 32;                          // sources per tile
+    static constexpr int TT = 16 / (int)sizeof(T);         // terms per thread (one 16-byte word)
+    static constexpr int TG = (NT + TT - 1) / TT;
+    static constexpr int RB = NB == 1 ? 1 : (sizeof(T) == 4 ? 4 : 2);   // right-hand sides per thread
+    static constexpr int RG = NB / RB;
+    static constexpr int split(int n) { return n >= 8 ? 8 : (n >= 4 ? 4 : (n >= 2 ? 2 : 1)); }
+    static constexpr int SP = split(128 / (TG * RG));      // source splits
+    static constexpr int THREADS = (TG * RG * SP + 31) / 32 * 32 < 64 ? 64 : (TG * RG * SP + 31) / 32 * 32;
+    static constexpr int ROW = TS + 1;                     // padded: lanes of one source read free of conflicts
+    static constexpr size_t GD = (size_t)2 * TG * ROW * 16;
+    static constexpr size_t W = (size_t)TS * NB * sizeof(typename Vec4<T>::type);
+    static constexpr size_t LM = (size_t)SP * NT * NB * sizeof(typename Vec4<T>::type);
+    static constexpr size_t BODY = GD + W > LM ? GD + W : LM;           // the sums reuse the tile's space
+    static constexpr size_t ANC = (size_t)(kMaxDepth + 1) * 2 * NT * sizeof(T);
+    static constexpr size_t SMEM = (BODY + 15) / 16 * 16 + ANC;
+};
+
+template <typename T, int TT> struct __align__(16) TermVec { T v[TT]; };
+
+template <typename T, int P, int NB>
+__global__ void __launch_bounds__(P2MShape<T, P, NB>::THREADS)
+    p2m_kernel(const int4 *__restrict__ items, int64_t nitems, int nbc, int B,
+               const typename Vec4<T>::type *__restrict__ spos, const typename Vec4<T>::type *__restrict__ snrm,
+               const typename Vec4<T>::type *__restrict__ sw, const typename Vec4<T>::type *__restrict__ box_c,
+               const int *__restrict__ parent, const int *__restrict__ used,
+               typename MomAcc<T>::type *__restrict__ mom, const int *nact) {
     using S = typename MomAcc<T>::scalar;
     using T4 = typename Vec4<T>::type;
-    constexpr int NT = n_terms(P);
-    __shared__ T pw[kP2MTile][3][P + 1];
-    __shared__ T4 shn[kP2MTile];
-    __shared__ T4 shw[kP2MTile][NB];
-    __shared__ T4 lm[NT][NB];
-    __shared__ T dpw[3][P + 1];
+    using Sh = P2MShape<T, P, NB>;
+    using TV = TermVec<T, Sh::TT>;
+    constexpr int NT = Sh::NT, TS = Sh::TS, TT = Sh::TT, TG = Sh::TG, RB = Sh::RB, RG = Sh::RG, SP = Sh::SP;
+    extern __shared__ __align__(16) unsigned char p2m_smem[];
+    TV *sg = (TV *)p2m_smem, *sd = sg + TG * Sh::ROW;       // [term group][source]
+    T4 *shw = (T4 *)(p2m_smem + Sh::GD);                    // [source][right-hand side]
+    T4 *lm = (T4 *)p2m_smem;                                // [split][term][right-hand side]
+    T *anc = (T *)(p2m_smem + (Sh::BODY + 15) / 16 * 16);   // [ancestor][g, d_3 g][term]
+    __shared__ int anc_box[kMaxDepth + 1], n_anc;
     const int64_t u = blockIdx.x;
     if (u >= nitems * nbc) return;
     const int64_t ii = u / nbc;
@@ -695,104 +781,156 @@ __global__ void p2m_kernel(const int4 *__restrict__ items, int64_t nitems, int n
     const int nb = min(NB, Bact - b0);
     const int4 item = items[ii];
     const T4 c = box_c[item.x];
-    const int t = threadIdx.x;
-    int k1 = 0, k2 = 0, k3 = 0;
-    if (t < NT) mi_decode(t, k1, k2, k3);
-    T acc[NB][4];
-#pragma unroll
-    for (int j = 0; j < NB; ++j)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[j][q] = T(0);
-    for (int base = item.y; base < item.z; base += kP2MTile) {
-        __syncthreads();
-        const int cnt = min(kP2MTile, item.z - base);
-        if (t < cnt) {
-            const T4 y = spos[base + t];
-            const T d[3] = {c.x - y.x, c.y - y.y, c.z - y.z};
-            for (int q = 0; q < 3; ++q) {
-                T v = 1;
-                for (int e = 0; e <= P; ++e) {
-                    pw[t][q][e] = v;
-                    v *= d[q];
-                }
-            }
-            shn[t] = snrm[base + t];
-#pragma unroll
-            for (int j = 0; j < NB; ++j) shw[t][j] = j < nb ? sw[(int64_t)(base + t) * B + b0 + j] : zero4<T4>();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tg = tid % TG, rg = (tid / TG) % RG, sp = tid / (TG * RG);
+    const bool on = sp < SP;
+    if (warp == 1) {   // the accepted ancestors' shift tables, one lane each
+        int mine = -1, k = 0;
+        for (int A = parent[item.x]; A >= 0; A = parent[A]) {
+            if (!used[A]) continue;
+            if (k == lane) mine = A;
+            ++k;
         }
-        __syncthreads();
-        if (t < NT) {
-            for (int s = 0; s < cnt; ++s) {
-                const T px = pw[s][0][k1], py = pw[s][1][k2], pz = pw[s][2][k3];
-                const T mono = px * py * pz;
-                const T4 n = shn[s];
-                T dm = 0;
-                if (k1) dm += n.x * T(k1) * pw[s][0][k1 - 1] * py * pz;
-                if (k2) dm += n.y * T(k2) * px * pw[s][1][k2 - 1] * pz;
-                if (k3) dm += n.z * T(k3) * px * py * pw[s][2][k3 - 1];
-#pragma unroll
-                for (int j = 0; j < NB; ++j) {
-                    const T4 w = shw[s][j];
-                    acc[j][0] += w.x * mono;
-                    acc[j][1] += w.y * mono;
-                    acc[j][2] -= w.z * dm;
-                    acc[j][3] -= w.w * dm;
-                }
-            }
+        if (lane == 0) n_anc = k;
+        if (mine >= 0) {
+            anc_box[lane] = mine;
+            const T4 ca = box_c[mine];
+            const T d[3] = {ca.x - c.x, ca.y - c.y, ca.z - c.z}, z[3] = {T(0), T(0), T(0)};
+            T *g = anc + (size_t)lane * 2 * NT;
+            harmonics<T, P>(d, z, [&](int t, const T &v, const T &, const T &d3) {
+                g[t] = v;
+                g[NT + t] = d3;
+            });
         }
     }
-    if (t < NT) {
-        const bool own = used[item.x] != 0;
+    T acc[TT][RB][4];
 #pragma unroll
-        for (int j = 0; j < NB; ++j) {
-            T4 o;
-            o.x = acc[j][0]; o.y = acc[j][1]; o.z = acc[j][2]; o.w = acc[j][3];
-            lm[t][j] = o;
-            if (own && j < nb) {
-                S *g = (S *)(mom + ((int64_t)item.x * NT + t) * B + b0 + j);
-                acc_add4(g, (S)acc[j][0], (S)acc[j][1], (S)acc[j][2], (S)acc[j][3]);
+    for (int i = 0; i < TT; ++i)
+#pragma unroll
+        for (int j = 0; j < RB; ++j)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[i][j][q] = T(0);
+    for (int base = item.y; base < item.z; base += TS) {
+        const int cnt = min(TS, item.z - base);
+        if (base > item.y) __syncthreads();   // the previous tile has been read
+        if (warp == 0) {
+            const int s = base + (lane < cnt ? lane : 0);
+            const T4 y = spos[s], nn = snrm[s];
+            const T d[3] = {c.x - y.x, c.y - y.y, c.z - y.z}, n[3] = {nn.x, nn.y, nn.z};
+            TV gv, dv;
+#pragma unroll
+            for (int i = 0; i < TT; ++i) gv.v[i] = dv.v[i] = T(0);
+            harmonics<T, P>(d, n, [&](int t, const T &g, const T &dn, const T &) {
+                gv.v[t % TT] = g;
+                dv.v[t % TT] = dn;
+                if (t % TT == TT - 1 || t == NT - 1) {
+                    sg[(t / TT) * Sh::ROW + lane] = gv;
+                    sd[(t / TT) * Sh::ROW + lane] = dv;
+                }
+            });
+        } else {
+            for (int q = tid - 32; q < cnt * NB; q += Sh::THREADS - 32) {
+                const int s = q / NB, j = q - s * NB;
+                shw[q] = j < nb ? sw[(int64_t)(base + s) * B + b0 + j] : zero4<T4>();
             }
         }
-    }
-    for (int A = parent[item.x]; A >= 0; A = parent[A]) {
-        if (!used[A]) continue;
         __syncthreads();
-        if (t < 3) {
-            const T4 ca = box_c[A];
-            const T delta = t == 0 ? ca.x - c.x : (t == 1 ? ca.y - c.y : ca.z - c.z);
-            T v = 1;
-            for (int e = 0; e <= P; ++e) {
-                dpw[t][e] = v;
-                v *= delta;
-            }
-        }
-        __syncthreads();
-        if (t < NT) {
+        if (on) {
+#pragma unroll 2
+            for (int s = sp; s < cnt; s += SP) {
+                const TV g = sg[tg * Sh::ROW + s], d = sd[tg * Sh::ROW + s];
 #pragma unroll
-            for (int j = 0; j < NB; ++j)
+                for (int j = 0; j < RB; ++j) {
+                    const T4 w = shw[s * NB + rg * RB + j];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[j][q] = T(0);
-            for (int l1 = 0; l1 <= k1; ++l1)
-                for (int l2 = 0; l2 <= k2; ++l2)
-                    for (int l3 = 0; l3 <= k3; ++l3) {
-                        const T coef = T(c_binom[k1][l1] * c_binom[k2][l2] * c_binom[k3][l3]) * dpw[0][k1 - l1] *
-                                       dpw[1][k2 - l2] * dpw[2][k3 - l3];
-                        const int li = mi_index(l1, l2, l3);
-#pragma unroll
-                        for (int j = 0; j < NB; ++j) {
-                            const T4 m = lm[li][j];
-                            acc[j][0] += coef * m.x;
-                            acc[j][1] += coef * m.y;
-                            acc[j][2] += coef * m.z;
-                            acc[j][3] += coef * m.w;
+                    for (int i = 0; i < TT; ++i) {
+                        if constexpr (std::is_same<T, float>::value) {
+                            const float2 v = __ffma2_rn(make_float2(g.v[i], g.v[i]), make_float2(w.x, w.y),
+                                                        make_float2(acc[i][j][0], acc[i][j][1]));
+                            const float2 k = __ffma2_rn(make_float2(d.v[i], d.v[i]), make_float2(w.z, w.w),
+                                                        make_float2(acc[i][j][2], acc[i][j][3]));
+                            acc[i][j][0] = v.x; acc[i][j][1] = v.y; acc[i][j][2] = k.x; acc[i][j][3] = k.y;
+                        } else if constexpr (std::is_same<T, ffloat>::value) {
+                            ff_mac(acc[i][j][0], g.v[i], w.x);
+                            ff_mac(acc[i][j][1], g.v[i], w.y);
+                            ff_mac(acc[i][j][2], d.v[i], w.z);
+                            ff_mac(acc[i][j][3], d.v[i], w.w);
+                        } else {
+                            acc[i][j][0] += g.v[i] * w.x;
+                            acc[i][j][1] += g.v[i] * w.y;
+                            acc[i][j][2] += d.v[i] * w.z;
+                            acc[i][j][3] += d.v[i] * w.w;
                         }
                     }
-#pragma unroll
-            for (int j = 0; j < NB; ++j) {
-                if (j >= nb) break;
-                S *g = (S *)(mom + ((int64_t)A * NT + t) * B + b0 + j);
-                acc_add4(g, (S)acc[j][0], (S)acc[j][1], (S)acc[j][2], (S)acc[j][3]);
+                }
             }
+        }
+    }
+    __syncthreads();   // the tile's space now takes the sums
+    if (on) {
+#pragma unroll
+        for (int i = 0; i < TT; ++i) {
+            const int t = tg * TT + i;
+            if (t >= NT) break;
+#pragma unroll
+            for (int j = 0; j < RB; ++j) {
+                if constexpr (std::is_same<T, ffloat>::value) {   // the running sums are unnormalised
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) ff_two_sum(acc[i][j][q].hi, acc[i][j][q].lo, acc[i][j][q].hi, acc[i][j][q].lo);
+                }
+                T4 o;
+                o.x = acc[i][j][0]; o.y = acc[i][j][1]; o.z = -acc[i][j][2]; o.w = -acc[i][j][3];
+                lm[((size_t)sp * NT + t) * NB + rg * RB + j] = o;
+            }
+        }
+    }
+    __syncthreads();
+    const bool own = used[item.x] != 0;
+    for (int q = tid; q < NT * NB; q += Sh::THREADS) {
+        const int t = q / NB, j = q - t * NB;
+        T4 o = lm[q];
+#pragma unroll
+        for (int k = 1; k < SP; ++k) {
+            const T4 p = lm[(size_t)k * NT * NB + q];
+            o.x += p.x; o.y += p.y; o.z += p.z; o.w += p.w;
+        }
+        if (SP > 1) lm[q] = o;
+        if (own && j < nb) {
+            const T f = T(c_terms.scale[t]);
+            S *g = (S *)(mom + ((int64_t)item.x * NT + t) * B + b0 + j);
+            acc_add4(g, (S)(f * o.x), (S)(f * o.y), (S)(f * o.z), (S)(f * o.w));
+        }
+    }
+    if (n_anc == 0) return;
+    __syncthreads();
+    for (int k = 0; k < n_anc; ++k) {
+        const T *ga = anc + (size_t)k * 2 * NT;
+        for (int q = tid; q < NT * NB; q += Sh::THREADS) {
+            const int t = q / NB, j = q - t * NB;
+            if (j >= nb) continue;
+            const int ka = c_terms.a[t], kb = c_terms.b[t], kc = c_terms.c[t];
+            T o[4] = {T(0), T(0), T(0), T(0)};
+            for (int i = 0; i <= ka; ++i)
+                for (int l = 0; l <= kb; ++l) {
+                    const int gi = mi_index(i, l, kc);
+                    const T g = ga[gi];
+                    const T4 m = lm[mi_index(ka - i, kb - l, 0) * NB + j];
+                    o[0] += g * m.x;
+                    o[1] += g * m.y;
+                    o[2] += g * m.z;
+                    o[3] += g * m.w;
+                    if (kc || i + l >= 2) {   // d_3 g vanishes for (0,0,0), (1,0,0) and (0,1,0)
+                        const T e = ga[NT + gi];
+                        const T4 m1 = lm[mi_index(ka - i, kb - l, 1) * NB + j];
+                        o[0] += e * m1.x;
+                        o[1] += e * m1.y;
+                        o[2] += e * m1.z;
+                        o[3] += e * m1.w;
+                    }
+                }
+            const T f = T(c_terms.scale[t]);
+            S *g = (S *)(mom + ((int64_t)anc_box[k] * NT + t) * B + b0 + j);
+            acc_add4(g, (S)(f * o[0]), (S)(f * o[1]), (S)(f * o[2]), (S)(f * o[3]));
         }
     }
 }
@@ -864,13 +1002,28 @@ static void p2p1_launch(lspr_ctx *ctx, const int4 *items, int64_t nitems, double
 }
 
 template <typename T, int P, int NB>
-static void p2m_launch(lspr_ctx *ctx, int B) {
+static void p2m_launch_nb(lspr_ctx *ctx, int B) {
+    static int smem_set[kSmemDevices] = {};
+    using Sh = P2MShape<T, P, NB>;
     Tree &tr = ctx->tree;
-    const int threads = ((n_terms(P) + 31) / 32) * 32;
     const int nbc = (B + NB - 1) / NB;
-    p2m_kernel<T, P, NB><<<(unsigned)(tr.n_p2m_items * nbc), threads, 0, ctx->stream>>>(
+    // a failure here shows as the launch's error, which the caller checks
+    if (Sh::SMEM > 47 * 1024) (void)allow_smem(p2m_kernel<T, P, NB>, (int)Sh::SMEM, ctx->device, smem_set);
+    p2m_kernel<T, P, NB><<<(unsigned)(tr.n_p2m_items * nbc), Sh::THREADS, Sh::SMEM, ctx->stream>>>(
         tr.p2m_items.p, tr.n_p2m_items, nbc, B, Views<T>::spos(ctx), Views<T>::snrm(ctx), Views<T>::w(ctx),
         Views<T>::bc(ctx), tr.box_parent.p, tr.box_used.p, Views<T>::mom_acc(ctx), ctx->rhs_nact);
+}
+
+template <typename T, int P, int NB>
+static void p2m_launch(lspr_ctx *ctx, int B) {
+    if constexpr (std::is_same<T, float>::value && NB > 1) {
+        // g is generated once per chunk of right-hand sides: the widest chunk that the batch fills
+        if (B > 16) p2m_launch_nb<T, P, 32>(ctx, B);
+        else if (B > 8) p2m_launch_nb<T, P, 16>(ctx, B);
+        else p2m_launch_nb<T, P, 8>(ctx, B);
+    } else {
+        p2m_launch_nb<T, P, NB>(ctx, B);
+    }
 }
 
 template <typename T, int P, int NB>

@@ -19,30 +19,27 @@ namespace {
 constexpr int kFfP2PChunk = 8;
 
 // one term k of the table: distances u - index(k - e_d) and u - index(k - 2 e_d) to the term's
-// own index u (0: absent), and the recurrence weights -(2n-1)/n and -(n-1)/n as float-float pairs
+// own index u (0: absent); and per degree the recurrence weight kappa_n as a float-float pair
 struct FfTerm {
-    unsigned char d1[3], d2[3];
-    short pad;
-    float c1h, c1l, c2h, c2l;
+    unsigned char d1[3], d2[2];
+    unsigned char pad[3];
 };
 struct FfTermTable {
     FfTerm t[n_terms(kMaxP)];
+    float kh[kMaxP + 1], kl[kMaxP + 1];
 };
 
 constexpr FfTermTable make_ff_terms() {
     FfTermTable tab{};
     constexpr MultiIndex<kMaxP> mi{};
-    for (int u = 0; u < n_terms(kMaxP); ++u) {
+    for (int u = 0; u < n_terms(kMaxP); ++u)
         for (int d = 0; d < 3; ++d) {
             tab.t[u].d1[d] = (unsigned char)(mi.m1[u][d] >= 0 ? u - mi.m1[u][d] : 0);
-            tab.t[u].d2[d] = (unsigned char)(mi.m2[u][d] >= 0 ? u - mi.m2[u][d] : 0);
+            if (d < 2) tab.t[u].d2[d] = (unsigned char)(mi.m2[u][d] >= 0 ? u - mi.m2[u][d] : 0);   // k_3 <= 1
         }
-        const double n = mi.deg[u];
-        const double c1 = u ? -(2.0 * n - 1.0) / n : 0.0, c2 = u ? -(n - 1.0) / n : 0.0;
-        tab.t[u].c1h = (float)c1;
-        tab.t[u].c1l = (float)(c1 - (double)(float)c1);
-        tab.t[u].c2h = (float)c2;
-        tab.t[u].c2l = (float)(c2 - (double)(float)c2);
+    for (int n = 0; n <= kMaxP; ++n) {
+        tab.kh[n] = (float)mi_kappa(n);
+        tab.kl[n] = (float)(mi_kappa(n) - (double)(float)mi_kappa(n));
     }
     return tab;
 }
@@ -52,7 +49,7 @@ __constant__ FfTermTable c_ff_terms = make_ff_terms();
 
 // The recurrence of a degree-n term reads terms of degrees n-1 and n-2 only, so each lane keeps
 // its coefficients in a ring of W slots (term u in slot u mod W), W = the terms of the three
-// highest degrees P-2, P-1, P (85 instead of 120 at P = 7): every term read is among the W
+// highest degrees P-2, P-1, P (39 instead of 64 at P = 7): every term read is among the W
 // written last.
 __host__ __device__ inline int ff_ring(int P) {
     return P < 2 ? n_terms(P) : n_terms(P) - n_terms(P - 3);
@@ -116,10 +113,13 @@ __global__ void __launch_bounds__(64)
                 __syncthreads();
             };
             stage(0);
-            const ffloat R[3] = {q.x - c.x, q.y - c.y, q.z - c.z};
-            const ffloat r2 = R[0] * R[0] + R[1] * R[1] + R[2] * R[2];
+            const ffloat d[3] = {q.x - c.x, q.y - c.y, q.z - c.z};
+            const ffloat r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
             const ffloat a0 = rsq(r2);
             const ffloat ir2 = a0 * a0;
+            const ffloat R[3] = {d[0] * ir2, d[1] * ir2, d[2] * ir2};
+            ffloat kap(0.f, 0.f);   // kappa_n / |R|^2 of the current degree n
+            int n = 0, tn = 1;      // degree, first term of the next one
             sa[lane] = a0;
             int su = 0;   // slot of term t
             int tpart = 0;   // first term of the staged part
@@ -134,21 +134,30 @@ __global__ void __launch_bounds__(64)
 #pragma unroll 1
             for (int t = 1; t < NT; ++t) {
                 if (t == tpart + TP) stage(tpart = t);
+                if (t == tn) {
+                    ++n;
+                    tn = (n + 1) * (n + 1);
+                    kap = ffloat(c_ff_terms.kh[n], c_ff_terms.kl[n]) * ir2;
+                }
                 const FfTerm &e = c_ff_terms.t[t];
                 su = su + 1 == W ? 0 : su + 1;
-                ffloat s1(0.f, 0.f), s2(0.f, 0.f);
+                ffloat at(0.f, 0.f);
+                if (e.d2[0] | e.d2[1]) {
+                    ffloat s2(0.f, 0.f);
 #pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    if (e.d1[d]) {
-                        const int sl = su - e.d1[d];
-                        s1 += R[d] * sa[(sl < 0 ? sl + W : sl) * 32 + lane];
-                    }
-                    if (e.d2[d]) {
-                        const int sl = su - e.d2[d];
-                        s2 += sa[(sl < 0 ? sl + W : sl) * 32 + lane];
-                    }
+                    for (int x = 0; x < 2; ++x)
+                        if (e.d2[x]) {
+                            const int sl = su - e.d2[x];
+                            s2 += sa[(sl < 0 ? sl + W : sl) * 32 + lane];
+                        }
+                    at = kap * s2;
                 }
-                const ffloat at = (ffloat(e.c1h, e.c1l) * s1 + ffloat(e.c2h, e.c2l) * s2) * ir2;
+#pragma unroll
+                for (int x = 0; x < 3; ++x)
+                    if (e.d1[x]) {
+                        const int sl = su - e.d1[x];
+                        at += R[x] * sa[(sl < 0 ? sl + W : sl) * 32 + lane];
+                    }
                 sa[su * 32 + lane] = at;
 #pragma unroll
                 for (int j = 0; j < NB; ++j) {

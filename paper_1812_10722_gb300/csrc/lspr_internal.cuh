@@ -49,8 +49,8 @@ constexpr int kMaxDepth = 10;                          // octree levels below th
 constexpr int kMaxNk = 32;
 constexpr int kMaxSurfaces = 16;                       // particle + analyte surfaces
 
-// number of multi-indices with |k| <= P
-__host__ __device__ constexpr int n_terms(int P) { return (P + 1) * (P + 2) * (P + 3) / 6; }
+// terms of an expansion of order P in the harmonic basis: the multi-indices |k| <= P with k_3 <= 1
+__host__ __device__ constexpr int n_terms(int P) { return (P + 1) * (P + 1); }
 
 // ---------------------------------------------------------------- device arrays
 // Counts device allocations made through DArr: captured CUDA graphs embed buffer
@@ -141,7 +141,7 @@ struct WorkOrder {   // sources/targets in the order the far-field kernels walk 
 struct Tree {
     bool ready = false;
     double theta = 0.5;
-    int P = 6, Ncrit = 300, NT = 84;
+    int P = 6, Ncrit = 300, NT = 49;
     int64_t nboxes = 0, ntblocks = 0;
     int64_t n_p2p_items = 0, n_m2p_items = 0, n_m2p_pairs = 0, n_p2m_items = 0;
     int64_t p2p_pairs = 0;

@@ -373,22 +373,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 const bool on = live && ((e.y >> blk) & 1);   // uniform over the warp but for the tail
                 float a[NT];
                 if (on) {
-                    constexpr MultiIndex<P> mi{};
-                    const float R[3] = {q.x - c.x, q.y - c.y, q.z - c.z};
-                    a[0] = rsq(R[0] * R[0] + R[1] * R[1] + R[2] * R[2]);
-                    const float ir2 = a[0] * a[0];
-#pragma unroll
-                    for (int t = 1; t < NT; ++t) {
-                        const int n = mi.deg[t];
-                        float s1 = 0.f, s2 = 0.f;
-#pragma unroll
-                        for (int d = 0; d < 3; ++d) {
-                            if (mi.m1[t][d] >= 0) s1 += R[d] * a[mi.m1[t][d]];
-                            if (mi.m2[t][d] >= 0) s2 += a[mi.m2[t][d]];
-                        }
-                        const float c1 = (float)(-(2.0 * n - 1.0) / n), c2 = (float)(-(n - 1.0) / n);
-                        a[t] = (c1 * s1 + c2 * s2) * ir2;
-                    }
+                    m2p_recurrence<float, P>(q.x - c.x, q.y - c.y, q.z - c.z, a, [](int, float) {});
                 } else {
 #pragma unroll
                     for (int t = 0; t < NT; ++t) a[t] = 0.f;
