@@ -175,7 +175,7 @@ struct Tree {
 };
 
 struct DirectItems {
-    int64_t n = 0;
+    int64_t n = 0, chunk = 0;   // items, sources per item
     DArr<int4> items;
 };
 
@@ -256,7 +256,8 @@ struct lspr_ctx {
     lspr::Mesh mesh;
     lspr::WorkOrder wo;
     lspr::Tree tree;
-    lspr::DirectItems direct;
+    lspr::DirectItems direct;          // one right-hand side
+    lspr::DirectItems direct_multi;    // several: fewer, longer items (n = 0: those of direct)
     lspr::Timing timing;
     // per-matvec scratch
     lspr::DArr<double> acc;            // [B][N][4]: V re/im, K re/im (far part)
@@ -309,6 +310,11 @@ struct lspr_ctx {
 };
 
 namespace lspr {
+
+// the direct-mode items of a product of BS channel sets
+inline const DirectItems &direct_items(const lspr_ctx *c, int64_t BS) {
+    return BS > 1 && c->direct_multi.n ? c->direct_multi : c->direct;
+}
 
 // -------------------------------------------------------------- error helpers
 int cuda_status(lspr_ctx *ctx, cudaError_t e, const char *what);

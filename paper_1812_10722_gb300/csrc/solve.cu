@@ -289,8 +289,8 @@ static int far_part(lspr_ctx *ctx, int mode, const double2 *x, int B) {
         LSPR_TRY_ST(launch_m2p(ctx, prec, ctx->acc.p, ctx->counters.p + 1, BS));
         LSPR_TRY(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
     } else {
-        LSPR_TRY_ST(launch_p2p(ctx, prec, ctx->direct.items.p, ctx->direct.n, ctx->acc.p, ctx->stream,
-                               ctx->counters.p, BS));
+        const DirectItems &d = direct_items(ctx, BS);
+        LSPR_TRY_ST(launch_p2p(ctx, prec, d.items.p, d.n, ctx->acc.p, ctx->stream, ctx->counters.p, BS));
     }
     ctx->matvec_count += B;
     return LSPR_OK;

@@ -588,6 +588,7 @@ int tree_build(lspr_ctx *ctx, double theta, int P, int Ncrit) {
     LSPR_TRY(ctx, cudaGetLastError());
     // the direct-mode items now address the Morton work order: refresh their own-panel flags
     LSPR_TRY_ST(launch_item_flags(ctx, ctx->direct.items.p, ctx->direct.n));
+    LSPR_TRY_ST(launch_item_flags(ctx, ctx->direct_multi.items.p, ctx->direct_multi.n));
     LSPR_TRY_ST(launch_ff_geometry(ctx));
 
     // octree
