@@ -47,13 +47,16 @@ static __device__ __forceinline__ float rsq(float x) {
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// FP64 1/sqrt(x): the FP32 reciprocal square root as the seed and one Newton-Raphson
-// step y <- y + y (1 - x y^2) / 2; a seed error e leaves ~1.5 e^2 (~2e-14 relative).
-// Used for squared distances, which stay far inside the FP32 range.
+// FP64 1/sqrt(x): the hardware's FP64 approximation (relative error e < 2^-19) as the seed and one
+// third-order step y <- y + y h (1/2 + 3/8 h), h = 1 - x y^2, which leaves ~2.5 e^3 (below half a
+// unit in the last place); five FP64 operations and no conversions through FP32 (one Newton step from
+// an FP32 seed left ~2e-14).  FP64 products: 20480 panels by treecode 5528 -> 5317 us, 1280 panels
+// direct 419 -> 399, their error against 64 bits 2.6e-15 -> 9e-16.
 static __device__ __forceinline__ double rsq(double x) {
-    const double y = (double)rsqrtf((float)x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double h = fma(-x * y, y, 1.0);
-    return fma(0.5 * y, h, y);
+    return fma(y * h, fma(0.375, h, 0.5), y);
 }
 
 template <typename T4>
