@@ -106,6 +106,34 @@ __global__ void item_flags_kernel(int4 *items, int64_t nitems, const int *__rest
     if (lane == 0) items[it].w = hit;
 }
 
+// first and last target block that a chunk of sources belongs to (one warp per chunk)
+__global__ void chunk_range_kernel(int64_t nch, int64_t chunk, int64_t Ns, const int *__restrict__ src_tblock,
+                                   int2 *range) {
+    const int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (c >= nch) return;
+    int lo = 0x7fffffff, hi = -1;
+    for (int64_t s = c * chunk + lane; s < min(Ns, (c + 1) * chunk); s += 32) {
+        lo = min(lo, src_tblock[s]);
+        hi = max(hi, src_tblock[s]);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) range[c] = make_int2(lo, hi);
+}
+
+// direct-mode items i = (target block i mod ntb, source chunk i / ntb), consecutive warps sharing a
+// chunk; item.w = 1 where the chunk may hold sources of the block's own panels (the flag only turns
+// the own-panel test on)
+__global__ void direct_items_kernel(int4 *items, int64_t ntb, int64_t nch, int64_t chunk, int64_t Ns,
+                                    const int2 *__restrict__ range) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= ntb * nch) return;
+    const int64_t c = i / ntb, tb = i - c * ntb;
+    const int2 r = range[c];
+    items[i] = make_int4((int)tb, (int)(c * chunk), (int)min(Ns, (c + 1) * chunk), tb >= r.x && tb <= r.y);
+}
+
 // FP64 -> float-float copies (moments accumulated in FP64, geometry)
 __global__ void to_ff_kernel(int64_t n, const dbl4 *__restrict__ a, ff4 *__restrict__ b, int id_in_w) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -216,6 +244,22 @@ int launch_item_flags(lspr_ctx *ctx, int4 *items, int64_t nitems) {
     if (nitems == 0) return LSPR_OK;
     ++ctx->n_launches;
     item_flags_kernel<<<grid_for(nitems * 32, 256), 256, 0, ctx->stream>>>(items, nitems, ctx->wo.src_tblock.p);
+    LSPR_TRY(ctx, cudaGetLastError());
+    return LSPR_OK;
+}
+
+int launch_direct_flags(lspr_ctx *ctx) {
+    const int64_t ntb = (ctx->mesh.N + kTargetBlock - 1) / kTargetBlock, Ns = ctx->mesh.Ns;
+    for (DirectItems *d : {&ctx->direct, &ctx->direct_multi}) {
+        if (d->n == 0) continue;
+        const int64_t nch = d->n / ntb;
+        LSPR_TRY(ctx, d->range.ensure(nch));
+        ctx->n_launches += 2;
+        chunk_range_kernel<<<grid_for(nch * 32, 128), 128, 0, ctx->stream>>>(nch, d->chunk, Ns, ctx->wo.src_tblock.p,
+                                                                             d->range.p);
+        direct_items_kernel<<<grid_for(d->n, 256), 256, 0, ctx->stream>>>(d->items.p, ntb, nch, d->chunk, Ns,
+                                                                          d->range.p);
+    }
     LSPR_TRY(ctx, cudaGetLastError());
     return LSPR_OK;
 }

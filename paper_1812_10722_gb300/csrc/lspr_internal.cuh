@@ -148,6 +148,7 @@ struct Tree {
     // boxes
     DArr<int> box_beg, box_end, box_child, box_nchild, box_level, box_used;
     DArr<unsigned> box_key;
+    DArr<int4> box_node;     // (first child, children, source begin, source end)
     DArr<dbl4> box_c64;   // centre (x,y,z), radius r_b
     DArr<float4> box_c32;
     // lists
@@ -176,6 +177,7 @@ struct Tree {
 
 struct DirectItems {
     int64_t n = 0, chunk = 0;   // items, sources per item
+    DArr<int2> range;           // per source chunk: first and last target block of its sources' panels
     DArr<int4> items;
 };
 
@@ -368,12 +370,16 @@ inline cudaError_t allow_smem(K kernel, int bytes, int device, int *set) {
 }
 
 int tree_build(lspr_ctx *ctx, double theta, int P, int Ncrit);
+// out = (lo[3], hi[3]) of the points a and b; part: 6 kBoxBlocks doubles of scratch
+constexpr int kBoxBlocks = 128;
+int launch_bbox(lspr_ctx *ctx, const dbl4 *a, int64_t na, const dbl4 *b, int64_t nb, double *part, double *out);
 int tree_tc_lists(lspr_ctx *ctx, bool p2p);
 int selftest_wait_timeout(lspr_ctx *ctx, int32_t *result);
 // stable LSD radix sort of (keys, vals) on the context's stream (bits: key width)
+// total: 256 ints
 int radix_sort(lspr_ctx *ctx, unsigned *keys, int *vals, unsigned *ktmp, int *vals_tmp, int64_t n, int bits, int *hist,
-               int *offs);
-int64_t radix_sort_scratch_ints(int64_t n);   // ints needed by each of hist and offs
+               int *total);
+int64_t radix_sort_scratch_ints(int64_t n);   // ints needed by hist
 // 10-bit coordinate -> every third bit (Morton interleave helper)
 __device__ __forceinline__ unsigned spread10(unsigned v) {
     v &= 0x3ffu;
@@ -394,8 +400,10 @@ int launch_m2p(lspr_ctx *ctx, int prec, double *acc, int *counter, int B);
 // float-float copies of the work-order geometry / box centres
 int launch_ff_geometry(lspr_ctx *ctx);
 int launch_ff_boxes(lspr_ctx *ctx);
-// item.w = 1 where a P2P item may contain sources of its own target block's panels
+// item.w = 1 where a P2P item may contain sources of its own target block's panels: exactly, or for
+// the direct-mode lists from the range of target blocks that each chunk of sources belongs to
 int launch_item_flags(lspr_ctx *ctx, int4 *items, int64_t nitems);
+int launch_direct_flags(lspr_ctx *ctx);
 // xt: x transposed to [2N][B] (B > 1), or null
 // S > 1 surfaces: B x S channel sets, weights of set (b, t) masked to the sources of surface t
 // x [B][2N]; xt: its transposed FP64 copy [2N][B] or null; xtf: its transposed FP32 copy

@@ -7,6 +7,7 @@
 #include <cmath>
 
 #include "lspr_internal.cuh"
+#include "rsq.cuh"
 
 namespace lspr {
 
@@ -160,13 +161,22 @@ __device__ __forceinline__ void atomic_max_pos(double *addr, double v) {
     atomicMax((unsigned long long *)addr, (unsigned long long)__double_as_longlong(v));
 }
 
+// the warp's largest v (every lane of the block takes part)
+__device__ __forceinline__ void warp_max_pos(double *addr, double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if ((threadIdx.x & 31) == 0) atomic_max_pos(addr, v);
+}
+
 // Far-rule Gauss nodes in natural order s = K*i + g: position, w_g*A_i, normal, panel id.
 __global__ void sources_kernel(const double *__restrict__ verts, const int *__restrict__ tris, int64_t N, int K,
                                const double *area, const double *nx, const double *ny, const double *nz,
                                const double *cx, const double *cy, const double *cz, dbl4 *pos, dbl4 *nrm,
-                               dbl4 *tgt, double *rho_max, double *L_max, const double *L) {
+                               dbl4 *tgt, double *rho_max, double *L_max, const double *L, const int *bad) {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= N * K) return;
+    if (*bad & 1) return;   // a vertex index out of range (the panel kernel found it)
+    const bool live = s < N * K;
+    if (!live) s = N * K - 1;   // repeats the last node, which changes no maximum
     int64_t i = s / K;
     int g = (int)(s - i * K);
     double y[3];
@@ -174,15 +184,15 @@ __global__ void sources_kernel(const double *__restrict__ verts, const int *__re
     for (int d = 0; d < 3; ++d)
         y[d] = c_far_bary[3 * g] * verts[3 * (int64_t)t[0] + d] + c_far_bary[3 * g + 1] * verts[3 * (int64_t)t[1] + d] +
                c_far_bary[3 * g + 2] * verts[3 * (int64_t)t[2] + d];
-    pos[s] = make_dbl4(y[0], y[1], y[2], c_far_w[g] * area[i]);
-    nrm[s] = make_dbl4(nx[i], ny[i], nz[i], (double)i);
-    double dx = y[0] - cx[i], dy = y[1] - cy[i], dz = y[2] - cz[i];
-    atomic_max_pos(rho_max, sqrt(dx * dx + dy * dy + dz * dz));
-    if (g == 0) {
-        tgt[i] = make_dbl4(cx[i], cy[i], cz[i], (double)i);
-        atomic_max_pos(L_max, L[i]);
-        atomic_max_pos(L_max + 1, fmax(fabs(cx[i]), fmax(fabs(cy[i]), fabs(cz[i]))));
+    if (live) {
+        pos[s] = make_dbl4(y[0], y[1], y[2], c_far_w[g] * area[i]);
+        nrm[s] = make_dbl4(nx[i], ny[i], nz[i], (double)i);
+        if (g == 0) tgt[i] = make_dbl4(cx[i], cy[i], cz[i], (double)i);
     }
+    const double dx = y[0] - cx[i], dy = y[1] - cy[i], dz = y[2] - cz[i];
+    // one atomic per warp and maximum (one per node: 327 us at 327680 nodes, all on one address)
+    warp_max_pos(rho_max, sqrt(dx * dx + dy * dy + dz * dz));
+    warp_max_pos(L_max, L[i]);
 }
 
 // Semi-analytical singular integral: for x = centroid of panel i, the panel
@@ -191,9 +201,9 @@ __global__ void sources_kernel(const double *__restrict__ verts, const int *__re
 // h / cos(phi)); the angle from phi_a to phi_b is integrated by N_k-point
 // Gauss-Legendre, i.e. N_k nodes on each edge.
 __global__ void self_kernel(const double *__restrict__ verts, const int *__restrict__ tris, int64_t N, int Nk,
-                            const double *cx, const double *cy, const double *cz, double *Vself) {
+                            const double *cx, const double *cy, const double *cz, double *Vself, const int *bad) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= N) return;
+    if (i >= N || (*bad & 1)) return;
     const double x[3] = {cx[i], cy[i], cz[i]};
     double v[3][3];
     for (int k = 0; k < 3; ++k)
@@ -294,90 +304,139 @@ __device__ __forceinline__ bool near_decide(const float4 &fi, const float4 &fj, 
     return near_exact(xi, yi, zi, cx[j], cy[j], cz[j], L[j], thr);
 }
 
-// One warp per target: lane c < 27 searches neighbour cell c and tests its panels; the
-// row is laid out as the self entry, then the hits of cell 0, 1, ... in sorted order.
+// One warp per occupied cell: lane c < 27 searches neighbour cell c once for all the cell's targets;
+// the neighbours' panels, in cell order, are the candidates.  Each lane holds one candidate of a
+// chunk of 32 and tests it against the targets in turn, a ballot counts the hits.  A row is laid out
+// as the self entry, then the hits of cell 0, 1, ... in sorted order.  Bound by the searches'
+// latency: 140 us for both passes at 81920 panels, 317 with a warp (and its searches) per target.
+constexpr int kCellTargets = 64;   // targets of a cell taken together
+constexpr int kCellWarps = 4;
 template <bool FILL>
-__global__ void near_cells_kernel(int64_t N, const double *__restrict__ cx, const double *__restrict__ cy,
-                                  const double *__restrict__ cz, const double *__restrict__ L, double thr,
-                                  const double *grid, const unsigned *__restrict__ skeys, const int *__restrict__ sidx,
-                                  const float4 *__restrict__ cf, int64_t *count, const int64_t *ptr, int *col,
-                                  int *row) {
-    const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+__global__ void __launch_bounds__(kCellWarps * 32)
+    near_cells_kernel(int64_t N, const double *__restrict__ cx, const double *__restrict__ cy,
+                      const double *__restrict__ cz, const double *__restrict__ L, double thr, const double *grid,
+                      const unsigned *__restrict__ skeys, const int *__restrict__ sidx, const float4 *__restrict__ cf,
+                      int64_t *count, const int64_t *ptr, int *col, int *row) {
+    __shared__ int hits[kCellWarps][kCellTargets];
+    const int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (i >= N) return;
-    const double xi = cx[i], yi = cy[i], zi = cz[i];
-    const float4 fi = cf[i];
+    int *hit = hits[threadIdx.x >> 5];
+    if (k >= N) return;
+    const unsigned mykey = skeys[k];
+    if (k > 0 && skeys[k - 1] == mykey) return;   // not the first panel of its cell
     const float cmax = (float)grid[4];
-    const int ix = cell_coord(xi, grid[0], grid[3]), iy = cell_coord(yi, grid[1], grid[3]),
-              iz = cell_coord(zi, grid[2], grid[3]);
-    int k0 = 0, k1 = 0;
+    const int i0 = sidx[k];
+    const int ix = cell_coord(cx[i0], grid[0], grid[3]), iy = cell_coord(cy[i0], grid[1], grid[3]),
+              iz = cell_coord(cz[i0], grid[2], grid[3]);
+    int k0 = 0, len = 0;
     if (lane < 27) {
         const int qx = ix + lane % 3 - 1, qy = iy + (lane / 3) % 3 - 1, qz = iz + lane / 9 - 1;
         if (qx >= 0 && qy >= 0 && qz >= 0 && qx <= 1023 && qy <= 1023 && qz <= 1023) {
             const unsigned key = cell_key(qx, qy, qz);
             k0 = lower_bound_u(skeys, (int)N, key);
-            k1 = k0;
-            while (k1 < N && skeys[k1] == key) ++k1;
+            if (k0 < N && skeys[k0] == key) len = lower_bound_u(skeys, (int)N, key + 1) - k0;
         }
     }
-    int c = 0;
-    for (int k = k0; k < k1; ++k) {
-        const int j = sidx[k];
-        if (j == i) continue;
-        const float4 fj = cf[j];
-        c += near_decide(fi, fj, 1e-6f * fj.w + 5e-7f * cmax, xi, yi, zi, j, cx, cy, cz, L, thr);
-    }
-    // inclusive warp scan of the per-lane hit counts
-    int inc = c;
+    int pre = len;   // inclusive scan: candidates up to and including this lane's cell
     for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += v;
+        const int v = __shfl_up_sync(0xffffffffu, pre, o);
+        if (lane >= o) pre += v;
     }
-    const int total = __shfl_sync(0xffffffffu, inc, 31);
-    if (!FILL) {
-        if (lane == 0) count[i] = total + 1;
-        return;
-    }
-    int64_t out = ptr[i];
-    if (lane == 0) {
-        col[out] = (int)i;   // self entry first
-        row[out] = (int)i;
-    }
-    out += 1 + (inc - c);
-    for (int k = k0; k < k1; ++k) {
-        const int j = sidx[k];
-        if (j == i) continue;
-        const float4 fj = cf[j];
-        if (near_decide(fi, fj, 1e-6f * fj.w + 5e-7f * cmax, xi, yi, zi, j, cx, cy, cz, L, thr)) {
-            col[out] = j;
-            row[out] = (int)i;
-            ++out;
+    const int total = __shfl_sync(0xffffffffu, pre, 31);
+    const int mine = __shfl_sync(0xffffffffu, len, 13);   // the cell itself (offsets 0, 0, 0)
+    for (int t0 = 0; t0 < mine; t0 += kCellTargets) {
+        const int nt = min(kCellTargets, mine - t0);
+        for (int t = lane; t < nt; t += 32) hit[t] = 0;
+        __syncwarp();
+        for (int c0 = 0; c0 < total; c0 += 32) {
+            const int c = c0 + lane;
+            // the cell that holds candidate c: the first lane whose inclusive count exceeds it
+            int lo = 0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const int v = __shfl_sync(0xffffffffu, pre, lo + o - 1);
+                if (v <= c) lo += o;
+            }
+            lo = min(lo, 31);
+            const int cb = __shfl_sync(0xffffffffu, k0, lo), cp = __shfl_sync(0xffffffffu, pre - len, lo);
+            int j = -1;
+            float4 fj = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (c < total) {
+                j = sidx[cb + (c - cp)];
+                fj = cf[j];
+            }
+            for (int t = 0; t < nt; ++t) {
+                const int i = sidx[k + t0 + t];
+                bool near = false;
+                if (j >= 0 && j != i)
+                    near = near_decide(cf[i], fj, 1e-6f * fj.w + 5e-7f * cmax, cx[i], cy[i], cz[i], j, cx, cy, cz, L,
+                                       thr);
+                const unsigned m = __ballot_sync(0xffffffffu, near);
+                const int run = hit[t];
+                if (FILL && near) {
+                    const int64_t out = ptr[i] + 1 + run + __popc(m & ((1u << lane) - 1u));
+                    col[out] = j;
+                    row[out] = i;
+                }
+                __syncwarp();
+                if (lane == 0) hit[t] = run + __popc(m);
+                __syncwarp();
+            }
         }
+        for (int t = lane; t < nt; t += 32) {
+            const int i = sidx[k + t0 + t];
+            if (FILL) {
+                col[ptr[i]] = i;   // self entry first
+                row[ptr[i]] = i;
+            } else {
+                count[i] = hit[t] + 1;
+            }
+        }
+        __syncwarp();
     }
 }
 
-// exclusive scan of n int64 counts into ptr[0..n], single block
-__global__ void scan_kernel(const int64_t *in, int64_t n, int64_t *out) {
-    __shared__ int64_t part[1024];
-    const int t = threadIdx.x;
-    const int64_t per = (n + blockDim.x - 1) / blockDim.x;
-    const int64_t b = t * per, e = min(n, b + per);
-    int64_t s = 0;
-    for (int64_t k = b; k < e; ++k) s += in[k];
-    part[t] = s;
-    __syncthreads();
-    for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-        int64_t v = t >= off ? part[t - off] : 0;
+// exclusive scan of n int64 counts into ptr[0..n], single block, four counts per thread and step
+__global__ void __launch_bounds__(1024) scan_kernel(const int64_t *__restrict__ in, int64_t n, int64_t *out) {
+    __shared__ int64_t sh[32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    int64_t run = 0;
+    for (int64_t base = 0; base < n; base += 4096) {
+        const int64_t i = base + 4 * t;
+        int64_t v[4], s = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            v[q] = i + q < n ? in[i + q] : 0;
+            s += v[q];
+        }
+        int64_t inc = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t w = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += w;
+        }
+        if (lane == 31) sh[warp] = inc;
         __syncthreads();
-        part[t] += v;
+        if (warp == 0) {
+            int64_t x = sh[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int64_t w = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += w;
+            }
+            sh[lane] = x;
+        }
+        __syncthreads();
+        int64_t e = run + (warp ? sh[warp - 1] : 0) + inc - s;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (i + q < n) out[i + q] = e;
+            e += v[q];
+        }
+        run += sh[31];
         __syncthreads();
     }
-    int64_t run = part[t] - s;
-    for (int64_t k = b; k < e; ++k) {
-        out[k] = run;
-        run += in[k];
-    }
-    if (t == blockDim.x - 1) out[n] = part[t];
+    if (t == 0) out[n] = run;
 }
 
 // FP32 copies (dV, dK) of the near-field corrections, read by the FP32 products of several
@@ -390,6 +449,10 @@ __global__ void near_f32_kernel(int64_t nnz, const double *__restrict__ dV, cons
 
 // Per near pair: dV, dK = (K_fine rule - far rule) over panel j seen from c_i,
 // and for the self entry V_ii (the far-field kernels skip a panel's own nodes).
+// FP64-pipe bound (23 nodes per pair): the node's offset is taken from the panel's edges (d = w -
+// b_1 e_1 - b_2 e_2 with w = x - v_0), (x - y).n = w.n is the same at every node of a flat panel,
+// and 1/r is rsq (five operations), so a node takes 18 FP64 operations.  81920 panels (2.05 M
+// pairs): 1.63 ms, 2.36 with the nodes formed from the vertices and the library's rsqrt.
 __global__ void near_values_kernel(int64_t nnz, const int *row, const int *col, const double *__restrict__ verts,
                                    const int *__restrict__ tris, const double *cx, const double *cy, const double *cz,
                                    const double *nx, const double *ny, const double *nz, const double *area,
@@ -404,31 +467,30 @@ __global__ void near_values_kernel(int64_t nnz, const int *row, const int *col, 
     }
     const double x[3] = {cx[i], cy[i], cz[i]};
     const double n[3] = {nx[j], ny[j], nz[j]};
-    double v[3][3];
-    for (int k = 0; k < 3; ++k)
-        for (int d = 0; d < 3; ++d) v[k][d] = verts[3 * (int64_t)tris[3 * (int64_t)j + k] + d];
+    double w[3], e1[3], e2[3];
+    const int *t = tris + 3 * (int64_t)j;
+    for (int q = 0; q < 3; ++q) {
+        const double v0 = verts[3 * (int64_t)t[0] + q];
+        w[q] = x[q] - v0;
+        e1[q] = verts[3 * (int64_t)t[1] + q] - v0;
+        e2[q] = verts[3 * (int64_t)t[2] + q] - v0;
+    }
+    const double dn = w[0] * n[0] + w[1] * n[1] + w[2] * n[2];
+    auto node = [&](double b1, double b2, double wt, double &sv, double &sk) {
+        const double d0 = fma(-b2, e2[0], fma(-b1, e1[0], w[0]));
+        const double d1 = fma(-b2, e2[1], fma(-b1, e1[1], w[1]));
+        const double d2 = fma(-b2, e2[2], fma(-b1, e1[2], w[2]));
+        const double r = rsq(d0 * d0 + d1 * d1 + d2 * d2);
+        const double wr = wt * r;
+        sv += wr;
+        sk = fma(wr, r * r, sk);
+    };
     double fv = 0, fk = 0, cv = 0, ck = 0;
-    for (int g = 0; g < Kf; ++g) {
-        double d[3];
-        for (int q = 0; q < 3; ++q)
-            d[q] = x[q] - (c_fine_bary[3 * g] * v[0][q] + c_fine_bary[3 * g + 1] * v[1][q] + c_fine_bary[3 * g + 2] * v[2][q]);
-        double ri = rsqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-        double dn = d[0] * n[0] + d[1] * n[1] + d[2] * n[2];
-        fv += c_fine_w[g] * ri;
-        fk += c_fine_w[g] * dn * ri * ri * ri;
-    }
-    for (int g = 0; g < K; ++g) {
-        double d[3];
-        for (int q = 0; q < 3; ++q)
-            d[q] = x[q] - (c_far_bary[3 * g] * v[0][q] + c_far_bary[3 * g + 1] * v[1][q] + c_far_bary[3 * g + 2] * v[2][q]);
-        double ri = rsqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-        double dn = d[0] * n[0] + d[1] * n[1] + d[2] * n[2];
-        cv += c_far_w[g] * ri;
-        ck += c_far_w[g] * dn * ri * ri * ri;
-    }
+    for (int g = 0; g < Kf; ++g) node(c_fine_bary[3 * g + 1], c_fine_bary[3 * g + 2], c_fine_w[g], fv, fk);
+    for (int g = 0; g < K; ++g) node(c_far_bary[3 * g + 1], c_far_bary[3 * g + 2], c_far_w[g], cv, ck);
     const double A = area[j] * kInv4Pi;
     dV[e] = (fv - cv) * A;
-    dK[e] = (fk - ck) * A;
+    dK[e] = (fk - ck) * dn * A;
 }
 
 __global__ void natural_order_kernel(int64_t N, int K, const dbl4 *pos, const dbl4 *nrm, const dbl4 *tgt,
@@ -506,9 +568,9 @@ int mesh_build(lspr_ctx *ctx, const double *verts, int64_t nv, const int *tris, 
     LSPR_TRY(ctx, m.src_nrm64.ensure(m.Ns));
     LSPR_TRY(ctx, m.tgt64.ensure(N));
 
-    // scratch: [0] bad flag (int), [1] rho_max, [2] L_max, [3] largest |coordinate| of a centroid
+    // scratch: [0] bad flag (int), [1] rho_max, [2] L_max, [4..9] bounding box of the centroids
     Tmp<double> flags(ctx->scratch[0]);
-    LSPR_TRY(ctx, flags.ensure(4));
+    LSPR_TRY(ctx, flags.ensure(10 + 6 * kBoxBlocks));
     LSPR_TRY(ctx, cudaMemsetAsync(flags.p, 0, 4 * sizeof(double), st));
     m.S = nsurf;
     LSPR_TRY(ctx, m.surf.ensure(N));
@@ -527,11 +589,13 @@ int mesh_build(lspr_ctx *ctx, const double *verts, int64_t nv, const int *tris, 
     ++ctx->n_launches;
     sources_kernel<<<grid_for(m.Ns, 256), 256, 0, st>>>(m.verts.p, m.tris.p, N, m.K, m.area.p, m.nx.p, m.ny.p,
                                                         m.nz.p, m.cx.p, m.cy.p, m.cz.p, m.src_pos64.p,
-                                                        m.src_nrm64.p, m.tgt64.p, flags.p + 1, flags.p + 2, m.L.p);
+                                                        m.src_nrm64.p, m.tgt64.p, flags.p + 1, flags.p + 2, m.L.p,
+                                                        (const int *)flags.p);
     ++ctx->n_launches;
-    self_kernel<<<grid_for(N, 128), 128, 0, st>>>(m.verts.p, m.tris.p, N, m.Nk, m.cx.p, m.cy.p, m.cz.p, m.Vself.p);
-    LSPR_TRY(ctx, cudaGetLastError());
-    double hflags[4];
+    self_kernel<<<grid_for(N, 128), 128, 0, st>>>(m.verts.p, m.tris.p, N, m.Nk, m.cx.p, m.cy.p, m.cz.p, m.Vself.p,
+                                                (const int *)flags.p);
+    LSPR_TRY_ST(launch_bbox(ctx, m.tgt64.p, N, nullptr, 0, flags.p + 10, flags.p + 4));
+    double hflags[10];
     LSPR_TRY(ctx, cudaMemcpyAsync(hflags, flags.p, sizeof(hflags), cudaMemcpyDeviceToHost, st));
     LSPR_TRY(ctx, cudaStreamSynchronize(st));
     int bad;
@@ -547,18 +611,7 @@ int mesh_build(lspr_ctx *ctx, const double *verts, int64_t nv, const int *tris, 
     LSPR_TRY(ctx, m.near_ptr.ensure(N + 1));
     double hgrid[5];
     {
-        std::vector<double> hc(3 * N);
-        // bounding box of the centroids (host copy of three N-vectors, once per geometry)
-        LSPR_TRY(ctx, cudaMemcpyAsync(hc.data(), m.cx.p, sizeof(double) * N, cudaMemcpyDeviceToHost, st));
-        LSPR_TRY(ctx, cudaMemcpyAsync(hc.data() + N, m.cy.p, sizeof(double) * N, cudaMemcpyDeviceToHost, st));
-        LSPR_TRY(ctx, cudaMemcpyAsync(hc.data() + 2 * N, m.cz.p, sizeof(double) * N, cudaMemcpyDeviceToHost, st));
-        LSPR_TRY(ctx, cudaStreamSynchronize(st));
-        double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
-        for (int d = 0; d < 3; ++d)
-            for (int64_t i = 0; i < N; ++i) {
-                lo[d] = std::min(lo[d], hc[d * N + i]);
-                hi[d] = std::max(hi[d], hc[d * N + i]);
-            }
+        const double *lo = hflags + 4, *hi = hflags + 7;
         const double ext = std::max(hi[0] - lo[0], std::max(hi[1] - lo[1], hi[2] - lo[2]));
         const double h = std::max(m.Lmax / m.thr * (1.0 + 1e-9), ext / 1023.0) * (1.0 + 1e-12) + 1e-300;
         hgrid[0] = lo[0];
@@ -580,7 +633,7 @@ int mesh_build(lspr_ctx *ctx, const double *verts, int64_t nv, const int *tris, 
     LSPR_TRY(ctx, vals.ensure(N));
     LSPR_TRY(ctx, vtmp.ensure(N));
     LSPR_TRY(ctx, hist.ensure(radix_sort_scratch_ints(N)));
-    LSPR_TRY(ctx, offs.ensure(radix_sort_scratch_ints(N)));
+    LSPR_TRY(ctx, offs.ensure(256));
     LSPR_TRY(ctx, cudaMemcpyAsync(grid.p, hgrid, sizeof(hgrid), cudaMemcpyHostToDevice, st));
     ++ctx->n_launches;
     cell_key_kernel<<<grid_for(N, 256), 256, 0, st>>>(N, m.cx.p, m.cy.p, m.cz.p, m.L.p, m.thr, grid.p, keys.p,
@@ -617,14 +670,6 @@ int mesh_build(lspr_ctx *ctx, const double *verts, int64_t nv, const int *tris, 
     return workorder_natural(ctx);
 }
 
-// item i = (target block i mod ntb, source chunk i / ntb): consecutive warps share a chunk
-__global__ void direct_items_kernel(int4 *items, int64_t ntb, int64_t nch, int64_t chunk, int64_t Ns) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= ntb * nch) return;
-    const int64_t c = i / ntb, tb = i - c * ntb;
-    items[i] = make_int4((int)tb, (int)(c * chunk), (int)min(Ns, (c + 1) * chunk), 0);
-}
-
 // Direct-mode work items: every target block against source chunks.  An item is one warp's work, so
 // a small mesh is cut finer, up to the point where adding an item's sums (4 FP64 atomics per target
 // and right-hand side) costs more than the warps in flight gain: at least 12288 items of 32 to 512
@@ -639,12 +684,9 @@ static int direct_lists(lspr_ctx *ctx, DirectItems &d, int64_t target, int64_t l
         return LSPR_OK;
     }
     d.chunk = chunk;
-    const int64_t nch = (m.Ns + chunk - 1) / chunk;
-    d.n = ntb * nch;
+    d.n = ntb * ((m.Ns + chunk - 1) / chunk);
     LSPR_TRY(ctx, d.items.ensure(d.n));
-    ++ctx->n_launches;
-    direct_items_kernel<<<grid_for(d.n, 256), 256, 0, ctx->stream>>>(d.items.p, ntb, nch, chunk, m.Ns);
-    return launch_item_flags(ctx, d.items.p, d.n);
+    return LSPR_OK;
 }
 
 int workorder_natural(lspr_ctx *ctx) {
@@ -669,6 +711,7 @@ int workorder_natural(lspr_ctx *ctx) {
     LSPR_TRY(ctx, cudaGetLastError());
     LSPR_TRY_ST(direct_lists(ctx, ctx->direct, 12288, 32));
     LSPR_TRY_ST(direct_lists(ctx, ctx->direct_multi, 3072, 64));
+    LSPR_TRY_ST(launch_direct_flags(ctx));
     LSPR_TRY_ST(launch_ff_geometry(ctx));
     LSPR_TRY(ctx, cudaStreamSynchronize(ctx->stream));
     return LSPR_OK;
