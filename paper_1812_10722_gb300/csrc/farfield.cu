@@ -35,9 +35,9 @@ namespace lspr {
 // (identity without a map; only the first *nact slots are formed when nact is given);
 // x is [B][2N] complex
 template <typename T4>
-// Several surfaces (S > 1): channel set slot = b * S + t carries the weights of the sources
-// of surface t only (zero elsewhere), so that each surface's layer potentials come out
-// separately; BS = B * S sets per source.
+// Several surfaces (S > 1): channel set slot = t K + k (surface t of the k-th of K running systems)
+// carries the weights of the sources of surface t only (zero elsewhere), so that each surface's
+// layer potentials come out separately; BS = B * S sets per source.
 __global__ void weights_kernel(int64_t Ns, int64_t N, int B, int S, const dbl4 *__restrict__ spos64,
                                const int *__restrict__ src_panel, const int *__restrict__ surf,
                                const double2 *__restrict__ x, const double2 *__restrict__ xt, T4 *__restrict__ w,
@@ -49,11 +49,10 @@ __global__ void weights_kernel(int64_t Ns, int64_t N, int B, int S, const dbl4 *
     const int slot = (int)(g - s * BS);
     if (nact && slot >= *nact) return;
     const int p = src_panel[s];
-    // set slot = k S + t: surface t of the k-th running system (map: k -> system)
-    const int k = slot / S, t = slot - k * S;
+    // set slot = t K + k: surface t of the k-th running system (map: k -> system)
+    const int K = nact ? *nact / S : B, t = slot / K, k = slot - t * K;
     const int b = map ? map[k] : k;
-    const int bs = b * S + t;
-    if (S > 1 && surf[p] != bs - b * S) {
+    if (S > 1 && surf[p] != t) {
         w[g] = zero4<T4>();
         return;
     }
@@ -83,7 +82,7 @@ __global__ void weights_f32t_kernel(int64_t Ns, int64_t N, int B, int S, const f
     const int slot = (int)(g - s * BS);
     if (nact && slot >= *nact) return;
     const int p = src_panel[s];
-    const int k = slot / S, t = slot - k * S;
+    const int K = nact ? *nact / S : B, t = slot / K, k = slot - t * K;
     const int b = map ? map[k] : k;
     if (S > 1 && surf[p] != t) {
         w[g] = zero4<float4>();
@@ -94,16 +93,21 @@ __global__ void weights_f32t_kernel(int64_t Ns, int64_t N, int B, int S, const f
     w[g] = make_float4(wa * dphi.x, wa * dphi.y, wa * phi.x, wa * phi.y);
 }
 
-// item.w = 1 iff some source of [item.y, item.z) belongs to a panel of the item's target block
-__global__ void item_flags_kernel(int4 *items, int64_t nitems, const int *__restrict__ src_tblock) {
+// item.w: bit 0 set iff some source of [item.y, item.z) belongs to a panel of the item's target block;
+// from bit kItemSurf the mask of the sources' surfaces (several surfaces)
+__global__ void item_flags_kernel(int4 *items, int64_t nitems, const int *__restrict__ src_tblock, int S,
+                                  const int *__restrict__ src_panel, const int *__restrict__ surf) {
     const int64_t it = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (it >= nitems) return;
     int4 item = items[it];
-    int hit = 0;
-    for (int s = item.y + lane; s < item.z; s += 32) hit |= src_tblock[s] == item.x;
-    hit = __any_sync(0xffffffffu, hit);
-    if (lane == 0) items[it].w = hit;
+    unsigned w = S > 1 ? 0u : 1u << kItemSurf;
+    for (int s = item.y + lane; s < item.z; s += 32) {
+        w |= src_tblock[s] == item.x;
+        if (S > 1) w |= 1u << (kItemSurf + surf[src_panel[s]]);
+    }
+    w = __reduce_or_sync(0xffffffffu, w);
+    if (lane == 0) items[it].w = (int)w;
 }
 
 // first and last target block that a chunk of sources belongs to (one warp per chunk)
@@ -131,7 +135,8 @@ __global__ void direct_items_kernel(int4 *items, int64_t ntb, int64_t nch, int64
     if (i >= ntb * nch) return;
     const int64_t c = i / ntb, tb = i - c * ntb;
     const int2 r = range[c];
-    items[i] = make_int4((int)tb, (int)(c * chunk), (int)min(Ns, (c + 1) * chunk), tb >= r.x && tb <= r.y);
+    items[i] = make_int4((int)tb, (int)(c * chunk), (int)min(Ns, (c + 1) * chunk),
+                          (tb >= r.x && tb <= r.y) | kAllSurf << kItemSurf);
 }
 
 // FP64 -> float-float copies (moments accumulated in FP64, geometry)
@@ -243,7 +248,8 @@ int launch_p2p(lspr_ctx *ctx, int prec, const int4 *items, int64_t nitems, doubl
 int launch_item_flags(lspr_ctx *ctx, int4 *items, int64_t nitems) {
     if (nitems == 0) return LSPR_OK;
     ++ctx->n_launches;
-    item_flags_kernel<<<grid_for(nitems * 32, 256), 256, 0, ctx->stream>>>(items, nitems, ctx->wo.src_tblock.p);
+    item_flags_kernel<<<grid_for(nitems * 32, 256), 256, 0, ctx->stream>>>(items, nitems, ctx->wo.src_tblock.p, ctx->mesh.S,
+                                                                          ctx->wo.src_panel.p, ctx->mesh.surf.p);
     LSPR_TRY(ctx, cudaGetLastError());
     return LSPR_OK;
 }
@@ -327,7 +333,7 @@ int launch_p2p_fp32_raw(cudaStream_t st, const int4 *items, int64_t nitems, cons
                         const float4 *spos, const float4 *snrm, const float4 *w, double *acc) {
     if (nitems == 0) return LSPR_OK;
     p2p_kernel<float, 1, false><<<grid_for(nitems, p2p_warps(1)), p2p_warps(1) * 32, 0, st>>>(
-        items, nitems, 1, 1, tgt, ntgt, spos, snrm, w, acc, nullptr, nullptr, 1 << 30);
+        items, nitems, 1, 1, tgt, ntgt, spos, snrm, w, acc, nullptr, nullptr, 1 << 30, 1);
     return cudaGetLastError() == cudaSuccess ? LSPR_OK : LSPR_E_CUDA;
 }
 

@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(p2p_warps(NB) * 32)
                const typename Vec4<T>::type *__restrict__ tgt, int64_t ntgt,
                const typename Vec4<T>::type *__restrict__ spos, const typename Vec4<T>::type *__restrict__ snrm,
                const typename Vec4<T>::type *__restrict__ sw, double *__restrict__ acc, int *counter,
-               const int *nact, int skip_from) {
+               const int *nact, int skip_from, int S) {
     using T4 = typename Vec4<T>::type;
     constexpr int W = p2p_warps(NB);
     __shared__ T4 sh[W][2][32];
@@ -178,6 +178,7 @@ __global__ void __launch_bounds__(p2p_warps(NB) * 32)
         const int64_t ii = it / nbc;
         const int b0 = (int)(it - ii * nbc) * NB, nb = min(NB, Bact - b0);
         const int4 item = __ldg(items + ii);
+        if (DYNAMIC && S > 1 && !((item.w >> kItemSurf) & set_surfaces(b0, nb, Bact, S))) continue;
         const int64_t t0 = (int64_t)item.x * kTargetBlock + lane, t1 = t0 + 32;
         const T4 q0 = t0 < ntgt ? tgt[t0] : tgt[0];
         const T4 q1 = t1 < ntgt ? tgt[t1] : tgt[0];
@@ -187,7 +188,7 @@ __global__ void __launch_bounds__(p2p_warps(NB) * 32)
         for (int k = 0; k < NB; ++k)
 #pragma unroll
             for (int c = 0; c < 4; ++c) a0[k][c] = a1[k][c] = T(0);
-        if (item.w)
+        if (item.w & 1)
             p2p_range<T, T4, NB, true>(item.y, item.z, lane, B, b0, nb, sh[warp], shw[warp], spos, snrm, sw, q0, q1,
                                        tp0, tp1, a0, a1);
         else
@@ -308,7 +309,7 @@ __global__ void __launch_bounds__(kP1Warps * 32)
         for (int u = 0; u < 2; ++u)
 #pragma unroll
             for (int c = 0; c < 2; ++c) av[u][c] = ak[u][c] = make_float2(0.f, 0.f);
-        if (item.w)
+        if (item.w & 1)
             p1_range<true>(item.y, item.z, lane, sh[warp], spos, snrm, sw, qx, qy, qz, tp, av, ak);
         else
             p1_range<false>(item.y, item.z, lane, sh[warp], spos, snrm, sw, qx, qy, qz, tp, av, ak);
@@ -625,7 +626,8 @@ __global__ void __launch_bounds__(kM2PGemmThreads)
     m2p_gemm_kernel(const int4 *__restrict__ items, int64_t nitems, int B,
                     const typename Vec4<T>::type *__restrict__ tgt, int64_t ntgt, const int *__restrict__ list,
                     const typename Vec4<T>::type *__restrict__ box_c, const typename Vec4<T>::type *__restrict__ mom,
-                    double *__restrict__ acc, int *counter, const int *nact) {
+                    double *__restrict__ acc, int *counter, const int *nact, const int *__restrict__ box_surf,
+                    int S) {
     using T4 = typename Vec4<T>::type;
     constexpr int NT = n_terms(P);
     constexpr int CH = 4 * NB;           // channels of a right-hand-side chunk
@@ -647,6 +649,7 @@ __global__ void __launch_bounds__(kM2PGemmThreads)
         if (it >= units) return;
         const int64_t ii = it / nbc;
         const int b0 = (int)(it - ii * nbc) * NB, nb = min(NB, Bact - b0);
+        const int um = set_surfaces(b0, nb, Bact, S);
         const int4 item = __ldg(items + ii);
         const int64_t tb = (int64_t)item.x * kTargetBlock;
         const int64_t ti = tb + tid;
@@ -659,6 +662,7 @@ __global__ void __launch_bounds__(kM2PGemmThreads)
 #pragma unroll 1
         for (int l = item.y; l < item.z; ++l) {
             const int b = __ldg(list + l);
+            if (S > 1 && !(box_surf[b] & um)) continue;
             const T4 bc = box_c[b];
             __syncthreads();   // phase 2 of the previous box is done with coef and ms
             for (int q2 = tid; q2 < NT * NB; q2 += kM2PGemmThreads) {
@@ -744,7 +748,8 @@ __global__ void __launch_bounds__(P2MShape<T, P, NB>::THREADS)
                const typename Vec4<T>::type *__restrict__ spos, const typename Vec4<T>::type *__restrict__ snrm,
                const typename Vec4<T>::type *__restrict__ sw, const typename Vec4<T>::type *__restrict__ box_c,
                const int *__restrict__ parent, const int *__restrict__ used,
-               typename MomAcc<T>::type *__restrict__ mom, const int *nact) {
+               typename MomAcc<T>::type *__restrict__ mom, const int *nact, const int *__restrict__ box_surf,
+               int NS) {
     using S = typename MomAcc<T>::scalar;
     using T4 = typename Vec4<T>::type;
     using Sh = P2MShape<T, P, NB>;
@@ -764,6 +769,7 @@ __global__ void __launch_bounds__(P2MShape<T, P, NB>::THREADS)
     if (b0 >= Bact) return;
     const int nb = min(NB, Bact - b0);
     const int4 item = items[ii];
+    if (NS > 1 && !(box_surf[item.x] & set_surfaces(b0, nb, Bact, NS))) return;
     const T4 c = box_c[item.x];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tg = tid % TG, rg = (tid / TG) % RG, sp = tid / (TG * RG);
@@ -971,7 +977,7 @@ static void p2p_launch(lspr_ctx *ctx, const int4 *items, int64_t nitems, int B, 
                                              persistent_grid(ctx, p2p_kernel<T, NB, true>, W * 32, &occ));
     p2p_kernel<T, NB, true><<<grid, W * 32, 0, st>>>(items, nitems, nbc, B, Views<T>::tgt(ctx), ctx->mesh.N,
                                                       Views<T>::spos(ctx), Views<T>::snrm(ctx), Views<T>::w(ctx),
-                                                      acc, counter, ctx->rhs_nact, skip_from);
+                                                      acc, counter, ctx->rhs_nact, skip_from, ctx->mesh.S);
 }
 
 // the packed single-right-hand-side P2P (FP32)
@@ -995,7 +1001,8 @@ static void p2m_launch_nb(lspr_ctx *ctx, int B) {
     if (Sh::SMEM > 47 * 1024) (void)allow_smem(p2m_kernel<T, P, NB>, (int)Sh::SMEM, ctx->device, smem_set);
     p2m_kernel<T, P, NB><<<(unsigned)(tr.n_p2m_items * nbc), Sh::THREADS, Sh::SMEM, ctx->stream>>>(
         tr.p2m_items.p, tr.n_p2m_items, nbc, B, Views<T>::spos(ctx), Views<T>::snrm(ctx), Views<T>::w(ctx),
-        Views<T>::bc(ctx), tr.box_parent.p, tr.box_used.p, Views<T>::mom_acc(ctx), ctx->rhs_nact);
+        Views<T>::bc(ctx), tr.box_parent.p, tr.box_used.p, Views<T>::mom_acc(ctx), ctx->rhs_nact,
+        tr.box_surf.p, ctx->mesh.S);
 }
 
 template <typename T, int P, int NB>
@@ -1031,7 +1038,7 @@ static void m2p_launch(lspr_ctx *ctx, double *acc, int *counter, int B) {
         const unsigned grid = (unsigned)std::min<int64_t>(tr.n_m2p_items * nbc, (int64_t)occ * std::max(1, ctx->num_sms));
         m2p_gemm_kernel<T, P, NB><<<grid, kM2PGemmThreads, smem, ctx->stream>>>(
             tr.m2p_items.p, tr.n_m2p_items, B, Views<T>::tgt(ctx), ctx->mesh.N, tr.m2p_list.p, Views<T>::bc(ctx),
-            Views<T>::mom(ctx), acc, counter, ctx->rhs_nact);
+            Views<T>::mom(ctx), acc, counter, ctx->rhs_nact, tr.box_surf.p, ctx->mesh.S);
         return;
     }
     constexpr int W = m2p_warps<T, P, NB>();

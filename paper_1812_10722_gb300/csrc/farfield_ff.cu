@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(64)
     m2p_ff_kernel(const int4 *__restrict__ items, int64_t nitems, int nbc, int B, int NT,
                   const ff4 *__restrict__ tgt, int64_t ntgt, const int *__restrict__ list,
                   const ff4 *__restrict__ box_c, const ff4 *__restrict__ mom, double *__restrict__ acc, int *counter,
-                  const int *nact, int W, int TP) {
+                  const int *nact, int W, int TP, const int *__restrict__ box_surf, int S) {
     extern __shared__ __align__(16) unsigned char ff_smem[];
     __shared__ int64_t unit;
     const int h = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -90,6 +90,7 @@ __global__ void __launch_bounds__(64)
         if (it >= units) return;
         const int64_t ii = it / nbc;
         const int b0 = (int)(it - ii * nbc) * NB, nb = min(NB, Bact - b0);
+        const int um = set_surfaces(b0, nb, Bact, S);
         const int4 item = __ldg(items + ii);
         const int64_t ti = (int64_t)item.x * kTargetBlock + lane + 32 * h;
         const ff4 q = ti < ntgt ? tgt[ti] : tgt[0];
@@ -101,6 +102,7 @@ __global__ void __launch_bounds__(64)
 #pragma unroll 1
         for (int l = item.y; l < item.z; ++l) {
             const int b = __ldg(list + l);
+            if (S > 1 && !(box_surf[b] & um)) continue;
             const ff4 c = box_c[b];
             // terms t0 .. t0 + TP - 1 of the box's moments into sm (the whole block, at the same t)
             auto stage = [&](int t0) {
@@ -217,7 +219,8 @@ int m2p_ff_launch(lspr_ctx *ctx, double *acc, int *counter, int B) {
         (unsigned)std::min<int64_t>(tr.n_m2p_items * nbc, (int64_t)occ * std::max(1, ctx->num_sms));
     m2p_ff_kernel<NB><<<grid, 64, smem, ctx->stream>>>(
         tr.m2p_items.p, tr.n_m2p_items, nbc, B, NT, Views<ffloat>::tgt(ctx), ctx->mesh.N, tr.m2p_list.p,
-        Views<ffloat>::bc(ctx), Views<ffloat>::mom(ctx), acc, counter, ctx->rhs_nact, W, tp_sel);
+        Views<ffloat>::bc(ctx), Views<ffloat>::mom(ctx), acc, counter, ctx->rhs_nact, W, tp_sel, tr.box_surf.p,
+        ctx->mesh.S);
     return LSPR_OK;
 }
 
@@ -231,7 +234,7 @@ template <int NB>
 __global__ void __launch_bounds__(kFfP2PWarps * 32)
     p2p_ff1_kernel(const int4 *__restrict__ items, int64_t nitems, int B, const ff4 *__restrict__ tgt, int64_t ntgt,
                    const ff4 *__restrict__ spos, const ff4 *__restrict__ snrm, const ff4 *__restrict__ sw,
-                   double *__restrict__ acc, int *counter, const int *nact) {
+                   double *__restrict__ acc, int *counter, const int *nact, int S) {
     __shared__ ff4 sh[kFfP2PWarps][2][32];
     __shared__ ff4 shw[kFfP2PWarps][32][NB];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -247,6 +250,7 @@ __global__ void __launch_bounds__(kFfP2PWarps * 32)
         const int rem = (int)(it - ii * 2 * nbc), h = rem / nbc;
         const int b0 = (rem - h * nbc) * NB, nb = min(NB, Bact - b0);
         const int4 item = __ldg(items + ii);
+        if (S > 1 && !((item.w >> kItemSurf) & set_surfaces(b0, nb, Bact, S))) continue;
         const int64_t t = (int64_t)item.x * kTargetBlock + 32 * h + lane;
         const ff4 q = t < ntgt ? tgt[t] : tgt[0];
         const int tp = panel_of(q.w);
@@ -270,7 +274,7 @@ __global__ void __launch_bounds__(kFfP2PWarps * 32)
                 const ff4 p = sh[warp][0][kk], n = sh[warp][1][kk];
                 const ffloat dx = q.x - p.x, dy = q.y - p.y, dz = q.z - p.z;
                 ffloat r = rsq(dx * dx + dy * dy + dz * dz);
-                if (item.w && panel_of(n.w) == tp) r = ffloat(0.f, 0.f);
+                if ((item.w & 1) && panel_of(n.w) == tp) r = ffloat(0.f, 0.f);
                 const ffloat tk = (dx * n.x + dy * n.y + dz * n.z) * (r * r) * r;
 #pragma unroll
                 for (int k = 0; k < NB; ++k) {
@@ -302,7 +306,7 @@ int p2p_ff1_launch(lspr_ctx *ctx, const int4 *items, int64_t nitems, int B, doub
                                              persistent_grid(ctx, p2p_ff1_kernel<NB>, kFfP2PWarps * 32, &occ));
     p2p_ff1_kernel<NB><<<grid, kFfP2PWarps * 32, 0, st>>>(items, nitems, B, Views<ffloat>::tgt(ctx), ctx->mesh.N,
                                                           Views<ffloat>::spos(ctx), Views<ffloat>::snrm(ctx),
-                                                          Views<ffloat>::w(ctx), acc, counter, ctx->rhs_nact);
+                                                          Views<ffloat>::w(ctx), acc, counter, ctx->rhs_nact, ctx->mesh.S);
     return LSPR_OK;
 }
 

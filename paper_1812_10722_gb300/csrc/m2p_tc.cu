@@ -93,7 +93,8 @@ __device__ __forceinline__ int core_off(int r, int k) {
 // or beyond the active count and terms beyond NT are zero.  One thread per 16 bytes of A_hi.
 template <int P, int RC>
 __global__ void tc_image_kernel(int64_t nbox, int B, int nrc, const float4 *__restrict__ mom,
-                                unsigned char *__restrict__ img, const int *nact) {
+                                unsigned char *__restrict__ img, const int *nact,
+                                const int *__restrict__ box_surf, int NS) {
     using S = TcShape<P, RC>;
     constexpr int per_chunk = S::A_CH / 16;
     const int Bact = nact ? *nact : B;
@@ -105,6 +106,8 @@ __global__ void tc_image_kernel(int64_t nbox, int B, int nrc, const float4 *__re
         const int64_t brc = c / S::NKC;
         const int rc = (int)(brc % nrc);
         const int64_t box = brc / nrc;
+        if (rc * RC >= Bact) continue;   // no right-hand side in use, or none of the box's surfaces: not read
+        if (NS > 1 && !(box_surf[box] & set_surfaces(rc * RC, min(RC, Bact - rc * RC), Bact, NS))) continue;
         // e enumerates the part's 16-byte segments in address order
         const int r = ((e >> 3) / (kKC / 4)) * 8 + (e & 7), k4 = (e >> 3) % (kKC / 4);
         const int j = rc * RC + (r >> 2), cpt = r & 3;
@@ -128,7 +131,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     m2p_tc_kernel(const int4 *__restrict__ items, int64_t nitems, int B, int nrc, const float4 *__restrict__ tgt,
                   int64_t ntgt, const int2 *__restrict__ list, const float4 *__restrict__ box_c,
                   const unsigned char *__restrict__ img, double *__restrict__ acc, int *counter, int *error,
-                  const int *nact) {
+                  const int *nact, int nsurf) {
     using S = TcShape<P, RC>;
     constexpr int NT = S::NT, NKC = S::NKC, NS = S::NS;
     extern __shared__ __align__(128) unsigned char tc_smem[];
@@ -177,6 +180,17 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const int Bact = nact ? *nact : B;   // right-hand sides in use (the first Bact slots)
     const int nbc = (Bact + RC - 1) / RC;
     const int64_t units = nitems * nbc;
+    // the A parts (bit h) of unit chunk rc that take list entry e: those with right-hand sides in use
+    // whose surfaces the box holds (entry.y: block mask, surface mask from bit 8); 0: the box is skipped
+    auto parts = [&](int rc, const int2 &e) -> int {
+        int m = 0;
+#pragma unroll
+        for (int h = 0; h < S::HALVES; ++h) {
+            const int b = rc * RC + h * S::HRC, n = min(S::HRC, Bact - b);
+            if (n > 0 && ((e.y >> kTcSurf) & set_surfaces(b, n, Bact, nsurf))) m |= 1 << h;
+        }
+        return m;
+    };
 
     if (warp == kProdWarp) {
         // ---- producer: work units and the A part of every stage
@@ -195,12 +209,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 const int rc = (int)(u - ii * nbc);
                 const int4 item = __ldg(items + ii);
                 bool ok = true;
-                int b_nx = item.y < item.z ? __ldg(&list[item.y].x) : 0;   // one box ahead
-                // A parts present: the halves of the unit holding right-hand sides in use
-                const int nh = min(S::HALVES, (Bact - rc * RC + S::HRC - 1) / S::HRC);
+                int2 e_nx = item.y < item.z ? __ldg(list + item.y) : make_int2(0, 0);   // one box ahead
                 for (int l = item.y; l < item.z && ok; ++l) {
-                    const unsigned char *src = img + ((int64_t)b_nx * nrc + rc * S::HALVES) * NKC * (2 * S::A_CH);
-                    if (l + 1 < item.z) b_nx = __ldg(&list[l + 1].x);
+                    const unsigned char *src = img + ((int64_t)e_nx.x * nrc + rc * S::HALVES) * NKC * (2 * S::A_CH);
+                    const int pm = parts(rc, e_nx);
+                    if (l + 1 < item.z) e_nx = __ldg(list + l + 1);
+                    if (!pm) continue;
                     for (int kc = 0; kc < NKC; ++kc, ++seq) {
                         const int s = (int)(seq % NS);
                         if (seq >= NS &&
@@ -210,10 +224,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         }
                         const uint32_t fb = smem_addr(&full_a[s]);
                         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb),
-                                     "r"((uint32_t)(nh * 2 * S::A_CH))
+                                     "r"((uint32_t)(__popc(pm) * 2 * S::A_CH))
                                      : "memory");
-                        for (int h = 0; h < nh; ++h)
-                            asm volatile(
+                        for (int h = 0; h < S::HALVES; ++h)
+                            if (pm >> h & 1) asm volatile(
                                 "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                                     sbase + (uint32_t)(s * S::STAGE + h * 2 * S::A_CH)),
                                 "l"(src + ((int64_t)h * NKC + kc) * 2 * S::A_CH), "r"(2 * S::A_CH), "r"(fb)
@@ -237,17 +251,26 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 const int64_t u = ring[slot];
                 if (u >= units) break;
                 const int4 item = __ldg(items + u / nbc);
-                if (item.y < item.z) {
+                {
                     const int ab = S::HALVES == 2 ? 0 : (nu & 1);
                     const bool wait = S::HALVES == 2 ? nu >= 1 : nu >= 2;
                     const uint32_t wpar = (uint32_t)(S::HALVES == 2 ? (nu - 1) : ((nu >> 1) - 1)) & 1u;
-                    if (wait && !bar_wait(smem_addr(&acc_empty[ab]), wpar, &abort_s)) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;");
                     const uint32_t d = tmem + (uint32_t)(ab * kTcN);
                     const int rc = (int)(u % nbc);
-                    const int nh = min(S::HALVES, (Bact - rc * RC + S::HRC - 1) / S::HRC);
                     bool ok = true;
+                    int begun = 0;   // A parts with an MMA so far
+                    int2 e_nx = item.y < item.z ? __ldg(list + item.y) : make_int2(0, 0);
                     for (int l = item.y; l < item.z && ok; ++l) {
+                        const int pm = parts(rc, e_nx);
+                        if (l + 1 < item.z) e_nx = __ldg(list + l + 1);
+                        if (!pm) continue;
+                        if (!begun) {   // the unit's accumulators are free
+                            if (wait && !bar_wait(smem_addr(&acc_empty[ab]), wpar, &abort_s)) {
+                                ok = false;
+                                break;
+                            }
+                            asm volatile("tcgen05.fence::after_thread_sync;");
+                        }
                         for (int kc = 0; kc < NKC; ++kc, ++seq) {
                             const int s = (int)(seq % NS);
                             const uint32_t par = (uint32_t)(seq / NS) & 1u;
@@ -263,8 +286,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                                 const uint32_t off = ks * 256;   // two 16-byte column groups per K step of 8
                                 const uint64_t dbh = umma_desc(st + S::OFF_B + off, 128, kChunkSBO);
                                 const uint64_t dbl = umma_desc(st + S::OFF_B + S::B_CH + off, 128, kChunkSBO);
-                                const uint32_t on = (l == item.y && kc == 0 && ks == 0) ? 0u : 1u;
-                                for (int h = 0; h < nh; ++h) {   // half h into accumulator d + h kTcN
+                                for (int h = 0; h < S::HALVES; ++h) {   // half h into accumulator d + h kTcN
+                                    if (!(pm >> h & 1)) continue;
+                                    const uint32_t on = (uint32_t)(begun >> h & 1);
+                                    begun |= 1 << h;
                                     const uint32_t ah = st + (uint32_t)(h * 2 * S::A_CH);
                                     const uint64_t dah = umma_desc(ah + off, 128, kChunkSBO);
                                     const uint64_t dal = umma_desc(ah + S::A_CH + off, 128, kChunkSBO);
@@ -278,8 +303,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         }
                     }
                     if (!ok) break;
-                    tc_commit(smem_addr(&acc_full[ab]));
-                    ++nu;
+                    if (begun) {
+                        tc_commit(smem_addr(&acc_full[ab]));
+                        ++nu;
+                    }
                 }
                 bar_arrive(smem_addr(&ring_empty[slot]));
             }
@@ -295,7 +322,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         int nu = 0;
         // the unit whose accumulator is still to be drained
         bool pend = false;
-        int p_ab = 0, p_par = 0, p_b0 = 0, p_nb = 0;
+        int p_ab = 0, p_par = 0, p_b0 = 0, p_nb = 0, p_parts = 0;
         int64_t p_tbase = 0;
         // epilogue: warp w reads lane quarter w % 4 (accumulator rows 32 (w % 4)..) and columns
         // 128 (w / 4)..; channel = row mod ROWS (both halves of a stacked accumulator are
@@ -307,7 +334,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll 1
             for (int hh = 0; hh < S::HALVES; ++hh) {   // the unit's A parts (accumulators)
             const int hnb = p_nb - hh * S::HRC;          // right-hand sides of this half
-            if ((32 * qd) % S::ROWS < 4 * hnb) {
+            if ((p_parts >> hh & 1) && (32 * qd) % S::ROWS < 4 * hnb) {
                 const int m = (32 * qd + lane) % S::ROWS, j = m >> 2, cpt = m & 3;
                 const int jb = p_b0 + hh * S::HRC + j;   // the right-hand side of row m
 #pragma unroll 1
@@ -363,6 +390,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             // the next box's list entry and centre are loaded one box ahead
             int2 e_nx = item.y < item.z ? __ldg(list + item.y) : make_int2(0, 0);
             float4 c_nx = item.y < item.z ? box_c[e_nx.x] : make_float4(0.f, 0.f, 0.f, 0.f);
+            int begun = 0;   // A parts with a box so far
             for (int l = item.y; l < item.z && ok; ++l) {
                 const int2 e = e_nx;
                 const float4 c = c_nx;
@@ -370,6 +398,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     e_nx = __ldg(list + l + 1);
                     c_nx = box_c[e_nx.x];
                 }
+                const int pm = parts(b0 / RC, e);
+                if (!pm) continue;
+                begun |= pm;
                 const bool on = live && ((e.y >> blk) & 1);   // uniform over the warp but for the tail
                 float a[NT];
                 if (on) {
@@ -412,8 +443,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
             if (ok && pend) ok = drain_acc();       // the previous unit, if this one had no box
             if (!ok) break;
-            if (item.y < item.z) {
+            if (begun) {
                 pend = true;
+                p_parts = begun;
                 p_ab = S::HALVES == 2 ? 0 : (nu & 1);
                 p_par = (S::HALVES == 2 ? nu : (nu >> 1)) & 1;
                 p_tbase = tbase;
@@ -449,12 +481,13 @@ int tc_launch(lspr_ctx *ctx, double *acc, int *counter, int B) {
     const unsigned gi =
         (unsigned)std::max<int64_t>(1, std::min<int64_t>((segs + 255) / 256, 8 * std::max(1, ctx->num_sms)));
     tc_image_kernel<P, S::HRC><<<gi, 256, 0, ctx->stream>>>(tr.nboxes, B, nrc, Views<float>::mom(ctx),
-                                                              ctx->tc_img.p, ctx->rhs_nact);
+                                                              ctx->tc_img.p, ctx->rhs_nact, tr.box_surf.p,
+                                                              ctx->mesh.S);
     const unsigned grid =
         (unsigned)std::max<int64_t>(1, std::min<int64_t>(tr.n_tc_items * nunit, std::max(1, ctx->num_sms)));
     m2p_tc_kernel<P, RC><<<grid, kTcThreads, S::SMEM, ctx->stream>>>(
         tr.tc_items.p, tr.n_tc_items, B, nrc, Views<float>::tgt(ctx), ctx->mesh.N, tr.tc_list.p,
-        Views<float>::bc(ctx), ctx->tc_img.p, acc, counter, ctx->dev_err.p, ctx->rhs_nact);
+        Views<float>::bc(ctx), ctx->tc_img.p, acc, counter, ctx->dev_err.p, ctx->rhs_nact, ctx->mesh.S);
     return LSPR_OK;
 }
 

@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     p2p_tc_kernel(const int4 *__restrict__ items, int64_t nitems, const int4 *__restrict__ ivl, int B,
                   const float4 *__restrict__ tgt, int64_t ntgt, const float4 *__restrict__ spos,
                   const float4 *__restrict__ snrm, const float4 *__restrict__ sw, double *__restrict__ acc,
-                  int *counter, int *error, const int *nact, int min_rhs) {
+                  int *counter, int *error, const int *nact, int min_rhs, int nsurf) {
     // fewer right-hand sides in use than min_rhs: the FP32-pipe P2P takes this product
     if ((nact ? *nact : B) < min_rhs) return;
     extern __shared__ __align__(128) unsigned char tc_smem[];
@@ -149,8 +149,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 const int b0 = (int)(u - ii * nbc) * kRC, nb = min(kRC, Bact - b0);
                 const int4 item = __ldg(items + ii);
                 bool ok = true;
+                const int um = set_surfaces(b0, nb, Bact, nsurf);
                 for (int iv = item.y; iv < item.z && ok; ++iv) {
                     const int4 e = __ldg(ivl + iv);
+                    if (!(e.w & um)) continue;   // no source of the unit's surfaces (all roles agree)
                     for (int sb = e.x; sb < e.y; sb += kSrc, ++seq) {
                         const int s = (int)(seq % kStages);
                         if (seq >= kStages &&
@@ -199,17 +201,24 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 const int64_t u = ring[slot];
                 if (u >= units) break;
                 const int64_t ii = u / nbc;
-                const int nb = min(kRC, Bact - (int)(u - ii * nbc) * kRC);
+                const int b0 = (int)(u - ii * nbc) * kRC, nb = min(kRC, Bact - b0);
                 const bool stacked = nb <= kRC / 2;
+                const int um = set_surfaces(b0, nb, Bact, nsurf);
                 const int4 item = __ldg(items + ii);
-                if (item.y < item.z) {
-                    // the accumulators are free once the previous unit is drained
-                    if (nu >= 1 && !bar_wait(smem_addr(&acc_empty), (uint32_t)((nu - 1) & 1), &abort_s)) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;");
+                {
                     const uint32_t dv = tmem, dk = tmem + (uint32_t)kTcN;
                     bool ok = true, first = true;
                     for (int iv = item.y; iv < item.z && ok; ++iv) {
                         const int4 e = __ldg(ivl + iv);
+                        if (!(e.w & um)) continue;
+                        // the accumulators are free once the previous unit is drained
+                        if (first && nu >= 1) {
+                            if (!bar_wait(smem_addr(&acc_empty), (uint32_t)((nu - 1) & 1), &abort_s)) {
+                                ok = false;
+                                break;
+                            }
+                            asm volatile("tcgen05.fence::after_thread_sync;");
+                        }
                         for (int sb = e.x; sb < e.y; sb += kSrc, ++seq) {
                             const int s = (int)(seq % kStages);
                             if (!bar_wait(smem_addr(&full_s[s]), (uint32_t)(seq / kStages) & 1u, &abort_s)) {
@@ -240,8 +249,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         }
                     }
                     if (!ok) break;
-                    tc_commit(smem_addr(&acc_full));
-                    ++nu;
+                    if (!first) {
+                        tc_commit(smem_addr(&acc_full));
+                        ++nu;
+                    }
                 }
                 bar_arrive(smem_addr(&ring_empty[slot]));
             }
@@ -333,8 +344,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const bool wr = wt >= 0 && wt < 128 && (!stacked || wt < 64);
             const int wj = stacked ? (wt & 31) : (wt & 31) + 32 * (wt >> 6);
             const int wk = stacked ? 4 * (wt >> 5) : 4 * ((wt >> 5) & 1);
+            const int um = set_surfaces(b0, nb, Bact, nsurf);
+            bool begun = false;
             for (int iv = item.y; iv < item.z && ok; ++iv) {
                 const int4 e = __ldg(ivl + iv);
+                if (!(e.w & um)) continue;
+                begun = true;
                 const bool on = live && ((e.z >> blk) & 1);   // uniform over the warp but for the tail
                 for (int sb = e.x; sb < e.y && ok; sb += kSrc) {
                     // the stage's inputs have landed (and its operands are free: the producer
@@ -422,7 +437,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
             if (ok && pend) ok = drain_acc();     // the previous unit, if this one had no source
             if (!ok) break;
-            if (item.y < item.z) {
+            if (begun) {
                 pend = true;
                 p_tbase = tbase;
                 p_b0 = b0;
@@ -458,7 +473,7 @@ int p2p_tc_launch(lspr_ctx *ctx, double *acc, cudaStream_t st, int *counter, int
     p2p_tc_kernel<<<grid, kTcThreads, kSmem, st>>>(tr.tcp_items.p, tr.n_tcp_items, tr.tcp_ivl.p, B,
                                                   Views<float>::tgt(ctx), ctx->mesh.N, Views<float>::spos(ctx),
                                                   Views<float>::snrm(ctx), Views<float>::w(ctx), acc, counter,
-                                                  ctx->dev_err.p, ctx->rhs_nact, min_rhs);
+                                                  ctx->dev_err.p, ctx->rhs_nact, min_rhs, ctx->mesh.S);
     return LSPR_OK;
 }
 

@@ -475,6 +475,36 @@ __global__ void box_final_kernel(int nboxes, const int *ext, dbl4 *c64, float4 *
     c32[b] = make_float4(cen[0], cen[1], cen[2], (float)(rb * (1.0 + 1e-6)));
 }
 
+// mask of the surfaces of each box's sources (several surfaces), one block per slice
+__global__ void __launch_bounds__(kGeomThreads) box_surf_kernel(const int2 *__restrict__ slices, const int *beg,
+                                                                const int *end, const int *__restrict__ src_panel,
+                                                                const int *__restrict__ surf, int *box_surf) {
+    const int2 sl = slices[blockIdx.x];
+    const int s0 = beg[sl.x] + sl.y * kSliceSrc, s1 = min(end[sl.x], s0 + kSliceSrc);
+    unsigned m = 0;
+    for (int s = s0 + threadIdx.x; s < s1; s += kGeomThreads) m |= 1u << surf[src_panel[s]];
+    m = __reduce_or_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m) atomicOr(&box_surf[sl.x], (int)m);
+}
+
+// the surface masks of the tensor-core work lists: M2P entries from their boxes, one warp per P2P
+// source range
+__global__ void tc_list_surf_kernel(int64_t n, int2 *list, const int *__restrict__ box_surf) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < n) list[i].y |= (box_surf ? box_surf[list[i].x] : 1) << kTcSurf;
+}
+__global__ void tc_ivl_surf_kernel(int64_t n, int4 *ivl, int S, const int *__restrict__ src_panel,
+                                   const int *__restrict__ surf) {
+    const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (i >= n) return;
+    unsigned m = S > 1 ? 0u : 1u;
+    if (S > 1)
+        for (int s = ivl[i].x + lane; s < ivl[i].y; s += 32) m |= 1u << surf[src_panel[s]];
+    m = __reduce_or_sync(0xffffffffu, m);
+    if (lane == 0) ivl[i].w = (int)m;
+}
+
 // box node of the list walk: (first child or -1, children, source begin, source end)
 __global__ void box_nodes_kernel(int nboxes, const int *beg, const int *end, const int *child, const int *nchild,
                                  int4 *node) {
@@ -782,6 +812,13 @@ int tree_build(lspr_ctx *ctx, double theta, int P, int Ncrit) {
     box_final_kernel<<<grid_for(nboxes, 256), 256, 0, st>>>(nboxes, ext.p, tr.box_c64.p, tr.box_c32.p);
     box_nodes_kernel<<<grid_for(nboxes, 256), 256, 0, st>>>(nboxes, tr.box_beg.p, tr.box_end.p, tr.box_child.p,
                                                             tr.box_nchild.p, tr.box_node.p);
+    if (m.S > 1) {
+        LSPR_TRY(ctx, tr.box_surf.ensure(nboxes));
+        LSPR_TRY(ctx, cudaMemsetAsync(tr.box_surf.p, 0, sizeof(int) * nboxes, st));
+        ++ctx->n_launches;
+        box_surf_kernel<<<nbs[1], kGeomThreads, 0, st>>>(slices.p, tr.box_beg.p, tr.box_end.p, w.src_panel.p, m.surf.p,
+                                                         tr.box_surf.p);
+    }
     LSPR_TRY_ST(launch_ff_boxes(ctx));
 
     // target blocks
@@ -891,6 +928,10 @@ int tree_tc_lists(lspr_ctx *ctx, bool p2p) {
             static_assert(sizeof(TcEntry) == sizeof(int2) && sizeof(TcItem) == sizeof(int4), "device layouts");
             LSPR_TRY(ctx, cudaMemcpyAsync(tr.tc_list.p, glist.data(), sizeof(int2) * glist.size(), cudaMemcpyHostToDevice, st));
             LSPR_TRY(ctx, cudaMemcpyAsync(tr.tc_items.p, gitems.data(), sizeof(int4) * gitems.size(), cudaMemcpyHostToDevice, st));
+            ++ctx->n_launches;
+            tc_list_surf_kernel<<<grid_for(glist.size(), 256), 256, 0, st>>>(
+                (int64_t)glist.size(), tr.tc_list.p, ctx->mesh.S > 1 ? tr.box_surf.p : nullptr);
+            LSPR_TRY(ctx, cudaGetLastError());
         }
         LSPR_TRY(ctx, cudaStreamSynchronize(st));
         tr.tc_built = true;
@@ -918,6 +959,10 @@ int tree_tc_lists(lspr_ctx *ctx, bool p2p) {
             LSPR_TRY(ctx, cudaMemcpyAsync(tr.tcp_items.p, pitems.data(), sizeof(int4) * pitems.size(),
                                           cudaMemcpyHostToDevice, st));
             LSPR_TRY(ctx, cudaMemcpyAsync(tr.tcp_ivl.p, pivl.data(), sizeof(int4) * pivl.size(), cudaMemcpyHostToDevice, st));
+            ++ctx->n_launches;
+            tc_ivl_surf_kernel<<<grid_for(pivl.size() * 32, 256), 256, 0, st>>>(
+                (int64_t)pivl.size(), tr.tcp_ivl.p, ctx->mesh.S, ctx->wo.src_panel.p, ctx->mesh.surf.p);
+            LSPR_TRY(ctx, cudaGetLastError());
         }
         LSPR_TRY(ctx, cudaStreamSynchronize(st));
         tr.tcp_built = true;
