@@ -232,7 +232,7 @@ int launch_p2p(lspr_ctx *ctx, int prec, const int4 *items, int64_t nitems, doubl
             if (B >= mn) LSPR_TRY_ST(p2p_tc_launch(ctx, acc, st, counter, B, 0));
             else p2p_launch<float, batch_chunk<float>(2)>(ctx, items, nitems, B, acc, st, counter);
         } else {
-            LSPR_TRY_ST(p2p_tc_launch(ctx, acc, st, counter, B, mn));
+            if (B >= mn) LSPR_TRY_ST(p2p_tc_launch(ctx, acc, st, counter, B, mn));
             p2p_launch<float, batch_chunk<float>(2)>(ctx, items, nitems, B, acc, st, counter, mn);
         }
     } else {

@@ -44,6 +44,7 @@ constexpr int kTargetBlock = 64;                       // targets per interactio
 constexpr int kTcGroup = 4;        // target blocks per tensor-core M2P group (256 targets)
 constexpr int kTcGroupSeg = 32;    // boxes per tensor-core M2P work unit at most
 constexpr int kTcP2PSrc = 2048;    // sources per tensor-core P2P work unit at most
+constexpr int kTcSrcRows = 8;      // tensor-core P2P source geometry per eight sources: rows -x, -y, -z, normal, panel, -
 constexpr int kTcSurf = 8;         // tensor-core M2P list entry.y: block mask, from this bit the box's surfaces
 constexpr int kMaxP = 8;                               // highest Taylor order compiled
 constexpr int kMaxDepth = 10;                          // octree levels below the root (10 bits per axis)
@@ -180,7 +181,9 @@ struct Tree {
     // the P2P source ranges of the same groups (tensor-core P2P): the union of the blocks'
     // ranges cut at every range end, each piece with the mask of the blocks that sum it
     DArr<int4> tcp_items;    // (group, interval begin, interval end, 0)
-    DArr<int4> tcp_ivl;      // (source begin, source end, block mask, 0)
+    DArr<int4> tcp_ivl;      // (source begin, source end, block mask, surface mask)
+    DArr<int> tcp_mask8;     // several surfaces: [eight sources] the surface masks of the ranges that hold them
+    DArr<float> tcp_src8;    // [eight sources][kTcSrcRows][8] their geometry
     int64_t n_tcp_items = 0, n_tcp_ivl = 0, n_tcp_sources = 0, n_tcp_stages = 0;   // stages of 8 sources
     bool tc_built = false, tcp_built = false;   // the group lists above match the tree
     DArr<int4> p2m_items;    // (leaf, source begin, source end, 0): leaves under an accepted box
@@ -302,6 +305,7 @@ struct lspr_ctx {
     int tc_p2p_min_rhs = 24;           // the tensor-core P2P takes products of at least this many
                                        // right-hand sides in use; fewer take the FP32-pipe P2P
     lspr::DArr<unsigned char> tc_img;  // split moments in tensor-core operand layout
+    lspr::DArr<unsigned char> tcp_img; // split source weights in tensor-core operand layout
     lspr::DArr<int> dev_err;           // [0] bounded device waits that ran out (never reset);
                                        // [1] failure-path check: tensor-core kernels give up at once
     int dev_err_seen = 0;              // [0] as last reported by a status (LSPR_E_TIMEOUT)

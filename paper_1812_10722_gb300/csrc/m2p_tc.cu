@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) {
             bar_init(smem_addr(&full_a[s]), 1);      // the producer's expect_tx (+ the copy's bytes)
-            bar_init(smem_addr(&full_b[s]), kTcN);   // one arrival per generating thread
+            bar_init(smem_addr(&full_b[s]), kGenWarps);   // one arrival per generating warp
             bar_init(smem_addr(&empty_s[s]), 1);     // the MMAs' commit
         }
         for (int a = 0; a < 2; ++a) {
@@ -436,7 +436,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         *(float4 *)(bl + core_off(tid, 4 * t4)) = sp.lo;
                     }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    bar_arrive(smem_addr(&full_b[s]));
+                    __syncwarp();   // one arrival per warp: a thread each would serialise on the barrier
+                    if (lane == 0) bar_arrive(smem_addr(&full_b[s]));
                     ++seq;
                 }
                 if (ok && pend) ok = drain_acc();   // the previous unit, behind this unit's first box

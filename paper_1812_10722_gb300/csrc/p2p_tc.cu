@@ -19,16 +19,25 @@
 // W_hi and W_lo are the two halves of one 128-row operand and two MMAs give all four products
 // (the epilogue adds both halves).
 //
+// The split weights are formed once per product in operand layout (p2p_image_kernel: 16 KB per eight
+// consecutive sources and 64 right-hand sides), so that staging them is one bulk copy; stages are
+// therefore aligned to multiples of eight sources, and a range that begins or ends inside one gets
+// zero kernel values for the rest.
+//
 // Roles (persistent, one CTA per SM, both accumulators in the SM's 512 tensor-memory columns):
 //   warp 16 (one lane) fetches work units into a small ring and bulk-copies every stage's inputs
-//     (the positions, normals and weights of its eight sources) into the stage;
+//     (the weight operands, and the positions and normals of its eight sources);
 //   warps 0-15 (two threads per target of the group, four of the stage's eight sources each)
-//     generate G and dG/dn of every stage in registers from those inputs, split them and write
-//     the B operands; warps 8-11 also write the split weights (the A operands); after the first
+//     generate G and dG/dn of every stage in registers, two sources at a time in packed f32x2
+//     arithmetic, split them and write the B operands; after the first
 //     stage of the next unit they drain the finished unit's accumulators (tcgen05.ld) into the
 //     FP64 accumulators;
 //   warp 17 (one lane) issues the MMAs of each stage once it is written, commits to the stage's
 //     "empty" barrier and, at the end of a unit, to the accumulator barrier.
+// 81920 panels, 64 right-hand sides: 3.44 ms with the image (0.15), 4.24 with the weights split by four
+// of the generating warps (which every stage waited for) and a barrier arrival per thread.  A stage
+// takes 0.86 us against 0.48 of its six MMAs and about as much of its 121 KB of shared-memory
+// traffic (operand reads, generated operands, copies).
 // Every wait is bounded (about a second): one that runs out raises an abort flag that the
 // other roles see, the block drains its bulk copies and MMAs in flight, frees its tensor memory
 // and returns,
@@ -58,13 +67,14 @@ constexpr int kRingConsumers = kGenWarps + 1;  // lane 0 of each consumer warp
 constexpr uint32_t kTmemCols = 2 * kTcN;       // D_V in columns [0, 256), D_K in [256, 512)
 constexpr int kAPart = (128 / 8) * kSBO;       // one split part of a weight operand (128 rows)
 constexpr int kBPart = (kTcN / 8) * kSBO;      // one split part of a kernel operand (256 rows)
-// stage: W_V hi | W_V lo | W_K hi | W_K lo | G hi | G lo | dG hi | dG lo | the stage's inputs as
-// bulk-copied from global memory: source positions (8 float4), normals (8 float4), weights
-// (8 sources x 64 right-hand sides float4)
-constexpr int kOffWV = 0, kOffWK = 2 * kAPart, kOffG = 4 * kAPart, kOffD = 4 * kAPart + 2 * kBPart;
-constexpr int kOffRaw = 4 * kAPart + 4 * kBPart;
-constexpr int kRawPos = 0, kRawNrm = kSrc * 16, kRawW = 2 * kSrc * 16;
-constexpr int kStage = kOffRaw + 2 * kSrc * 16 + kSrc * kRC * 16;
+// stage: the weight operands as bulk-copied from the image (W_V hi | W_V lo | W_K hi | W_K lo, or
+// stacked W_V | W_K) | G hi | G lo | dG hi | dG lo | the geometry of the stage's sources (kTcSrcRows
+// rows of eight floats)
+constexpr int kOffG = 4 * kAPart, kOffD = 4 * kAPart + 2 * kBPart;
+constexpr int kOffSrc = 4 * kAPart + 4 * kBPart;
+constexpr int kImgBlock = 4 * kAPart;          // image bytes per eight sources and 64 right-hand sides
+constexpr int kSrcBytes = kTcSrcRows * kSrc * 4;
+constexpr int kStage = kOffSrc + kSrcBytes;
 constexpr int kStages = 4;
 constexpr int kSmem = kStages * kStage;
 static_assert(kSmem + 1024 <= 232448, "the stages and the static shared memory fit one SM");
@@ -79,10 +89,62 @@ __device__ __forceinline__ int core_off(int r, int k) {
     return (r >> 3) * kSBO + (k >> 2) * 128 + (r & 7) * 16 + (k & 3) * 4;
 }
 
+// The split weights of every eight consecutive sources in operand layout.  One thread per (eight
+// sources, unit chunk, half of the eight, right-hand side).  Sources past the end have zero weights;
+// rows of right-hand sides not in use are not written (their accumulator rows are not read).
+__global__ void __launch_bounds__(128)
+    p2p_image_kernel(int64_t Ns, int B, int nrc, const float4 *__restrict__ sw, unsigned char *__restrict__ img,
+                     const int *nact, int min_rhs, int nsurf, const int *__restrict__ mask8) {
+    const int Bact = nact ? *nact : B;
+    if (Bact < min_rhs) return;
+    const int64_t blk = blockIdx.x;   // (eight sources, chunk)
+    const int64_t g8 = blk / nrc;
+    const int rc = (int)(blk - g8 * nrc), b0 = rc * kRC, nb = min(kRC, Bact - b0);
+    if (nb <= 0) return;
+    const int q = threadIdx.x >> 6, j = threadIdx.x & 63;
+    const int64_t s0 = g8 * kSrc + 4 * q;
+    // no range that holds these sources has one of the chunk's surfaces: no unit reads the block
+    if (nsurf > 1 && !(mask8[g8] & set_surfaces(b0, nb, Bact, nsurf))) return;
+    if (j >= nb) return;
+    float4 w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        w[i] = s0 + i < Ns ? __ldg(sw + (s0 + i) * B + b0 + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const TfPair vr = tf32_split(make_float4(w[0].x, w[1].x, w[2].x, w[3].x));
+    const TfPair vi = tf32_split(make_float4(w[0].y, w[1].y, w[2].y, w[3].y));
+    const TfPair kr = tf32_split(make_float4(w[0].z, w[1].z, w[2].z, w[3].z));
+    const TfPair ki = tf32_split(make_float4(w[0].w, w[1].w, w[2].w, w[3].w));
+    unsigned char *o = img + blk * kImgBlock;
+    const int c = 4 * q;
+    if (nb <= kRC / 2) {
+        // stacked: rows re hi j, im hi 32 + j, re lo 64 + j, im lo 96 + j
+        *(float4 *)(o + core_off(j, c)) = vr.hi;
+        *(float4 *)(o + core_off(32 + j, c)) = vi.hi;
+        *(float4 *)(o + core_off(64 + j, c)) = vr.lo;
+        *(float4 *)(o + core_off(96 + j, c)) = vi.lo;
+        o += kAPart;
+        *(float4 *)(o + core_off(j, c)) = kr.hi;
+        *(float4 *)(o + core_off(32 + j, c)) = ki.hi;
+        *(float4 *)(o + core_off(64 + j, c)) = kr.lo;
+        *(float4 *)(o + core_off(96 + j, c)) = ki.lo;
+    } else {
+        // rows re j, im 64 + j; the high part, then the low part
+        *(float4 *)(o + core_off(j, c)) = vr.hi;
+        *(float4 *)(o + core_off(64 + j, c)) = vi.hi;
+        *(float4 *)(o + kAPart + core_off(j, c)) = vr.lo;
+        *(float4 *)(o + kAPart + core_off(64 + j, c)) = vi.lo;
+        o += 2 * kAPart;
+        *(float4 *)(o + core_off(j, c)) = kr.hi;
+        *(float4 *)(o + core_off(64 + j, c)) = ki.hi;
+        *(float4 *)(o + kAPart + core_off(j, c)) = kr.lo;
+        *(float4 *)(o + kAPart + core_off(64 + j, c)) = ki.lo;
+    }
+}
+
 __global__ void __launch_bounds__(kTcThreads, 1)
     p2p_tc_kernel(const int4 *__restrict__ items, int64_t nitems, const int4 *__restrict__ ivl, int B,
-                  const float4 *__restrict__ tgt, int64_t ntgt, const float4 *__restrict__ spos,
-                  const float4 *__restrict__ snrm, const float4 *__restrict__ sw, double *__restrict__ acc,
+                  const float4 *__restrict__ tgt, int64_t ntgt, const float *__restrict__ src8,
+                  const unsigned char *__restrict__ img, int nrc, double *__restrict__ acc,
                   int *counter, int *error, const int *nact, int min_rhs, int nsurf) {
     // fewer right-hand sides in use than min_rhs: the FP32-pipe P2P takes this product
     if ((nact ? *nact : B) < min_rhs) return;
@@ -96,7 +158,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const uint32_t sbase = smem_addr(tc_smem);
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
-            bar_init(smem_addr(&full_s[s]), kGenThreads);   // one arrival per generating thread
+            bar_init(smem_addr(&full_s[s]), kGenWarps);   // one arrival per generating warp
             bar_init(smem_addr(&empty_s[s]), 1);     // the MMAs' commit
             bar_init(smem_addr(&raw_s[s]), 1);       // the producer's expect_tx (+ the copies' bytes)
         }
@@ -146,42 +208,35 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 bar_arrive(smem_addr(&ring_full[slot]));
                 if (u >= units) break;
                 const int64_t ii = u / nbc;
-                const int b0 = (int)(u - ii * nbc) * kRC, nb = min(kRC, Bact - b0);
+                const int rc = (int)(u - ii * nbc), b0 = rc * kRC, nb = min(kRC, Bact - b0);
+                const uint32_t abytes = nb <= kRC / 2 ? 2 * kAPart : 4 * kAPart;
                 const int4 item = __ldg(items + ii);
                 bool ok = true;
                 const int um = set_surfaces(b0, nb, Bact, nsurf);
                 for (int iv = item.y; iv < item.z && ok; ++iv) {
                     const int4 e = __ldg(ivl + iv);
                     if (!(e.w & um)) continue;   // no source of the unit's surfaces (all roles agree)
-                    for (int sb = e.x; sb < e.y; sb += kSrc, ++seq) {
+                    for (int g = e.x / kSrc; g * kSrc < e.y; ++g, ++seq) {
                         const int s = (int)(seq % kStages);
                         if (seq >= kStages &&
                             !bar_wait(smem_addr(&empty_s[s]), (uint32_t)((seq / kStages) - 1) & 1u, &abort_s)) {
                             ok = false;
                             break;
                         }
-                        const int n = min(kSrc, e.y - sb);
-                        const uint32_t rb = smem_addr(&raw_s[s]);
-                        const uint32_t dst = sbase + (uint32_t)(s * kStage + kOffRaw);
+                        const uint32_t rb = smem_addr(&raw_s[s]), dst = sbase + (uint32_t)(s * kStage);
                         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(rb),
-                                     "r"((uint32_t)(n * 32 + n * nb * 16))
+                                     "r"((uint32_t)(abytes + kSrcBytes))
                                      : "memory");
                         asm volatile(
                             "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                                dst + kRawPos),
-                            "l"(spos + sb), "r"(n * 16), "r"(rb)
+                                dst + kOffSrc),
+                            "l"(src8 + (int64_t)g * (kTcSrcRows * kSrc)), "r"(kSrcBytes), "r"(rb)
                             : "memory");
                         asm volatile(
                             "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                                dst + kRawNrm),
-                            "l"(snrm + sb), "r"(n * 16), "r"(rb)
+                                dst),
+                            "l"(img + ((int64_t)g * nrc + rc) * kImgBlock), "r"(abytes), "r"(rb)
                             : "memory");
-                        for (int k = 0; k < n; ++k)
-                            asm volatile(
-                                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                                    dst + kRawW + (uint32_t)(k * kRC * 16)),
-                                "l"(sw + (int64_t)(sb + k) * B + b0), "r"(nb * 16), "r"(rb)
-                                : "memory");
                     }
                 }
                 if (!ok) break;
@@ -219,18 +274,21 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                             }
                             asm volatile("tcgen05.fence::after_thread_sync;");
                         }
-                        for (int sb = e.x; sb < e.y; sb += kSrc, ++seq) {
+                        for (int g = e.x / kSrc; g * kSrc < e.y; ++g, ++seq) {
                             const int s = (int)(seq % kStages);
-                            if (!bar_wait(smem_addr(&full_s[s]), (uint32_t)(seq / kStages) & 1u, &abort_s)) {
+                            const uint32_t par = (uint32_t)(seq / kStages) & 1u;
+                            if (!bar_wait(smem_addr(&raw_s[s]), par, &abort_s) ||
+                                !bar_wait(smem_addr(&full_s[s]), par, &abort_s)) {
                                 ok = false;
                                 break;
                             }
                             asm volatile("tcgen05.fence::after_thread_sync;");
                             const uint32_t st = sbase + (uint32_t)(s * kStage);
-                            const uint64_t wvh = umma_desc(st + kOffWV, 128, kSBO);
-                            const uint64_t wvl = umma_desc(st + kOffWV + kAPart, 128, kSBO);
-                            const uint64_t wkh = umma_desc(st + kOffWK, 128, kSBO);
-                            const uint64_t wkl = umma_desc(st + kOffWK + kAPart, 128, kSBO);
+                            const uint32_t koff = stacked ? kAPart : 2 * kAPart;
+                            const uint64_t wvh = umma_desc(st, 128, kSBO);
+                            const uint64_t wvl = umma_desc(st + kAPart, 128, kSBO);
+                            const uint64_t wkh = umma_desc(st + koff, 128, kSBO);
+                            const uint64_t wkl = umma_desc(st + koff + kAPart, 128, kSBO);
                             const uint64_t gh = umma_desc(st + kOffG, 128, kSBO);
                             const uint64_t gl = umma_desc(st + kOffG + kBPart, 128, kSBO);
                             const uint64_t hh = umma_desc(st + kOffD, 128, kSBO);
@@ -262,9 +320,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
     } else {
         // ---- generators: thread tid owns target tt = tid mod 256 of the group (row tt of the
-        // kernel operands) for the four sources 4 hf .. 4 hf + 3 of each stage, hf = tid / 256;
-        // threads 256..383 also stage the weights of one right-hand side for four sources
-        const int tt = tid & (kTcN - 1), hf = tid / kTcN, wt = tid - kTcN;
+        // kernel operands) for the four sources 4 hf .. 4 hf + 3 of each stage, hf = tid / 256
+        const int tt = tid & (kTcN - 1), hf = tid / kTcN;
         const int blk = tt / kTargetBlock;
         int64_t seq = 0;
         int nu = 0;
@@ -339,11 +396,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const bool live = ti < ntgt;
             const float4 q = live ? tgt[ti] : tgt[0];
             const int tp = live ? panel_of(q.w) : -1;
-            // weight staging (rows of the weight operands as documented at drain_acc): right-hand
-            // side wj at the sources of columns wk..wk+3; stacked units need threads 0..63 only
-            const bool wr = wt >= 0 && wt < 128 && (!stacked || wt < 64);
-            const int wj = stacked ? (wt & 31) : (wt & 31) + 32 * (wt >> 6);
-            const int wk = stacked ? 4 * (wt >> 5) : 4 * ((wt >> 5) & 1);
+            const float2 qx = make_float2(q.x, q.x), qy = make_float2(q.y, q.y), qz = make_float2(q.z, q.z);
             const int um = set_surfaces(b0, nb, Bact, nsurf);
             bool begun = false;
             for (int iv = item.y; iv < item.z && ok; ++iv) {
@@ -351,7 +404,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 if (!(e.w & um)) continue;
                 begun = true;
                 const bool on = live && ((e.z >> blk) & 1);   // uniform over the warp but for the tail
-                for (int sb = e.x; sb < e.y && ok; sb += kSrc) {
+                for (int g8 = e.x / kSrc; g8 * kSrc < e.y && ok; ++g8) {
                     // the stage's inputs have landed (and its operands are free: the producer
                     // armed the copies after the stage's previous MMAs completed)
                     const int s = (int)(seq % kStages);
@@ -360,63 +413,39 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         break;
                     }
                     unsigned char *stg = tc_smem + s * kStage;
-                    const float4 *rpos = (const float4 *)(stg + kOffRaw + kRawPos);
-                    const float4 *rnrm = (const float4 *)(stg + kOffRaw + kRawNrm);
-                    const float4 *rw = (const float4 *)(stg + kOffRaw + kRawW);
+                    const float4 *src = (const float4 *)(stg + kOffSrc) + hf;   // row r: src[2 r]
                     // this thread's part of the kernel operand row of its target: G and dG/dn of
-                    // the stage's sources 4 hf .. 4 hf + 3
+                    // the stage's sources 4 hf .. 4 hf + 3 (positions are stored negated)
                     constexpr int kPart = kSrc / kGenSplit;
                     float g[kPart], h[kPart];
+                    if (on) {
+                        const float4 px = src[0], py = src[2], pz = src[4], nx = src[6], ny = src[8], nz = src[10];
+                        const float4 id = src[12];
+                        const int pid[4] = {__float_as_int(id.x), __float_as_int(id.y), __float_as_int(id.z),
+                                            __float_as_int(id.w)};
 #pragma unroll
-                    for (int kk = 0; kk < kPart; ++kk) {
-                        const int k = kPart * hf + kk;
-                        g[kk] = 0.f;
-                        h[kk] = 0.f;
-                        if (on && sb + k < e.y) {
-                            const float4 p = rpos[k], n = rnrm[k];
-                            const float dx = q.x - p.x, dy = q.y - p.y, dz = q.z - p.z;
-                            float r = rsq(dx * dx + dy * dy + dz * dz);
-                            r = panel_of(n.w) == tp ? 0.f : r;
-                            g[kk] = r;
-                            h[kk] = (dx * n.x + dy * n.y + dz * n.z) * (r * r) * r;
+                        for (int p = 0; p < 2; ++p) {
+                            const float2 dx = __fadd2_rn(qx, p ? make_float2(px.z, px.w) : make_float2(px.x, px.y));
+                            const float2 dy = __fadd2_rn(qy, p ? make_float2(py.z, py.w) : make_float2(py.x, py.y));
+                            const float2 dz = __fadd2_rn(qz, p ? make_float2(pz.z, pz.w) : make_float2(pz.x, pz.y));
+                            const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+                            // zero for the target's own panel and for sources outside the range
+                            const int k = g8 * kSrc + kPart * hf + 2 * p;
+                            const float r0 = pid[2 * p] == tp || k < e.x || k >= e.y ? 0.f : rsq(r2.x);
+                            const float r1 = pid[2 * p + 1] == tp || k + 1 < e.x || k + 1 >= e.y ? 0.f : rsq(r2.y);
+                            const float2 r = make_float2(r0, r1);
+                            const float2 dn = __ffma2_rn(dz, p ? make_float2(nz.z, nz.w) : make_float2(nz.x, nz.y),
+                                              __ffma2_rn(dy, p ? make_float2(ny.z, ny.w) : make_float2(ny.x, ny.y),
+                                              __fmul2_rn(dx, p ? make_float2(nx.z, nx.w) : make_float2(nx.x, nx.y))));
+                            const float2 t = __fmul2_rn(__fmul2_rn(dn, __fmul2_rn(r, r)), r);
+                            g[2 * p] = r.x;
+                            g[2 * p + 1] = r.y;
+                            h[2 * p] = t.x;
+                            h[2 * p + 1] = t.y;
                         }
-                    }
-                    // the weights of right-hand side wj at the four sources from column wk
-                    float4 w[4];
+                    } else {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        w[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (wr && wj < nb && sb + wk + i < e.y) w[i] = rw[(wk + i) * kRC + wj];
-                    }
-                    if (wr) {
-                        const float4 vre = make_float4(w[0].x, w[1].x, w[2].x, w[3].x);
-                        const float4 vim = make_float4(w[0].y, w[1].y, w[2].y, w[3].y);
-                        const float4 kre = make_float4(w[0].z, w[1].z, w[2].z, w[3].z);
-                        const float4 kim = make_float4(w[0].w, w[1].w, w[2].w, w[3].w);
-                        const TfPair svr = tf32_split(vre), svi = tf32_split(vim);
-                        const TfPair skr = tf32_split(kre), ski = tf32_split(kim);
-                        unsigned char *av = stg + kOffWV, *ak = stg + kOffWK;
-                        if (stacked) {
-                            // rows: re hi wj, im hi 32 + wj, re lo 64 + wj, im lo 96 + wj
-                            *(float4 *)(av + core_off(wj, wk)) = svr.hi;
-                            *(float4 *)(av + core_off(32 + wj, wk)) = svi.hi;
-                            *(float4 *)(av + core_off(64 + wj, wk)) = svr.lo;
-                            *(float4 *)(av + core_off(96 + wj, wk)) = svi.lo;
-                            *(float4 *)(ak + core_off(wj, wk)) = skr.hi;
-                            *(float4 *)(ak + core_off(32 + wj, wk)) = ski.hi;
-                            *(float4 *)(ak + core_off(64 + wj, wk)) = skr.lo;
-                            *(float4 *)(ak + core_off(96 + wj, wk)) = ski.lo;
-                        } else {
-                            // rows: re wj, im 64 + wj; the high part, then the low part
-                            *(float4 *)(av + core_off(wj, wk)) = svr.hi;
-                            *(float4 *)(av + core_off(64 + wj, wk)) = svi.hi;
-                            *(float4 *)(av + kAPart + core_off(wj, wk)) = svr.lo;
-                            *(float4 *)(av + kAPart + core_off(64 + wj, wk)) = svi.lo;
-                            *(float4 *)(ak + core_off(wj, wk)) = skr.hi;
-                            *(float4 *)(ak + core_off(64 + wj, wk)) = ski.hi;
-                            *(float4 *)(ak + kAPart + core_off(wj, wk)) = skr.lo;
-                            *(float4 *)(ak + kAPart + core_off(64 + wj, wk)) = ski.lo;
-                        }
+                        for (int k = 0; k < kPart; ++k) g[k] = h[k] = 0.f;
                     }
                     unsigned char *bg = stg + kOffG, *bd = stg + kOffD;
                     static_assert(kPart == 4, "a thread writes one 4-column slice of its row");
@@ -430,7 +459,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         *(float4 *)(bd + kBPart + core_off(tt, kPart * hf)) = sh.lo;
                     }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    bar_arrive(smem_addr(&full_s[s]));
+                    __syncwarp();   // one arrival per warp: a thread each would serialise on the barrier
+                    if (lane == 0) bar_arrive(smem_addr(&full_s[s]));
                     ++seq;
                     if (pend) ok = drain_acc();   // the previous unit, behind this unit's first stage
                 }
@@ -468,12 +498,17 @@ int p2p_tc_launch(lspr_ctx *ctx, double *acc, cudaStream_t st, int *counter, int
     if (!ctx->dev_err.p) return LSPR_E_STATE;
     LSPR_TRY(ctx, allow_smem(p2p_tc_kernel, kSmem, ctx->device, smem_set));
     const int nrc = (B + kRC - 1) / kRC;
+    const int64_t Ns = ctx->mesh.Ns, ng = (Ns + kSrc - 1) / kSrc;
+    LSPR_TRY(ctx, ctx->tcp_img.ensure((size_t)(ng * nrc) * kImgBlock));
+    ++ctx->n_launches;   // the image; the caller counts the P2P launch
+    p2p_image_kernel<<<(unsigned)(ng * nrc), 128, 0, st>>>(Ns, B, nrc, Views<float>::w(ctx), ctx->tcp_img.p,
+                                                          ctx->rhs_nact, min_rhs, ctx->mesh.S, tr.tcp_mask8.p);
     const unsigned grid =
         (unsigned)std::max<int64_t>(1, std::min<int64_t>(tr.n_tcp_items * nrc, std::max(1, ctx->num_sms)));
     p2p_tc_kernel<<<grid, kTcThreads, kSmem, st>>>(tr.tcp_items.p, tr.n_tcp_items, tr.tcp_ivl.p, B,
-                                                  Views<float>::tgt(ctx), ctx->mesh.N, Views<float>::spos(ctx),
-                                                  Views<float>::snrm(ctx), Views<float>::w(ctx), acc, counter,
-                                                  ctx->dev_err.p, ctx->rhs_nact, min_rhs, ctx->mesh.S);
+                                                  Views<float>::tgt(ctx), ctx->mesh.N, tr.tcp_src8.p, ctx->tcp_img.p,
+                                                  nrc, acc, counter, ctx->dev_err.p, ctx->rhs_nact, min_rhs,
+                                                  ctx->mesh.S);
     return LSPR_OK;
 }
 

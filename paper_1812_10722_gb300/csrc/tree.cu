@@ -494,7 +494,7 @@ __global__ void tc_list_surf_kernel(int64_t n, int2 *list, const int *__restrict
     if (i < n) list[i].y |= (box_surf ? box_surf[list[i].x] : 1) << kTcSurf;
 }
 __global__ void tc_ivl_surf_kernel(int64_t n, int4 *ivl, int S, const int *__restrict__ src_panel,
-                                   const int *__restrict__ surf) {
+                                   const int *__restrict__ surf, int *mask8) {
     const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (i >= n) return;
@@ -503,6 +503,27 @@ __global__ void tc_ivl_surf_kernel(int64_t n, int4 *ivl, int S, const int *__res
         for (int s = ivl[i].x + lane; s < ivl[i].y; s += 32) m |= 1u << surf[src_panel[s]];
     m = __reduce_or_sync(0xffffffffu, m);
     if (lane == 0) ivl[i].w = (int)m;
+    if (S > 1)
+        for (int g = ivl[i].x / 8 + lane; g * 8 < ivl[i].y; g += 32) atomicOr(&mask8[g], (int)m);
+}
+
+// geometry of eight consecutive sources, one row per component (positions negated), in the layout
+// that the tensor-core P2P reads; sources past the end repeat the last one
+__global__ void tc_src8_kernel(int64_t Ns, const float4 *__restrict__ spos, const float4 *__restrict__ snrm,
+                               float *src8) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= (Ns + 7) / 8 * 8) return;
+    const int64_t s = min(i, Ns - 1);
+    const float4 p = spos[s], n = snrm[s];
+    float *o = src8 + (i >> 3) * (kTcSrcRows * 8) + (i & 7);
+    o[0] = -p.x;
+    o[8] = -p.y;
+    o[16] = -p.z;
+    o[24] = n.x;
+    o[32] = n.y;
+    o[40] = n.z;
+    o[48] = n.w;
+    o[56] = 0.f;
 }
 
 // box node of the list walk: (first child or -1, children, source begin, source end)
@@ -952,8 +973,16 @@ int tree_tc_lists(lspr_ctx *ctx, bool p2p) {
         tr.n_tcp_ivl = (int64_t)pivl.size();
         tr.n_tcp_sources = psrc;
         tr.n_tcp_stages = 0;
-        for (const TcRange &r : pivl) tr.n_tcp_stages += (r.s1 - r.s0 + 7) / 8;
+        for (const TcRange &r : pivl) tr.n_tcp_stages += (r.s1 + 7) / 8 - r.s0 / 8;   // aligned to eight sources
         LSPR_TRY(ctx, tr.tcp_items.ensure(std::max<size_t>(1, pitems.size())));
+        const int64_t Ns = ctx->mesh.Ns;
+        if (ctx->mesh.S > 1) {
+            LSPR_TRY(ctx, tr.tcp_mask8.ensure((size_t)(Ns + 7) / 8));
+            LSPR_TRY(ctx, cudaMemsetAsync(tr.tcp_mask8.p, 0, sizeof(int) * ((Ns + 7) / 8), st));
+        }
+        LSPR_TRY(ctx, tr.tcp_src8.ensure((size_t)(Ns + 7) / 8 * (kTcSrcRows * 8)));
+        ++ctx->n_launches;
+        tc_src8_kernel<<<grid_for(Ns + 7, 256), 256, 0, st>>>(Ns, ctx->wo.spos32.p, ctx->wo.snrm32.p, tr.tcp_src8.p);
         LSPR_TRY(ctx, tr.tcp_ivl.ensure(std::max<size_t>(1, pivl.size())));
         if (!pitems.empty()) {
             LSPR_TRY(ctx, cudaMemcpyAsync(tr.tcp_items.p, pitems.data(), sizeof(int4) * pitems.size(),
@@ -961,7 +990,7 @@ int tree_tc_lists(lspr_ctx *ctx, bool p2p) {
             LSPR_TRY(ctx, cudaMemcpyAsync(tr.tcp_ivl.p, pivl.data(), sizeof(int4) * pivl.size(), cudaMemcpyHostToDevice, st));
             ++ctx->n_launches;
             tc_ivl_surf_kernel<<<grid_for(pivl.size() * 32, 256), 256, 0, st>>>(
-                (int64_t)pivl.size(), tr.tcp_ivl.p, ctx->mesh.S, ctx->wo.src_panel.p, ctx->mesh.surf.p);
+                (int64_t)pivl.size(), tr.tcp_ivl.p, ctx->mesh.S, ctx->wo.src_panel.p, ctx->mesh.surf.p, tr.tcp_mask8.p);
             LSPR_TRY(ctx, cudaGetLastError());
         }
         LSPR_TRY(ctx, cudaStreamSynchronize(st));
