@@ -193,7 +193,9 @@ __global__ void assemble_rhs_f32_kernel(int64_t N, int B, int L, const double *_
 // transposed right-hand sides xt [2N][B] contiguously in b.  The entries of the row's own surface
 // (nearly all) are summed first and enter with one complex product.  FP64 throughout: bound by the
 // FP64 pipe (4 multiply-adds per entry and right-hand side).  145920 panels, 32 right-hand sides:
-// 3.43 ms, 3.74 with one thread per (row, right-hand side) gathering from x [B][2N].
+// 1.23 ms (3.43 with both surfaces' cases in one loop, whose
+// branches the compiler merges into 18 FP64 operations per entry; 3.74 with one thread per (row,
+// right-hand side) gathering from x [B][2N]).
 __global__ void assemble_surf_rhs_kernel(int64_t N, int B, int S, int L, const int *__restrict__ surf,
                                          const double *__restrict__ acc, const int64_t *__restrict__ ptr,
                                          const int *__restrict__ col, const double *__restrict__ dV,
@@ -210,21 +212,29 @@ __global__ void assemble_surf_rhs_kernel(int64_t N, int B, int S, int L, const i
         if (k < 0) continue;   // converged system: row left untouched
         double2 Vs = make_double2(0, 0), Ks = make_double2(0, 0);   // own surface
         double2 Ka = make_double2(0, 0), Vw = make_double2(0, 0);   // the others
+        bool others = false;
         for (int64_t e = e0; e < e1; ++e) {
             const int64_t j = col[e];
-            const int t = surf[j];
             const double a = dV[e], c = dK[e];
             const double2 ph = xt[j * B + b], dp = xt[(N + j) * B + b];
-            if (t == si) {
+            if (surf[j] == si) {
                 Vs.x = fma(a, dp.x, Vs.x);
                 Vs.y = fma(a, dp.y, Vs.y);
                 Ks.x = fma(c, ph.x, Ks.x);
                 Ks.y = fma(c, ph.y, Ks.y);
             } else {
-                Ka = cadd(Ka, cscale(ph, c));
-                Vw = cadd(Vw, cmul(s[b * S + t], cscale(dp, a)));
+                others = true;
             }
         }
+        // in a loop of its own: beside the sums above, its 14 operations were issued for every entry
+        if (others)
+            for (int64_t e = e0; e < e1; ++e) {
+                const int64_t j = col[e];
+                const int t = surf[j];
+                if (t == si) continue;
+                Ka = cadd(Ka, cscale(xt[j * B + b], dK[e]));
+                Vw = cadd(Vw, cmul(s[b * S + t], cscale(xt[(N + j) * B + b], dV[e])));
+            }
         for (int t = 0; t < S; ++t) {
             const double *f = acc + 4 * (i * ((int64_t)B * S) + (int64_t)t * K + k);
             const double2 V = make_double2(f[0], f[1]), Kt = make_double2(f[2], f[3]);
