@@ -568,21 +568,39 @@ __device__ __forceinline__ bool mac_accept(const dbl4 &c, const dbl4 &lo, const 
     return c.w < theta * r && r - c.w > clear;
 }
 
+// The same decision from FP32 copies where they settle it (the box centres are FP32 values, the
+// block's bounds are rounded), else in FP64: margin bounds the difference of both sides of each
+// comparison, from 2^-24 of the coordinates (at most cmax), the radius's 1e-6 enlargement and the
+// arithmetic, twice over.  The FP64 test alone made the list walk FP64-bound.
+__device__ __forceinline__ bool mac_decide(const float4 &c, const float4 &lo, const float4 &hi, float cmax, float theta,
+                                           float clear, const dbl4 *c64, const dbl4 &lo64, const dbl4 &hi64,
+                                           double theta64, double clear64) {
+    const float dx = fmaxf(0.f, fmaxf(lo.x - c.x, c.x - hi.x));
+    const float dy = fmaxf(0.f, fmaxf(lo.y - c.y, c.y - hi.y));
+    const float dz = fmaxf(0.f, fmaxf(lo.z - c.z, c.z - hi.z));
+    const float r = sqrtf(dx * dx + dy * dy + dz * dz);
+    const float margin = 1e-6f * cmax + 3e-6f * r + 6e-6f * c.w + 1e-6f * clear;
+    const float a = fminf(theta * r - c.w, r - c.w - clear);
+    if (a > margin) return true;
+    if (a < -margin) return false;
+    return mac_accept(*c64, lo64, hi64, theta64, clear64);
+}
+
 // One warp per target block walks the tree depth first.  A popped box is known to be
 // rejected by the MAC: a leaf becomes a direct (P2P) source range, merged with the
 // previous range when contiguous; for an internal box the lanes test its children in
 // parallel, accepted children join the block's M2P list and rejected ones are pushed in
 // reverse octant order, so leaves come out in Morton order.
 // The stack holds the boxes' nodes, loaded together with their acceptance test, so that a pop costs
-// one dependent load (the children's centres and nodes) instead of three:
-// 245 us a walk at 81920 panels, 283 before.
+// one dependent load (the children's centres and nodes) instead of three.  81920 panels:
+// 63 us (counting) and 98 us (filling) a walk, 245 with the acceptance test in FP64, 283 before that.
 // FILL = false: count P2P items, M2P boxes and M2P items per target block.
 // FILL = true: write them at the scanned offsets and mark accepted boxes as used.
 constexpr int kListWarps = 4;
 template <bool FILL>
 __global__ void __launch_bounds__(kListWarps * 32) lists_kernel(
     int64_t ntb, int64_t N, const dbl4 *lo, const dbl4 *hi, const dbl4 *__restrict__ bc,
-    const int4 *__restrict__ node, double theta, double clear, int *n_p2p, int *n_m2p, int *n_m2pi,
+    const float4 *__restrict__ bc32, const int4 *__restrict__ node, double theta, double clear, int *n_p2p, int *n_m2p, int *n_m2pi,
     const int *o_p2p, const int *o_m2p, const int *o_m2pi, int4 *p2p_items, int *m2p_list, int4 *m2p_items,
     int *used, unsigned long long *pairs, int *overflow) {
     __shared__ int4 stk[kListWarps][kStack];
@@ -591,6 +609,11 @@ __global__ void __launch_bounds__(kListWarps * 32) lists_kernel(
     if (tb >= ntb) return;
     int4 *stack = stk[warp];
     const dbl4 l = lo[tb], h = hi[tb];
+    const float4 lf = make_float4((float)l.x, (float)l.y, (float)l.z, 0.f);
+    const float4 hf = make_float4((float)h.x, (float)h.y, (float)h.z, 0.f);
+    const float cmax = fmaxf(fmaxf(fmaxf(fabsf(lf.x), fabsf(hf.x)), fmaxf(fabsf(lf.y), fabsf(hf.y))),
+                             fmaxf(fabsf(lf.z), fabsf(hf.z)));
+    const float thf = (float)theta, clf = (float)clear;
     const int ntgt = (int)min((int64_t)kTargetBlock, N - tb * kTargetBlock);
     if (lane == 0) stack[0] = node[0];
     __syncwarp();
@@ -631,7 +654,7 @@ __global__ void __launch_bounds__(kListWarps * 32) lists_kernel(
         if (lane < nc) {
             ch = bn.x + lane;
             cn = node[ch];
-            acc = mac_accept(bc[ch], l, h, theta, clear);
+            acc = mac_decide(bc32[ch], lf, hf, cmax, thf, clf, bc + ch, l, h, theta, clear);
             push = !acc;
         }
         const unsigned am = __ballot_sync(0xffffffffu, acc), pm = __ballot_sync(0xffffffffu, push);
@@ -867,7 +890,7 @@ int tree_build(lspr_ctx *ctx, double theta, int P, int Ncrit) {
     LSPR_TRY(ctx, cudaMemsetAsync(tr.box_used.p, 0, sizeof(int) * nboxes, st));
     ++ctx->n_launches;
     lists_kernel<false><<<grid_for(ntb, kListWarps), kListWarps * 32, 0, st>>>(
-        ntb, N, tlo.p, thi.p, tr.box_c64.p, tr.box_node.p, theta, clear,
+        ntb, N, tlo.p, thi.p, tr.box_c64.p, tr.box_c32.p, tr.box_node.p, theta, clear,
         cnt3.p, cnt3.p + ntb, cnt3.p + 2 * ntb, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
         pairs.p, ovf.p);
     ++ctx->n_launches;
@@ -893,7 +916,7 @@ int tree_build(lspr_ctx *ctx, double theta, int P, int Ncrit) {
     LSPR_TRY(ctx, tr.m2p_items.ensure(std::max<int64_t>(1, tot[2])));
     ++ctx->n_launches;
     lists_kernel<true><<<grid_for(ntb, kListWarps), kListWarps * 32, 0, st>>>(
-        ntb, N, tlo.p, thi.p, tr.box_c64.p, tr.box_node.p, theta, clear,
+        ntb, N, tlo.p, thi.p, tr.box_c64.p, tr.box_c32.p, tr.box_node.p, theta, clear,
         nullptr, nullptr, nullptr, off3.p, off3.p + ntb, off3.p + 2 * ntb, tr.p2p_items.p, tr.m2p_list.p,
         tr.m2p_items.p, tr.box_used.p, pairs.p, ovf.p);
     LSPR_TRY(ctx, cudaGetLastError());
