@@ -154,6 +154,12 @@ LSPR_API int lspr_tree_build(lspr_ctx *ctx, double theta, int32_t P, int32_t Ncr
 LSPR_API int lspr_matvec(lspr_ctx *ctx, const double *x, double *y, int32_t B, const double *eps_ratio,
                 int32_t mode, int32_t on_device);
 
+/* The same product for x and y on the device and eps_ratio on the host (the few permittivity ratios
+ * of a product usually are): they are copied behind the caller's earlier work on the context's
+ * stream, without a transfer of the caller's own.  Errors as lspr_matvec. */
+LSPR_API int lspr_matvec_device(lspr_ctx *ctx, const double *x, double *y, int32_t B, const double *eps_ratio,
+                                int32_t mode);
+
 /* Solve the interface problem for B wavelengths and return the induced dipole
  * and the extinction cross-section of each (host pointers):
  *   eps_in   [B][nsurf] complex  permittivity of every surface per wavelength

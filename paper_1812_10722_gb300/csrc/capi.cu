@@ -70,10 +70,24 @@ namespace lspr {
 
 // LSPR_E_TIMEOUT if a bounded device wait ran out since the last status that reported one
 // (the stream is synchronised by the caller); otherwise rc
+static int judge_count(lspr_ctx *c, int count, int rc);
 int timeout_status(lspr_ctx *c, int rc) {
     int count = 0;
     if (cudaMemcpy(&count, c->dev_err.p, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
         return cuda_status(c, cudaGetLastError(), "reading the device error count");
+    c->tc_launched = false;
+    return judge_count(c, count, rc);
+}
+
+int finish_status(lspr_ctx *c) {
+    const bool read = c->tc_launched;   // only the tensor-core kernels hold bounded waits
+    if (read) LSPR_TRY(c, cudaMemcpyAsync(c->host_err, c->dev_err.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    LSPR_TRY(c, cudaStreamSynchronize(c->stream));
+    c->tc_launched = false;
+    return read ? judge_count(c, *c->host_err, LSPR_OK) : LSPR_OK;
+}
+
+static int judge_count(lspr_ctx *c, int count, int rc) {
     if (count == c->dev_err_seen) return rc;
     c->dev_err_seen = count;
     c->last_error = "a bounded device wait ran out: the product is incomplete";
@@ -121,7 +135,7 @@ int lspr_create(lspr_ctx **out, int device, void *cuda_stream) {
     if (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess ||
-        c->dev_err.ensure(2) != cudaSuccess || cudaMemset(c->dev_err.p, 0, 2 * sizeof(int)) != cudaSuccess) {
+        cudaMallocHost((void **)&c->host_err, sizeof(int)) != cudaSuccess || c->dev_err.ensure(2) != cudaSuccess || cudaMemset(c->dev_err.p, 0, 2 * sizeof(int)) != cudaSuccess) {
         lspr_destroy(c);
         return LSPR_E_CUDA;
     }
@@ -141,6 +155,7 @@ int lspr_destroy(lspr_ctx *c) {
         if (e) cudaEventDestroy(e);
     if (c->side) cudaStreamDestroy(c->side);
     if (c->gstream) cudaStreamDestroy(c->gstream);
+    if (c->host_err) cudaFreeHost(c->host_err);
     delete c;   // device arrays free themselves
     return LSPR_OK;
 }
@@ -162,8 +177,8 @@ int lspr_tree_build(lspr_ctx *c, double theta, int32_t P, int32_t Ncrit) {
     return tree_build(c, theta, P, Ncrit);
 }
 
-int lspr_matvec(lspr_ctx *c, const double *x, double *y, int32_t B, const double *eps_ratio, int32_t mode,
-                int32_t on_device) {
+static int matvec(lspr_ctx *c, const double *x, double *y, int32_t B, const double *eps_ratio, int32_t mode,
+                  bool vectors_on_device, bool ratio_on_device) {
     if (!c || !x || !y || !eps_ratio || B < 1 || mode < 0 || mode > 5) return LSPR_E_ARG;
     if (!c->mesh.ready) return LSPR_E_STATE;
     if (mode_tree(mode) && !c->tree.ready) return LSPR_E_STATE;
@@ -172,24 +187,35 @@ int lspr_matvec(lspr_ctx *c, const double *x, double *y, int32_t B, const double
     const double2 *xd = (const double2 *)x;
     double2 *yd = (double2 *)y;
     const double2 *sd = (const double2 *)eps_ratio;
-    if (!on_device) {
-        LSPR_TRY(c, c->xbuf.ensure((size_t)B * n2));
-        LSPR_TRY(c, c->ybuf.ensure((size_t)B * n2));
+    if (!ratio_on_device) {
         const int S = c->mesh.S;   // eps_ratio is [B][S]
         LSPR_TRY(c, c->sbuf.ensure((size_t)B * S));
-        LSPR_TRY(c, cudaMemcpyAsync(c->xbuf.p, x, sizeof(double2) * B * n2, cudaMemcpyHostToDevice, c->stream));
         LSPR_TRY(c, cudaMemcpyAsync(c->sbuf.p, eps_ratio, sizeof(double2) * B * S, cudaMemcpyHostToDevice,
                                     c->stream));
-        xd = c->xbuf.p;
-        yd = c->ybuf.p;
         sd = c->sbuf.p;
     }
+    if (!vectors_on_device) {
+        LSPR_TRY(c, c->xbuf.ensure((size_t)B * n2));
+        LSPR_TRY(c, c->ybuf.ensure((size_t)B * n2));
+        LSPR_TRY(c, cudaMemcpyAsync(c->xbuf.p, x, sizeof(double2) * B * n2, cudaMemcpyHostToDevice, c->stream));
+        xd = c->xbuf.p;
+        yd = c->ybuf.p;
+    }
     LSPR_TRY_ST(apply_operator(c, mode, xd, yd, sd, B));
-    if (!on_device)
+    if (!vectors_on_device)
         LSPR_TRY(c, cudaMemcpyAsync(y, yd, sizeof(double2) * B * n2, cudaMemcpyDeviceToHost, c->stream));
-    LSPR_TRY(c, cudaStreamSynchronize(c->stream));
+    const int rc = finish_status(c);
     timer_collect(c);
-    return timeout_status(c, LSPR_OK);
+    return rc;
+}
+
+int lspr_matvec(lspr_ctx *c, const double *x, double *y, int32_t B, const double *eps_ratio, int32_t mode,
+                int32_t on_device) {
+    return matvec(c, x, y, B, eps_ratio, mode, on_device != 0, on_device != 0);
+}
+
+int lspr_matvec_device(lspr_ctx *c, const double *x, double *y, int32_t B, const double *eps_ratio, int32_t mode) {
+    return matvec(c, x, y, B, eps_ratio, mode, true, false);
 }
 
 int lspr_solve(lspr_ctx *c, const double *eps_in, double eps_out_re, double eps_out_im, const double *E0,

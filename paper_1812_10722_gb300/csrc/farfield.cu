@@ -34,6 +34,18 @@ namespace lspr {
 // w[s][slot] = w_s A_s / (4 pi) * (dphi_b, phi_b) at the source's panel, b = map[slot]
 // (identity without a map; only the first *nact slots are formed when nact is given);
 // x is [B][2N] complex
+// The kernels also clear the product's sums (accumulators and counters, moments): zero.p[0..n).
+struct ZeroRanges {
+    float4 *p[2];
+    int64_t n[2];
+};
+__device__ __forceinline__ void clear_ranges(const ZeroRanges &z, int64_t g) {
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+        for (int64_t i = g; i < z.n[q]; i += step) z.p[q][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 template <typename T4>
 // Several surfaces (S > 1): channel set slot = t K + k (surface t of the k-th of K running systems)
 // carries the weights of the sources of surface t only (zero elsewhere), so that each surface's
@@ -41,9 +53,10 @@ template <typename T4>
 __global__ void weights_kernel(int64_t Ns, int64_t N, int B, int S, const dbl4 *__restrict__ spos64,
                                const int *__restrict__ src_panel, const int *__restrict__ surf,
                                const double2 *__restrict__ x, const double2 *__restrict__ xt, T4 *__restrict__ w,
-                               const int *map, const int *nact) {
+                               const int *map, const int *nact, ZeroRanges zero) {
     const int BS = B * S;
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    clear_ranges(zero, g);
     if (g >= Ns * BS) return;
     const int64_t s = g / BS;
     const int slot = (int)(g - s * BS);
@@ -74,9 +87,10 @@ __global__ void weights_kernel(int64_t Ns, int64_t N, int B, int S, const dbl4 *
 __global__ void weights_f32t_kernel(int64_t Ns, int64_t N, int B, int S, const float4 *__restrict__ spos32,
                                     const int *__restrict__ src_panel, const int *__restrict__ surf,
                                     const float2 *__restrict__ xt, float4 *__restrict__ w, const int *map,
-                                    const int *nact) {
+                                    const int *nact, ZeroRanges zero) {
     const int BS = B * S;
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    clear_ranges(zero, g);
     if (g >= Ns * BS) return;
     const int64_t s = g / BS;
     const int slot = (int)(g - s * BS);
@@ -154,9 +168,24 @@ __global__ void to_ff_kernel(int64_t n, const dbl4 *__restrict__ a, ff4 *__restr
 
 // --------------------------------------------------------------- launchers
 int launch_weights(lspr_ctx *ctx, int prec, const double2 *x, const double2 *xt, int64_t N, int B, int S,
-                   const float2 *xtf) {
+                   const float2 *xtf, bool tree) {
     const int64_t Ns = ctx->mesh.Ns;
     const int BS = B * S;
+    ZeroRanges z = {{(float4 *)ctx->acc.p, nullptr}, {(int64_t)(4 * N * BS * sizeof(double) + kCounters * sizeof(int)) / 16, 0}};
+    static_assert(kCounters * sizeof(int) % 16 == 0, "cleared in words of 16 bytes");
+    if (tree) {
+        Tree &tr = ctx->tree;
+        const int64_t nm = tr.nboxes * tr.NT * BS;
+        if (prec == PREC_F32) {
+            LSPR_TRY(ctx, tr.mom32.ensure(nm));
+            z.p[1] = tr.mom32.p;
+            z.n[1] = nm;
+        } else {
+            LSPR_TRY(ctx, tr.mom64.ensure(nm));
+            z.p[1] = (float4 *)tr.mom64.p;
+            z.n[1] = 2 * nm;
+        }
+    }
     const unsigned grid = grid_for(Ns * BS, 256);
     cudaEvent_t ev;
     timer_begin(ctx, T_WEIGHTS, &ev);
@@ -164,20 +193,20 @@ int launch_weights(lspr_ctx *ctx, int prec, const double2 *x, const double2 *xt,
     if (prec == PREC_F64) {
         LSPR_TRY(ctx, ctx->w64.ensure(Ns * BS));
         weights_kernel<dbl4><<<grid, 256, 0, ctx->stream>>>(Ns, N, B, S, ctx->wo.spos64.p, ctx->wo.src_panel.p, ctx->mesh.surf.p, x, xt,
-                                                            ctx->w64.p, ctx->rhs_map, ctx->rhs_nact);
+                                                            ctx->w64.p, ctx->rhs_map, ctx->rhs_nact, z);
     } else if (prec == PREC_FF) {
         LSPR_TRY(ctx, ctx->w_ff.ensure(Ns * BS));
         weights_kernel<ff4><<<grid, 256, 0, ctx->stream>>>(Ns, N, B, S, ctx->wo.spos64.p, ctx->wo.src_panel.p, ctx->mesh.surf.p, x, xt,
-                                                           ctx->w_ff.p, ctx->rhs_map, ctx->rhs_nact);
+                                                           ctx->w_ff.p, ctx->rhs_map, ctx->rhs_nact, z);
     } else if (xtf) {
         LSPR_TRY(ctx, ctx->w32.ensure(Ns * BS));
         weights_f32t_kernel<<<grid, 256, 0, ctx->stream>>>(Ns, N, B, S, ctx->wo.spos32.p, ctx->wo.src_panel.p,
                                                            ctx->mesh.surf.p, xtf, ctx->w32.p, ctx->rhs_map,
-                                                           ctx->rhs_nact);
+                                                           ctx->rhs_nact, z);
     } else {
         LSPR_TRY(ctx, ctx->w32.ensure(Ns * BS));
         weights_kernel<float4><<<grid, 256, 0, ctx->stream>>>(Ns, N, B, S, ctx->wo.spos64.p, ctx->wo.src_panel.p, ctx->mesh.surf.p, x, xt,
-                                                              ctx->w32.p, ctx->rhs_map, ctx->rhs_nact);
+                                                              ctx->w32.p, ctx->rhs_map, ctx->rhs_nact, z);
     }
     timer_end(ctx, T_WEIGHTS, ev);
     LSPR_TRY(ctx, cudaGetLastError());
@@ -279,12 +308,8 @@ int launch_p2m(lspr_ctx *ctx, int prec, int B) {
     timer_begin(ctx, slot, &ev);
     ++ctx->n_launches;
     if (prec == PREC_F32) {
-        LSPR_TRY(ctx, tr.mom32.ensure(nm));
-        LSPR_TRY(ctx, cudaMemsetAsync(tr.mom32.p, 0, sizeof(float4) * nm, ctx->stream));
         LSPR_TRY_ST(p2m_orders_f32(ctx, B));
     } else {
-        LSPR_TRY(ctx, tr.mom64.ensure(nm));
-        LSPR_TRY(ctx, cudaMemsetAsync(tr.mom64.p, 0, sizeof(dbl4) * nm, ctx->stream));
         if (prec == PREC_F64) {
             LSPR_TRY_ST(p2m_orders_f64(ctx, B));
         } else {
@@ -325,7 +350,7 @@ int launch_m2p(lspr_ctx *ctx, int prec, double *acc, int *counter, int B) {
 int launch_weights_fp32_raw(cudaStream_t st, int64_t Ns, int64_t N, const dbl4 *spos64, const int *src_panel,
                             const double2 *x, float4 *w) {
     weights_kernel<float4><<<grid_for(Ns, 256), 256, 0, st>>>(Ns, N, 1, 1, spos64, src_panel, nullptr, x, nullptr, w, nullptr,
-                                                               nullptr);
+                                                               nullptr, ZeroRanges{});
     return cudaGetLastError() == cudaSuccess ? LSPR_OK : LSPR_E_CUDA;
 }
 

@@ -272,7 +272,7 @@ struct lspr_ctx {
     cudaStream_t stream = nullptr;
     cudaStream_t side = nullptr;       // second stream: P2P overlaps P2M -> M2P
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    lspr::DArr<int> counters;          // work-item counters of the persistent kernels
+    lspr::DArr<int> counters;          // selftest results
     int num_sms = 0;
     lspr::Mesh mesh;
     lspr::WorkOrder wo;
@@ -281,7 +281,7 @@ struct lspr_ctx {
     lspr::DirectItems direct_multi;    // several: fewer, longer items (n = 0: those of direct)
     lspr::Timing timing;
     // per-matvec scratch
-    lspr::DArr<double> acc;            // [B][N][4]: V re/im, K re/im (far part)
+    lspr::DArr<double> acc;            // [N][B][4]: V re/im, K re/im (far part), then the work-item counters
     lspr::DArr<float4> w32;            // [Ns] source weights
     lspr::DArr<dbl4> w64;
     lspr::DArr<ff4> w_ff;
@@ -309,6 +309,8 @@ struct lspr_ctx {
     lspr::DArr<int> dev_err;           // [0] bounded device waits that ran out (never reset);
                                        // [1] failure-path check: tensor-core kernels give up at once
     int dev_err_seen = 0;              // [0] as last reported by a status (LSPR_E_TIMEOUT)
+    int *host_err = nullptr;           // pinned copy of [0]
+    bool tc_launched = false;          // a tensor-core kernel was launched since [0] was last read
     // point charges inside the surfaces (lspr_set_charges): (x, y, z, q) and the surface of each
     lspr::DArr<dbl4> charges;
     lspr::DArr<int> charge_surf;
@@ -343,6 +345,9 @@ int cuda_status(lspr_ctx *ctx, cudaError_t e, const char *what);
 // LSPR_E_TIMEOUT in place of rc (LSPR_OK or LSPR_E_NOT_CONVERGED) when a bounded device wait ran
 // out since the last status that reported one; call with the context's stream synchronised
 int timeout_status(lspr_ctx *ctx, int rc);
+// the same for a product whose stream is not synchronised yet: the count is fetched behind the
+// product's kernels (only when a kernel with bounded waits was launched) and the stream synchronised
+int finish_status(lspr_ctx *ctx);
 #define LSPR_TRY(ctx, expr)                                              \
     do {                                                                 \
         cudaError_t e__ = (expr);                                        \
@@ -415,7 +420,9 @@ __device__ __forceinline__ unsigned spread10(unsigned v) {
 // B right-hand sides: weights [source][B], accumulators acc [panel][B][4]
 int launch_p2p(lspr_ctx *ctx, int prec, const int4 *items, int64_t nitems, double *acc, cudaStream_t st,
                int *counter, int B);
+// the moments are zero on entry (launch_weights clears them)
 int launch_p2m(lspr_ctx *ctx, int prec, int B);
+constexpr int kCounters = 8;   // work-item counters behind the accumulators
 int launch_m2p(lspr_ctx *ctx, int prec, double *acc, int *counter, int B);
 // float-float copies of the work-order geometry / box centres
 int launch_ff_geometry(lspr_ctx *ctx);
@@ -427,9 +434,10 @@ int launch_direct_flags(lspr_ctx *ctx);
 // xt: x transposed to [2N][B] (B > 1), or null
 // S > 1 surfaces: B x S channel sets, weights of set (b, t) masked to the sources of surface t
 // x [B][2N]; xt: its transposed FP64 copy [2N][B] or null; xtf: its transposed FP32 copy
-// (FP32 products of several right-hand sides) or null
+// (FP32 products of several right-hand sides) or null.  Clears the accumulators and counters of the
+// product and, with tree set, its moments.
 int launch_weights(lspr_ctx *ctx, int prec, const double2 *x, const double2 *xt, int64_t N, int B, int S,
-                   const float2 *xtf = nullptr);
+                   const float2 *xtf, bool tree);
 int launch_weights_fp32_raw(cudaStream_t st, int64_t Ns, int64_t N, const dbl4 *spos64, const int *src_panel,
                             const double2 *x, float4 *w);
 int launch_p2p_fp32_raw(cudaStream_t st, const int4 *items, int64_t nitems, const float4 *tgt, int64_t ntgt,

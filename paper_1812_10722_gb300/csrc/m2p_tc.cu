@@ -477,6 +477,7 @@ int tc_launch(lspr_ctx *ctx, double *acc, int *counter, int B) {
     const int64_t segs = tr.nboxes * nrc * S::NKC * (S::A_CH / 16);
     LSPR_TRY(ctx, ctx->tc_img.ensure((size_t)segs * 32));
     if (!ctx->dev_err.p) return LSPR_E_STATE;
+    ctx->tc_launched = true;
     LSPR_TRY(ctx, allow_smem(m2p_tc_kernel<P, RC>, S::SMEM, ctx->device, smem_set));
     ++ctx->n_launches;   // the image; the caller counts the M2P launch
     const unsigned gi =

@@ -496,6 +496,7 @@ int p2p_tc_launch(lspr_ctx *ctx, double *acc, cudaStream_t st, int *counter, int
     if (!tr.tcp_built) LSPR_TRY_ST(tree_tc_lists(ctx, true));
     if (tr.n_tcp_items == 0) return LSPR_OK;
     if (!ctx->dev_err.p) return LSPR_E_STATE;
+    ctx->tc_launched = true;
     LSPR_TRY(ctx, allow_smem(p2p_tc_kernel, kSmem, ctx->device, smem_set));
     const int nrc = (B + kRC - 1) / kRC;
     const int64_t Ns = ctx->mesh.Ns, ng = (Ns + kSrc - 1) / kSrc;

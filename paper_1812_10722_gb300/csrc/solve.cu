@@ -285,10 +285,8 @@ static int far_part(lspr_ctx *ctx, int mode, const double2 *x, int B) {
     const int S = ctx->mesh.S;
     const int BS = B * S;
     if (tree && !ctx->tree.ready) return LSPR_E_STATE;
-    LSPR_TRY(ctx, ctx->acc.ensure(4 * N * BS));
-    LSPR_TRY(ctx, ctx->counters.ensure(8));
-    LSPR_TRY(ctx, cudaMemsetAsync(ctx->acc.p, 0, sizeof(double) * 4 * N * BS, ctx->stream));
-    LSPR_TRY(ctx, cudaMemsetAsync(ctx->counters.p, 0, sizeof(int) * 8, ctx->stream));
+    LSPR_TRY(ctx, ctx->acc.ensure(4 * N * BS + kCounters * sizeof(int) / sizeof(double)));
+    int *counters = (int *)(ctx->acc.p + 4 * N * BS);
     const double2 *xt = nullptr;
     const float2 *xtf = nullptr;
     const dim3 tg(grid_for(2 * N, 32), grid_for(B, 32)), tb(32, 8);
@@ -304,27 +302,27 @@ static int far_part(lspr_ctx *ctx, int mode, const double2 *x, int B) {
         transpose_kernel<double2><<<tg, tb, 0, ctx->stream>>>(B, 2 * N, x, ctx->xt.p, nullptr);
         xt = ctx->xt.p;
     }
-    LSPR_TRY_ST(launch_weights(ctx, prec, x, xt, N, B, S, xtf));
+    LSPR_TRY_ST(launch_weights(ctx, prec, x, xt, N, B, S, xtf, tree));
     if (tree && ctx->timing.enabled) {
         // kernel timing: every far-field kernel on the main stream, one after another, so that
         // the events around a launch measure that kernel alone (no overlap, no waiting)
         LSPR_TRY_ST(launch_p2p(ctx, prec, ctx->tree.p2p_items.p, ctx->tree.n_p2p_items, ctx->acc.p, ctx->stream,
-                               ctx->counters.p, BS));
+                               counters, BS));
         LSPR_TRY_ST(launch_p2m(ctx, prec, BS));
-        LSPR_TRY_ST(launch_m2p(ctx, prec, ctx->acc.p, ctx->counters.p + 1, BS));
+        LSPR_TRY_ST(launch_m2p(ctx, prec, ctx->acc.p, counters + 1, BS));
     } else if (tree) {
         // P2P on the side stream overlaps P2M -> M2P on the main stream; both add into acc
         LSPR_TRY(ctx, cudaEventRecord(ctx->ev_fork, ctx->stream));
         LSPR_TRY(ctx, cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
         LSPR_TRY_ST(launch_p2p(ctx, prec, ctx->tree.p2p_items.p, ctx->tree.n_p2p_items, ctx->acc.p, ctx->side,
-                               ctx->counters.p, BS));
+                               counters, BS));
         LSPR_TRY(ctx, cudaEventRecord(ctx->ev_join, ctx->side));
         LSPR_TRY_ST(launch_p2m(ctx, prec, BS));
-        LSPR_TRY_ST(launch_m2p(ctx, prec, ctx->acc.p, ctx->counters.p + 1, BS));
+        LSPR_TRY_ST(launch_m2p(ctx, prec, ctx->acc.p, counters + 1, BS));
         LSPR_TRY(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
     } else {
         const DirectItems &d = direct_items(ctx, BS);
-        LSPR_TRY_ST(launch_p2p(ctx, prec, d.items.p, d.n, ctx->acc.p, ctx->stream, ctx->counters.p, BS));
+        LSPR_TRY_ST(launch_p2p(ctx, prec, d.items.p, d.n, ctx->acc.p, ctx->stream, counters, BS));
     }
     ctx->matvec_count += B;
     return LSPR_OK;

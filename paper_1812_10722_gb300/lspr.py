@@ -80,6 +80,7 @@ def lib():
             L.lspr_mesh_upload.argtypes = [_vp, _vp, _i64, _vp, _i64, _vp, _i32, ctypes.POINTER(QuadOpts), _i32]
             L.lspr_tree_build.argtypes = [_vp, _d, _i32, _i32]
             L.lspr_matvec.argtypes = [_vp, _vp, _vp, _i32, _vp, _i32, _i32]
+            L.lspr_matvec_device.argtypes = [_vp, _vp, _vp, _i32, _vp, _i32]
             L.lspr_solve.argtypes = [_vp, _vp, _d, _d, _vp, _vp, _i32, ctypes.POINTER(SolveOpts), _vp, _vp,
                                      ctypes.POINTER(SolveStats)]
             L.lspr_get_info.argtypes = [_vp] + [ctypes.POINTER(_i64)] * 7
@@ -100,7 +101,7 @@ def lib():
             L.lspr_selftest_wait_timeout.argtypes = [_vp, ctypes.POINTER(_i32)]
             L.lspr_selftest_gate_waits.argtypes = [_vp, _i32]
             L.lspr_set_charges.argtypes = [_vp, _vp, _i64, _vp]
-            for f in ("lspr_create", "lspr_destroy", "lspr_mesh_upload", "lspr_tree_build", "lspr_matvec",
+            for f in ("lspr_create", "lspr_destroy", "lspr_mesh_upload", "lspr_tree_build", "lspr_matvec", "lspr_matvec_device",
                       "lspr_solve", "lspr_get_info", "lspr_set_timing", "lspr_get_timing", "lspr_launch_count",
                       "lspr_set_graphs", "lspr_graph_stats", "lspr_autotune", "lspr_set_tensor_cores",
                       "lspr_device_errors", "lspr_selftest_wait_timeout", "lspr_selftest_gate_waits",
@@ -163,7 +164,8 @@ class Context:
                     stream = torch.cuda.current_stream(device).cuda_stream
             except ImportError:
                 stream = None
-        _check(lib().lspr_create(ctypes.byref(self._h), device, ctypes.c_void_p(stream or 0)), "lspr_create")
+        self._stream = int(stream or 0)
+        _check(lib().lspr_create(ctypes.byref(self._h), device, ctypes.c_void_p(self._stream)), "lspr_create")
         self.n = 0
 
     def close(self):
@@ -233,10 +235,12 @@ class Context:
             squeeze = x.dim() == 1
             xx = x.reshape(-1, 2 * self.n).contiguous()
             B = xx.shape[0]
-            s = torch.as_tensor(self._per_surface(eps_ratio, B).copy(), device=x.device)
+            s = self._per_surface(eps_ratio, B)
             y = torch.empty_like(xx)
-            rc = lib().lspr_matvec(self._h, ctypes.c_void_p(xx.data_ptr()), ctypes.c_void_p(y.data_ptr()), B,
-                                   ctypes.c_void_p(s.data_ptr()), m, 1)
+            own = torch.cuda.current_stream(x.device)
+            if own.cuda_stream != self._stream:   # x may still be in the making on the caller's stream
+                own.synchronize()
+            rc = lib().lspr_matvec_device(self._h, xx.data_ptr(), y.data_ptr(), B, s.ctypes.data, m)
             _check(rc, "lspr_matvec", self._h)
             return y[0] if squeeze else y
         x = np.ascontiguousarray(x, dtype=np.complex128)
