@@ -171,8 +171,7 @@ int launch_weights(lspr_ctx *ctx, int prec, const double2 *x, const double2 *xt,
                    const float2 *xtf, bool tree) {
     const int64_t Ns = ctx->mesh.Ns;
     const int BS = B * S;
-    ZeroRanges z = {{(float4 *)ctx->acc.p, nullptr}, {(int64_t)(4 * N * BS * sizeof(double) + kCounters * sizeof(int)) / 16, 0}};
-    static_assert(kCounters * sizeof(int) % 16 == 0, "cleared in words of 16 bytes");
+    ZeroRanges z = {{(float4 *)ctx->acc.p, nullptr}, {(int64_t)(4 * N * BS * sizeof(double) + acc_tail_ints(BS) * sizeof(int)) / 16, 0}};
     if (tree) {
         Tree &tr = ctx->tree;
         const int64_t nm = tr.nboxes * tr.NT * BS;

@@ -421,14 +421,15 @@ constexpr TermInfo make_term_info() {
 }
 static __constant__ TermInfo c_terms = make_term_info();
 
-// A_k(R) of every term, each handed to use(t, A_t) as soon as it is made
+// lead A_k(R) of every term, each handed to use(t, lead A_t) as soon as it is made
 template <typename T, int P, class F>
-__device__ __forceinline__ void m2p_recurrence(T Rx, T Ry, T Rz, T (&a)[n_terms(P)], F &&use) {
+__device__ __forceinline__ void m2p_recurrence(T Rx, T Ry, T Rz, T (&a)[n_terms(P)], F &&use, T lead = T(1)) {
     constexpr MultiIndex<P> mi{};
     constexpr int NT = MultiIndex<P>::NT;
     a[0] = rsq(Rx * Rx + Ry * Ry + Rz * Rz);
     const T ir2 = a[0] * a[0];
     const T R[3] = {Rx * ir2, Ry * ir2, Rz * ir2};
+    a[0] = lead * a[0];
     use(0, a[0]);
 #pragma unroll
     for (int t = 1; t < NT; ++t) {

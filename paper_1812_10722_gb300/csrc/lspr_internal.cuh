@@ -168,6 +168,7 @@ struct Tree {
     DArr<int> box_surf;      // several surfaces: mask of the surfaces of the box's sources
     DArr<dbl4> box_c64;   // centre (x,y,z), radius r_b
     DArr<float4> box_c32;
+    float rho_min = 0.f;     // least scale length of a box's expansion (box_scale)
     // lists
     DArr<int4> p2p_items;    // (target block, source begin, source end, 0)
     DArr<int4> m2p_items;    // (target block, list begin, list end, 0)
@@ -422,7 +423,10 @@ int launch_p2p(lspr_ctx *ctx, int prec, const int4 *items, int64_t nitems, doubl
                int *counter, int B);
 // the moments are zero on entry (launch_weights clears them)
 int launch_p2m(lspr_ctx *ctx, int prec, int B);
-constexpr int kCounters = 8;   // work-item counters behind the accumulators
+// behind the accumulators of a product, cleared with them: the work-item counters, then per layer and
+// channel set the largest magnitudes that scale the tensor-core operands
+constexpr int kCounters = 8;
+inline int64_t acc_tail_ints(int64_t BS) { return kCounters + (2 * BS + 3) / 4 * 4; }
 int launch_m2p(lspr_ctx *ctx, int prec, double *acc, int *counter, int B);
 // float-float copies of the work-order geometry / box centres
 int launch_ff_geometry(lspr_ctx *ctx);

@@ -7,18 +7,29 @@
 // its shape, so N is made as wide as the instruction allows: a work unit is a group of four
 // consecutive 64-target blocks (N = 256) and walks the sorted union of their M2P lists; the
 // coefficients of a block that did not accept a box are zero, so every block still receives
-// exactly the boxes its own acceptance test chose.  Both operands are split into TF32 high
+// exactly the boxes its own acceptance test chose.  Both operands are split into FP16 high
 // and low parts (FP32 accumulation in tensor memory): with 32 right-hand sides per unit
-// (128 channels) the product is A_hi B_hi + A_hi B_lo + A_lo B_hi (3xTF32); with 16 (64
+// (128 channels) the product is A_hi B_hi + A_hi B_lo + A_lo B_hi; with 16 (64
 // channels) A_hi and A_lo are stacked into the 128 rows of one operand and two MMAs give all
-// four products.
-//
-// Two kernels per product:
+// four products.  The FP16 parts hold the 22 bits of a TF32 split as long as the operands are
+// scaled into range, all by powers of two:
+//   - lengths of a box are measured in rho_b (box_scale): with rho_b / r < theta the coefficients
+//     A_k rho_b^(n+1) stay below 1.2 (the largest |A_k| r^(n+1) of any degree up to 8 and direction),
+//     and are carried times 2^15;
+//   - the moments M_k / rho_b^(n+1) of one right-hand side and layer are scaled by their largest
+//     magnitude over all boxes (m2p_max_kernel) into [2^14, 2^15).
+// What falls below full precision is then at most 2^-25 absolute in both: 2^-40 of the largest.
+// Against TF32 parts the MMAs take half the K steps and the operands half the bytes: 81920 panels, P 7,
+// 64 right-hand sides 2.57 -> 1.58 ms with both preparing kernels; sensor of 145920 panels 6.12 -> 4.38.
+// Error of the product against the float-float operator of the same tree, over batches of 2 to 28 on
+// spheres and sensors: 0.4 to 0.9 of the TF32 form's (half as many accumulation steps).
+// Three kernels per product:
+//   - m2p_max_kernel finds the scales;
 //   - tc_image_kernel writes, once per product, the split moments of every box in the
 //     operand layout of one pipeline stage (K-major 8x16-byte core matrices, no swizzle),
 //     so that staging A is a single bulk copy;
 //   - m2p_tc_kernel is persistent and warp-specialised.  The terms of each (unit, box) are
-//     cut into chunks of 16, one pipeline stage each (a ring of NS stages in shared memory):
+//     cut into chunks of 32, one pipeline stage each (a ring of NS stages in shared memory):
 //       warps 0-7 (one thread per target of the group) compute the coefficients a_k by the
 //         recurrence of m2p_kernel and write the split B part of each stage; they drain each
 //         unit's accumulator (tcgen05.ld) into the FP64 accumulators once the next unit's
@@ -42,9 +53,9 @@ namespace {
 
 using namespace tc;
 
-constexpr int kKC = 16;                        // terms per pipeline stage (two MMA K steps)
+constexpr int kKC = 32;                        // terms per pipeline stage (two MMA K steps)
 constexpr int kTcN = kTcGroup * kTargetBlock;  // targets per work unit (the MMA's N)
-constexpr int kChunkSBO = (kKC / 4) * 128;     // bytes per 8-row group of a stage operand
+constexpr int kChunkSBO = (kKC / 8) * 128;     // bytes per 8-row group of a stage operand
 constexpr int kGenWarps = kTcN / 32;           // one thread per target
 constexpr int kProdWarp = kGenWarps, kMmaWarp = kGenWarps + 1;
 constexpr int kTcThreads = 32 * (kGenWarps + 2);
@@ -71,7 +82,7 @@ struct TcShape {
     static constexpr int HRC = RC / HALVES;               // right-hand sides per A part
     static constexpr int ROWS = 4 * HRC;
     static constexpr bool STACKED = ROWS == 64;           // hi and lo halves of one operand
-    static constexpr uint32_t IDESC = idesc_tf32(128, kTcN);
+    static constexpr uint32_t IDESC = idesc_f16(128, kTcN);
     static constexpr int A_CH = (ROWS / 8) * kChunkSBO;   // one split part of one A per stage
     static constexpr int B_CH = (kTcN / 8) * kChunkSBO;   // one split part of B per stage
     static constexpr int OFF_B = HALVES * 2 * A_CH;       // [A_hi | A_lo] per half, then B_hi | B_lo
@@ -83,18 +94,73 @@ struct TcShape {
     static_assert(NS >= 2, "at least two stages");
 };
 
+struct TermDegrees {
+    signed char d[n_terms(kMaxP)];
+    __host__ __device__ constexpr int operator[](int t) const { return d[t]; }
+};
+constexpr TermDegrees make_degrees() {
+    TermDegrees r{};
+    constexpr MultiIndex<kMaxP> mi{};
+    for (int t = 0; t < n_terms(kMaxP); ++t) r.d[t] = (signed char)mi.deg[t];
+    return r;
+}
+__constant__ TermDegrees c_deg = make_degrees();
+
 // byte offset of (row r, term k) inside one split part of a stage operand
 __device__ __forceinline__ int core_off(int r, int k) {
-    return (r >> 3) * kChunkSBO + (k >> 2) * 128 + (r & 7) * 16 + (k & 3) * 4;
+    return (r >> 3) * kChunkSBO + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2;
+}
+
+// scale length of a box's expansion, a power of two: its radius (c.w), but at least theta times the
+// distance that the acceptance test keeps clear, so that the coefficients of a box of few sources,
+// accepted far beyond its radius / theta, keep their size
+__device__ __forceinline__ float box_scale(const float4 &c, float rho_min) {
+    return __int_as_float(__float_as_int(fmaxf(c.w, rho_min)) & 0x7f800000);
+}
+__device__ __forceinline__ float inv_pow2(float p) { return __int_as_float((254 << 23) - __float_as_int(p)); }
+
+// largest |M_k| / rho^(n+1) per layer and right-hand side over the accepted boxes: mx[2 j] single layer,
+// mx[2 j + 1] double layer, as the bits of non-negative floats.  One block per box (grid stride).
+constexpr int kMaxSets = 512;   // channel sets per block column of m2p_max_kernel
+__global__ void __launch_bounds__(256)
+    m2p_max_kernel(int64_t nbox, int NT, int B, const float4 *__restrict__ mom, const float4 *__restrict__ box_c,
+                   float rho_min, const int *__restrict__ used, int *mx, const int *nact,
+                   const int *__restrict__ box_surf, int NS) {
+    __shared__ int smax[2 * kMaxSets];
+    const int Bact = nact ? *nact : B, j0 = blockIdx.y * kMaxSets, nj = min(kMaxSets, Bact - j0);
+    if (nj <= 0) return;
+    for (int j = threadIdx.x; j < 2 * nj; j += blockDim.x) smax[j] = 0;
+    __syncthreads();
+    for (int64_t box = blockIdx.x; box < nbox; box += gridDim.x) {
+        if (!used[box]) continue;
+        const float ir = inv_pow2(box_scale(box_c[box], rho_min));
+        const float4 *m = mom + box * NT * B;
+        for (int q = threadIdx.x; q < NT * nj; q += blockDim.x) {
+            const int t = q / nj, j = q - t * nj;
+            if (NS > 1 && !(box_surf[box] & set_surfaces(j0 + j, 1, Bact, NS))) continue;
+            float f = ir;
+            for (int n = c_deg[t]; n > 0; --n) f *= ir;
+            const float4 v = __ldg(m + (int64_t)t * B + j0 + j);
+            const int a = __float_as_int(fmaxf(fabsf(v.x), fabsf(v.y)) * f);
+            const int b = __float_as_int(fmaxf(fabsf(v.z), fabsf(v.w)) * f);
+            // (a NaN loses against the other component in fmaxf; its rows are NaN whatever the scale)
+            if (a > smax[2 * j]) atomicMax(&smax[2 * j], a);
+            if (b > smax[2 * j + 1]) atomicMax(&smax[2 * j + 1], b);
+        }
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < 2 * nj; j += blockDim.x)
+        if (smax[j] > 0) atomicMax(&mx[2 * j0 + j], smax[j]);
 }
 
 // The split moments of every box in stage layout: image[((box * nrc + rc) * NKC + kc)] holds
-// A_hi then A_lo of right-hand sides rc*RC.. and terms kc*16..; rows of right-hand sides at
+// A_hi then A_lo of right-hand sides rc*RC.. and terms kc*32..; rows of right-hand sides at
 // or beyond the active count and terms beyond NT are zero.  One thread per 16 bytes of A_hi.
 template <int P, int RC>
 __global__ void tc_image_kernel(int64_t nbox, int B, int nrc, const float4 *__restrict__ mom,
                                 unsigned char *__restrict__ img, const int *nact,
-                                const int *__restrict__ box_surf, int NS) {
+                                const int *__restrict__ box_surf, int NS, const float4 *__restrict__ box_c,
+                                float rho_min, const int *__restrict__ mx) {
     using S = TcShape<P, RC>;
     constexpr int per_chunk = S::A_CH / 16;
     const int Bact = nact ? *nact : B;
@@ -109,20 +175,24 @@ __global__ void tc_image_kernel(int64_t nbox, int B, int nrc, const float4 *__re
         if (rc * RC >= Bact) continue;   // no right-hand side in use, or none of the box's surfaces: not read
         if (NS > 1 && !(box_surf[box] & set_surfaces(rc * RC, min(RC, Bact - rc * RC), Bact, NS))) continue;
         // e enumerates the part's 16-byte segments in address order
-        const int r = ((e >> 3) / (kKC / 4)) * 8 + (e & 7), k4 = (e >> 3) % (kKC / 4);
-        const int j = rc * RC + (r >> 2), cpt = r & 3;
-        float v[4];
+        const int r = ((e >> 3) / (kKC / 8)) * 8 + (e & 7), k8 = (e >> 3) % (kKC / 8);
+        const int j = rc * RC + (r >> 2), cpt = r & 3, t0 = kc * kKC + 8 * k8;
+        float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (t0 < S::NT && j < Bact) {
+            const float ir = inv_pow2(box_scale(__ldg(box_c + box), rho_min));
+            float f = f16_scale(__ldg(mx + 2 * j + (cpt >> 1))) * ir;
+            int n = 0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int t = kc * kKC + 4 * k4 + u;
-            float x = 0.f;
-            if (t < S::NT && j < Bact) x = __ldg((const float *)(mom + (box * S::NT + t) * B + j) + cpt);
-            v[u] = x;
+            for (int u = 0; u < 8; ++u)
+                if (t0 + u < S::NT) {
+                    for (const int d = c_deg[t0 + u]; n < d; ++n) f *= ir;
+                    v[u] = __ldg((const float *)(mom + (box * S::NT + t0 + u) * B + j) + cpt) * f;
+                }
         }
-        const TfPair sp = tf32_split(make_float4(v[0], v[1], v[2], v[3]));
+        const HalfPair sp = f16_split(v);
         unsigned char *dst = img + c * (2 * S::A_CH) + 16 * e;
-        *(float4 *)dst = sp.hi;
-        *(float4 *)(dst + S::A_CH) = sp.lo;
+        *(uint4 *)dst = sp.hi;
+        *(uint4 *)(dst + S::A_CH) = sp.lo;
     }
 }
 
@@ -131,7 +201,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     m2p_tc_kernel(const int4 *__restrict__ items, int64_t nitems, int B, int nrc, const float4 *__restrict__ tgt,
                   int64_t ntgt, const int2 *__restrict__ list, const float4 *__restrict__ box_c,
                   const unsigned char *__restrict__ img, double *__restrict__ acc, int *counter, int *error,
-                  const int *nact, int nsurf) {
+                  const int *nact, int nsurf, float rho_min, const int *__restrict__ mx) {
     using S = TcShape<P, RC>;
     constexpr int NT = S::NT, NKC = S::NKC, NS = S::NS;
     extern __shared__ __align__(128) unsigned char tc_smem[];
@@ -281,9 +351,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                             }
                             asm volatile("tcgen05.fence::after_thread_sync;");
                             const uint32_t st = sbase + (uint32_t)(s * S::STAGE);
-                            const int ksteps = (min(kKC, NT - kc * kKC) + 7) / 8;
+                            const int ksteps = (min(kKC, NT - kc * kKC) + 15) / 16;
                             for (int ks = 0; ks < ksteps; ++ks) {
-                                const uint32_t off = ks * 256;   // two 16-byte column groups per K step of 8
+                                const uint32_t off = ks * 256;   // two 16-byte column groups per K step of 16
                                 const uint64_t dbh = umma_desc(st + S::OFF_B + off, 128, kChunkSBO);
                                 const uint64_t dbl = umma_desc(st + S::OFF_B + S::B_CH + off, 128, kChunkSBO);
                                 for (int h = 0; h < S::HALVES; ++h) {   // half h into accumulator d + h kTcN
@@ -294,9 +364,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                                     const uint64_t dah = umma_desc(ah + off, 128, kChunkSBO);
                                     const uint64_t dal = umma_desc(ah + S::A_CH + off, 128, kChunkSBO);
                                     const uint32_t dh = d + (uint32_t)(h * kTcN);
-                                    tc_mma(dh, dah, dbh, S::IDESC, on);
-                                    tc_mma(dh, dah, dbl, S::IDESC, 1u);
-                                    if (!S::STACKED) tc_mma(dh, dal, dbh, S::IDESC, 1u);
+                                    tc_mma_f16(dh, dah, dbh, S::IDESC, on);
+                                    tc_mma_f16(dh, dah, dbl, S::IDESC, 1u);
+                                    if (!S::STACKED) tc_mma_f16(dh, dal, dbh, S::IDESC, 1u);
                                 }
                             }
                             tc_commit(smem_addr(&empty_s[s]));
@@ -337,6 +407,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if ((p_parts >> hh & 1) && (32 * qd) % S::ROWS < 4 * hnb) {
                 const int m = (32 * qd + lane) % S::ROWS, j = m >> 2, cpt = m & 3;
                 const int jb = p_b0 + hh * S::HRC + j;   // the right-hand side of row m
+                // both operands' scales undone: 2^-15 for the coefficients, 1 / f16_scale for the moments
+                const float undo = j < hnb ? inv_pow2(f16_scale(__ldg(mx + 2 * jb + (cpt >> 1)))) * 0x1p-15f : 0.f;
 #pragma unroll 1
                 for (int c0 = 0; c0 < kTcN / 2; c0 += 32) {
                     const int64_t tc = p_tbase + half * (kTcN / 2) + c0 + lane;   // this lane's column's target
@@ -358,7 +430,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         for (int x = 0; x < 16; ++x) {
                             const int p = __shfl_sync(0xffffffffu, pc, h16 + x);
                             if (j < hnb && p >= 0)
-                                atomicAdd(acc + 4 * ((int64_t)p * B + jb) + cpt, (double)__uint_as_float(v[x]));
+                                atomicAdd(acc + 4 * ((int64_t)p * B + jb) + cpt, (double)(__uint_as_float(v[x]) * undo));
                         }
                     }
                 }
@@ -404,7 +476,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 const bool on = live && ((e.y >> blk) & 1);   // uniform over the warp but for the tail
                 float a[NT];
                 if (on) {
-                    m2p_recurrence<float, P>(q.x - c.x, q.y - c.y, q.z - c.z, a, [](int, float) {});
+                    const float ir = inv_pow2(box_scale(c, rho_min));
+                    m2p_recurrence<float, P>((q.x - c.x) * ir, (q.y - c.y) * ir, (q.z - c.z) * ir, a,
+                                             [](int, float) {}, 0x1p15f);
                 } else {
 #pragma unroll
                     for (int t = 0; t < NT; ++t) a[t] = 0.f;
@@ -421,19 +495,21 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         break;
                     }
                     unsigned char *bh = tc_smem + s * S::STAGE + S::OFF_B, *bl = bh + S::B_CH;
-                    // four terms per 16-byte store: the eight lanes of a quarter warp fill one
-                    // core matrix, free of bank conflicts
+                    // eight terms per 16-byte store: the eight lanes of a quarter warp fill one
+                    // core matrix, free of bank conflicts; only the columns of the stage's MMAs
+                    const int kmax = min(kKC, (NT - kc * kKC + 15) / 16 * 16);
 #pragma unroll
-                    for (int t4 = 0; t4 < kKC / 4; ++t4) {
-                        float v[4];
+                    for (int t8 = 0; t8 < kKC / 8; ++t8) {
+                        if (8 * t8 >= kmax) break;
+                        float v[8];
 #pragma unroll
-                        for (int w = 0; w < 4; ++w) {
-                            const int t = kc * kKC + 4 * t4 + w;
+                        for (int w = 0; w < 8; ++w) {
+                            const int t = kc * kKC + 8 * t8 + w;
                             v[w] = t < NT ? a[t < NT ? t : 0] : 0.f;
                         }
-                        const TfPair sp = tf32_split(make_float4(v[0], v[1], v[2], v[3]));
-                        *(float4 *)(bh + core_off(tid, 4 * t4)) = sp.hi;
-                        *(float4 *)(bl + core_off(tid, 4 * t4)) = sp.lo;
+                        const HalfPair sp = f16_split(v);
+                        *(uint4 *)(bh + core_off(tid, 8 * t8)) = sp.hi;
+                        *(uint4 *)(bl + core_off(tid, 8 * t8)) = sp.lo;
                     }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();   // one arrival per warp: a thread each would serialise on the barrier
@@ -479,17 +555,23 @@ int tc_launch(lspr_ctx *ctx, double *acc, int *counter, int B) {
     if (!ctx->dev_err.p) return LSPR_E_STATE;
     ctx->tc_launched = true;
     LSPR_TRY(ctx, allow_smem(m2p_tc_kernel<P, RC>, S::SMEM, ctx->device, smem_set));
-    ++ctx->n_launches;   // the image; the caller counts the M2P launch
+    ctx->n_launches += 2;   // scales and image; the caller counts the M2P launch
+    int *mx = (int *)(acc + 4 * ctx->mesh.N * B) + kCounters;   // cleared with the accumulators
+    const dim3 gm((unsigned)std::min<int64_t>(tr.nboxes, 8 * std::max(1, ctx->num_sms)), (B + kMaxSets - 1) / kMaxSets);
+    m2p_max_kernel<<<gm, 256, 0, ctx->stream>>>(tr.nboxes, S::NT, B, Views<float>::mom(ctx),
+                                                         Views<float>::bc(ctx), tr.rho_min, tr.box_used.p, mx,
+                                                         ctx->rhs_nact, tr.box_surf.p, ctx->mesh.S);
     const unsigned gi =
         (unsigned)std::max<int64_t>(1, std::min<int64_t>((segs + 255) / 256, 8 * std::max(1, ctx->num_sms)));
     tc_image_kernel<P, S::HRC><<<gi, 256, 0, ctx->stream>>>(tr.nboxes, B, nrc, Views<float>::mom(ctx),
                                                               ctx->tc_img.p, ctx->rhs_nact, tr.box_surf.p,
-                                                              ctx->mesh.S);
+                                                              ctx->mesh.S, Views<float>::bc(ctx), tr.rho_min, mx);
     const unsigned grid =
         (unsigned)std::max<int64_t>(1, std::min<int64_t>(tr.n_tc_items * nunit, std::max(1, ctx->num_sms)));
     m2p_tc_kernel<P, RC><<<grid, kTcThreads, S::SMEM, ctx->stream>>>(
         tr.tc_items.p, tr.n_tc_items, B, nrc, Views<float>::tgt(ctx), ctx->mesh.N, tr.tc_list.p,
-        Views<float>::bc(ctx), ctx->tc_img.p, acc, counter, ctx->dev_err.p, ctx->rhs_nact, ctx->mesh.S);
+        Views<float>::bc(ctx), ctx->tc_img.p, acc, counter, ctx->dev_err.p, ctx->rhs_nact, ctx->mesh.S, tr.rho_min,
+        mx);
     return LSPR_OK;
 }
 

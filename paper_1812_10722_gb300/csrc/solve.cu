@@ -285,7 +285,7 @@ static int far_part(lspr_ctx *ctx, int mode, const double2 *x, int B) {
     const int S = ctx->mesh.S;
     const int BS = B * S;
     if (tree && !ctx->tree.ready) return LSPR_E_STATE;
-    LSPR_TRY(ctx, ctx->acc.ensure(4 * N * BS + kCounters * sizeof(int) / sizeof(double)));
+    LSPR_TRY(ctx, ctx->acc.ensure(4 * N * BS + acc_tail_ints(BS) / 2));
     int *counters = (int *)(ctx->acc.p + 4 * N * BS);
     const double2 *xt = nullptr;
     const float2 *xtf = nullptr;

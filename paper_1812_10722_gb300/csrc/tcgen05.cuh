@@ -1,8 +1,10 @@
 // tcgen05 / mbarrier building blocks of the tensor-core far-field kernels (inline PTX):
-// shared-memory matrix and instruction descriptors for K-major TF32 operands without swizzle,
-// the TF32 high/low split (both parts rounded to nearest), bounded mbarrier waits and the MMA /
+// shared-memory matrix and instruction descriptors for K-major TF32 and FP16 operands without swizzle,
+// their high/low splits (both parts rounded to nearest), bounded mbarrier waits and the MMA /
 // commit instructions.
 #pragma once
+#include <cuda_fp16.h>
+
 #include <cstdint>
 
 namespace lspr {
@@ -38,6 +40,32 @@ __device__ __forceinline__ TfPair tf32_split(const float4 v) {
     return p;
 }
 
+
+// FP16 split x = hi + lo of eight values, both parts rounded to nearest: within the FP16 range (and
+// down to 2^-2 for x itself) hi + lo holds 22 bits as the TF32 split does, at twice the MMA rate and
+// half the operand bytes; below, |x - hi - lo| <= 2^-25
+struct HalfPair {
+    uint4 hi, lo;
+};
+__device__ __forceinline__ HalfPair f16_split(const float (&v)[8]) {
+    HalfPair p;
+    uint32_t *h = &p.hi.x, *l = &p.lo.x;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const __half2 a = __floats2half2_rn(v[2 * i], v[2 * i + 1]);
+        const float2 b = __half22float2(a);
+        const __half2 c = __floats2half2_rn(v[2 * i] - b.x, v[2 * i + 1] - b.y);
+        h[i] = *(const uint32_t *)&a;
+        l[i] = *(const uint32_t *)&c;
+    }
+    return p;
+}
+// the power of two that brings a largest magnitude (the bits of a non-negative float) into
+// [2^14, 2^15); 1 for infinities and NaN
+__device__ __forceinline__ float f16_scale(int bits) {
+    const int e = bits >> 23;
+    return e >= 255 ? 1.f : __int_as_float(min(254, 268 - e) << 23);
+}
 
 __device__ __forceinline__ uint64_t now_ns() {
     uint64_t t;
@@ -91,6 +119,16 @@ __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint3
 }
 
 
+__device__ __forceinline__ void tc_mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+    asm volatile("{ .reg .pred p; setp.ne.b32 p, %4, 0;\n"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(d),
+                 "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
+}
+
+// instruction descriptor: FP32 accumulator, FP16 A and B, both K-major, N and M
+constexpr uint32_t idesc_f16(int m, int n) {
+    return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+}
 // instruction descriptor: FP32 accumulator, TF32 A and B, both K-major, N and M
 constexpr uint32_t idesc_tf32(int m, int n) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);

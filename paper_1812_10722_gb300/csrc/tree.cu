@@ -876,6 +876,7 @@ int tree_build(lspr_ctx *ctx, double theta, int P, int Ncrit) {
 
     // lists: count
     const double clear = m.Lmax / m.thr + m.rho_max;
+    tr.rho_min = (float)(theta * clear);   // an accepted box is at least clear away
     Tmp<int> cnt3(ctx->scratch[11]), off3(ctx->scratch[12]);
     Tmp<int64_t> tot3(ctx->scratch[13]);
     Tmp<unsigned long long> pairs(ctx->scratch[14]);
