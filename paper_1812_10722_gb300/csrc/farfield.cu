@@ -236,6 +236,159 @@ int launch_ff_boxes(lspr_ctx *ctx) {
     return LSPR_OK;
 }
 
+// ---------------------------------------------- P2P, several right-hand sides in FP32
+// Per tile of kPgTile sources, a block of 64 threads forms G and dG/dn of the 64-target block in shared
+// memory (one target per thread, two sources at a time in packed f32x2 arithmetic) and multiplies them
+// with the tile's weights as two small matrix products, V += G W_V and K += dG/dn W_K: a thread holds
+// 8 targets x RB/2 channels of one layer (RB right-hand sides per chunk: 16, or 8 or 4 where no more are
+// left, as in a solve whose number in use falls), so four shared-memory reads feed 64 multiply-adds.
+// The FP32 pipe's share is 12 + 4 RB operations per pair.  20480 panels (86 M pairs), 16 right-hand
+// sides: 381 us, 476 with two targets per lane and the weights read by broadcast (bound by the
+// shared-memory reads, ten 16-byte reads per 32 packed multiply-adds); four targets per lane and 8
+// right-hand sides took 453 (217 registers, two warps per scheduler).
+constexpr int kPgTile = 32, kPgThreads = 64, kPgRB = 16;
+struct PgSmem {
+    float G[kPgTile][kTargetBlock], T[kPgTile][kTargetBlock];
+    float wv[kPgTile][2 * kPgRB], wk[kPgTile][2 * kPgRB];   // (re, im) per right-hand side
+    float src[6][kPgTile];                                  // -x, -y, -z, normal
+    int pid[kPgTile], tpid[kTargetBlock];
+};
+
+template <int RB, bool CHECK>
+__device__ __forceinline__ void pg_unit(const int4 &item, int B, int b0, int nb, PgSmem &sm, const float4 &q, int64_t t0,
+                                        int64_t ntgt, const float4 *__restrict__ spos,
+                                        const float4 *__restrict__ snrm, const float4 *__restrict__ sw,
+                                        double *__restrict__ acc) {
+    constexpr int NP = RB / 4;   // right-hand sides per thread
+    const int tid = threadIdx.x, tx = tid & 7, layer = tid >> 5, cg = (tid >> 3) & 3;
+    const int tp = panel_of(q.w);
+    const float2 qx = make_float2(q.x, q.x), qy = make_float2(q.y, q.y), qz = make_float2(q.z, q.z);
+    float2 a[8][NP];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int p = 0; p < NP; ++p) a[i][p] = make_float2(0.f, 0.f);
+    for (int base = item.y; base < item.z; base += kPgTile) {
+        const int cnt = min(kPgTile, item.z - base);
+        __syncthreads();   // the previous tile has been read
+        if (tid < kPgTile) {   // past the end: the first source again, with zero weights
+            const int s = base + (tid < cnt ? tid : 0);
+            const float4 p = spos[s], n = snrm[s];
+            sm.src[0][tid] = -p.x; sm.src[1][tid] = -p.y; sm.src[2][tid] = -p.z;
+            sm.src[3][tid] = n.x; sm.src[4][tid] = n.y; sm.src[5][tid] = n.z;
+            sm.pid[tid] = panel_of(n.w);
+        }
+#pragma unroll 4
+        for (int e = tid; e < kPgTile * RB; e += kPgThreads) {
+            const int s = e / RB, j = e - s * RB;
+            const float4 w = s < cnt && j < nb ? sw[(int64_t)(base + s) * B + b0 + j] : zero4<float4>();
+            *(float2 *)&sm.wv[s][2 * j] = make_float2(w.x, w.y);
+            *(float2 *)&sm.wk[s][2 * j] = make_float2(w.z, w.w);
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int s = 0; s < kPgTile; s += 2) {
+            const float2 dx = __fadd2_rn(qx, *(const float2 *)&sm.src[0][s]);
+            const float2 dy = __fadd2_rn(qy, *(const float2 *)&sm.src[1][s]);
+            const float2 dz = __fadd2_rn(qz, *(const float2 *)&sm.src[2][s]);
+            const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+            float2 r = make_float2(rsq(r2.x), rsq(r2.y));
+            if (CHECK) {   // the far-rule terms of the target's own panel are skipped
+                r.x = sm.pid[s] == tp ? 0.f : r.x;
+                r.y = sm.pid[s + 1] == tp ? 0.f : r.y;
+            }
+            const float2 dn = __ffma2_rn(dz, *(const float2 *)&sm.src[5][s],
+                              __ffma2_rn(dy, *(const float2 *)&sm.src[4][s],
+                              __fmul2_rn(dx, *(const float2 *)&sm.src[3][s])));
+            const float2 t = __fmul2_rn(__fmul2_rn(dn, __fmul2_rn(r, r)), r);
+            sm.G[s][tid] = r.x;
+            sm.G[s + 1][tid] = r.y;
+            sm.T[s][tid] = t.x;
+            sm.T[s + 1][tid] = t.y;
+        }
+        __syncthreads();
+        const float (*m)[kTargetBlock] = layer ? sm.T : sm.G;
+        const float (*w)[2 * kPgRB] = layer ? sm.wk : sm.wv;
+#pragma unroll 4
+        for (int s = 0; s < kPgTile; ++s) {
+            const float4 g0 = *(const float4 *)&m[s][4 * tx], g1 = *(const float4 *)&m[s][32 + 4 * tx];
+            const float g[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                const float2 wp = *(const float2 *)&w[s][2 * (NP * cg + p)];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) a[i][p] = __ffma2_rn(make_float2(g[i], g[i]), wp, a[i][p]);
+            }
+        }
+    }
+    // target (i < 4: 4 tx + i, else 28 + 4 tx + i), right-hand side NP cg + p, components 2 layer, + 1
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int t = (i < 4 ? 0 : 28) + 4 * tx + i;
+        if (t0 + t >= ntgt) continue;
+        double *o = acc + 4 * ((int64_t)sm.tpid[t] * B + b0) + 2 * layer;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const int j = NP * cg + p;
+            if (j < nb) {
+                atomicAdd(o + 4 * j, (double)a[i][p].x);
+                atomicAdd(o + 4 * j + 1, (double)a[i][p].y);
+            }
+        }
+    }
+}
+
+template <int RB, class... A>
+__device__ __forceinline__ void pg_check(const int4 &item, A &&...a) {
+    if (item.w & 1) pg_unit<RB, true>(item, a...);
+    else pg_unit<RB, false>(item, a...);
+}
+
+// Work units (item, chunk of kPgRB right-hand sides) from an atomic counter; nothing is done when at
+// least skip_from right-hand sides are in use (the tensor-core P2P then takes the product)
+__global__ void __launch_bounds__(kPgThreads, 8)
+    p2p_multi_kernel(const int4 *__restrict__ items, int64_t nitems, int B, const float4 *__restrict__ tgt, int64_t ntgt,
+                     const float4 *__restrict__ spos, const float4 *__restrict__ snrm, const float4 *__restrict__ sw,
+                     double *__restrict__ acc, int *counter, const int *nact, int skip_from, int S) {
+    __shared__ __align__(16) PgSmem sm;
+    __shared__ int64_t unit_s;
+    const int tid = threadIdx.x;
+    const int Bact = nact ? *nact : B;   // right-hand sides in use (the first Bact slots)
+    if (Bact >= skip_from) return;
+    const int nbc = (Bact + kPgRB - 1) / kPgRB;
+    const int64_t units = nitems * nbc;
+    while (true) {
+        __syncthreads();   // the previous unit's readers are done with unit_s and tpid
+        if (tid == 0) unit_s = atomicAdd(counter, 1);
+        __syncthreads();
+        const int64_t it = unit_s;
+        if (it >= units) return;
+        const int64_t ii = it / nbc;
+        const int b0 = (int)(it - ii * nbc) * kPgRB, nb = min(kPgRB, Bact - b0);
+        const int4 item = __ldg(items + ii);
+        if (S > 1 && !((item.w >> kItemSurf) & set_surfaces(b0, nb, Bact, S))) continue;
+        const int64_t t0 = (int64_t)item.x * kTargetBlock, ti = t0 + tid;
+        const float4 q = ti < ntgt ? tgt[ti] : tgt[0];
+        sm.tpid[tid] = panel_of(q.w);   // read after the tile's barriers
+        if (nb > 8) pg_check<16>(item, B, b0, nb, sm, q, t0, ntgt, spos, snrm, sw, acc);
+        else if (nb > 4) pg_check<8>(item, B, b0, nb, sm, q, t0, ntgt, spos, snrm, sw, acc);
+        else pg_check<4>(item, B, b0, nb, sm, q, t0, ntgt, spos, snrm, sw, acc);
+    }
+}
+
+static int p2p_multi_launch(lspr_ctx *ctx, const int4 *items, int64_t nitems, int B, double *acc, cudaStream_t st,
+                            int *counter, int skip_from = 1 << 30) {
+    static int occ = 0;
+    const int64_t units = nitems * ((B + kPgRB - 1) / kPgRB);
+    const unsigned grid =
+        (unsigned)std::min<int64_t>(units, persistent_grid(ctx, p2p_multi_kernel, kPgThreads, &occ));
+    p2p_multi_kernel<<<grid, kPgThreads, 0, st>>>(items, nitems, B, Views<float>::tgt(ctx), ctx->mesh.N,
+                                                  Views<float>::spos(ctx), Views<float>::snrm(ctx),
+                                                  Views<float>::w(ctx), acc, counter, ctx->rhs_nact, skip_from,
+                                                  ctx->mesh.S);
+    return LSPR_OK;
+}
+
 static int slot_of(int prec, int f32, int f64, int ff) { return prec == PREC_F64 ? f64 : (prec == PREC_FF ? ff : f32); }
 
 int launch_p2p(lspr_ctx *ctx, int prec, const int4 *items, int64_t nitems, double *acc, cudaStream_t st,
@@ -258,14 +411,14 @@ int launch_p2p(lspr_ctx *ctx, int prec, const int4 *items, int64_t nitems, doubl
         const int mn = std::max(2, ctx->tc_p2p_min_rhs);
         if (!ctx->rhs_nact) {
             if (B >= mn) LSPR_TRY_ST(p2p_tc_launch(ctx, acc, st, counter, B, 0));
-            else p2p_launch<float, batch_chunk<float>(2)>(ctx, items, nitems, B, acc, st, counter);
+            else LSPR_TRY_ST(p2p_multi_launch(ctx, items, nitems, B, acc, st, counter));
         } else {
             if (B >= mn) LSPR_TRY_ST(p2p_tc_launch(ctx, acc, st, counter, B, mn));
-            p2p_launch<float, batch_chunk<float>(2)>(ctx, items, nitems, B, acc, st, counter, mn);
+            LSPR_TRY_ST(p2p_multi_launch(ctx, items, nitems, B, acc, st, counter, mn));
         }
     } else {
         if (B == 1) p2p1_launch(ctx, items, nitems, acc, st, counter);
-        else p2p_launch<float, batch_chunk<float>(2)>(ctx, items, nitems, B, acc, st, counter);
+        else LSPR_TRY_ST(p2p_multi_launch(ctx, items, nitems, B, acc, st, counter));
     }
     timer_end_on(ctx, slot, ev, st);
     timer_rhs(ctx, slot, B);
@@ -357,7 +510,7 @@ int launch_p2p_fp32_raw(cudaStream_t st, const int4 *items, int64_t nitems, cons
                         const float4 *spos, const float4 *snrm, const float4 *w, double *acc) {
     if (nitems == 0) return LSPR_OK;
     p2p_kernel<float, 1, false><<<grid_for(nitems, p2p_warps(1)), p2p_warps(1) * 32, 0, st>>>(
-        items, nitems, 1, 1, tgt, ntgt, spos, snrm, w, acc, nullptr, nullptr, 1 << 30, 1);
+        items, nitems, 1, 1, tgt, ntgt, spos, snrm, w, acc, nullptr, nullptr, 1);
     return cudaGetLastError() == cudaSuccess ? LSPR_OK : LSPR_E_CUDA;
 }
 

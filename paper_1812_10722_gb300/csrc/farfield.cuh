@@ -149,22 +149,21 @@ __device__ __forceinline__ void p2p_range(int beg, int end, int lane, int B, int
 
 // Work units: (item, right-hand-side chunk), item = (target block, source begin, source
 // end, own-panel flag); one per warp.  DYNAMIC: a persistent grid whose warps take units
-// from an atomic counter.  acc is [panel][B][4].  The kernel does nothing when at least
-// skip_from right-hand sides are in use (the tensor-core P2P then takes the product).
+// from an atomic counter.  acc is [panel][B][4].  FP32 products of several right-hand sides take
+// p2p_multi_kernel (farfield.cu) instead.
 template <typename T, int NB, bool DYNAMIC>
 __global__ void __launch_bounds__(p2p_warps(NB) * 32)
     p2p_kernel(const int4 *__restrict__ items, int64_t nitems, int nbc, int B,
                const typename Vec4<T>::type *__restrict__ tgt, int64_t ntgt,
                const typename Vec4<T>::type *__restrict__ spos, const typename Vec4<T>::type *__restrict__ snrm,
                const typename Vec4<T>::type *__restrict__ sw, double *__restrict__ acc, int *counter,
-               const int *nact, int skip_from, int S) {
+               const int *nact, int S) {
     using T4 = typename Vec4<T>::type;
     constexpr int W = p2p_warps(NB);
     __shared__ T4 sh[W][2][32];
     __shared__ T4 shw[W][32][NB];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int Bact = nact ? *nact : B;   // right-hand sides in use (the first Bact slots)
-    if (Bact >= skip_from) return;       // the tensor-core P2P takes this product
     nbc = (Bact + NB - 1) / NB;
     const int64_t units = nitems * nbc;
     int64_t it = (int64_t)blockIdx.x * W + warp;
@@ -970,7 +969,7 @@ template <> struct Views<ffloat> {
 
 template <typename T, int NB>
 static void p2p_launch(lspr_ctx *ctx, const int4 *items, int64_t nitems, int B, double *acc, cudaStream_t st,
-                       int *counter, int skip_from = 1 << 30) {
+                       int *counter) {
     static int occ = 0;
     constexpr int W = p2p_warps(NB);
     const int nbc = (B + NB - 1) / NB;
@@ -978,7 +977,7 @@ static void p2p_launch(lspr_ctx *ctx, const int4 *items, int64_t nitems, int B, 
                                              persistent_grid(ctx, p2p_kernel<T, NB, true>, W * 32, &occ));
     p2p_kernel<T, NB, true><<<grid, W * 32, 0, st>>>(items, nitems, nbc, B, Views<T>::tgt(ctx), ctx->mesh.N,
                                                       Views<T>::spos(ctx), Views<T>::snrm(ctx), Views<T>::w(ctx),
-                                                      acc, counter, ctx->rhs_nact, skip_from, ctx->mesh.S);
+                                                      acc, counter, ctx->rhs_nact, ctx->mesh.S);
 }
 
 // the packed single-right-hand-side P2P (FP32)
