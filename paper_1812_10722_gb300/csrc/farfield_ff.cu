@@ -15,7 +15,7 @@ namespace {
 // right-hand sides per float-float P2P work unit: 95.9 ms per 64-right-hand-side product on the
 // 81920-panel sphere's tree (theta 0.4, P 7, Ncrit 512) against 120.6 ms for chunks of 4 and
 // 281.6 ms for the two-targets-per-lane kernel with chunks of 2; chunks of 16 spill (162
-// registers at 8)
+// registers at 8 before the channels were packed)
 constexpr int kFfP2PChunk = 8;
 
 // one term k of the table: distances u - index(k - e_d) and u - index(k - 2 e_d) to the term's
@@ -62,12 +62,119 @@ __host__ __device__ inline size_t ff_m2p_smem(int TP, int W, int NB) {
     return (size_t)TP * NB * sizeof(ff4) + 2 * (size_t)W * 32 * sizeof(ffloat);
 }
 
+// a ff4 with its parts grouped for ff_mac2: (x.hi, y.hi, x.lo, y.lo), (z.hi, w.hi, z.lo, w.lo)
+struct __align__(16) ff4p {
+    float4 xy, zw;
+};
+__device__ __forceinline__ ff4p packed(const ff4 &m) {
+    return {make_float4(m.x.hi, m.y.hi, m.x.lo, m.y.lo), make_float4(m.z.hi, m.w.hi, m.z.lo, m.w.lo)};
+}
+// the two channels of each layer of one right-hand side += f m
+__device__ __forceinline__ void mac4(ff2 (&a)[2], float2 fh, float2 nfh, float2 fl, const ff4p &m) {
+    ff_mac2(a[0], fh, nfh, fl, make_float2(m.xy.x, m.xy.y), make_float2(m.xy.z, m.xy.w));
+    ff_mac2(a[1], fh, nfh, fl, make_float2(m.zw.x, m.zw.y), make_float2(m.zw.z, m.zw.w));
+}
+__device__ __forceinline__ double ff2_x(const ff2 &a) { return (double)a.hi.x + (double)a.lo.x; }
+__device__ __forceinline__ double ff2_y(const ff2 &a) { return (double)a.hi.y + (double)a.lo.y; }
+
+// One work unit for up to NB right-hand sides; see m2p_ff_kernel
+template <int NB>
+__device__ __forceinline__ void m2p_ff_unit(const int4 &item, int B, int b0, int nb, int um, int NT,
+                                            const ff4 *__restrict__ tgt, int64_t ntgt, const int *__restrict__ list,
+                                            const ff4 *__restrict__ box_c, const ff4 *__restrict__ mom,
+                                            double *__restrict__ acc, int W, int TP,
+                                            const int *__restrict__ box_surf, int S, ff4p *sm, ffloat *sa) {
+    const int h = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t ti = (int64_t)item.x * kTargetBlock + lane + 32 * h;
+    const ff4 q = ti < ntgt ? tgt[ti] : tgt[0];
+    ff2 a[NB][2];
+#pragma unroll
+    for (int j = 0; j < NB; ++j)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) a[j][c].hi = a[j][c].lo = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int l = item.y; l < item.z; ++l) {
+        const int b = __ldg(list + l);
+        if (S > 1 && !(box_surf[b] & um)) continue;
+        const ff4 c = box_c[b];
+        // terms t0 .. t0 + TP - 1 of the box's moments into sm (the whole block, at the same t)
+        auto stage = [&](int t0) {
+            __syncthreads();   // the previous part's moments are no longer read
+            const int nq = min(TP, NT - t0) * NB;
+            for (int q2 = threadIdx.x; q2 < nq; q2 += 64) {
+                const int t = q2 / NB, j = q2 - t * NB;
+                sm[q2] = packed(j < nb ? mom[((int64_t)b * NT + t0 + t) * B + b0 + j] : zero4<ff4>());
+            }
+            __syncthreads();
+        };
+        stage(0);
+        const ffloat d[3] = {q.x - c.x, q.y - c.y, q.z - c.z};
+        const ffloat r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+        const ffloat a0 = rsq(r2);
+        const ffloat ir2 = a0 * a0;
+        const ffloat R[3] = {d[0] * ir2, d[1] * ir2, d[2] * ir2};
+        ffloat kap(0.f, 0.f);   // kappa_n / |R|^2 of the current degree n
+        int n = 0, tn = 1;      // degree, first term of the next one
+        sa[lane] = a0;
+        int su = 0;      // slot of term t
+        int tpart = 0;   // first term of the staged part
+        {
+            const float2 fh = both(a0.hi), nfh = both(-a0.hi), fl = both(a0.lo);
+#pragma unroll
+            for (int j = 0; j < NB; ++j) mac4(a[j], fh, nfh, fl, sm[j]);
+        }
+#pragma unroll 1
+        for (int t = 1; t < NT; ++t) {
+            if (t == tpart + TP) stage(tpart = t);
+            if (t == tn) {
+                ++n;
+                tn = (n + 1) * (n + 1);
+                kap = ffloat(c_ff_terms.kh[n], c_ff_terms.kl[n]) * ir2;
+            }
+            const FfTerm &e = c_ff_terms.t[t];
+            su = su + 1 == W ? 0 : su + 1;
+            ffloat at(0.f, 0.f);
+            if (e.d2[0] | e.d2[1]) {
+                ffloat s2(0.f, 0.f);
+#pragma unroll
+                for (int x = 0; x < 2; ++x)
+                    if (e.d2[x]) {
+                        const int sl = su - e.d2[x];
+                        s2 += sa[(sl < 0 ? sl + W : sl) * 32 + lane];
+                    }
+                at = kap * s2;
+            }
+#pragma unroll
+            for (int x = 0; x < 3; ++x)
+                if (e.d1[x]) {
+                    const int sl = su - e.d1[x];
+                    at += R[x] * sa[(sl < 0 ? sl + W : sl) * 32 + lane];
+                }
+            sa[su * 32 + lane] = at;
+            const float2 fh = both(at.hi), nfh = both(-at.hi), fl = both(at.lo);
+#pragma unroll
+            for (int j = 0; j < NB; ++j) mac4(a[j], fh, nfh, fl, sm[(t - tpart) * NB + j]);
+        }
+    }
+    if (ti < ntgt) {
+        const int64_t tp = panel_of(q.w);
+#pragma unroll
+        for (int j = 0; j < NB; ++j)
+            if (j < nb)
+                atomic_add4(acc + 4 * (tp * B + b0 + j), ff2_x(a[j][0]), ff2_y(a[j][0]), ff2_x(a[j][1]),
+                            ff2_y(a[j][1]));
+    }
+}
+
 // Work units and accumulation as in m2p_kernel; NT = n_terms(P) at run time.  A block of two
 // warps takes a unit: warp h the targets 32 h .. 32 h + 31 of the 64-target block, both on the
 // same boxes, so each box's moments are staged once for the two, in parts of TP terms (the
 // launcher picks TP so that more blocks fit per SM).  The recurrence is rolled (each lane's
 // coefficients live in its column of the warp's ring), and the contraction accumulates with
-// ff_mac.
+// ff_mac2, the real and imaginary channel at once.  A unit takes the narrowest of NB, NB / 2 and
+// NB / 4 that holds its right-hand sides (the contraction is 9/10 of the work).  Issue-bound.
+// 40500 panels, 12 right-hand sides: 11.7 ms, 15.0 with units of eight and scalar parts (20480 panels,
+// 16: 4.32 after 4.63).
 template <int NB>
 __global__ void __launch_bounds__(64)
     m2p_ff_kernel(const int4 *__restrict__ items, int64_t nitems, int nbc, int B, int NT,
@@ -76,9 +183,8 @@ __global__ void __launch_bounds__(64)
                   const int *nact, int W, int TP, const int *__restrict__ box_surf, int S) {
     extern __shared__ __align__(16) unsigned char ff_smem[];
     __shared__ int64_t unit;
-    const int h = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    ff4 *sm = (ff4 *)ff_smem;
-    ffloat *sa = (ffloat *)(sm + TP * NB) + (size_t)h * W * 32;   // sa[(t mod W) * 32 + lane]
+    ff4p *sm = (ff4p *)ff_smem;
+    ffloat *sa = (ffloat *)(sm + TP * NB) + (size_t)(threadIdx.x >> 5) * W * 32;   // sa[(t mod W) * 32 + lane]
     const int Bact = nact ? *nact : B;   // right-hand sides in use (the first Bact slots)
     nbc = (Bact + NB - 1) / NB;
     const int64_t units = nitems * nbc;
@@ -92,93 +198,14 @@ __global__ void __launch_bounds__(64)
         const int b0 = (int)(it - ii * nbc) * NB, nb = min(NB, Bact - b0);
         const int um = set_surfaces(b0, nb, Bact, S);
         const int4 item = __ldg(items + ii);
-        const int64_t ti = (int64_t)item.x * kTargetBlock + lane + 32 * h;
-        const ff4 q = ti < ntgt ? tgt[ti] : tgt[0];
-        ffloat a[NB][4];
-#pragma unroll
-        for (int j = 0; j < NB; ++j)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) a[j][c] = ffloat(0.f, 0.f);
-#pragma unroll 1
-        for (int l = item.y; l < item.z; ++l) {
-            const int b = __ldg(list + l);
-            if (S > 1 && !(box_surf[b] & um)) continue;
-            const ff4 c = box_c[b];
-            // terms t0 .. t0 + TP - 1 of the box's moments into sm (the whole block, at the same t)
-            auto stage = [&](int t0) {
-                __syncthreads();   // the previous part's moments are no longer read
-                const int nq = min(TP, NT - t0) * NB;
-                for (int q2 = threadIdx.x; q2 < nq; q2 += 64) {
-                    const int t = q2 / NB, j = q2 - t * NB;
-                    sm[q2] = j < nb ? mom[((int64_t)b * NT + t0 + t) * B + b0 + j] : zero4<ff4>();
-                }
-                __syncthreads();
-            };
-            stage(0);
-            const ffloat d[3] = {q.x - c.x, q.y - c.y, q.z - c.z};
-            const ffloat r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-            const ffloat a0 = rsq(r2);
-            const ffloat ir2 = a0 * a0;
-            const ffloat R[3] = {d[0] * ir2, d[1] * ir2, d[2] * ir2};
-            ffloat kap(0.f, 0.f);   // kappa_n / |R|^2 of the current degree n
-            int n = 0, tn = 1;      // degree, first term of the next one
-            sa[lane] = a0;
-            int su = 0;   // slot of term t
-            int tpart = 0;   // first term of the staged part
-#pragma unroll
-            for (int j = 0; j < NB; ++j) {
-                const ff4 m = sm[j];
-                ff_mac(a[j][0], a0, m.x);
-                ff_mac(a[j][1], a0, m.y);
-                ff_mac(a[j][2], a0, m.z);
-                ff_mac(a[j][3], a0, m.w);
-            }
-#pragma unroll 1
-            for (int t = 1; t < NT; ++t) {
-                if (t == tpart + TP) stage(tpart = t);
-                if (t == tn) {
-                    ++n;
-                    tn = (n + 1) * (n + 1);
-                    kap = ffloat(c_ff_terms.kh[n], c_ff_terms.kl[n]) * ir2;
-                }
-                const FfTerm &e = c_ff_terms.t[t];
-                su = su + 1 == W ? 0 : su + 1;
-                ffloat at(0.f, 0.f);
-                if (e.d2[0] | e.d2[1]) {
-                    ffloat s2(0.f, 0.f);
-#pragma unroll
-                    for (int x = 0; x < 2; ++x)
-                        if (e.d2[x]) {
-                            const int sl = su - e.d2[x];
-                            s2 += sa[(sl < 0 ? sl + W : sl) * 32 + lane];
-                        }
-                    at = kap * s2;
-                }
-#pragma unroll
-                for (int x = 0; x < 3; ++x)
-                    if (e.d1[x]) {
-                        const int sl = su - e.d1[x];
-                        at += R[x] * sa[(sl < 0 ? sl + W : sl) * 32 + lane];
-                    }
-                sa[su * 32 + lane] = at;
-#pragma unroll
-                for (int j = 0; j < NB; ++j) {
-                    const ff4 m = sm[(t - tpart) * NB + j];
-                    ff_mac(a[j][0], at, m.x);
-                    ff_mac(a[j][1], at, m.y);
-                    ff_mac(a[j][2], at, m.z);
-                    ff_mac(a[j][3], at, m.w);
-                }
-            }
-        }
-        if (ti < ntgt) {
-            const int64_t tp = panel_of(q.w);
-#pragma unroll
-            for (int j = 0; j < NB; ++j)
-                if (j < nb)
-                    atomic_add4(acc + 4 * (tp * B + b0 + j), (double)a[j][0], (double)a[j][1], (double)a[j][2],
-                                (double)a[j][3]);
-        }
+        if (NB < 4 || nb > NB / 2)
+            m2p_ff_unit<NB>(item, B, b0, nb, um, NT, tgt, ntgt, list, box_c, mom, acc, W, TP, box_surf, S, sm, sa);
+        else if (nb > NB / 4)
+            m2p_ff_unit<(NB < 4 ? 1 : NB / 2)>(item, B, b0, nb, um, NT, tgt, ntgt, list, box_c, mom, acc, W, TP, box_surf, S,
+                                              sm, sa);
+        else
+            m2p_ff_unit<(NB < 4 ? 1 : NB / 4)>(item, B, b0, nb, um, NT, tgt, ntgt, list, box_c, mom, acc, W, TP, box_surf, S,
+                                              sm, sa);
     }
 }
 
@@ -230,13 +257,65 @@ int m2p_ff_launch(lspr_ctx *ctx, double *acc, int *counter, int B) {
 // the two-targets-per-lane kernel.  Sources are staged per warp in chunks of 32 and read by
 // broadcast; sums and the own-panel rule are those of p2p_kernel.
 constexpr int kFfP2PWarps = 4;
+template <int NBW, int NB>
+__device__ __forceinline__ void p2p_ff1_unit(const int4 &item, int B, int b0, int nb, int64_t t,
+                                             const ff4 *__restrict__ tgt, int64_t ntgt, const ff4 *__restrict__ spos,
+                                             const ff4 *__restrict__ snrm, const ff4 *__restrict__ sw,
+                                             double *__restrict__ acc, ff4 (*sh)[32], ff4p (*shw)[NB]) {
+    const int lane = threadIdx.x & 31;
+    const ff4 q = t < ntgt ? tgt[t] : tgt[0];
+    const int tp = panel_of(q.w);
+    ff2 a[NBW][2];
+#pragma unroll
+    for (int k = 0; k < NBW; ++k)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) a[k][c].hi = a[k][c].lo = make_float2(0.f, 0.f);
+    for (int base = item.y; base < item.z; base += 32) {
+        const int s = base + lane;
+        if (s < item.z) {
+            sh[0][lane] = spos[s];
+            sh[1][lane] = snrm[s];
+#pragma unroll
+            for (int k = 0; k < NBW; ++k)
+                shw[lane][k] = packed(k < nb ? sw[(int64_t)s * B + b0 + k] : zero4<ff4>());
+        }
+        __syncwarp();
+        const int cnt = min(32, item.z - base);
+#pragma unroll 2
+        for (int kk = 0; kk < cnt; ++kk) {
+            const ff4 p = sh[0][kk], n = sh[1][kk];
+            const ffloat dx = q.x - p.x, dy = q.y - p.y, dz = q.z - p.z;
+            ffloat r = rsq(dx * dx + dy * dy + dz * dz);
+            if ((item.w & 1) && panel_of(n.w) == tp) r = ffloat(0.f, 0.f);
+            const ffloat tk = (dx * n.x + dy * n.y + dz * n.z) * (r * r) * r;
+            const float2 rh = both(r.hi), nrh = both(-r.hi), rl = both(r.lo);
+            const float2 th = both(tk.hi), nth = both(-tk.hi), tl = both(tk.lo);
+#pragma unroll
+            for (int k = 0; k < NBW; ++k) {
+                const ff4p w = shw[kk][k];
+                ff_mac2(a[k][0], rh, nrh, rl, make_float2(w.xy.x, w.xy.y), make_float2(w.xy.z, w.xy.w));
+                ff_mac2(a[k][1], th, nth, tl, make_float2(w.zw.x, w.zw.y), make_float2(w.zw.z, w.zw.w));
+            }
+        }
+        __syncwarp();
+    }
+    if (t < ntgt) {
+#pragma unroll
+        for (int k = 0; k < NBW; ++k)
+            if (k < nb)
+                atomic_add4(acc + 4 * ((int64_t)tp * B + b0 + k), ff2_x(a[k][0]), ff2_y(a[k][0]), ff2_x(a[k][1]),
+                            ff2_y(a[k][1]));
+    }
+}
+
+// 40500 panels, 12 right-hand sides: 7.88 ms, 9.52 with units of eight and scalar parts.
 template <int NB>
 __global__ void __launch_bounds__(kFfP2PWarps * 32)
     p2p_ff1_kernel(const int4 *__restrict__ items, int64_t nitems, int B, const ff4 *__restrict__ tgt, int64_t ntgt,
                    const ff4 *__restrict__ spos, const ff4 *__restrict__ snrm, const ff4 *__restrict__ sw,
                    double *__restrict__ acc, int *counter, const int *nact, int S) {
     __shared__ ff4 sh[kFfP2PWarps][2][32];
-    __shared__ ff4 shw[kFfP2PWarps][32][NB];
+    __shared__ ff4p shw[kFfP2PWarps][32][NB];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int Bact = nact ? *nact : B;
     const int nbc = (Bact + NB - 1) / NB;
@@ -252,48 +331,11 @@ __global__ void __launch_bounds__(kFfP2PWarps * 32)
         const int4 item = __ldg(items + ii);
         if (S > 1 && !((item.w >> kItemSurf) & set_surfaces(b0, nb, Bact, S))) continue;
         const int64_t t = (int64_t)item.x * kTargetBlock + 32 * h + lane;
-        const ff4 q = t < ntgt ? tgt[t] : tgt[0];
-        const int tp = panel_of(q.w);
-        ffloat a[NB][4];
-#pragma unroll
-        for (int k = 0; k < NB; ++k)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) a[k][c] = ffloat(0.f, 0.f);
-        for (int base = item.y; base < item.z; base += 32) {
-            const int s = base + lane;
-            if (s < item.z) {
-                sh[warp][0][lane] = spos[s];
-                sh[warp][1][lane] = snrm[s];
-#pragma unroll
-                for (int k = 0; k < NB; ++k) shw[warp][lane][k] = k < nb ? sw[(int64_t)s * B + b0 + k] : zero4<ff4>();
-            }
-            __syncwarp();
-            const int cnt = min(32, item.z - base);
-#pragma unroll 2
-            for (int kk = 0; kk < cnt; ++kk) {
-                const ff4 p = sh[warp][0][kk], n = sh[warp][1][kk];
-                const ffloat dx = q.x - p.x, dy = q.y - p.y, dz = q.z - p.z;
-                ffloat r = rsq(dx * dx + dy * dy + dz * dz);
-                if ((item.w & 1) && panel_of(n.w) == tp) r = ffloat(0.f, 0.f);
-                const ffloat tk = (dx * n.x + dy * n.y + dz * n.z) * (r * r) * r;
-#pragma unroll
-                for (int k = 0; k < NB; ++k) {
-                    const ff4 w = shw[warp][kk][k];
-                    ff_mac(a[k][0], r, w.x);
-                    ff_mac(a[k][1], r, w.y);
-                    ff_mac(a[k][2], tk, w.z);
-                    ff_mac(a[k][3], tk, w.w);
-                }
-            }
-            __syncwarp();
-        }
-        if (t < ntgt) {
-#pragma unroll
-            for (int k = 0; k < NB; ++k)
-                if (k < nb)
-                    atomic_add4(acc + 4 * ((int64_t)tp * B + b0 + k), (double)a[k][0], (double)a[k][1],
-                                (double)a[k][2], (double)a[k][3]);
-        }
+        // the narrowest of NB and NB / 2 that holds the unit's right-hand sides
+        if (nb > NB / 2)
+            p2p_ff1_unit<NB, NB>(item, B, b0, nb, t, tgt, ntgt, spos, snrm, sw, acc, sh[warp], shw[warp]);
+        else
+            p2p_ff1_unit<NB / 2, NB>(item, B, b0, nb, t, tgt, ntgt, spos, snrm, sw, acc, sh[warp], shw[warp]);
     }
 }
 

@@ -76,6 +76,29 @@ __device__ __forceinline__ void ff_mac(ffloat &acc, const ffloat &a, const ffloa
     acc.lo = __fadd_rn(acc.lo, __fadd_rn(e, pe));
 }
 
+// Two float-float values side by side, their parts packed (f32x2): the operations of ff_mac in half
+// the instructions.  The FP32 pipe takes the same time, but the issue slots it leaves go to the
+// loads and address arithmetic around it.
+struct ff2 {
+    float2 hi, lo;
+};
+// acc += a b elementwise with a = (ah, al) given as one factor for both and nah = -ah; every rounding
+// is that of ff_mac (a difference x - y is the fused -1 y + x, rounded once)
+__device__ __forceinline__ void ff_mac2(ff2 &acc, float2 ah, float2 nah, float2 al, float2 bh, float2 bl) {
+    const float2 m1 = make_float2(-1.f, -1.f);
+    const float2 np = __fmul2_rn(nah, bh);                  // -p
+    float2 pe = __ffma2_rn(ah, bh, np);                     // exact error of p
+    pe = __ffma2_rn(ah, bl, pe);
+    pe = __ffma2_rn(al, bh, pe);
+    const float2 s = __ffma2_rn(np, m1, acc.hi);            // acc.hi + p
+    const float2 v = __ffma2_rn(acc.hi, m1, s);
+    const float2 t = __ffma2_rn(__ffma2_rn(v, m1, s), m1, acc.hi);   // acc.hi - (s - v)
+    const float2 e = __ffma2_rn(__fadd2_rn(np, v), m1, t);           // + (p - v)
+    acc.hi = s;
+    acc.lo = __fadd2_rn(acc.lo, __fadd2_rn(e, pe));
+}
+__device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
+
 __device__ __forceinline__ ffloat &operator+=(ffloat &x, const ffloat &y) { return x = x + y; }
 __device__ __forceinline__ ffloat &operator-=(ffloat &x, const ffloat &y) { return x = x - y; }
 __device__ __forceinline__ ffloat &operator*=(ffloat &x, const ffloat &y) { return x = x * y; }
