@@ -546,6 +546,17 @@ __global__ void arn_precond_setup_kernel(int64_t N, int BS, const double *Vself,
     if (t < BS) pq[t] = cdiv(make_double2(1.0, 0.0), make_double2(1.0 + s[t].x, s[t].y));
 }
 
+// the scales that the tensor-core launches carry by value (powers of two) and their operand parts
+uint64_t tc_scales(const Tree &tr) {
+    uint64_t k = tr.tcp_f16 ? 1 : 0;
+    for (const float f : {tr.rho_min, tr.tcp_gs, tr.tcp_ts}) {
+        uint32_t b;
+        std::memcpy(&b, &f, sizeof(b));
+        k = k << 9 | b >> 23;
+    }
+    return k;
+}
+
 int small_kernel_warps(int B, int m) {
     const int by_smem = (int)(45000 / tail_smem_per_warp(m));
     return std::max(1, std::min({B, kMaxWarpsSmall, by_smem}));
@@ -857,7 +868,8 @@ int gmres_graph_solve(lspr_ctx *ctx, int mode, int B, int m, int maxiter, double
                             (uint64_t)tr.n_m2p_items, (uint64_t)tr.n_p2m_items,
                             (uint64_t)direct_items(ctx, (int64_t)B * me.S).n,
                             (uint64_t)(uintptr_t)ctx->gm_V.p, (uint64_t)ctx->num_sms, (uint64_t)me.S,
-                            (uint64_t)ctx->tensor_cores, (uint64_t)tr.n_tc_items, (uint64_t)tr.n_tcp_items};
+                            (uint64_t)ctx->tensor_cores | tc_scales(tr) << 8, (uint64_t)tr.n_tc_items,
+                            (uint64_t)tr.n_tcp_items};
         GraphCache *gc = nullptr;
         const bool graphs = ctx->use_graphs && !ctx->timing.enabled;
         for (GraphCache &c : ctx->gcache)

@@ -44,7 +44,8 @@ constexpr int kTargetBlock = 64;                       // targets per interactio
 constexpr int kTcGroup = 4;        // target blocks per tensor-core M2P group (256 targets)
 constexpr int kTcGroupSeg = 32;    // boxes per tensor-core M2P work unit at most
 constexpr int kTcP2PSrc = 2048;    // sources per tensor-core P2P work unit at most
-constexpr int kTcSrcRows = 8;      // tensor-core P2P source geometry per eight sources: rows -x, -y, -z, normal, panel, -
+constexpr int kTcSrcRows = 8;      // tensor-core P2P source geometry per stage: rows -x, -y, -z, normal, panel, -
+constexpr float kTcP2PRange = 4096.f;   // largest ratio of P2P distances for FP16 parts
 constexpr int kTcSurf = 8;         // tensor-core M2P list entry.y: block mask, from this bit the box's surfaces
 constexpr int kMaxP = 8;                               // highest Taylor order compiled
 constexpr int kMaxDepth = 10;                          // octree levels below the root (10 bits per axis)
@@ -183,8 +184,11 @@ struct Tree {
     // ranges cut at every range end, each piece with the mask of the blocks that sum it
     DArr<int4> tcp_items;    // (group, interval begin, interval end, 0)
     DArr<int4> tcp_ivl;      // (source begin, source end, block mask, surface mask)
-    DArr<int> tcp_mask8;     // several surfaces: [eight sources] the surface masks of the ranges that hold them
-    DArr<float> tcp_src8;    // [eight sources][kTcSrcRows][8] their geometry
+    DArr<int> tcp_mask;      // several surfaces: [stage's sources] the surface masks of the ranges that hold them
+    DArr<float> tcp_src;     // [stage's sources][kTcSrcRows][sources] their geometry, scaled
+    DArr<int> tcp_stat;      // bits of the smallest and largest squared P2P distance, the largest source weight
+    bool tcp_f16 = false;    // FP16 parts (16 sources per stage) rather than TF32 (8)
+    float tcp_gs = 1.f, tcp_ts = 1.f;   // scales of G and dG/dn
     int64_t n_tcp_items = 0, n_tcp_ivl = 0, n_tcp_sources = 0, n_tcp_stages = 0;   // stages of 8 sources
     bool tc_built = false, tcp_built = false;   // the group lists above match the tree
     DArr<int4> p2m_items;    // (leaf, source begin, source end, 0): leaves under an accepted box
@@ -426,7 +430,7 @@ int launch_p2m(lspr_ctx *ctx, int prec, int B);
 // behind the accumulators of a product, cleared with them: the work-item counters, then per layer and
 // channel set the largest magnitudes that scale the tensor-core operands
 constexpr int kCounters = 8;
-inline int64_t acc_tail_ints(int64_t BS) { return kCounters + (2 * BS + 3) / 4 * 4; }
+inline int64_t acc_tail_ints(int64_t BS) { return kCounters + 4 * BS; }   // M2P's, then P2P's
 int launch_m2p(lspr_ctx *ctx, int prec, double *acc, int *counter, int B);
 // float-float copies of the work-order geometry / box centres
 int launch_ff_geometry(lspr_ctx *ctx);

@@ -7,37 +7,50 @@
 //   D_V[channel][target] += W_V[channel][source] G[source][target]
 //   D_K[channel][target] += W_K[channel][source] dG/dn[source][target]
 // with the channels (re and im of each of up to 64 right-hand sides: 128 rows) as the MMA's M,
-// the 256 targets of a group of four consecutive 64-target blocks as its N, and 8 sources per
+// the 256 targets of a group of four consecutive 64-target blocks as its N, and the sources of a
 // pipeline stage as its K.  W_V holds only single-layer weights and W_K only double-layer ones,
 // so no operand carries structural zeros, and one kernel tile serves 64 right-hand sides.
 // The group walks the union of its blocks' P2P source ranges; a target whose block does not sum
 // a range gets zero kernel values there, and a target's own panel is skipped (its exact integral
-// is in the near correction), as in p2p_kernel.  Both operands are split into TF32 high and low
+// is in the near correction), as in p2p_kernel.  Both operands are split into high and low
 // parts (each rounded to nearest) with FP32 accumulation in tensor memory: with more than 32
 // right-hand sides in the unit, three MMAs per operand pair give W_hi G_hi + W_hi G_lo +
-// W_lo G_hi (3xTF32); with at most 32,
+// W_lo G_hi; with at most 32,
 // W_hi and W_lo are the two halves of one 128-row operand and two MMAs give all four products
 // (the epilogue adds both halves).
 //
-// The split weights are formed once per product in operand layout (p2p_image_kernel: 16 KB per eight
-// consecutive sources and 64 right-hand sides), so that staging them is one bulk copy; stages are
-// therefore aligned to multiples of eight sources, and a range that begins or ends inside one gets
+// The parts are FP16 (16 sources per stage) where the kernel values' range allows it, else TF32 (8
+// sources; FP16 parts hold the same 22 bits at twice the rate).  The smallest and the largest distance
+// of a P2P pair (pair_range_kernel, once per tree) set powers of two that bring G and dG/dn (at most
+// 1/r and 1/r^2) below 2^15.  With their ratio at most kTcP2PRange = 4096, G stays above 2^3 and loses
+// nothing; dG/dn falls to 2^-9 at the largest distances, where its parts keep 2^-25 absolute: summed
+// over the sources of a P2P region of area a that is below 2^-40 a / r_min^2 of a potential of order 2 pi
+// (2^-27 at a = 10 nm^2, r_min = 0.04 nm), less than the accumulation rounds off.  The weights of one
+// right-hand side and layer are scaled by a bound of their largest magnitude.  All scales are powers of
+// two: those of G and dG/dn are folded into the positions and normals, all are undone as the
+// accumulators are drained.
+//
+// The split weights are formed once per product in operand layout (p2p_image_kernel: 16 KB per stage's
+// sources and 64 right-hand sides), so that staging them is one bulk copy; stages are
+// therefore aligned to multiples of their sources, and a range that begins or ends inside one gets
 // zero kernel values for the rest.
 //
 // Roles (persistent, one CTA per SM, both accumulators in the SM's 512 tensor-memory columns):
 //   warp 16 (one lane) fetches work units into a small ring and bulk-copies every stage's inputs
-//     (the weight operands, and the positions and normals of its eight sources);
-//   warps 0-15 (two threads per target of the group, four of the stage's eight sources each)
+//     (the weight operands, and the positions and normals of its sources);
+//   warps 0-15 (two threads per target of the group, half of the stage's sources each)
 //     generate G and dG/dn of every stage in registers, two sources at a time in packed f32x2
 //     arithmetic, split them and write the B operands; after the first
 //     stage of the next unit they drain the finished unit's accumulators (tcgen05.ld) into the
 //     FP64 accumulators;
 //   warp 17 (one lane) issues the MMAs of each stage once it is written, commits to the stage's
 //     "empty" barrier and, at the end of a unit, to the accumulator barrier.
-// 81920 panels, 64 right-hand sides: 3.44 ms with the image (0.15), 4.24 with the weights split by four
-// of the generating warps (which every stage waited for) and a barrier arrival per thread.  A stage
-// takes 0.86 us against 0.48 of its six MMAs and about as much of its 121 KB of shared-memory
-// traffic (operand reads, generated operands, copies).
+// 81920 panels, 64 right-hand sides, with the preparing kernels: 2.19 ms; 3.44 with TF32 parts (a stage
+// of 8 sources took 0.86 us, 0.48 of it the MMAs and as much its 121 KB of shared-memory traffic; FP16
+// halves both per source); 4.24 with the weights split by four of the generating warps (which every
+// stage waited for) and a barrier arrival per thread.  Error of the product of 28 right-hand sides
+// against the float-float operator: 2.3e-6 with FP16 parts, 4.4e-6 with TF32 (half as many
+// accumulation steps).
 // Every wait is bounded (about a second): one that runs out raises an abort flag that the
 // other roles see, the block drains its bulk copies and MMAs in flight, frees its tensor memory
 // and returns,
@@ -53,11 +66,10 @@ namespace {
 
 using namespace tc;
 
-constexpr int kSrc = 8;                        // sources per stage (the MMA's K)
 constexpr int kRC = 64;                        // right-hand sides per work unit
 constexpr int kTcN = kTcGroup * kTargetBlock;  // targets per work unit (the MMA's N)
-constexpr int kSBO = (kSrc / 4) * 128;         // bytes per 8-row group of a stage operand
-constexpr int kGenSplit = 2;                   // generating threads per target (4 of the 8 sources each)
+constexpr int kSBO = 256;                      // bytes per 8-row group of a stage operand (two 16-byte columns)
+constexpr int kGenSplit = 2;                   // generating threads per target (one column each)
 constexpr int kGenThreads = kGenSplit * kTcN;
 constexpr int kGenWarps = kGenThreads / 32;
 constexpr int kProdWarp = kGenWarps, kMmaWarp = kGenWarps + 1;
@@ -69,83 +81,128 @@ constexpr int kAPart = (128 / 8) * kSBO;       // one split part of a weight ope
 constexpr int kBPart = (kTcN / 8) * kSBO;      // one split part of a kernel operand (256 rows)
 // stage: the weight operands as bulk-copied from the image (W_V hi | W_V lo | W_K hi | W_K lo, or
 // stacked W_V | W_K) | G hi | G lo | dG hi | dG lo | the geometry of the stage's sources (kTcSrcRows
-// rows of eight floats)
+// rows of a float per source)
 constexpr int kOffG = 4 * kAPart, kOffD = 4 * kAPart + 2 * kBPart;
 constexpr int kOffSrc = 4 * kAPart + 4 * kBPart;
-constexpr int kImgBlock = 4 * kAPart;          // image bytes per eight sources and 64 right-hand sides
-constexpr int kSrcBytes = kTcSrcRows * kSrc * 4;
-constexpr int kStage = kOffSrc + kSrcBytes;
+constexpr int kImgBlock = 4 * kAPart;          // image bytes per stage's sources and 64 right-hand sides
+constexpr int kStage = kOffSrc + kTcSrcRows * 16 * 4;
 constexpr int kStages = 4;
 constexpr int kSmem = kStages * kStage;
 static_assert(kSmem + 1024 <= 232448, "the stages and the static shared memory fit one SM");
-constexpr uint32_t kIdesc = idesc_tf32(128, kTcN);
+// operand parts: FP16 with 16 sources per stage, or TF32 with 8
+template <bool F16>
+struct P2PShape {
+    static constexpr int SRC = F16 ? 16 : 8;           // sources per stage (the MMA's K)
+    static constexpr int PART = SRC / kGenSplit;       // sources per generating thread and 16-byte column
+    static constexpr uint32_t SRC_BYTES = kTcSrcRows * SRC * 4;
+    static constexpr uint32_t IDESC = F16 ? idesc_f16(128, kTcN) : idesc_tf32(128, kTcN);
+    static __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t acc) {
+        if (F16) tc_mma_f16(d, a, b, IDESC, acc);
+        else tc_mma(d, a, b, IDESC, acc);
+    }
+    // the high and low parts of PART values to their columns
+    static __device__ __forceinline__ void split(const float (&v)[PART], unsigned char *hi, unsigned char *lo) {
+        if constexpr (F16) {
+            const HalfPair p = f16_split(v);
+            *(uint4 *)hi = p.hi;
+            *(uint4 *)lo = p.lo;
+        } else {
+            const TfPair p = tf32_split(make_float4(v[0], v[1], v[2], v[3]));
+            *(float4 *)hi = p.hi;
+            *(float4 *)lo = p.lo;
+        }
+    }
+};
 static_assert(kTmemCols <= 512 && kTcN <= 256, "both accumulators fit the tensor memory");
 static_assert(kStages >= 2, "at least two stages");
 static_assert(kRC * 2 == 128, "re and im of the unit's right-hand sides fill the MMA's M");
 
-// byte offset of (row r, column k) inside one split part of a stage operand (K-major 8 x 16-byte
-// core matrices, no swizzle)
-__device__ __forceinline__ int core_off(int r, int k) {
-    return (r >> 3) * kSBO + (k >> 2) * 128 + (r & 7) * 16 + (k & 3) * 4;
-}
+// byte offset of (row r, 16-byte column c) inside one split part of a stage operand (K-major 8 x
+// 16-byte core matrices, no swizzle)
+__device__ __forceinline__ int core_off(int r, int c) { return (r >> 3) * kSBO + c * 128 + (r & 7) * 16; }
 
-// The split weights of every eight consecutive sources in operand layout.  One thread per (eight
-// sources, unit chunk, half of the eight, right-hand side).  Sources past the end have zero weights;
-// rows of right-hand sides not in use are not written (their accumulator rows are not read).
-__global__ void __launch_bounds__(128)
-    p2p_image_kernel(int64_t Ns, int B, int nrc, const float4 *__restrict__ sw, unsigned char *__restrict__ img,
-                     const int *nact, int min_rhs, int nsurf, const int *__restrict__ mask8) {
-    const int Bact = nact ? *nact : B;
-    if (Bact < min_rhs) return;
-    const int64_t blk = blockIdx.x;   // (eight sources, chunk)
-    const int64_t g8 = blk / nrc;
-    const int rc = (int)(blk - g8 * nrc), b0 = rc * kRC, nb = min(kRC, Bact - b0);
-    if (nb <= 0) return;
-    const int q = threadIdx.x >> 6, j = threadIdx.x & 63;
-    const int64_t s0 = g8 * kSrc + 4 * q;
-    // no range that holds these sources has one of the chunk's surfaces: no unit reads the block
-    if (nsurf > 1 && !(mask8[g8] & set_surfaces(b0, nb, Bact, nsurf))) return;
-    if (j >= nb) return;
-    float4 w[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        w[i] = s0 + i < Ns ? __ldg(sw + (s0 + i) * B + b0 + j) : make_float4(0.f, 0.f, 0.f, 0.f);
-    const TfPair vr = tf32_split(make_float4(w[0].x, w[1].x, w[2].x, w[3].x));
-    const TfPair vi = tf32_split(make_float4(w[0].y, w[1].y, w[2].y, w[3].y));
-    const TfPair kr = tf32_split(make_float4(w[0].z, w[1].z, w[2].z, w[3].z));
-    const TfPair ki = tf32_split(make_float4(w[0].w, w[1].w, w[2].w, w[3].w));
-    unsigned char *o = img + blk * kImgBlock;
-    const int c = 4 * q;
-    if (nb <= kRC / 2) {
-        // stacked: rows re hi j, im hi 32 + j, re lo 64 + j, im lo 96 + j
-        *(float4 *)(o + core_off(j, c)) = vr.hi;
-        *(float4 *)(o + core_off(32 + j, c)) = vi.hi;
-        *(float4 *)(o + core_off(64 + j, c)) = vr.lo;
-        *(float4 *)(o + core_off(96 + j, c)) = vi.lo;
-        o += kAPart;
-        *(float4 *)(o + core_off(j, c)) = kr.hi;
-        *(float4 *)(o + core_off(32 + j, c)) = ki.hi;
-        *(float4 *)(o + core_off(64 + j, c)) = kr.lo;
-        *(float4 *)(o + core_off(96 + j, c)) = ki.lo;
-    } else {
-        // rows re j, im 64 + j; the high part, then the low part
-        *(float4 *)(o + core_off(j, c)) = vr.hi;
-        *(float4 *)(o + core_off(64 + j, c)) = vi.hi;
-        *(float4 *)(o + kAPart + core_off(j, c)) = vr.lo;
-        *(float4 *)(o + kAPart + core_off(64 + j, c)) = vi.lo;
-        o += 2 * kAPart;
-        *(float4 *)(o + core_off(j, c)) = kr.hi;
-        *(float4 *)(o + core_off(64 + j, c)) = ki.hi;
-        *(float4 *)(o + kAPart + core_off(j, c)) = kr.lo;
-        *(float4 *)(o + kAPart + core_off(64 + j, c)) = ki.lo;
+// largest magnitude per layer and system of the right-hand sides xt [2N][B], times the largest source
+// weight: a bound of the weights of the system's sets, as the bits of a non-negative float in mx[2 set]
+// (single layer) and mx[2 set + 1]
+constexpr int kMaxSets = 512;   // right-hand sides per block column
+__global__ void __launch_bounds__(256)
+    p2p_max_kernel(int64_t N, int B, int S, const float2 *__restrict__ xt, const int *__restrict__ stat, int *mx,
+                   const int *inv, const int *nact, int min_rhs) {
+    __shared__ int smax[2 * kMaxSets];
+    const int sets = nact ? *nact : B * S;
+    if (sets < min_rhs) return;
+    const int j0 = blockIdx.y * kMaxSets, nj = min(kMaxSets, B - j0), K = sets / S;
+    for (int j = threadIdx.x; j < 2 * nj; j += blockDim.x) smax[j] = 0;
+    __syncthreads();
+    const float wa = __int_as_float(stat[2]);
+    const int64_t rows = (2 * N + gridDim.x - 1) / gridDim.x;
+    const int64_t r0 = blockIdx.x * rows, r1 = min(2 * N, r0 + rows);
+    for (int64_t q = threadIdx.x; q < (r1 - r0) * nj; q += blockDim.x) {
+        const int64_t r = r0 + q / nj;
+        const int j = (int)(q % nj), layer = r < N ? 1 : 0;
+        const float2 v = __ldg(xt + r * B + j0 + j);
+        const int a = __float_as_int(fmaxf(fabsf(v.x), fabsf(v.y)) * wa);
+        if (a > smax[2 * j + layer]) atomicMax(&smax[2 * j + layer], a);
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < 2 * nj; j += blockDim.x) {
+        const int b = j0 + (j >> 1), k = inv ? inv[b] : b;
+        if (k < 0 || smax[j] == 0) continue;
+        for (int t = 0; t < S; ++t) atomicMax(&mx[2 * (t * K + k) + (j & 1)], smax[j]);
     }
 }
 
+// The split weights of every stage's sources in operand layout.  One thread per (sources of a
+// stage, unit chunk, half of them, right-hand side).  Sources past the end have zero weights;
+// rows of right-hand sides not in use are not written (their accumulator rows are not read).
+template <bool F16>
+__global__ void __launch_bounds__(128)
+    p2p_image_kernel(int64_t Ns, int B, int nrc, const float4 *__restrict__ sw, unsigned char *__restrict__ img,
+                     const int *nact, int min_rhs, int nsurf, const int *__restrict__ mask, const int *__restrict__ mx) {
+    using H = P2PShape<F16>;
+    const int Bact = nact ? *nact : B;
+    if (Bact < min_rhs) return;
+    const int64_t blk = blockIdx.x;   // (sources of a stage, chunk)
+    const int64_t g = blk / nrc;
+    const int rc = (int)(blk - g * nrc), b0 = rc * kRC, nb = min(kRC, Bact - b0);
+    if (nb <= 0) return;
+    const int q = threadIdx.x >> 6, j = threadIdx.x & 63;
+    const int64_t s0 = g * H::SRC + H::PART * q;
+    // no range that holds these sources has one of the chunk's surfaces: no unit reads the block
+    if (nsurf > 1 && !(mask[g] & set_surfaces(b0, nb, Bact, nsurf))) return;
+    if (j >= nb) return;
+    const float fv = F16 ? f16_scale(__ldg(mx + 2 * (b0 + j))) : 1.f;
+    const float fk = F16 ? f16_scale(__ldg(mx + 2 * (b0 + j) + 1)) : 1.f;
+    float w[4][H::PART];
+#pragma unroll
+    for (int i = 0; i < H::PART; ++i) {
+        const float4 v = s0 + i < Ns ? __ldg(sw + (s0 + i) * B + b0 + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+        w[0][i] = v.x * fv;
+        w[1][i] = v.y * fv;
+        w[2][i] = v.z * fk;
+        w[3][i] = v.w * fk;
+    }
+    const bool stacked = nb <= kRC / 2;
+    // rows: re j, im 64 + j, the high part, then the low part; stacked: re hi j, im hi 32 + j, re lo
+    // 64 + j, im lo 96 + j
+    const int im = stacked ? 32 : 64;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        unsigned char *o = img + blk * kImgBlock + (c >> 1) * (stacked ? kAPart : 2 * kAPart);
+        unsigned char *hi = o + core_off((c & 1) * im + j, q);
+        H::split(w[c], hi, stacked ? o + core_off(64 + (c & 1) * im + j, q) : hi + kAPart);
+    }
+}
+
+template <bool F16>
 __global__ void __launch_bounds__(kTcThreads, 1)
     p2p_tc_kernel(const int4 *__restrict__ items, int64_t nitems, const int4 *__restrict__ ivl, int B,
-                  const float4 *__restrict__ tgt, int64_t ntgt, const float *__restrict__ src8,
+                  const float4 *__restrict__ tgt, int64_t ntgt, const float *__restrict__ srcs,
                   const unsigned char *__restrict__ img, int nrc, double *__restrict__ acc,
-                  int *counter, int *error, const int *nact, int min_rhs, int nsurf) {
+                  int *counter, int *error, const int *nact, int min_rhs, int nsurf, float gs, float ts,
+                  const int *__restrict__ mx) {
+    using H = P2PShape<F16>;
+    constexpr int kSrc = H::SRC;
     // fewer right-hand sides in use than min_rhs: the FP32-pipe P2P takes this product
     if ((nact ? *nact : B) < min_rhs) return;
     extern __shared__ __align__(128) unsigned char tc_smem[];
@@ -225,12 +282,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         }
                         const uint32_t rb = smem_addr(&raw_s[s]), dst = sbase + (uint32_t)(s * kStage);
                         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(rb),
-                                     "r"((uint32_t)(abytes + kSrcBytes))
+                                     "r"((uint32_t)(abytes + H::SRC_BYTES))
                                      : "memory");
                         asm volatile(
                             "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                                 dst + kOffSrc),
-                            "l"(src8 + (int64_t)g * (kTcSrcRows * kSrc)), "r"(kSrcBytes), "r"(rb)
+                            "l"(srcs + (int64_t)g * (kTcSrcRows * kSrc)), "r"(H::SRC_BYTES), "r"(rb)
                             : "memory");
                         asm volatile(
                             "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -295,13 +352,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                             const uint64_t hl = umma_desc(st + kOffD + kBPart, 128, kSBO);
                             const uint32_t on = first ? 0u : 1u;
                             first = false;
-                            tc_mma(dv, wvh, gh, kIdesc, on);
-                            tc_mma(dv, wvh, gl, kIdesc, 1u);
-                            tc_mma(dk, wkh, hh, kIdesc, on);
-                            tc_mma(dk, wkh, hl, kIdesc, 1u);
+                            H::mma(dv, wvh, gh, on);
+                            H::mma(dv, wvh, gl, 1u);
+                            H::mma(dk, wkh, hh, on);
+                            H::mma(dk, wkh, hl, 1u);
                             if (!stacked) {
-                                tc_mma(dv, wvl, gh, kIdesc, 1u);
-                                tc_mma(dk, wkl, hh, kIdesc, 1u);
+                                H::mma(dv, wvl, gh, 1u);
+                                H::mma(dk, wkl, hh, 1u);
                             }
                             tc_commit(smem_addr(&empty_s[s]));
                         }
@@ -320,7 +377,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
     } else {
         // ---- generators: thread tid owns target tt = tid mod 256 of the group (row tt of the
-        // kernel operands) for the four sources 4 hf .. 4 hf + 3 of each stage, hf = tid / 256
+        // kernel operands) for the sources of 16-byte column hf of each stage, hf = tid / 256
         const int tt = tid & (kTcN - 1), hf = tid / kTcN;
         const int blk = tt / kTargetBlock;
         int64_t seq = 0;
@@ -341,6 +398,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const int j = p_stacked ? (m & 31) : (m & 63);
             const int cpt = p_stacked ? ((m >> 5) & 1) : (m >> 6);
             const bool row_on = j < p_nb;
+            // the scales undone: of the kernel values and of the weights
+            float undo_v = 1.f, undo_k = 1.f;
+            if (F16 && row_on) {
+                undo_v = 1.f / gs * (1.f / f16_scale(__ldg(mx + 2 * (p_b0 + j))));
+                undo_k = 1.f / ts * (1.f / f16_scale(__ldg(mx + 2 * (p_b0 + j) + 1)));
+            }
             if (__any_sync(0xffffffffu, row_on)) {
 #pragma unroll 1
                 for (int c0 = 0; c0 < kTcN / 4; c0 += 32) {
@@ -366,7 +429,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                                 const int p = __shfl_sync(0xffffffffu, pc, h16 + x);
                                 if (row_on && p >= 0)
                                     atomicAdd(acc + 4 * ((int64_t)p * B + p_b0 + j) + 2 * op + cpt,
-                                              (double)__uint_as_float(v[x]));
+                                              (double)(F16 ? __uint_as_float(v[x]) * (op ? undo_k : undo_v) : __uint_as_float(v[x])));
                             }
                         }
                     }
@@ -396,7 +459,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const bool live = ti < ntgt;
             const float4 q = live ? tgt[ti] : tgt[0];
             const int tp = live ? panel_of(q.w) : -1;
-            const float2 qx = make_float2(q.x, q.x), qy = make_float2(q.y, q.y), qz = make_float2(q.z, q.z);
+            // lengths are taken in units of gs (1 for TF32): r, then, is gs / |x - y|
+            const float ig = F16 ? 1.f / gs : 1.f;
+            const float2 qx = make_float2(q.x * ig, q.x * ig), qy = make_float2(q.y * ig, q.y * ig);
+            const float2 qz = make_float2(q.z * ig, q.z * ig);
             const int um = set_surfaces(b0, nb, Bact, nsurf);
             bool begun = false;
             for (int iv = item.y; iv < item.z && ok; ++iv) {
@@ -413,51 +479,47 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         break;
                     }
                     unsigned char *stg = tc_smem + s * kStage;
-                    const float4 *src = (const float4 *)(stg + kOffSrc) + hf;   // row r: src[2 r]
-                    // this thread's part of the kernel operand row of its target: G and dG/dn of
-                    // the stage's sources 4 hf .. 4 hf + 3 (positions are stored negated)
-                    constexpr int kPart = kSrc / kGenSplit;
+                    // row r of this thread's sources: src[r * kSrc / 4 + quad] (positions are stored
+                    // negated; the normals carry dG/dn's scale)
+                    constexpr int kPart = H::PART, kRow = kSrc / 4;
+                    const float4 *src = (const float4 *)(stg + kOffSrc) + hf * (kPart / 4);
                     float g[kPart], h[kPart];
                     if (on) {
-                        const float4 px = src[0], py = src[2], pz = src[4], nx = src[6], ny = src[8], nz = src[10];
-                        const float4 id = src[12];
-                        const int pid[4] = {__float_as_int(id.x), __float_as_int(id.y), __float_as_int(id.z),
-                                            __float_as_int(id.w)};
 #pragma unroll
-                        for (int p = 0; p < 2; ++p) {
-                            const float2 dx = __fadd2_rn(qx, p ? make_float2(px.z, px.w) : make_float2(px.x, px.y));
-                            const float2 dy = __fadd2_rn(qy, p ? make_float2(py.z, py.w) : make_float2(py.x, py.y));
-                            const float2 dz = __fadd2_rn(qz, p ? make_float2(pz.z, pz.w) : make_float2(pz.x, pz.y));
-                            const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-                            // zero for the target's own panel and for sources outside the range
-                            const int k = g8 * kSrc + kPart * hf + 2 * p;
-                            const float r0 = pid[2 * p] == tp || k < e.x || k >= e.y ? 0.f : rsq(r2.x);
-                            const float r1 = pid[2 * p + 1] == tp || k + 1 < e.x || k + 1 >= e.y ? 0.f : rsq(r2.y);
-                            const float2 r = make_float2(r0, r1);
-                            const float2 dn = __ffma2_rn(dz, p ? make_float2(nz.z, nz.w) : make_float2(nz.x, nz.y),
-                                              __ffma2_rn(dy, p ? make_float2(ny.z, ny.w) : make_float2(ny.x, ny.y),
-                                              __fmul2_rn(dx, p ? make_float2(nx.z, nx.w) : make_float2(nx.x, nx.y))));
-                            const float2 t = __fmul2_rn(__fmul2_rn(dn, __fmul2_rn(r, r)), r);
-                            g[2 * p] = r.x;
-                            g[2 * p + 1] = r.y;
-                            h[2 * p] = t.x;
-                            h[2 * p + 1] = t.y;
+                        for (int k4 = 0; k4 < kPart / 4; ++k4) {
+                            const float4 px = src[k4], py = src[kRow + k4], pz = src[2 * kRow + k4];
+                            const float4 nx = src[3 * kRow + k4], ny = src[4 * kRow + k4], nz = src[5 * kRow + k4];
+                            const float4 id = src[6 * kRow + k4];
+                            const int pid[4] = {__float_as_int(id.x), __float_as_int(id.y), __float_as_int(id.z),
+                                                __float_as_int(id.w)};
+#pragma unroll
+                            for (int p = 0; p < 2; ++p) {
+                                const float2 dx = __fadd2_rn(qx, p ? make_float2(px.z, px.w) : make_float2(px.x, px.y));
+                                const float2 dy = __fadd2_rn(qy, p ? make_float2(py.z, py.w) : make_float2(py.x, py.y));
+                                const float2 dz = __fadd2_rn(qz, p ? make_float2(pz.z, pz.w) : make_float2(pz.x, pz.y));
+                                const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+                                // zero for the target's own panel and for sources outside the range
+                                const int k = g8 * kSrc + kPart * hf + 4 * k4 + 2 * p;
+                                const float r0 = pid[2 * p] == tp || k < e.x || k >= e.y ? 0.f : rsq(r2.x);
+                                const float r1 = pid[2 * p + 1] == tp || k + 1 < e.x || k + 1 >= e.y ? 0.f : rsq(r2.y);
+                                const float2 r = make_float2(r0, r1);
+                                const float2 dn = __ffma2_rn(dz, p ? make_float2(nz.z, nz.w) : make_float2(nz.x, nz.y),
+                                                  __ffma2_rn(dy, p ? make_float2(ny.z, ny.w) : make_float2(ny.x, ny.y),
+                                                  __fmul2_rn(dx, p ? make_float2(nx.z, nx.w) : make_float2(nx.x, nx.y))));
+                                const float2 t = __fmul2_rn(__fmul2_rn(dn, __fmul2_rn(r, r)), r);
+                                g[4 * k4 + 2 * p] = r.x;
+                                g[4 * k4 + 2 * p + 1] = r.y;
+                                h[4 * k4 + 2 * p] = t.x;
+                                h[4 * k4 + 2 * p + 1] = t.y;
+                            }
                         }
                     } else {
 #pragma unroll
                         for (int k = 0; k < kPart; ++k) g[k] = h[k] = 0.f;
                     }
                     unsigned char *bg = stg + kOffG, *bd = stg + kOffD;
-                    static_assert(kPart == 4, "a thread writes one 4-column slice of its row");
-                    {
-                        const float4 gv = make_float4(g[0], g[1], g[2], g[3]);
-                        const float4 hv = make_float4(h[0], h[1], h[2], h[3]);
-                        const TfPair sg = tf32_split(gv), sh = tf32_split(hv);
-                        *(float4 *)(bg + core_off(tt, kPart * hf)) = sg.hi;
-                        *(float4 *)(bg + kBPart + core_off(tt, kPart * hf)) = sg.lo;
-                        *(float4 *)(bd + core_off(tt, kPart * hf)) = sh.hi;
-                        *(float4 *)(bd + kBPart + core_off(tt, kPart * hf)) = sh.lo;
-                    }
+                    H::split(g, bg + core_off(tt, hf), bg + kBPart + core_off(tt, hf));
+                    H::split(h, bd + core_off(tt, hf), bd + kBPart + core_off(tt, hf));
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();   // one arrival per warp: a thread each would serialise on the barrier
                     if (lane == 0) bar_arrive(smem_addr(&full_s[s]));
@@ -487,30 +549,46 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     if (tid == 0 && abort_s) atomicAdd(error, 1);
 }
 
+template <bool F16>
+int launch_parts(lspr_ctx *ctx, double *acc, cudaStream_t st, int *counter, int B, int min_rhs) {
+    static int smem_set[kSmemDevices] = {};
+    using H = P2PShape<F16>;
+    Tree &tr = ctx->tree;
+    LSPR_TRY(ctx, allow_smem(p2p_tc_kernel<F16>, kSmem, ctx->device, smem_set));
+    const int nrc = (B + kRC - 1) / kRC;
+    const int64_t Ns = ctx->mesh.Ns, N = ctx->mesh.N, ng = (Ns + H::SRC - 1) / H::SRC;
+    LSPR_TRY(ctx, ctx->tcp_img.ensure((size_t)(ng * nrc) * kImgBlock));
+    int *mx = (int *)(acc + 4 * N * B) + kCounters + 2 * B;   // cleared with the accumulators
+    if (F16) {
+        const int S = ctx->mesh.S, nsys = B / S;
+        ++ctx->n_launches;
+        p2p_max_kernel<<<dim3(4 * std::max(1, ctx->num_sms), (nsys + kMaxSets - 1) / kMaxSets), 256, 0, st>>>(
+            N, nsys, S, ctx->xtf.p, tr.tcp_stat.p, mx, ctx->rhs_inv, ctx->rhs_nact, min_rhs);
+    }
+    ++ctx->n_launches;   // the image; the caller counts the P2P launch
+    p2p_image_kernel<F16><<<(unsigned)(ng * nrc), 128, 0, st>>>(Ns, B, nrc, Views<float>::w(ctx), ctx->tcp_img.p,
+                                                               ctx->rhs_nact, min_rhs, ctx->mesh.S, tr.tcp_mask.p, mx);
+    const unsigned grid =
+        (unsigned)std::max<int64_t>(1, std::min<int64_t>(tr.n_tcp_items * nrc, std::max(1, ctx->num_sms)));
+    p2p_tc_kernel<F16><<<grid, kTcThreads, kSmem, st>>>(tr.tcp_items.p, tr.n_tcp_items, tr.tcp_ivl.p, B,
+                                                       Views<float>::tgt(ctx), N, tr.tcp_src.p, ctx->tcp_img.p, nrc, acc,
+                                                       counter, ctx->dev_err.p, ctx->rhs_nact, min_rhs, ctx->mesh.S,
+                                                       tr.tcp_gs, tr.tcp_ts, mx);
+    LSPR_TRY(ctx, cudaGetLastError());
+    return LSPR_OK;
+}
+
 }  // namespace
 
 // FP32 tree P2P of B >= 2 right-hand sides on the tensor cores
 int p2p_tc_launch(lspr_ctx *ctx, double *acc, cudaStream_t st, int *counter, int B, int min_rhs) {
-    static int smem_set[kSmemDevices] = {};
     Tree &tr = ctx->tree;
     if (!tr.tcp_built) LSPR_TRY_ST(tree_tc_lists(ctx, true));
     if (tr.n_tcp_items == 0) return LSPR_OK;
     if (!ctx->dev_err.p) return LSPR_E_STATE;
     ctx->tc_launched = true;
-    LSPR_TRY(ctx, allow_smem(p2p_tc_kernel, kSmem, ctx->device, smem_set));
-    const int nrc = (B + kRC - 1) / kRC;
-    const int64_t Ns = ctx->mesh.Ns, ng = (Ns + kSrc - 1) / kSrc;
-    LSPR_TRY(ctx, ctx->tcp_img.ensure((size_t)(ng * nrc) * kImgBlock));
-    ++ctx->n_launches;   // the image; the caller counts the P2P launch
-    p2p_image_kernel<<<(unsigned)(ng * nrc), 128, 0, st>>>(Ns, B, nrc, Views<float>::w(ctx), ctx->tcp_img.p,
-                                                          ctx->rhs_nact, min_rhs, ctx->mesh.S, tr.tcp_mask8.p);
-    const unsigned grid =
-        (unsigned)std::max<int64_t>(1, std::min<int64_t>(tr.n_tcp_items * nrc, std::max(1, ctx->num_sms)));
-    p2p_tc_kernel<<<grid, kTcThreads, kSmem, st>>>(tr.tcp_items.p, tr.n_tcp_items, tr.tcp_ivl.p, B,
-                                                  Views<float>::tgt(ctx), ctx->mesh.N, tr.tcp_src8.p, ctx->tcp_img.p,
-                                                  nrc, acc, counter, ctx->dev_err.p, ctx->rhs_nact, min_rhs,
-                                                  ctx->mesh.S);
-    return LSPR_OK;
+    return tr.tcp_f16 ? launch_parts<true>(ctx, acc, st, counter, B, min_rhs)
+                      : launch_parts<false>(ctx, acc, st, counter, B, min_rhs);
 }
 
 }  // namespace lspr

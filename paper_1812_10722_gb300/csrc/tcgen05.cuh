@@ -61,10 +61,10 @@ __device__ __forceinline__ HalfPair f16_split(const float (&v)[8]) {
     return p;
 }
 // the power of two that brings a largest magnitude (the bits of a non-negative float) into
-// [2^14, 2^15); 1 for infinities and NaN
+// [2^14, 2^15), at most 2^126 so that its reciprocal is normal; 1 for infinities and NaN
 __device__ __forceinline__ float f16_scale(int bits) {
     const int e = bits >> 23;
-    return e >= 255 ? 1.f : __int_as_float(min(254, 268 - e) << 23);
+    return e >= 255 ? 1.f : __int_as_float(min(253, 268 - e) << 23);
 }
 
 __device__ __forceinline__ uint64_t now_ns() {

@@ -494,7 +494,7 @@ __global__ void tc_list_surf_kernel(int64_t n, int2 *list, const int *__restrict
     if (i < n) list[i].y |= (box_surf ? box_surf[list[i].x] : 1) << kTcSurf;
 }
 __global__ void tc_ivl_surf_kernel(int64_t n, int4 *ivl, int S, const int *__restrict__ src_panel,
-                                   const int *__restrict__ surf, int *mask8) {
+                                   const int *__restrict__ surf, int *mask, int per) {
     const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (i >= n) return;
@@ -504,26 +504,59 @@ __global__ void tc_ivl_surf_kernel(int64_t n, int4 *ivl, int S, const int *__res
     m = __reduce_or_sync(0xffffffffu, m);
     if (lane == 0) ivl[i].w = (int)m;
     if (S > 1)
-        for (int g = ivl[i].x / 8 + lane; g * 8 < ivl[i].y; g += 32) atomicOr(&mask8[g], (int)m);
+        for (int g = ivl[i].x / per + lane; g * per < ivl[i].y; g += 32) atomicOr(&mask[g], (int)m);
 }
 
-// geometry of eight consecutive sources, one row per component (positions negated), in the layout
-// that the tensor-core P2P reads; sources past the end repeat the last one
-__global__ void tc_src8_kernel(int64_t Ns, const float4 *__restrict__ spos, const float4 *__restrict__ snrm,
-                               float *src8) {
+// stat[0], stat[1]: smallest and largest squared distance (FP32 bits) between a target and a source of
+// another panel over the P2P items, one warp per item (stat[0] starts at the largest int)
+__global__ void __launch_bounds__(128)
+    pair_range_kernel(int64_t nitems, const int4 *__restrict__ items, int64_t N, const float4 *__restrict__ tgt,
+                      const float4 *__restrict__ spos, const int *__restrict__ src_panel, int *stat) {
+    const int64_t it = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (it >= nitems) return;
+    const int4 item = items[it];
+    const int64_t t0 = (int64_t)item.x * kTargetBlock + lane;
+    const float4 q0 = tgt[min(t0, N - 1)], q1 = tgt[min(t0 + 32, N - 1)];
+    float lo = 3e38f, hi = 0.f;
+#pragma unroll 4
+    for (int s = item.y; s < item.z; ++s) {
+        const float4 p = __ldg(spos + s);
+        const int id = __ldg(src_panel + s);
+        const float ax = q0.x - p.x, ay = q0.y - p.y, az = q0.z - p.z;
+        const float bx = q1.x - p.x, by = q1.y - p.y, bz = q1.z - p.z;
+        const float ra = ax * ax + ay * ay + az * az, rb = bx * bx + by * by + bz * bz;
+        if (id != __float_as_int(q0.w)) { lo = fminf(lo, ra); hi = fmaxf(hi, ra); }
+        if (id != __float_as_int(q1.w)) { lo = fminf(lo, rb); hi = fmaxf(hi, rb); }
+    }
+    const int l = __reduce_min_sync(0xffffffffu, __float_as_int(lo)), h = __reduce_max_sync(0xffffffffu, __float_as_int(hi));
+    if (lane == 0) {
+        if (l < __ldcg(stat)) atomicMin(stat, l);
+        if (h > __ldcg(stat + 1)) atomicMax(stat + 1, h);
+    }
+}
+
+// geometry of the sources of every stage (n of them), one row per component, in the layout that the
+// tensor-core P2P reads: positions negated and divided by gs, normals times ts / gs^2 (the scales of G
+// and dG/dn, see p2p_tc.cu); sources past the end repeat the last one.  stat[2]: the largest weight.
+__global__ void tc_src_kernel(int64_t Ns, int n, float gs, float ts, const float4 *__restrict__ spos,
+                              const float4 *__restrict__ snrm, float *src, int *stat) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= (Ns + 7) / 8 * 8) return;
     const int64_t s = min(i, Ns - 1);
-    const float4 p = spos[s], n = snrm[s];
-    float *o = src8 + (i >> 3) * (kTcSrcRows * 8) + (i & 7);
-    o[0] = -p.x;
-    o[8] = -p.y;
-    o[16] = -p.z;
-    o[24] = n.x;
-    o[32] = n.y;
-    o[40] = n.z;
-    o[48] = n.w;
-    o[56] = 0.f;
+    const float4 p = spos[s], v = snrm[s];
+    const int w = __reduce_max_sync(0xffffffffu, __float_as_int(fabsf(p.w * (float)kInv4Pi)));
+    if ((threadIdx.x & 31) == 0) atomicMax(stat + 2, w);
+    if (i >= (Ns + n - 1) / n * n) return;
+    const float ig = 1.f / gs, f = ts * ig * ig;
+    float *o = src + i / n * (kTcSrcRows * n) + i % n;
+    o[0] = -p.x * ig;
+    o[n] = -p.y * ig;
+    o[2 * n] = -p.z * ig;
+    o[3 * n] = v.x * f;
+    o[4 * n] = v.y * f;
+    o[5 * n] = v.z * f;
+    o[6 * n] = v.w;
+    o[7 * n] = 0.f;
 }
 
 // box node of the list walk: (first child or -1, children, source begin, source end)
@@ -876,7 +909,8 @@ int tree_build(lspr_ctx *ctx, double theta, int P, int Ncrit) {
 
     // lists: count
     const double clear = m.Lmax / m.thr + m.rho_max;
-    tr.rho_min = (float)(theta * clear);   // an accepted box is at least clear away
+    // an accepted box is at least clear away; a power of two, since recorded graphs are told apart by it
+    tr.rho_min = (float)std::exp2(std::floor(std::log2(theta * clear)));
     Tmp<int> cnt3(ctx->scratch[11]), off3(ctx->scratch[12]);
     Tmp<int64_t> tot3(ctx->scratch[13]);
     Tmp<unsigned long long> pairs(ctx->scratch[14]);
@@ -932,7 +966,8 @@ int tree_build(lspr_ctx *ctx, double theta, int P, int Ncrit) {
     int np2m = 0;
     LSPR_TRY(ctx, cudaMemcpyAsync(&np2m, ovf.p, sizeof(int), cudaMemcpyDeviceToHost, st));
     // the group lists of the tensor-core far field are formed on first use (tree_tc_lists)
-    tr.tc_built = tr.tcp_built = false;
+    tr.tc_built = tr.tcp_built = tr.tcp_f16 = false;
+    tr.tcp_gs = tr.tcp_ts = 1.f;
     tr.n_tc_items = tr.n_tc_pairs = tr.n_tcp_items = tr.n_tcp_ivl = tr.n_tcp_sources = tr.n_tcp_stages = 0;
     timer_end(ctx, T_TREE, ev);
     LSPR_TRY(ctx, cudaGetLastError());
@@ -997,16 +1032,39 @@ int tree_tc_lists(lspr_ctx *ctx, bool p2p) {
         tr.n_tcp_ivl = (int64_t)pivl.size();
         tr.n_tcp_sources = psrc;
         tr.n_tcp_stages = 0;
-        for (const TcRange &r : pivl) tr.n_tcp_stages += (r.s1 + 7) / 8 - r.s0 / 8;   // aligned to eight sources
-        LSPR_TRY(ctx, tr.tcp_items.ensure(std::max<size_t>(1, pitems.size())));
+        // the range of distances chooses the operand parts and their scales
         const int64_t Ns = ctx->mesh.Ns;
-        if (ctx->mesh.S > 1) {
-            LSPR_TRY(ctx, tr.tcp_mask8.ensure((size_t)(Ns + 7) / 8));
-            LSPR_TRY(ctx, cudaMemsetAsync(tr.tcp_mask8.p, 0, sizeof(int) * ((Ns + 7) / 8), st));
+        int stat[3] = {0x7fffffff, 0, 0};
+        LSPR_TRY(ctx, tr.tcp_stat.ensure(3));
+        LSPR_TRY(ctx, cudaMemcpyAsync(tr.tcp_stat.p, stat, sizeof(stat), cudaMemcpyHostToDevice, st));
+        if (tr.n_p2p_items > 0) {
+            ++ctx->n_launches;
+            pair_range_kernel<<<grid_for(tr.n_p2p_items * 32, 128), 128, 0, st>>>(
+                tr.n_p2p_items, tr.p2p_items.p, ctx->mesh.N, ctx->wo.tgt32.p, ctx->wo.spos32.p, ctx->wo.src_panel.p,
+                tr.tcp_stat.p);
+            LSPR_TRY(ctx, cudaGetLastError());
+            LSPR_TRY(ctx, cudaMemcpyAsync(stat, tr.tcp_stat.p, sizeof(stat), cudaMemcpyDeviceToHost, st));
+            LSPR_TRY(ctx, cudaStreamSynchronize(st));
         }
-        LSPR_TRY(ctx, tr.tcp_src8.ensure((size_t)(Ns + 7) / 8 * (kTcSrcRows * 8)));
+        float r2lo, r2hi;
+        std::memcpy(&r2lo, &stat[0], sizeof(float));
+        std::memcpy(&r2hi, &stat[1], sizeof(float));
+        // moderate lengths only, so that no scale leaves the FP32 range
+        tr.tcp_f16 = r2lo > 1e-12f && r2hi < 1e12f && r2hi <= kTcP2PRange * kTcP2PRange * r2lo;
+        tr.tcp_gs = tr.tcp_f16 ? std::exp2(std::floor(std::log2(32768.f * std::sqrt(r2lo)))) : 1.f;
+        tr.tcp_ts = tr.tcp_f16 ? std::exp2(std::floor(std::log2(32768.f * r2lo))) : 1.f;
+        const int per = tr.tcp_f16 ? 16 : 8;   // sources per stage
+        for (const TcRange &r : pivl) tr.n_tcp_stages += (r.s1 + per - 1) / per - r.s0 / per;
+        LSPR_TRY(ctx, tr.tcp_items.ensure(std::max<size_t>(1, pitems.size())));
+        const int64_t ng = (Ns + per - 1) / per;
+        if (ctx->mesh.S > 1) {
+            LSPR_TRY(ctx, tr.tcp_mask.ensure((size_t)ng));
+            LSPR_TRY(ctx, cudaMemsetAsync(tr.tcp_mask.p, 0, sizeof(int) * ng, st));
+        }
+        LSPR_TRY(ctx, tr.tcp_src.ensure((size_t)ng * (kTcSrcRows * per)));
         ++ctx->n_launches;
-        tc_src8_kernel<<<grid_for(Ns + 7, 256), 256, 0, st>>>(Ns, ctx->wo.spos32.p, ctx->wo.snrm32.p, tr.tcp_src8.p);
+        tc_src_kernel<<<grid_for(ng * per, 256), 256, 0, st>>>(Ns, per, tr.tcp_gs, tr.tcp_ts, ctx->wo.spos32.p,
+                                                               ctx->wo.snrm32.p, tr.tcp_src.p, tr.tcp_stat.p);
         LSPR_TRY(ctx, tr.tcp_ivl.ensure(std::max<size_t>(1, pivl.size())));
         if (!pitems.empty()) {
             LSPR_TRY(ctx, cudaMemcpyAsync(tr.tcp_items.p, pitems.data(), sizeof(int4) * pitems.size(),
@@ -1014,7 +1072,7 @@ int tree_tc_lists(lspr_ctx *ctx, bool p2p) {
             LSPR_TRY(ctx, cudaMemcpyAsync(tr.tcp_ivl.p, pivl.data(), sizeof(int4) * pivl.size(), cudaMemcpyHostToDevice, st));
             ++ctx->n_launches;
             tc_ivl_surf_kernel<<<grid_for(pivl.size() * 32, 256), 256, 0, st>>>(
-                (int64_t)pivl.size(), tr.tcp_ivl.p, ctx->mesh.S, ctx->wo.src_panel.p, ctx->mesh.surf.p, tr.tcp_mask8.p);
+                (int64_t)pivl.size(), tr.tcp_ivl.p, ctx->mesh.S, ctx->wo.src_panel.p, ctx->mesh.surf.p, tr.tcp_mask.p, per);
             LSPR_TRY(ctx, cudaGetLastError());
         }
         LSPR_TRY(ctx, cudaStreamSynchronize(st));
