@@ -214,6 +214,7 @@ __global__ void __launch_bounds__(p2p_warps(NB) * 32)
 // partial sums are added with one exchange and each lane adds two targets into the FP64
 // accumulators.  The sums and the own-panel rule are those of p2p_kernel.
 constexpr int kP1Warps = 8;
+constexpr int64_t kP1Halves = 12288;   // 20480 panels (7433 items): 72.6 us in halves, 77.3 whole; 56180 (19849): no gain
 struct P1Src {   // one staged source, 96 bytes: duplicated pairs (the position negated)
     float4 pxy;   // (-px, -px, -py, -py)
     float4 pzn;   // (-pz, -pz, nx, nx)
@@ -278,7 +279,7 @@ template <bool DYNAMIC>
 __global__ void __launch_bounds__(kP1Warps * 32)
     p2p1_kernel(const int4 *__restrict__ items, int64_t nitems, const float4 *__restrict__ tgt, int64_t ntgt,
                 const float4 *__restrict__ spos, const float4 *__restrict__ snrm, const float4 *__restrict__ sw,
-                double *__restrict__ acc, int *counter, const int *nact) {
+                double *__restrict__ acc, int *counter, const int *nact, int parts) {
     __shared__ P1Src sh[kP1Warps][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane & 15, h = lane >> 4;
     if (nact && *nact < 1) return;   // no right-hand side in use
@@ -289,8 +290,13 @@ __global__ void __launch_bounds__(kP1Warps * 32)
             if (lane == 0) v = atomicAdd(counter, 1);
             it = __shfl_sync(0xffffffffu, v, 0);
         }
-        if (it >= nitems) return;
-        const int4 item = __ldg(items + it);
+        if (it >= nitems * parts) return;
+        int4 item = __ldg(items + it / parts);
+        if (parts > 1) {   // this unit's part of the item's sources
+            const int n = item.z - item.y, p = (int)(it % parts), y = item.y;
+            item.y = y + n * p / parts;
+            item.z = y + n * (p + 1) / parts;
+        }
         const int64_t t0 = (int64_t)item.x * kTargetBlock + l;
         float4 q[4];
         int tp[4];
@@ -984,11 +990,13 @@ static void p2p_launch(lspr_ctx *ctx, const int4 *items, int64_t nitems, int B, 
 static void p2p1_launch(lspr_ctx *ctx, const int4 *items, int64_t nitems, double *acc, cudaStream_t st,
                         int *counter) {
     static int occ = 0;
-    const unsigned grid = std::min<unsigned>(grid_for(nitems, kP1Warps),
+    // few items for the warps in flight (about 5000): halves, for a shorter last wave
+    const int parts = nitems < kP1Halves ? 2 : 1;
+    const unsigned grid = std::min<unsigned>(grid_for(nitems * parts, kP1Warps),
                                              persistent_grid(ctx, p2p1_kernel<true>, kP1Warps * 32, &occ));
     p2p1_kernel<true><<<grid, kP1Warps * 32, 0, st>>>(items, nitems, Views<float>::tgt(ctx), ctx->mesh.N,
                                                        Views<float>::spos(ctx), Views<float>::snrm(ctx),
-                                                       Views<float>::w(ctx), acc, counter, ctx->rhs_nact);
+                                                       Views<float>::w(ctx), acc, counter, ctx->rhs_nact, parts);
 }
 
 template <typename T, int P, int NB>
