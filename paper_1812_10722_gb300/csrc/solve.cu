@@ -29,36 +29,57 @@ __device__ __forceinline__ double2 csqrt_p(double2 z) {
 }
 
 // ------------------------------------------------------------------ assembly
-// RAW = true writes the layer potentials (V dphi, K phi) instead of the block rows.
-// kRowLanes lanes per (row, right-hand side) read the row's near entries coalesced
-// (rows hold ~25 entries); groups are ordered row-major so the B right-hand sides of a
-// row reuse its CSR entries from cache.  acc is [panel][B][4], x and y are [B][2N].
+// One right-hand side.  kRowLanes lanes per row read the row's near entries coalesced (rows hold
+// ~25 entries), four each at a time with their gathers issued together.  acc is [panel][4], x and y
+// are [2N].  What becomes of the sums:
+//   ROWS the block rows, RAW the layer potentials (V dphi, K phi), both with the far part;
+//   ADD  added to the far part: treecode products run this beside the P2P (it waits on memory, the
+//        P2P on the FP32 pipe) and form the rows from acc afterwards (block_rows_kernel).
 constexpr int kRowLanes = 8;
-template <bool RAW>
-__global__ void assemble_kernel(int64_t N, int B, const double *__restrict__ acc, const int64_t *__restrict__ ptr,
+enum { NEAR_ROWS, NEAR_RAW, NEAR_ADD };
+__device__ __forceinline__ void put_rows(int64_t N, int64_t i, double2 ph, double2 V, double2 K, double2 s, double2 *y) {
+    const double2 sv = cmul(s, V);
+    y[i] = make_double2(0.5 * ph.x + K.x - V.x, 0.5 * ph.y + K.y - V.y);
+    y[N + i] = make_double2(0.5 * ph.x - K.x + sv.x, 0.5 * ph.y - K.y + sv.y);
+}
+template <int WHAT>
+__global__ void assemble_kernel(int64_t N, double *__restrict__ acc, const int64_t *__restrict__ ptr,
                                 const int *__restrict__ col, const double *__restrict__ dV,
                                 const double *__restrict__ dK, const double2 *__restrict__ x, const double2 *s,
                                 double2 *y, double2 *Vd, double2 *Kp, const int *inv) {
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t grp = g / kRowLanes;
+    const int64_t i = g / kRowLanes;
     const int lane = (int)(g % kRowLanes);
-    const int64_t i = grp / B;
-    const int b = (int)(grp - i * B);
-    // the far part of system b sits in slot inv[b] of acc (identity without a map); rows
-    // of converged systems (slot -1) are left untouched
-    const int slot = i < N ? (inv ? inv[b] : b) : -1;
-    const bool valid = i < N && slot >= 0;
-    const double2 *xb = x + (int64_t)b * 2 * N;
+    const bool valid = i < N && (!inv || inv[0] >= 0);   // the row of a converged system is left untouched
     double vr = 0, vi = 0, kr = 0, ki = 0;
     if (valid) {
-        for (int64_t e = ptr[i] + lane; e < ptr[i + 1]; e += kRowLanes) {
-            const int j = col[e];
-            const double a = dV[e], c = dK[e];
-            const double2 ph = xb[j], dp = xb[N + j];
-            vr += a * dp.x;
-            vi += a * dp.y;
-            kr += c * ph.x;
-            ki += c * ph.y;
+        const int64_t e1 = ptr[i + 1];
+        for (int64_t e = ptr[i] + lane; e < e1; e += 4 * kRowLanes) {
+            int j[4];
+            double a[4], c[4];
+            double2 ph[4], dp[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t q = e + u * kRowLanes;
+                if (q >= e1) continue;
+                j[u] = col[q];
+                a[u] = dV[q];
+                c[u] = dK[q];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (e + u * kRowLanes >= e1) continue;
+                ph[u] = x[j[u]];
+                dp[u] = x[N + j[u]];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (e + u * kRowLanes >= e1) continue;
+                vr = fma(a[u], dp[u].x, vr);
+                vi = fma(a[u], dp[u].y, vi);
+                kr = fma(c[u], ph[u].x, kr);
+                ki = fma(c[u], ph[u].y, ki);
+            }
         }
     }
 #pragma unroll
@@ -69,19 +90,31 @@ __global__ void assemble_kernel(int64_t N, int B, const double *__restrict__ acc
         ki += __shfl_xor_sync(0xffffffffu, ki, o, kRowLanes);
     }
     if (!valid || lane != 0) return;
-    const double *ai = acc + 4 * (i * B + slot);
-    const double2 V = make_double2(ai[0] + vr, ai[1] + vi);
-    const double2 K = make_double2(ai[2] + kr, ai[3] + ki);
-    if (RAW) {
-        Vd[(int64_t)b * N + i] = V;
-        Kp[(int64_t)b * N + i] = K;
+    double *ai = acc + 4 * i;
+    if (WHAT == NEAR_ADD) {
+        atomicAdd(ai, vr);
+        atomicAdd(ai + 1, vi);
+        atomicAdd(ai + 2, kr);
+        atomicAdd(ai + 3, ki);
         return;
     }
-    const double2 ph = xb[i];
-    const double2 sv = cmul(s[b], V);
-    double2 *yb = y + (int64_t)b * 2 * N;
-    yb[i] = make_double2(0.5 * ph.x + K.x - V.x, 0.5 * ph.y + K.y - V.y);
-    yb[N + i] = make_double2(0.5 * ph.x - K.x + sv.x, 0.5 * ph.y - K.y + sv.y);
+    const double2 V = make_double2(ai[0] + vr, ai[1] + vi);
+    const double2 K = make_double2(ai[2] + kr, ai[3] + ki);
+    if (WHAT == NEAR_RAW) {
+        Vd[i] = V;
+        Kp[i] = K;
+        return;
+    }
+    put_rows(N, i, x[i], V, K, s[0], y);
+}
+
+// the block rows of one right-hand side from acc, which holds the near sums too
+__global__ void block_rows_kernel(int64_t N, const double *__restrict__ acc, const double2 *__restrict__ x,
+                                  const double2 *s, double2 *y, const int *inv) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= N || (inv && inv[0] < 0)) return;
+    const double2 V = make_double2(acc[4 * i], acc[4 * i + 1]), K = make_double2(acc[4 * i + 2], acc[4 * i + 3]);
+    put_rows(N, i, x[i], V, K, s[0], y);
 }
 
 // Several right-hand sides: x [B][2N] is transposed to xt [2N][B] once per product, so
@@ -190,17 +223,16 @@ __global__ void assemble_rhs_f32_kernel(int64_t N, int B, int L, const double *_
 // near corrections, the latter split by the source panel's surface t:
 //   y_top = phi/2 + (K phi)_s - (V dphi)_s,  y_bot = phi/2 - sum_t (K phi)_t + sum_t s_bt (V dphi)_t
 // L lanes per row (L <= 32, a power of two), lane r handling b = r, r + L, ...; the gathers read the
-// transposed right-hand sides xt [2N][B] contiguously in b.  The entries of the row's own surface
-// (nearly all) are summed first and enter with one complex product.  FP64 throughout: bound by the
-// FP64 pipe (4 multiply-adds per entry and right-hand side).  145920 panels, 32 right-hand sides:
-// 1.23 ms (3.43 with both surfaces' cases in one loop, whose
-// branches the compiler merges into 18 FP64 operations per entry; 3.74 with one thread per (row,
-// right-hand side) gathering from x [B][2N]).
-__global__ void assemble_surf_rhs_kernel(int64_t N, int B, int S, int L, const int *__restrict__ surf,
-                                         const double *__restrict__ acc, const int64_t *__restrict__ ptr,
-                                         const int *__restrict__ col, const double *__restrict__ dV,
-                                         const double *__restrict__ dK, const double2 *__restrict__ xt,
-                                         const double2 *__restrict__ s, double2 *y, const int *inv, const int *nact) {
+// transposed right-hand sides xt [2N][B] contiguously in b.  The near sums are added to acc (treecode
+// products run this beside the P2P, whose tensor cores leave the FP64 pipe free), the rows formed from
+// it afterwards.  FP64 throughout: bound by the FP64 pipe (4 multiply-adds per entry and right-hand
+// side).  145920 panels, 32 right-hand sides: 1.23 ms in one kernel (3.43 with both cases below in one
+// loop, whose branches the compiler merges into 18 FP64 operations per entry; 3.74 with one thread per
+// (row, right-hand side) gathering from x [B][2N]).
+__global__ void near_surf_kernel(int64_t N, int B, int S, int L, const int *__restrict__ surf, double *__restrict__ acc,
+                                 const int64_t *__restrict__ ptr, const int *__restrict__ col,
+                                 const double *__restrict__ dV, const double *__restrict__ dK,
+                                 const double2 *__restrict__ xt, const int *inv, const int *nact) {
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t i = g / L;
     const int r = (int)(g - i * L);
@@ -210,44 +242,64 @@ __global__ void assemble_surf_rhs_kernel(int64_t N, int B, int S, int L, const i
     for (int b = r; b < B; b += L) {
         const int k = inv ? inv[b] : b;
         if (k < 0) continue;   // converged system: row left untouched
-        double2 Vs = make_double2(0, 0), Ks = make_double2(0, 0);   // own surface
-        double2 Ka = make_double2(0, 0), Vw = make_double2(0, 0);   // the others
+        double *f = acc + 4 * (i * ((int64_t)B * S) + k);   // set t K + k at f + 4 t K
+        double vr = 0, vi = 0, kr = 0, ki = 0;   // own surface: nearly all entries
         bool others = false;
         for (int64_t e = e0; e < e1; ++e) {
             const int64_t j = col[e];
             const double a = dV[e], c = dK[e];
             const double2 ph = xt[j * B + b], dp = xt[(N + j) * B + b];
             if (surf[j] == si) {
-                Vs.x = fma(a, dp.x, Vs.x);
-                Vs.y = fma(a, dp.y, Vs.y);
-                Ks.x = fma(c, ph.x, Ks.x);
-                Ks.y = fma(c, ph.y, Ks.y);
+                vr = fma(a, dp.x, vr);
+                vi = fma(a, dp.y, vi);
+                kr = fma(c, ph.x, kr);
+                ki = fma(c, ph.y, ki);
             } else {
                 others = true;
             }
         }
-        // in a loop of its own: beside the sums above, its 14 operations were issued for every entry
+        double *o = f + 4 * (int64_t)si * K;
+        atomicAdd(o, vr);
+        atomicAdd(o + 1, vi);
+        atomicAdd(o + 2, kr);
+        atomicAdd(o + 3, ki);
         if (others)
             for (int64_t e = e0; e < e1; ++e) {
                 const int64_t j = col[e];
                 const int t = surf[j];
                 if (t == si) continue;
-                Ka = cadd(Ka, cscale(xt[j * B + b], dK[e]));
-                Vw = cadd(Vw, cmul(s[b * S + t], cscale(xt[(N + j) * B + b], dV[e])));
+                const double2 ph = xt[j * B + b], dp = xt[(N + j) * B + b];
+                o = f + 4 * (int64_t)t * K;
+                atomicAdd(o, dV[e] * dp.x);
+                atomicAdd(o + 1, dV[e] * dp.y);
+                atomicAdd(o + 2, dK[e] * ph.x);
+                atomicAdd(o + 3, dK[e] * ph.y);
             }
+    }
+}
+
+__global__ void block_rows_surf_kernel(int64_t N, int B, int S, int L, const int *__restrict__ surf,
+                                       const double *__restrict__ acc, const double2 *__restrict__ xt,
+                                       const double2 *__restrict__ s, double2 *y, const int *inv, const int *nact) {
+    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = g / L;
+    const int r = (int)(g - i * L);
+    if (i >= N) return;
+    const int K = nact ? *nact / S : B, si = surf[i];
+    for (int b = r; b < B; b += L) {
+        const int k = inv ? inv[b] : b;
+        if (k < 0) continue;
+        double2 Vs = make_double2(0, 0), Ks = Vs, Ka = Vs, Vw = Vs;
         for (int t = 0; t < S; ++t) {
             const double *f = acc + 4 * (i * ((int64_t)B * S) + (int64_t)t * K + k);
             const double2 V = make_double2(f[0], f[1]), Kt = make_double2(f[2], f[3]);
             if (t == si) {
-                Vs = cadd(Vs, V);
-                Ks = cadd(Ks, Kt);
-            } else {
-                Ka = cadd(Ka, Kt);
-                Vw = cadd(Vw, cmul(s[b * S + t], V));
+                Vs = V;
+                Ks = Kt;
             }
+            Ka = cadd(Ka, Kt);
+            Vw = cadd(Vw, cmul(s[b * S + t], V));
         }
-        Ka = cadd(Ka, Ks);
-        Vw = cadd(Vw, cmul(s[b * S + si], Vs));
         const double2 ph = xt[i * B + b];
         double2 *yb = y + (int64_t)b * 2 * N;
         yb[i] = make_double2(0.5 * ph.x + Ks.x - Vs.x, 0.5 * ph.y + Ks.y - Vs.y);
@@ -278,7 +330,33 @@ __global__ void raw_surf_kernel(int64_t N, int S, const int *__restrict__ surf, 
 // far-field parts of B right-hand sides x [B][2N] into ctx->acc [panel][B S][4] (S surfaces:
 // channel set t B + b holds the potentials of surface t's sources); with B > 1 the
 // transposed copy xt of x is formed first (the block assembly reads it too)
-static int far_part(lspr_ctx *ctx, int mode, const double2 *x, int B) {
+// near: the near sums are added to acc as well, in treecode modes beside the P2P
+static bool near_in_acc(const lspr_ctx *ctx, int mode, int B) {
+    return ctx->mesh.S > 1 || (B == 1 && mode_tree(mode));
+}
+static int near_part(lspr_ctx *ctx, const double2 *x, int B) {
+    const Mesh &m = ctx->mesh;
+    const int64_t N = m.N;
+    cudaEvent_t ev;
+    timer_begin(ctx, T_NEAR, &ev);
+    ++ctx->n_launches;
+    if (m.S > 1) {
+        int L = 1;
+        while (L < B && L < 32) L *= 2;
+        near_surf_kernel<<<grid_for(N * L, 256), 256, 0, ctx->stream>>>(   // xt of one right-hand side is x itself
+            N, B, m.S, L, m.surf.p, ctx->acc.p, m.near_ptr.p, m.near_col.p, m.near_dV.p, m.near_dK.p,
+            B > 1 ? ctx->xt.p : x, ctx->rhs_inv, ctx->rhs_nact);
+    } else {
+        assemble_kernel<NEAR_ADD><<<grid_for(N * kRowLanes, 256), 256, 0, ctx->stream>>>(
+            N, ctx->acc.p, m.near_ptr.p, m.near_col.p, m.near_dV.p, m.near_dK.p, x, nullptr, nullptr, nullptr, nullptr,
+            ctx->rhs_inv);
+    }
+    timer_end(ctx, T_NEAR, ev);
+    LSPR_TRY(ctx, cudaGetLastError());
+    return LSPR_OK;
+}
+
+static int far_part(lspr_ctx *ctx, int mode, const double2 *x, int B, bool near) {
     const int prec = mode_prec(mode);
     const bool tree = mode_tree(mode);
     const int64_t N = ctx->mesh.N;
@@ -310,6 +388,7 @@ static int far_part(lspr_ctx *ctx, int mode, const double2 *x, int B) {
                                counters, BS));
         LSPR_TRY_ST(launch_p2m(ctx, prec, BS));
         LSPR_TRY_ST(launch_m2p(ctx, prec, ctx->acc.p, counters + 1, BS));
+        if (near) LSPR_TRY_ST(near_part(ctx, x, B));
     } else if (tree) {
         // P2P on the side stream overlaps P2M -> M2P on the main stream; both add into acc
         LSPR_TRY(ctx, cudaEventRecord(ctx->ev_fork, ctx->stream));
@@ -319,10 +398,12 @@ static int far_part(lspr_ctx *ctx, int mode, const double2 *x, int B) {
         LSPR_TRY(ctx, cudaEventRecord(ctx->ev_join, ctx->side));
         LSPR_TRY_ST(launch_p2m(ctx, prec, BS));
         LSPR_TRY_ST(launch_m2p(ctx, prec, ctx->acc.p, counters + 1, BS));
+        if (near) LSPR_TRY_ST(near_part(ctx, x, B));
         LSPR_TRY(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
     } else {
         const DirectItems &d = direct_items(ctx, BS);
         LSPR_TRY_ST(launch_p2p(ctx, prec, d.items.p, d.n, ctx->acc.p, ctx->stream, counters, BS));
+        if (near) LSPR_TRY_ST(near_part(ctx, x, B));
     }
     ctx->matvec_count += B;
     return LSPR_OK;
@@ -331,20 +412,21 @@ static int far_part(lspr_ctx *ctx, int mode, const double2 *x, int B) {
 int apply_operator(lspr_ctx *ctx, int mode, const double2 *x, double2 *y, const double2 *s, int B) {
     const Mesh &m = ctx->mesh;
     const int64_t N = m.N;
-    LSPR_TRY_ST(far_part(ctx, mode, x, B));
+    const bool near = near_in_acc(ctx, mode, B);
+    LSPR_TRY_ST(far_part(ctx, mode, x, B, near));
     cudaEvent_t ev;
     timer_begin(ctx, T_NEAR, &ev);
     ++ctx->n_launches;
     int L = 1;
     while (L < B && L < 32) L *= 2;
     if (m.S > 1) {
-        // xt of one right-hand side is x itself
-        assemble_surf_rhs_kernel<<<grid_for(N * L, 256), 256, 0, ctx->stream>>>(
-            N, B, m.S, L, m.surf.p, ctx->acc.p, m.near_ptr.p, m.near_col.p, m.near_dV.p, m.near_dK.p,
-            B > 1 ? ctx->xt.p : x, s, y, ctx->rhs_inv, ctx->rhs_nact);
+        block_rows_surf_kernel<<<grid_for(N * L, 256), 256, 0, ctx->stream>>>(
+            N, B, m.S, L, m.surf.p, ctx->acc.p, B > 1 ? ctx->xt.p : x, s, y, ctx->rhs_inv, ctx->rhs_nact);
+    } else if (near) {
+        block_rows_kernel<<<grid_for(N, 256), 256, 0, ctx->stream>>>(N, ctx->acc.p, x, s, y, ctx->rhs_inv);
     } else if (B == 1) {
-        assemble_kernel<false><<<grid_for(N * kRowLanes, 256), 256, 0, ctx->stream>>>(
-            N, B, ctx->acc.p, m.near_ptr.p, m.near_col.p, m.near_dV.p, m.near_dK.p, x, s, y, nullptr, nullptr,
+        assemble_kernel<NEAR_ROWS><<<grid_for(N * kRowLanes, 256), 256, 0, ctx->stream>>>(
+            N, ctx->acc.p, m.near_ptr.p, m.near_col.p, m.near_dV.p, m.near_dK.p, x, s, y, nullptr, nullptr,
             ctx->rhs_inv);
     } else {
         if (mode_prec(mode) == PREC_F32)
@@ -362,16 +444,15 @@ int apply_operator(lspr_ctx *ctx, int mode, const double2 *x, double2 *y, const 
 
 int layer_potentials(lspr_ctx *ctx, int mode, const double2 *x, double2 *Vd, double2 *Kp) {
     const Mesh &m = ctx->mesh;
-    LSPR_TRY_ST(far_part(ctx, mode, x, 1));
+    LSPR_TRY_ST(far_part(ctx, mode, x, 1, false));
     ++ctx->n_launches;
     if (m.S > 1)
         raw_surf_kernel<<<grid_for(m.N, 128), 128, 0, ctx->stream>>>(m.N, m.S, m.surf.p, ctx->acc.p, m.near_ptr.p,
                                                                      m.near_col.p, m.near_dV.p, m.near_dK.p, x, Vd,
                                                                      Kp);
     else
-        assemble_kernel<true><<<grid_for(m.N * kRowLanes, 256), 256, 0, ctx->stream>>>(
-            m.N, 1, ctx->acc.p, m.near_ptr.p, m.near_col.p, m.near_dV.p, m.near_dK.p, x, nullptr, nullptr, Vd, Kp,
-            nullptr);
+        assemble_kernel<NEAR_RAW><<<grid_for(m.N * kRowLanes, 256), 256, 0, ctx->stream>>>(
+            m.N, ctx->acc.p, m.near_ptr.p, m.near_col.p, m.near_dV.p, m.near_dK.p, x, nullptr, nullptr, Vd, Kp, nullptr);
     LSPR_TRY(ctx, cudaGetLastError());
     return LSPR_OK;
 }
