@@ -720,11 +720,15 @@ __global__ void __launch_bounds__(kM2PGemmThreads)
 // sides (the sources split over SP thread groups where the tile leaves the block small).  The sums
 // are added to the leaf if some target block accepted it, and shifted into every accepted ancestor
 // A (upward pass folded in): with delta = c_A - c, the Taylor expansion of g_k about delta gives
-//   M_(a,b,c)(A) = sum_{i<=a, j<=b} g_(i,j,c)(delta) M_(a-i,b-j,0) + d_3 g_(i,j,c)(delta) M_(a-i,b-j,1).
+//   M_(a,b,c)(A) = sum_{i<=a, j<=b} g_(i,j,c)(delta) M_(a-i,b-j,0) + d_3 g_(i,j,c)(delta) M_(a-i,b-j,1),
+// a convolution in a for each pair of lines (b, c), (b - j, 0 or 1): a thread takes the outputs of one
+// line and right-hand side four at a time, so that a moment read from shared memory serves four.
 // Stored moments carry the factor gamma_n k_1! k_2! of their term.
 // Bound by the FP32 pipe and the shared-memory reads of the tile product.  81920 panels, P 7,
-// 64 right-hand sides: 769 us, 1913 before (one thread per Cartesian term, every monomial and its
-// derivative formed per right-hand-side chunk of 8); 56180 panels, P 6, one right-hand side: 65 us
+// 64 right-hand sides: 538 us; 775 with a thread per output term of the shifts (a moment read per
+// product), 1913 before (one thread per Cartesian term, every monomial and its
+// derivative formed per right-hand-side chunk of 8); 145920 panels, 32 right-hand sides: 730 us, 1030
+// before the shifts by lines; 56180 panels, P 6, one right-hand side: 65 us
 // after 135.
 template <typename T, int P, int NB>
 struct P2MShape {
@@ -742,7 +746,11 @@ struct P2MShape {
     static constexpr size_t W = (size_t)TS * NB * sizeof(typename Vec4<T>::type);
     static constexpr size_t LM = (size_t)SP * NT * NB * sizeof(typename Vec4<T>::type);
     static constexpr size_t BODY = GD + W > LM ? GD + W : LM;           // the sums reuse the tile's space
-    static constexpr size_t ANC = (size_t)(kMaxDepth + 1) * 2 * NT * sizeof(T);
+    // shift table of an ancestor: [g, d_3 g][c][j][i], each line preceded by three zeros (i < 0)
+    static constexpr int LINE = P + 4;
+    static constexpr int TAB = 2 * 2 * (P + 1) * LINE;
+    static constexpr int ANCS = 4;                         // ancestors tabulated at a time
+    static constexpr size_t ANC = (size_t)ANCS * TAB * sizeof(T);
     static constexpr size_t SMEM = (BODY + 15) / 16 * 16 + ANC;
 };
 
@@ -765,7 +773,7 @@ __global__ void __launch_bounds__(P2MShape<T, P, NB>::THREADS)
     TV *sg = (TV *)p2m_smem, *sd = sg + TG * Sh::ROW;       // [term group][source]
     T4 *shw = (T4 *)(p2m_smem + Sh::GD);                    // [source][right-hand side]
     T4 *lm = (T4 *)p2m_smem;                                // [split][term][right-hand side]
-    T *anc = (T *)(p2m_smem + (Sh::BODY + 15) / 16 * 16);   // [ancestor][g, d_3 g][term]
+    T *anc = (T *)(p2m_smem + (Sh::BODY + 15) / 16 * 16);   // [ancestor][TAB]
     __shared__ int anc_box[kMaxDepth + 1], n_anc;
     const int64_t u = blockIdx.x;
     if (u >= nitems * nbc) return;
@@ -780,25 +788,30 @@ __global__ void __launch_bounds__(P2MShape<T, P, NB>::THREADS)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tg = tid % TG, rg = (tid / TG) % RG, sp = tid / (TG * RG);
     const bool on = sp < SP;
-    if (warp == 1) {   // the accepted ancestors' shift tables, one lane each
+    // the shift tables of the accepted ancestors first .. first + ANCS - 1, one lane of warp 1 each
+    auto tabulate = [&](int first) {
+        if (warp != 1) return;
         int mine = -1, k = 0;
         for (int A = parent[item.x]; A >= 0; A = parent[A]) {
             if (!used[A]) continue;
-            if (k == lane) mine = A;
+            if (k == first + lane) mine = A;
             ++k;
         }
         if (lane == 0) n_anc = k;
-        if (mine >= 0) {
-            anc_box[lane] = mine;
-            const T4 ca = box_c[mine];
-            const T d[3] = {ca.x - c.x, ca.y - c.y, ca.z - c.z}, z[3] = {T(0), T(0), T(0)};
-            T *g = anc + (size_t)lane * 2 * NT;
-            harmonics<T, P>(d, z, [&](int t, const T &v, const T &, const T &d3) {
-                g[t] = v;
-                g[NT + t] = d3;
-            });
-        }
-    }
+        if (mine < 0 || lane >= Sh::ANCS) return;
+        anc_box[lane] = mine;
+        const T4 ca = box_c[mine];
+        const T d[3] = {ca.x - c.x, ca.y - c.y, ca.z - c.z}, z[3] = {T(0), T(0), T(0)};
+        T *g = anc + (size_t)lane * Sh::TAB;
+        for (int i = 0; i < Sh::TAB; ++i) g[i] = T(0);
+        constexpr MultiIndex<P> mi{};
+        harmonics<T, P>(d, z, [&](int t, const T &v, const T &, const T &d3) {
+            const int o = (mi.k[t][2] * (P + 1) + mi.k[t][1]) * Sh::LINE + 3 + mi.k[t][0];
+            g[o] = v;
+            g[2 * (P + 1) * Sh::LINE + o] = d3;
+        });
+    };
+    tabulate(0);
     T acc[TT][RB][4];
 #pragma unroll
     for (int i = 0; i < TT; ++i)
@@ -900,33 +913,51 @@ __global__ void __launch_bounds__(P2MShape<T, P, NB>::THREADS)
     if (n_anc == 0) return;
     __syncthreads();
     for (int k = 0; k < n_anc; ++k) {
-        const T *ga = anc + (size_t)k * 2 * NT;
-        for (int q = tid; q < NT * NB; q += Sh::THREADS) {
-            const int t = q / NB, j = q - t * NB;
+        const int kk = k % Sh::ANCS;
+        if (k > 0 && kk == 0) {
+            __syncthreads();
+            tabulate(k);
+            __syncthreads();
+        }
+        const T *tab = anc + (size_t)kk * Sh::TAB;
+        typename MomAcc<T>::type *dst = mom + (int64_t)anc_box[kk] * NT * B + b0;
+        for (int q = tid; q < (2 * P + 1) * NB; q += Sh::THREADS) {
+            const int line = q / NB, j = q - line * NB;
             if (j >= nb) continue;
-            const int ka = c_terms.a[t], kb = c_terms.b[t], kc = c_terms.c[t];
-            T o[4] = {T(0), T(0), T(0), T(0)};
-            for (int i = 0; i <= ka; ++i)
-                for (int l = 0; l <= kb; ++l) {
-                    const int gi = mi_index(i, l, kc);
-                    const T g = ga[gi];
-                    const T4 m = lm[mi_index(ka - i, kb - l, 0) * NB + j];
-                    o[0] += g * m.x;
-                    o[1] += g * m.y;
-                    o[2] += g * m.z;
-                    o[3] += g * m.w;
-                    if (kc || i + l >= 2) {   // d_3 g vanishes for (0,0,0), (1,0,0) and (0,1,0)
-                        const T e = ga[NT + gi];
-                        const T4 m1 = lm[mi_index(ka - i, kb - l, 1) * NB + j];
-                        o[0] += e * m1.x;
-                        o[1] += e * m1.y;
-                        o[2] += e * m1.z;
-                        o[3] += e * m1.w;
+            const int c = line > P ? 1 : 0, b = line - c * (P + 1), amax = P - c - b;
+            for (int a0 = 0; a0 <= amax; a0 += 4) {
+                T o[4][4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) o[r][x] = T(0);
+#pragma unroll
+                for (int c1 = 0; c1 < 2; ++c1)
+                    for (int b1 = 0; b1 <= b; ++b1) {
+                        // moments (l, b1, c1) times table entry i = a0 + r - l of line (b - b1, c)
+                        const T *g = tab + ((c1 * 2 + c) * (P + 1) + (b - b1)) * Sh::LINE + 3 + a0;
+                        const int lmax = min(min(a0 + 3, amax), P - c1 - b1);
+                        for (int l = 0; l <= lmax; ++l) {
+                            const T4 m = lm[mi_index(l, b1, c1) * NB + j];
+#pragma unroll
+                            for (int r = 0; r < 4; ++r) {
+                                const T f = g[r - l];
+                                o[r][0] += f * m.x;
+                                o[r][1] += f * m.y;
+                                o[r][2] += f * m.z;
+                                o[r][3] += f * m.w;
+                            }
+                        }
                     }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    if (a0 + r > amax) break;
+                    const int t = mi_index(a0 + r, b, c);
+                    const T f = T(c_terms.scale[t]);
+                    acc_add4((S *)(dst + (int64_t)t * B + j), (S)(f * o[r][0]), (S)(f * o[r][1]), (S)(f * o[r][2]),
+                             (S)(f * o[r][3]));
                 }
-            const T f = T(c_terms.scale[t]);
-            S *g = (S *)(mom + ((int64_t)anc_box[k] * NT + t) * B + b0 + j);
-            acc_add4(g, (S)(f * o[0]), (S)(f * o[1]), (S)(f * o[2]), (S)(f * o[3]));
+            }
         }
     }
 }
