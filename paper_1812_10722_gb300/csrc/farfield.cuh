@@ -721,14 +721,19 @@ __global__ void __launch_bounds__(kM2PGemmThreads)
 // are added to the leaf if some target block accepted it, and shifted into every accepted ancestor
 // A (upward pass folded in): with delta = c_A - c, the Taylor expansion of g_k about delta gives
 //   M_(a,b,c)(A) = sum_{i<=a, j<=b} g_(i,j,c)(delta) M_(a-i,b-j,0) + d_3 g_(i,j,c)(delta) M_(a-i,b-j,1),
-// a convolution in a for each pair of lines (b, c), (b - j, 0 or 1): a thread takes the outputs of one
-// line and right-hand side four at a time, so that a moment read from shared memory serves four.
+// a convolution in a for each pair of lines (b, c), (b - j, 0 or 1): with 8 or more FP32 right-hand sides
+// a thread takes the outputs of one line and right-hand side four at a time, so that a moment read from
+// shared memory serves four.  With one right-hand side a line each leaves most threads idle (56180 panels:
+// 79 us after 63), and in FP64 and float-float the sixteen sums cost more registers than the reads
+// (20480 panels, one FP64: 248 after 175 us; 40500 panels, 12 float-float: 1480 after 1075): there a
+// thread takes one output term.
 // Stored moments carry the factor gamma_n k_1! k_2! of their term.
 // Bound by the FP32 pipe and the shared-memory reads of the tile product.  81920 panels, P 7,
-// 64 right-hand sides: 538 us; 775 with a thread per output term of the shifts (a moment read per
+// 64 right-hand sides: 514 us; 775 with a thread per output term of the shifts (a moment read per
 // product), 1913 before (one thread per Cartesian term, every monomial and its
-// derivative formed per right-hand-side chunk of 8); 145920 panels, 32 right-hand sides: 730 us, 1030
-// before the shifts by lines; 56180 panels, P 6, one right-hand side: 65 us
+// derivative formed per right-hand-side chunk of 8); 145920 panels, 32 right-hand sides: 674 us, 1030
+// before the shifts by lines (541 and 730 with the table read for every product; 20480 panels, 16
+// right-hand sides: 55 us so, 68 with the table values sliding, whose unrolling costs more there); 56180 panels, P 6, one right-hand side: 65 us
 // after 135.
 template <typename T, int P, int NB>
 struct P2MShape {
@@ -746,10 +751,14 @@ struct P2MShape {
     static constexpr size_t W = (size_t)TS * NB * sizeof(typename Vec4<T>::type);
     static constexpr size_t LM = (size_t)SP * NT * NB * sizeof(typename Vec4<T>::type);
     static constexpr size_t BODY = GD + W > LM ? GD + W : LM;           // the sums reuse the tile's space
-    // shift table of an ancestor: [g, d_3 g][c][j][i], each line preceded by three zeros (i < 0)
-    static constexpr int LINE = P + 4;
-    static constexpr int TAB = 2 * 2 * (P + 1) * LINE;
-    static constexpr int ANCS = 4;                         // ancestors tabulated at a time
+    // shifts by lines (else a thread per output term): several FP32 right-hand sides
+    static constexpr bool LINES = sizeof(T) == 4 && NB >= 8;
+    static constexpr int UNROLL = NB >= 32 ? 4 : 1;
+    // shift table of an ancestor: [g, d_3 g][term]; by lines [g, d_3 g][c][j][i], each line preceded by
+    // four zeros (i < 0)
+    static constexpr int LINE = P + 5;
+    static constexpr int TAB = LINES ? 2 * 2 * (P + 1) * LINE : 2 * NT;
+    static constexpr int ANCS = LINES ? 4 : kMaxDepth + 1;   // ancestors tabulated at a time
     static constexpr size_t ANC = (size_t)ANCS * TAB * sizeof(T);
     static constexpr size_t SMEM = (BODY + 15) / 16 * 16 + ANC;
 };
@@ -798,17 +807,20 @@ __global__ void __launch_bounds__(P2MShape<T, P, NB>::THREADS)
             ++k;
         }
         if (lane == 0) n_anc = k;
+        if (Sh::LINES) {
+            for (int i = lane; i < Sh::ANCS * Sh::TAB; i += 32) anc[i] = T(0);
+            __syncwarp();
+        }
         if (mine < 0 || lane >= Sh::ANCS) return;
         anc_box[lane] = mine;
         const T4 ca = box_c[mine];
         const T d[3] = {ca.x - c.x, ca.y - c.y, ca.z - c.z}, z[3] = {T(0), T(0), T(0)};
         T *g = anc + (size_t)lane * Sh::TAB;
-        for (int i = 0; i < Sh::TAB; ++i) g[i] = T(0);
         constexpr MultiIndex<P> mi{};
         harmonics<T, P>(d, z, [&](int t, const T &v, const T &, const T &d3) {
-            const int o = (mi.k[t][2] * (P + 1) + mi.k[t][1]) * Sh::LINE + 3 + mi.k[t][0];
+            const int o = Sh::LINES ? (mi.k[t][2] * (P + 1) + mi.k[t][1]) * Sh::LINE + 4 + mi.k[t][0] : t;
             g[o] = v;
-            g[2 * (P + 1) * Sh::LINE + o] = d3;
+            g[Sh::TAB / 2 + o] = d3;
         });
     };
     tabulate(0);
@@ -921,42 +933,76 @@ __global__ void __launch_bounds__(P2MShape<T, P, NB>::THREADS)
         }
         const T *tab = anc + (size_t)kk * Sh::TAB;
         typename MomAcc<T>::type *dst = mom + (int64_t)anc_box[kk] * NT * B + b0;
-        for (int q = tid; q < (2 * P + 1) * NB; q += Sh::THREADS) {
-            const int line = q / NB, j = q - line * NB;
-            if (j >= nb) continue;
-            const int c = line > P ? 1 : 0, b = line - c * (P + 1), amax = P - c - b;
-            for (int a0 = 0; a0 <= amax; a0 += 4) {
-                T o[4][4];
+        if constexpr (Sh::LINES) {
+            for (int q = tid; q < (2 * P + 1) * NB; q += Sh::THREADS) {
+                const int line = q / NB, j = q - line * NB;
+                if (j >= nb) continue;
+                const int c = line > P ? 1 : 0, b = line - c * (P + 1), amax = P - c - b;
+                for (int a0 = 0; a0 <= amax; a0 += 4) {
+                    T o[4][4];
 #pragma unroll
-                for (int r = 0; r < 4; ++r)
+                    for (int r = 0; r < 4; ++r)
 #pragma unroll
-                    for (int x = 0; x < 4; ++x) o[r][x] = T(0);
+                        for (int x = 0; x < 4; ++x) o[r][x] = T(0);
 #pragma unroll
-                for (int c1 = 0; c1 < 2; ++c1)
-                    for (int b1 = 0; b1 <= b; ++b1) {
-                        // moments (l, b1, c1) times table entry i = a0 + r - l of line (b - b1, c)
-                        const T *g = tab + ((c1 * 2 + c) * (P + 1) + (b - b1)) * Sh::LINE + 3 + a0;
-                        const int lmax = min(min(a0 + 3, amax), P - c1 - b1);
-                        for (int l = 0; l <= lmax; ++l) {
-                            const T4 m = lm[mi_index(l, b1, c1) * NB + j];
+                    for (int c1 = 0; c1 < 2; ++c1)
+                        for (int b1 = 0; b1 <= b; ++b1) {
+                            // moments (l, b1, c1) times the table entries i = a0 + r - l of line (b - b1, c)
+                            const T *g = tab + ((c1 * 2 + c) * (P + 1) + (b - b1)) * Sh::LINE + 4 + a0;
+                            const int lmax = min(min(a0 + 3, amax), P - c1 - b1);
+                            T f[4] = {g[0], g[1], g[2], g[3]};   // slides along the line
+#pragma unroll Sh::UNROLL
+                            for (int l = 0; l <= lmax; ++l) {
+                                const T4 m = lm[mi_index(l, b1, c1) * NB + j];
 #pragma unroll
-                            for (int r = 0; r < 4; ++r) {
-                                const T f = g[r - l];
-                                o[r][0] += f * m.x;
-                                o[r][1] += f * m.y;
-                                o[r][2] += f * m.z;
-                                o[r][3] += f * m.w;
+                                for (int r = 0; r < 4; ++r) {
+                                    const T fr = Sh::UNROLL > 1 ? f[r] : g[r - l];
+                                    o[r][0] += fr * m.x;
+                                    o[r][1] += fr * m.y;
+                                    o[r][2] += fr * m.z;
+                                    o[r][3] += fr * m.w;
+                                }
+#pragma unroll
+                                for (int r = 3; r > 0; --r) f[r] = f[r - 1];
+                                f[0] = g[-1 - l];
                             }
                         }
-                    }
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    if (a0 + r > amax) break;
-                    const int t = mi_index(a0 + r, b, c);
-                    const T f = T(c_terms.scale[t]);
-                    acc_add4((S *)(dst + (int64_t)t * B + j), (S)(f * o[r][0]), (S)(f * o[r][1]), (S)(f * o[r][2]),
-                             (S)(f * o[r][3]));
+                    for (int r = 0; r < 4; ++r) {
+                        if (a0 + r > amax) break;
+                        const int t = mi_index(a0 + r, b, c);
+                        const T f = T(c_terms.scale[t]);
+                        acc_add4((S *)(dst + (int64_t)t * B + j), (S)(f * o[r][0]), (S)(f * o[r][1]),
+                                 (S)(f * o[r][2]), (S)(f * o[r][3]));
+                    }
                 }
+            }
+        } else {
+            for (int q = tid; q < NT * NB; q += Sh::THREADS) {
+                const int t = q / NB, j = q - t * NB;
+                if (j >= nb) continue;
+                const int ka = c_terms.a[t], kb = c_terms.b[t], kc = c_terms.c[t];
+                T o[4] = {T(0), T(0), T(0), T(0)};
+                for (int i = 0; i <= ka; ++i)
+                    for (int l = 0; l <= kb; ++l) {
+                        const int gi = mi_index(i, l, kc);
+                        const T g = tab[gi];
+                        const T4 m = lm[mi_index(ka - i, kb - l, 0) * NB + j];
+                        o[0] += g * m.x;
+                        o[1] += g * m.y;
+                        o[2] += g * m.z;
+                        o[3] += g * m.w;
+                        if (kc || i + l >= 2) {   // d_3 g vanishes for (0,0,0), (1,0,0) and (0,1,0)
+                            const T e = tab[NT + gi];
+                            const T4 m1 = lm[mi_index(ka - i, kb - l, 1) * NB + j];
+                            o[0] += e * m1.x;
+                            o[1] += e * m1.y;
+                            o[2] += e * m1.z;
+                            o[3] += e * m1.w;
+                        }
+                    }
+                const T f = T(c_terms.scale[t]);
+                acc_add4((S *)(dst + (int64_t)t * B + j), (S)(f * o[0]), (S)(f * o[1]), (S)(f * o[2]), (S)(f * o[3]));
             }
         }
     }
