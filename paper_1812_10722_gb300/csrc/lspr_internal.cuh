@@ -42,8 +42,12 @@ inline bool mode_tree(int mode) { return mode == LSPR_TREE_FP64 || mode == LSPR_
 constexpr double kInv4Pi = 0.079577471545947667884;   // 1 / (4 pi)
 constexpr int kTargetBlock = 64;                       // targets per interaction block (2 per lane)
 constexpr int kTcGroup = 4;        // target blocks per tensor-core M2P group (256 targets)
-constexpr int kTcGroupSeg = 32;    // boxes per tensor-core M2P work unit at most
-constexpr int kTcP2PSrc = 2048;    // sources per tensor-core P2P work unit at most
+// Boxes per tensor-core M2P work unit and sources per P2P unit (stages of 16, of 8 with TF32 parts), at most
+// (tc_unit).  A unit ends with its accumulators added in FP64, which no MMA overlaps; the upper limits bound
+// the steps added in FP32 (at most 672 K steps of boxes, 256 stages of sources).
+constexpr int kTcSegMin = 32;
+constexpr int tc_seg_max(int P) { return P < 7 ? 64 : 112; }
+constexpr int kTcSrcMin = 1024, kTcSrcMax = 4096;
 constexpr int kTcSrcRows = 8;      // tensor-core P2P source geometry per stage: rows -x, -y, -z, normal, panel, -
 constexpr float kTcP2PRange = 4096.f;   // largest ratio of P2P distances for FP16 parts
 constexpr int kTcSurf = 8;         // tensor-core M2P list entry.y: block mask, from this bit the box's surfaces

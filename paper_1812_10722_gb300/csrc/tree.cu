@@ -988,7 +988,7 @@ int tree_tc_lists(lspr_ctx *ctx, bool p2p) {
     const int64_t ntb = tr.ntblocks;
     if (!tr.ready) return LSPR_E_STATE;
     if (!tr.tc_built) {
-        // M2P lists of the groups (tc_group_m2p)
+        // M2P lists of the groups
         std::vector<int> hlist((size_t)tr.n_m2p_pairs);
         std::vector<int4> hitems((size_t)tr.n_m2p_items);
         if (tr.n_m2p_pairs > 0) {
@@ -998,9 +998,9 @@ int tree_tc_lists(lspr_ctx *ctx, bool p2p) {
         }
         std::vector<TcEntry> glist;
         std::vector<TcItem> gitems;
-        tc_group_m2p(ntb, kTcGroup, kTcGroupSeg, hlist.data(), (const int *)hitems.data(), tr.n_m2p_items, glist,
-                     gitems);
+        tc_union_m2p(ntb, kTcGroup, hlist.data(), (const int *)hitems.data(), tr.n_m2p_items, glist, gitems);
         tr.n_tc_pairs = (int64_t)glist.size();
+        tc_cut_m2p(tc_unit(tr.n_tc_pairs, ctx->num_sms, kTcSegMin, tc_seg_max(tr.P)), gitems);
         tr.n_tc_items = (int64_t)gitems.size();
         LSPR_TRY(ctx, tr.tc_list.ensure(std::max<size_t>(1, glist.size())));
         LSPR_TRY(ctx, tr.tc_items.ensure(std::max<size_t>(1, gitems.size())));
@@ -1017,7 +1017,7 @@ int tree_tc_lists(lspr_ctx *ctx, bool p2p) {
         tr.tc_built = true;
     }
     if (p2p && !tr.tcp_built) {
-        // P2P source ranges of the same groups (tc_group_p2p)
+        // P2P source ranges of the same groups
         std::vector<int4> hp2p((size_t)tr.n_p2p_items);
         if (tr.n_p2p_items > 0) {
             LSPR_TRY(ctx, cudaMemcpyAsync(hp2p.data(), tr.p2p_items.p, sizeof(int4) * tr.n_p2p_items,
@@ -1027,9 +1027,7 @@ int tree_tc_lists(lspr_ctx *ctx, bool p2p) {
         std::vector<TcRange> pivl;
         std::vector<TcItem> pitems;
         static_assert(sizeof(TcRange) == sizeof(int4), "device layout");
-        const int64_t psrc = tc_group_p2p(ntb, kTcGroup, kTcP2PSrc, (const int *)hp2p.data(), tr.n_p2p_items, pivl, pitems);
-        tr.n_tcp_items = (int64_t)pitems.size();
-        tr.n_tcp_ivl = (int64_t)pivl.size();
+        const int64_t psrc = tc_union_p2p(ntb, kTcGroup, (const int *)hp2p.data(), tr.n_p2p_items, pivl, pitems);
         tr.n_tcp_sources = psrc;
         tr.n_tcp_stages = 0;
         // the range of distances chooses the operand parts and their scales
@@ -1054,6 +1052,9 @@ int tree_tc_lists(lspr_ctx *ctx, bool p2p) {
         tr.tcp_gs = tr.tcp_f16 ? std::exp2(std::floor(std::log2(32768.f * std::sqrt(r2lo)))) : 1.f;
         tr.tcp_ts = tr.tcp_f16 ? std::exp2(std::floor(std::log2(32768.f * r2lo))) : 1.f;
         const int per = tr.tcp_f16 ? 16 : 8;   // sources per stage
+        tc_cut_p2p(tc_unit(psrc, ctx->num_sms, kTcSrcMin, kTcSrcMax / 16 * per), pivl, pitems);
+        tr.n_tcp_items = (int64_t)pitems.size();
+        tr.n_tcp_ivl = (int64_t)pivl.size();
         for (const TcRange &r : pivl) tr.n_tcp_stages += (r.s1 + per - 1) / per - r.s0 / per;
         LSPR_TRY(ctx, tr.tcp_items.ensure(std::max<size_t>(1, pitems.size())));
         const int64_t ng = (Ns + per - 1) / per;
