@@ -418,13 +418,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         uint32_t v[16];
                         const uint32_t addr = tmem + ((uint32_t)(32 * qd) << 16) +
                                               (uint32_t)((p_ab + hh) * kTcN + half * (kTcN / 2) + c0 + h16);
-                        asm volatile(
-                            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-                            "%14,%15}, [%16];"
-                            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-                              "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-                              "=r"(v[14]), "=r"(v[15])
-                            : "r"(addr));
+                        tc_ld16(addr, v);
                         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                         for (int x = 0; x < 16; ++x) {

@@ -45,7 +45,12 @@
 //     FP64 accumulators;
 //   warp 17 (one lane) issues the MMAs of each stage once it is written, commits to the stage's
 //     "empty" barrier and, at the end of a unit, to the accumulator barrier.
-// 81920 panels, 64 right-hand sides, with the preparing kernels: 2.19 ms; 3.44 with TF32 parts (a stage
+// While a unit's accumulators are drained no MMA runs, so units are long (tc_unit) and the drain adds
+// whole 32-byte sectors: rows 2 j and 2 j + 1 of an operand are re and im of right-hand side j, and a
+// warp exchanges halves of D_V and D_K so that one instruction adds all four components of eight.
+// 81920 panels, 64 right-hand sides, with the preparing kernels: 1.77 ms; 1.92 with the sectors
+// touched by two instructions each and every range's bounds loaded when it begins instead of one range
+// ahead, 2.19 with units of 2048 sources besides; 3.44 with TF32 parts (a stage
 // of 8 sources took 0.86 us, 0.48 of it the MMAs and as much its 121 KB of shared-memory traffic; FP16
 // halves both per source); 4.24 with the weights split by four of the generating warps (which every
 // stage waited for) and a barrier arrival per thread.  Error of the product of 28 right-hand sides
@@ -183,14 +188,12 @@ __global__ void __launch_bounds__(128)
         w[3][i] = v.w * fk;
     }
     const bool stacked = nb <= kRC / 2;
-    // rows: re j, im 64 + j, the high part, then the low part; stacked: re hi j, im hi 32 + j, re lo
-    // 64 + j, im lo 96 + j
-    const int im = stacked ? 32 : 64;
+    // rows: 2 j + (0: re, 1: im), the high part, then the low part; stacked: the low rows are 64 + 2 j + ..
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         unsigned char *o = img + blk * kImgBlock + (c >> 1) * (stacked ? kAPart : 2 * kAPart);
-        unsigned char *hi = o + core_off((c & 1) * im + j, q);
-        H::split(w[c], hi, stacked ? o + core_off(64 + (c & 1) * im + j, q) : hi + kAPart);
+        unsigned char *hi = o + core_off(2 * j + (c & 1), q);
+        H::split(w[c], hi, stacked ? o + core_off(64 + 2 * j + (c & 1), q) : hi + kAPart);
     }
 }
 
@@ -270,8 +273,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 const int4 item = __ldg(items + ii);
                 bool ok = true;
                 const int um = set_surfaces(b0, nb, Bact, nsurf);
+                int4 e_nx = item.y < item.z ? __ldg(ivl + item.y) : make_int4(0, 0, 0, 0);   // one range ahead
                 for (int iv = item.y; iv < item.z && ok; ++iv) {
-                    const int4 e = __ldg(ivl + iv);
+                    const int4 e = e_nx;
+                    if (iv + 1 < item.z) e_nx = __ldg(ivl + iv + 1);
                     if (!(e.w & um)) continue;   // no source of the unit's surfaces (all roles agree)
                     for (int g = e.x / kSrc; g * kSrc < e.y; ++g, ++seq) {
                         const int s = (int)(seq % kStages);
@@ -320,8 +325,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 {
                     const uint32_t dv = tmem, dk = tmem + (uint32_t)kTcN;
                     bool ok = true, first = true;
+                    int4 e_nx = item.y < item.z ? __ldg(ivl + item.y) : make_int4(0, 0, 0, 0);
                     for (int iv = item.y; iv < item.z && ok; ++iv) {
-                        const int4 e = __ldg(ivl + iv);
+                        const int4 e = e_nx;
+                        if (iv + 1 < item.z) e_nx = __ldg(ivl + iv + 1);
                         if (!(e.w & um)) continue;
                         // the accumulators are free once the previous unit is drained
                         if (first && nu >= 1) {
@@ -390,47 +397,44 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         // targets from column 64 (w / 4) of both accumulators; false: a wait ran out
         auto drain_acc = [&]() -> bool {
             const int qd = warp & 3, part = warp >> 2;
-            if (!warp_wait(smem_addr(&acc_full), (uint32_t)((nu - 1) & 1), &abort_s)) return false;
-            asm volatile("tcgen05.fence::after_thread_sync;");
-            const int m = 32 * qd + lane;
-            // row m: without stacking re (m < 64) / im of right-hand side m % 64; stacked: re / im
-            // of m % 32 in the high (m < 64) or the low half
-            const int j = p_stacked ? (m & 31) : (m & 63);
-            const int cpt = p_stacked ? ((m >> 5) & 1) : (m >> 6);
-            const bool row_on = j < p_nb;
+            const int64_t tc0 = p_tbase + part * (kTcN / 4) + lane;   // the targets of this lane's columns
+            const int pc0 = tc0 < ntgt ? panel_of(tgt[tc0].w) : -1;
+            const int pc1 = tc0 + 32 < ntgt ? panel_of(tgt[tc0 + 32].w) : -1;
+            // row m: 2 j + (0: re, 1: im) of right-hand side j; stacked: of the high (m < 64) or the low half
+            const int m = (32 * qd + lane) & (p_stacked ? 63 : 127), j = m >> 1;
             // the scales undone: of the kernel values and of the weights
             float undo_v = 1.f, undo_k = 1.f;
-            if (F16 && row_on) {
+            if (F16 && j < p_nb) {
                 undo_v = 1.f / gs * (1.f / f16_scale(__ldg(mx + 2 * (p_b0 + j))));
                 undo_k = 1.f / ts * (1.f / f16_scale(__ldg(mx + 2 * (p_b0 + j) + 1)));
             }
-            if (__any_sync(0xffffffffu, row_on)) {
+            if (!warp_wait(smem_addr(&acc_full), (uint32_t)((nu - 1) & 1), &abort_s)) return false;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            // The 16 right-hand sides of the warp's rows are added eight at a time, all four components of
+            // each by one instruction (whole 32-byte sectors; a warp per accumulator would touch every
+            // sector twice): lanes 0-15 take D_V, lanes 16-31 D_K, after one exchange between the halves.
+            const bool dk = lane >= 16;
+            const int jw = (m - lane) >> 1, ja = jw + ((lane & 15) >> 1), jb = ja + 8;   // the lane's right-hand sides
+            double *const dst = acc + 4 * (p_b0 + ja) + 2 * (int)dk + (lane & 1);
+            if (jw < p_nb) {
 #pragma unroll 1
-                for (int c0 = 0; c0 < kTcN / 4; c0 += 32) {
-                    const int64_t tc = p_tbase + part * (kTcN / 4) + c0 + lane;   // this lane's column's target
-                    const int pc = tc < ntgt ? panel_of(tgt[tc].w) : -1;
-#pragma unroll 1
-                    for (int op = 0; op < 2; ++op) {   // D_V, then D_K
+                for (int c0 = 0; c0 < kTcN / 4; c0 += 16) {
+                    uint32_t v[16], k[16];
+                    const uint32_t addr = tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(part * (kTcN / 4) + c0);
+                    tc_ld16(addr, v);
+                    tc_ld16(addr + kTcN, k);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    const int pc = c0 < 32 ? pc0 : pc1;
 #pragma unroll
-                        for (int h16 = 0; h16 < 32; h16 += 16) {
-                            uint32_t v[16];
-                            const uint32_t addr = tmem + ((uint32_t)(32 * qd) << 16) +
-                                                  (uint32_t)(op * kTcN + part * (kTcN / 4) + c0 + h16);
-                            asm volatile(
-                                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-                                "%14,%15}, [%16];"
-                                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-                                  "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
-                                  "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                                : "r"(addr));
-                            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                            for (int x = 0; x < 16; ++x) {
-                                const int p = __shfl_sync(0xffffffffu, pc, h16 + x);
-                                if (row_on && p >= 0)
-                                    atomicAdd(acc + 4 * ((int64_t)p * B + p_b0 + j) + 2 * op + cpt,
-                                              (double)(F16 ? __uint_as_float(v[x]) * (op ? undo_k : undo_v) : __uint_as_float(v[x])));
-                            }
+                    for (int x = 0; x < 16; ++x) {
+                        const int p = __shfl_sync(0xffffffffu, pc, (c0 & 16) + x);
+                        float fv = __uint_as_float(v[x]), fk = __uint_as_float(k[x]);
+                        if (F16) fv *= undo_v, fk *= undo_k;
+                        const float y = __shfl_xor_sync(0xffffffffu, dk ? fv : fk, 16);
+                        if (p >= 0) {
+                            double *const o = dst + 4 * (int64_t)p * B;
+                            if (ja < p_nb) atomicAdd(o, (double)(dk ? y : fv));
+                            if (jb < p_nb) atomicAdd(o + 32, (double)(dk ? fk : y));
                         }
                     }
                 }
@@ -465,8 +469,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const float2 qz = make_float2(q.z * ig, q.z * ig);
             const int um = set_surfaces(b0, nb, Bact, nsurf);
             bool begun = false;
+            int4 e_nx = item.y < item.z ? __ldg(ivl + item.y) : make_int4(0, 0, 0, 0);
             for (int iv = item.y; iv < item.z && ok; ++iv) {
-                const int4 e = __ldg(ivl + iv);
+                const int4 e = e_nx;
+                if (iv + 1 < item.z) e_nx = __ldg(ivl + iv + 1);
                 if (!(e.w & um)) continue;
                 begun = true;
                 const bool on = live && ((e.z >> blk) & 1);   // uniform over the warp but for the tail
