@@ -173,8 +173,8 @@ __device__ __forceinline__ void m2p_ff_unit(const int4 &item, int B, int b0, int
 // coefficients live in its column of the warp's ring), and the contraction accumulates with
 // ff_mac2, the real and imaginary channel at once.  A unit takes the narrowest of NB, NB / 2 and
 // NB / 4 that holds its right-hand sides (the contraction is 9/10 of the work).  Issue-bound.
-// 40500 panels, 12 right-hand sides: 11.7 ms, 15.0 with units of eight and scalar parts (20480 panels,
-// 16: 4.32 after 4.63).
+// 40500 panels, 12 right-hand sides: 10.5 ms (11.7 with 12 operations per product, 15.0 with units of
+// eight and scalar parts).
 template <int NB>
 __global__ void __launch_bounds__(64)
     m2p_ff_kernel(const int4 *__restrict__ items, int64_t nitems, int nbc, int B, int NT,
@@ -284,7 +284,7 @@ __device__ __forceinline__ void p2p_ff1_unit(const int4 &item, int B, int b0, in
 #pragma unroll 2
         for (int kk = 0; kk < cnt; ++kk) {
             const ff4 p = sh[0][kk], n = sh[1][kk];
-            const ffloat dx = q.x - p.x, dy = q.y - p.y, dz = q.z - p.z;
+            const ffloat dx = ff_diff(q.x, p.x), dy = ff_diff(q.y, p.y), dz = ff_diff(q.z, p.z);
             ffloat r = rsq(dx * dx + dy * dy + dz * dz);
             if ((item.w & 1) && panel_of(n.w) == tp) r = ffloat(0.f, 0.f);
             const ffloat tk = (dx * n.x + dy * n.y + dz * n.z) * (r * r) * r;
@@ -308,7 +308,8 @@ __device__ __forceinline__ void p2p_ff1_unit(const int4 &item, int B, int b0, in
     }
 }
 
-// 40500 panels, 12 right-hand sides: 7.88 ms, 9.52 with units of eight and scalar parts.
+// 40500 panels, 12 right-hand sides: 7.1 ms (7.88 with 12 operations per product, 9.52 with units of eight
+// and scalar parts).
 template <int NB>
 __global__ void __launch_bounds__(kFfP2PWarps * 32)
     p2p_ff1_kernel(const int4 *__restrict__ items, int64_t nitems, int B, const ff4 *__restrict__ tgt, int64_t ntgt,

@@ -50,6 +50,18 @@ __device__ __forceinline__ ffloat operator+(const ffloat &x, const ffloat &y) {
 __device__ __forceinline__ ffloat operator-(const ffloat &x) { return ffloat(-x.hi, -x.lo); }
 __device__ __forceinline__ ffloat operator-(const ffloat &x, const ffloat &y) { return x + (-y); }
 
+// x - y with the difference of the low parts kept whole: for coordinates of close points, whose leading
+// parts cancel, so that only the rounding of the coordinates themselves is left
+__device__ __forceinline__ ffloat ff_diff(const ffloat &x, const ffloat &y) {
+    float s, e, l, le;
+    ff_two_sum(x.hi, -y.hi, s, e);
+    ff_two_sum(x.lo, -y.lo, l, le);
+    ffloat r;
+    ff_quick_two_sum(s, __fadd_rn(e, l), r.hi, r.lo);
+    r.lo = __fadd_rn(r.lo, le);
+    return r;
+}
+
 __device__ __forceinline__ ffloat operator*(const ffloat &x, const ffloat &y) {
     const float p = __fmul_rn(x.hi, y.hi);
     float e = __fmaf_rn(x.hi, y.hi, -p);   // exact error of the leading product
@@ -76,26 +88,27 @@ __device__ __forceinline__ void ff_mac(ffloat &acc, const ffloat &a, const ffloa
     acc.lo = __fadd_rn(acc.lo, __fadd_rn(e, pe));
 }
 
-// Two float-float values side by side, their parts packed (f32x2): the operations of ff_mac in half
-// the instructions.  The FP32 pipe takes the same time, but the issue slots it leaves go to the
-// loads and address arithmetic around it.
+// Two float-float values side by side, their parts packed (f32x2): half the instructions, the same
+// FP32 operations.
 struct ff2 {
     float2 hi, lo;
 };
-// acc += a b elementwise with a = (ah, al) given as one factor for both and nah = -ah; every rounding
-// is that of ff_mac (a difference x - y is the fused -1 y + x, rounded once)
+// acc += a b elementwise with a = (ah, al) given as one factor for both and nah = -ah, in 10 operations
+// instead of ff_mac's 12: with p = RN(ah bh), s = RN(acc.hi + p) and v = RN(s - acc.hi) the error of the
+// sum is u + (p - v), u = acc.hi - (s - v), both exact (two-sum), so the fused t = ah bh - v gives p - v
+// and the product's own error in one rounding of a number of the size of s's last place.  A difference
+// x - y is the fused -1 y + x, rounded once; s takes that form too, since a packed product and addition
+// side by side would be contracted, and an unrounded p breaks the two-sum (errors of 5e-9).  The
+// kernels that use it are bound by the FP32 pipe: 40500 panels, 12 right-hand sides 20.9 -> 19.1 ms.
 __device__ __forceinline__ void ff_mac2(ff2 &acc, float2 ah, float2 nah, float2 al, float2 bh, float2 bl) {
     const float2 m1 = make_float2(-1.f, -1.f);
-    const float2 np = __fmul2_rn(nah, bh);                  // -p
-    float2 pe = __ffma2_rn(ah, bh, np);                     // exact error of p
-    pe = __ffma2_rn(ah, bl, pe);
-    pe = __ffma2_rn(al, bh, pe);
-    const float2 s = __ffma2_rn(np, m1, acc.hi);            // acc.hi + p
-    const float2 v = __ffma2_rn(acc.hi, m1, s);
-    const float2 t = __ffma2_rn(__ffma2_rn(v, m1, s), m1, acc.hi);   // acc.hi - (s - v)
-    const float2 e = __ffma2_rn(__fadd2_rn(np, v), m1, t);           // + (p - v)
+    const float2 s = __ffma2_rn(__fmul2_rn(nah, bh), m1, acc.hi);
+    const float2 nv = __ffma2_rn(s, m1, acc.hi);                     // -v
+    const float2 u = __ffma2_rn(__fadd2_rn(s, nv), m1, acc.hi);
+    const float2 t = __ffma2_rn(ah, bh, nv);
+    const float2 x = __ffma2_rn(al, bh, __ffma2_rn(ah, bl, u));
     acc.hi = s;
-    acc.lo = __fadd2_rn(acc.lo, __fadd2_rn(e, pe));
+    acc.lo = __fadd2_rn(acc.lo, __fadd2_rn(x, t));
 }
 __device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
 
@@ -103,15 +116,14 @@ __device__ __forceinline__ ffloat &operator+=(ffloat &x, const ffloat &y) { retu
 __device__ __forceinline__ ffloat &operator-=(ffloat &x, const ffloat &y) { return x = x - y; }
 __device__ __forceinline__ ffloat &operator*=(ffloat &x, const ffloat &y) { return x = x * y; }
 
-// 1/sqrt(x): FP32 seed y0, then one Newton-Raphson step y0 (1 + h/2), h = 1 - x y0^2
-// formed in float-float (1 - leading part is exact since x y0^2 is close to 1); the
-// step leaves a relative error of about (3/8) h^2 ~ 1e-13.
+// 1/sqrt(x): FP32 seed y0, then one third-order step y0 (1 + h/2 + 3 h^2/8), h = 1 - x y0^2
+// formed in float-float (1 - leading part is exact since x y0^2 is close to 1).
 __device__ __forceinline__ ffloat rsq(const ffloat &x) {
     const float y0 = rsqrtf(x.hi);
     const ffloat xy2 = x * (ffloat(y0) * ffloat(y0));
     const float h = __fsub_rn(__fsub_rn(1.f, xy2.hi), xy2.lo);
     ffloat r;
-    ff_quick_two_sum(y0, __fmul_rn(__fmul_rn(0.5f, y0), h), r.hi, r.lo);
+    ff_quick_two_sum(y0, __fmul_rn(__fmul_rn(y0, h), __fmaf_rn(0.375f, h, 0.5f)), r.hi, r.lo);
     return r;
 }
 
