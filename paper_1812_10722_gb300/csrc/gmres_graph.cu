@@ -39,10 +39,10 @@ namespace lspr {
 namespace {
 
 constexpr int kT = 256;                 // threads per block of the vector kernels
-constexpr int kPer = 8;                 // entries per thread of an inner-product block's chunk
 constexpr double kReorthEta = 0.70710678118654752;   // second pass when ||w_1|| < eta ||w_0||
-constexpr int kDotChunk = kT * kPer;    // elements per inner-product block
-constexpr int kMaxWarpsSmall = 16;      // warps of the per-system (rotation, back substitution) kernels
+constexpr int kDotChunk = 1024;         // entries per inner-product block
+constexpr int kDotSub = 4;              // parts of a chunk: a warp's task is four basis vectors on one part
+constexpr int kAxpyPer = 2;             // entries per thread of the update
 
 // one complex entry in float-float: re = rh + rl, im = ih + il
 struct __align__(16) cff {
@@ -71,18 +71,26 @@ __device__ __forceinline__ cff pack(const ffloat &re, const ffloat &im) {
     return {r.hi, i.hi, r.lo, i.lo};
 }
 
-// (sr, si) += conj(v) w
-__device__ __forceinline__ void cff_conj_mac(ffloat &sr, ffloat &si, const cff &v, const cff &w) {
-    const ffloat vr = re_of(v), vi = im_of(v), wr = re_of(w), wi = im_of(w);
-    ff_mac(sr, vr, wr);
-    ff_mac(sr, vi, wi);
-    ff_mac(si, vr, wi);
-    ff_mac(si, -vi, wr);
+// Packed products of a complex factor f with v: a += f_re (v_re, v_im), b += f_im (v_re, v_im), so that
+// f v = (a.x - b.y, a.y + b.x) and f conj(v) = (a.x + b.y, b.x - a.y).  f's parts come in both halves of
+// a pair, the leading ones with their negatives (ff_mac2).
+struct CPair {
+    ff2 a, b;
+};
+struct __align__(16) CFactor {
+    float2 rh, nrh, rl, ih, nih, il;
+};
+__device__ __forceinline__ CFactor factor(const cff &f) {
+    return {both(f.rh), both(-f.rh), both(f.rl), both(f.ih), both(-f.ih), both(f.il)};
 }
-// (ar, ai) += v h, or -= v h with SUB
-template <bool SUB>
+__device__ __forceinline__ void cff_mac2(CPair &p, const CFactor &f, const float4 &v) {
+    const float2 vh = make_float2(v.x, v.y), vl = make_float2(v.z, v.w);
+    ff_mac2(p.a, f.rh, f.nrh, f.rl, vh, vl);
+    ff_mac2(p.b, f.ih, f.nih, f.il, vh, vl);
+}
+// (ar, ai) += v h
 __device__ __forceinline__ void cff_mac(ffloat &ar, ffloat &ai, const cff &v, const cff &h) {
-    const ffloat vr = SUB ? -re_of(v) : re_of(v), vi = SUB ? -im_of(v) : im_of(v);
+    const ffloat vr = re_of(v), vi = im_of(v);
     const ffloat hr = re_of(h), hi = im_of(h);
     ff_mac(ar, vr, hr);
     ff_mac(ar, -vi, hi);
@@ -113,7 +121,7 @@ struct Arn {
     double *npart, *nrm, *cs, *res, *npart0, *nrm0;
     int *reorth;
     const double *bn, *par;
-    unsigned *tick;
+    unsigned *tick;      // [2B + 1] last-block tickets
     int *jdev, *active, *jb, *iters;
     int *rmap;   // [2B + 2]: slot -> system, system -> slot (-1: not running), running count,
                  // channel sets in use (running count x surfaces)
@@ -124,20 +132,25 @@ struct Arn {
 
 __device__ __forceinline__ cff *wff(const Arn &a, int b) { return (cff *)(a.w + (int64_t)b * a.n2); }
 
-// packs the running systems into the first slots (single thread)
-__device__ __forceinline__ void pack_running(const Arn &a) {
+// packs the running systems into the first slots (one whole warp); returns their number
+__device__ __forceinline__ int pack_running(const Arn &a) {
+    const int lane = threadIdx.x & 31;
     int n = 0;
-    for (int b = 0; b < a.B; ++b) {
-        if (a.active[b]) {
-            a.rmap[n] = b;
-            a.rmap[a.B + b] = n++;
-        } else {
-            a.rmap[a.B + b] = -1;
-        }
+    for (int b0 = 0; b0 < a.B; b0 += 32) {
+        const int b = b0 + lane;
+        const bool on = b < a.B && __ldcg(a.active + b);
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        const int slot = n + __popc(m & ((1u << lane) - 1));
+        if (on) a.rmap[slot] = b;
+        if (b < a.B) a.rmap[a.B + b] = on ? slot : -1;
+        n += __popc(m);
     }
-    for (int q = n; q < a.B; ++q) a.rmap[q] = 0;
-    a.rmap[2 * a.B] = n;
-    a.rmap[2 * a.B + 1] = n * a.S;
+    for (int q = n + lane; q < a.B; q += 32) a.rmap[q] = 0;
+    if (lane == 0) {
+        a.rmap[2 * a.B] = n;
+        a.rmap[2 * a.B + 1] = n * a.S;
+    }
+    return n;
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -190,9 +203,9 @@ __device__ __forceinline__ bool last_block(unsigned *t, unsigned count) {
 
 // final sum of the squared-norm partials of system b into nrm[b] and 1/nrm[b] (last block
 // only); decide: the first Gram-Schmidt pass decides whether the second runs
-__device__ __forceinline__ void norm_final(const Arn &a, int b, double *sh, bool decide = false) {
+__device__ __forceinline__ void norm_final(const Arn &a, int b, int nblk, double *sh, bool decide = false) {
     double t = 0.0;
-    for (int c = threadIdx.x; c < a.nblk; c += kT) t += __ldcg(a.npart + (int64_t)b * a.nblk + c);
+    for (int c = threadIdx.x; c < nblk; c += kT) t += __ldcg(a.npart + (int64_t)b * a.nblk + c);
     t = block_sum(t, sh);
     if (threadIdx.x == 0) {
         const double r = sqrt(t);
@@ -228,7 +241,7 @@ __global__ void __launch_bounds__(kT) arn_resid_kernel(Arn a, int x_zero) {
     }
     q = block_sum(q, sh);
     if (threadIdx.x == 0) a.npart[(int64_t)b * a.nblk + blockIdx.x] = q;
-    if (last_block(a.tick + a.B + b, a.nblk)) norm_final(a, b, sh);
+    if (last_block(a.tick + a.B + b, a.nblk)) norm_final(a, b, a.nblk, sh);
 }
 
 // v_0 = -w / beta for the running systems (w = A x - b); cycle state reset
@@ -246,9 +259,10 @@ __global__ void __launch_bounds__(kT) arn_init_kernel(Arn a) {
             a.tick[a.B + b] = 0;
             if (b == 0) {
                 *a.jdev = 0;
-                pack_running(a);
+                a.tick[2 * a.B] = 0;
             }
         }
+        if (b == 0 && threadIdx.x < 32) pack_running(a);
     }
 }
 
@@ -280,15 +294,79 @@ __global__ void __launch_bounds__(kT) arn_precond_kernel(Arn a) {
 
 // One classical Gram-Schmidt pass, first half: h_i = <v_i, w> for i <= j.  A block takes a
 // chunk of kDotChunk entries of one system: its threads stage the chunk of w in shared memory
-// (pass 0 converts w to float-float in place and forms ||w||^2 of the chunk), then warp q takes
-// the basis vectors q, q + 8, ...: its lanes stride over the chunk (64 entries each, with four
-// independent float-float accumulator pairs, so many loads are in flight) and one warp reduction
-// per vector gives the chunk's partial product.  The last block of the system sums the chunks
-// into h (FP64 and float-float) and into the Hessenberg column (hcol = h on pass 0, hcol += h on
-// pass 1).
-__global__ void __launch_bounds__(kT) arn_dot_kernel(Arn a, int pass) {
-    __shared__ cff ws[kDotChunk];
-    __shared__ double2 red[kMaxRestart + 1];
+// (pass 0 converts w to float-float in place and forms ||w||^2 of the chunk), then a warp takes
+// tasks of four basis vectors on a kDotSub-th of the chunk, so that an entry of w read from shared
+// memory serves four products and eight loads per lane are in flight.  The 8 sums of a task are
+// reduced over the warp by halves (9 exchanges instead of 40).  The last block of the system sums
+// the chunks into h (FP64 and float-float) and into the Hessenberg column (hcol = h on pass 0,
+// hcol += h on pass 1).
+// 20480 panels, 16 systems, mid-cycle, cold caches: 51 us (81 with one vector per warp, chunks of 2048 and
+// unpacked products, whose 320 blocks left SMs idle).
+constexpr int kDotVec = 4;
+inline size_t dot_smem(int m) {   // w and the sums of the parts
+    return kDotChunk * sizeof(cff) + (size_t)kDotSub * (m + 1) * sizeof(double2);
+}
+template <int NV>
+__device__ __forceinline__ void dot_task(const cff *__restrict__ v, int64_t stride, const cff *ws, int e0, int len,
+                                         double2 *red) {
+    const int lane = threadIdx.x & 31;
+    CPair p[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+        p[k].a.hi = p[k].a.lo = p[k].b.hi = p[k].b.lo = make_float2(0.f, 0.f);
+    constexpr int kU = 2;   // entries loaded together
+#pragma unroll 1
+    for (int e = e0 + lane; e < e0 + kDotChunk / kDotSub; e += 32 * kU) {
+        float4 x[kU][NV];
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+#pragma unroll
+            for (int k = 0; k < NV; ++k)
+                x[u][k] = e + 32 * u < len ? __ldg((const float4 *)(v + k * stride + e + 32 * u))
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const CFactor f = factor(ws[e + 32 * u]);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) cff_mac2(p[k], f, x[u][k]);
+        }
+    }
+    // w conj(v): (a.x + b.y, b.x - a.y)
+    ffloat t[2 * NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        t[2 * k] = ff_norm(ffloat(p[k].a.hi.x, p[k].a.lo.x)) + ff_norm(ffloat(p[k].b.hi.y, p[k].b.lo.y));
+        t[2 * k + 1] = ff_norm(ffloat(p[k].b.hi.x, p[k].b.lo.x)) - ff_norm(ffloat(p[k].a.hi.y, p[k].a.lo.y));
+    }
+    if (NV == 4) {   // each exchange halves the values a lane holds: lanes with the same lane >> 2 end with one
+#pragma unroll
+        for (int o = 16, n = NV; o >= 4; o >>= 1, n >>= 1) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int q = 0; q < n; ++q) {
+                const ffloat send = up ? t[q] : t[q + n], keep = up ? t[q + n] : t[q];
+                t[q] = keep + shfl_xor(send, o);
+            }
+        }
+        ffloat s = t[0] + shfl_xor(t[0], 2);
+        s = s + shfl_xor(s, 1);
+        if ((lane & 3) == 0) {   // value 4 (bit 4) + 2 (bit 3) + (bit 2) of the lane
+            const int q = ((lane & 16) >> 2) | ((lane & 8) >> 2) | ((lane & 4) >> 2);
+            ((double *)red)[q] = (double)s;
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < 2 * NV; ++q) {
+            const ffloat s = ff_warp_sum(t[q]);
+            if (lane == 0) ((double *)red)[q] = (double)s;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kT, 2) arn_dot_kernel(Arn a, int pass) {
+    extern __shared__ double2 dsm[];
+    cff *ws = (cff *)dsm;
+    double2 *red = dsm + kDotChunk;   // [kDotSub][m + 1]
     __shared__ double shn[kT / 32];
     const int b = blockIdx.y, chunk = blockIdx.x;
     if (!a.active[b] || (pass && !a.reorth[b])) return;
@@ -317,36 +395,27 @@ __global__ void __launch_bounds__(kT) arn_dot_kernel(Arn a, int pass) {
     }
     __syncthreads();
     const cff *Vb = a.V + (int64_t)b * a.vstride + c0;
-    for (int i = warp; i < nv; i += kT / 32) {
+    const int tasks = kDotSub * ((nv + kDotVec - 1) / kDotVec);
+    for (int q = warp; q < tasks; q += kT / 32) {
+        const int sub = q % kDotSub, i = q / kDotSub * kDotVec;
         const cff *v = Vb + (int64_t)i * a.n2;
-        ffloat sr[4], si[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) sr[u] = si[u] = ffloat(0.f, 0.f);
-        if (len == kDotChunk) {
-            // eight entries per lane loaded together before they are used (more bytes in flight)
-#pragma unroll 1
-            for (int e0 = lane; e0 < kDotChunk; e0 += 256) {
-                float4 vv[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) vv[u] = __ldg((const float4 *)(v + e0 + 32 * u));
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const cff x = {vv[u].x, vv[u].y, vv[u].z, vv[u].w};
-                    cff_conj_mac(sr[u & 3], si[u & 3], x, ws[e0 + 32 * u]);
-                }
-            }
-        } else {   // the ragged last chunk
-            for (int e = lane; e < len; e += 32) cff_conj_mac(sr[0], si[0], v[e], ws[e]);
+        double2 *r = red + sub * (a.m + 1) + i;
+        const int e0 = sub * (kDotChunk / kDotSub);
+        switch (min(kDotVec, nv - i)) {
+            case 4: dot_task<4>(v, a.n2, ws, e0, len, r); break;
+            case 3: dot_task<3>(v, a.n2, ws, e0, len, r); break;
+            case 2: dot_task<2>(v, a.n2, ws, e0, len, r); break;
+            default: dot_task<1>(v, a.n2, ws, e0, len, r); break;
         }
-        ffloat tr = ff_norm(sr[0]) + ff_norm(sr[1]) + (ff_norm(sr[2]) + ff_norm(sr[3]));
-        ffloat ti = ff_norm(si[0]) + ff_norm(si[1]) + (ff_norm(si[2]) + ff_norm(si[3]));
-        tr = ff_warp_sum(tr);
-        ti = ff_warp_sum(ti);
-        if (lane == 0) red[i] = make_double2((double)tr, (double)ti);
     }
     __syncthreads();
     double2 *pb = a.part + (int64_t)b * (a.m + 1) * a.nch;
-    for (int i = threadIdx.x; i < nv; i += kT) pb[(int64_t)i * a.nch + chunk] = red[i];
+    for (int i = threadIdx.x; i < nv; i += kT) {
+        double2 t = red[i];
+#pragma unroll
+        for (int s = 1; s < kDotSub; ++s) t = cadd(t, red[s * (a.m + 1) + i]);
+        pb[(int64_t)i * a.nch + chunk] = t;
+    }
     if (!last_block(a.tick + b, a.nch)) return;
     if (pass == 0) {
         double t = 0.0;
@@ -384,50 +453,68 @@ __global__ void __launch_bounds__(kT) arn_dot_kernel(Arn a, int pass) {
 // decides whether the second runs (reorth[b])
 __global__ void __launch_bounds__(kT) arn_axpy_kernel(Arn a, int pass) {
     __shared__ double sh[kT / 32];
-    __shared__ cff hs[kMaxRestart + 1];
+    __shared__ CFactor hs[kMaxRestart + 1];
     const int b = blockIdx.y;
     if (!a.active[b] || (pass && !a.reorth[b])) return;
     const int nv = *a.jdev + 1;
-    for (int i = threadIdx.x; i < nv; i += kT) hs[i] = a.hff[(int64_t)b * (a.m + 1) + i];
+    for (int i = threadIdx.x; i < nv; i += kT) {
+        const cff h = a.hff[(int64_t)b * (a.m + 1) + i];
+        hs[i] = factor({-h.rh, -h.ih, -h.rl, -h.il});
+    }
     __syncthreads();
-    const int64_t k = blockIdx.x * (int64_t)kT + threadIdx.x;
-    ffloat q(0.f, 0.f);
-    if (k < a.n2) {
-        const cff *Vb = a.V + (int64_t)b * a.vstride + k;
-        cff *wk = wff(a, b) + k;
-        const cff w0 = *wk;
-        ffloat ar = re_of(w0), ai = im_of(w0);
+    const int64_t k0 = blockIdx.x * (int64_t)(kT * kAxpyPer) + threadIdx.x;
+    const cff *Vb = a.V + (int64_t)b * a.vstride;
+    cff *wb = wff(a, b);
+    CPair p[kAxpyPer];
+    bool on[kAxpyPer];
+    int64_t k[kAxpyPer];
+#pragma unroll
+    for (int u = 0; u < kAxpyPer; ++u) {
+        on[u] = k0 + u * kT < a.n2;
+        k[u] = on[u] ? k0 + u * kT : a.n2 - 1;   // the entry of a thread past the end is read and dropped
+        const cff w0 = wb[k[u]];
+        p[u].a.hi = make_float2(w0.rh, w0.ih);
+        p[u].a.lo = make_float2(w0.rl, w0.il);
+        p[u].b.hi = p[u].b.lo = make_float2(0.f, 0.f);
+    }
 #pragma unroll 4
-        for (int i = 0; i < nv; ++i) cff_mac<true>(ar, ai, Vb[(int64_t)i * a.n2], hs[i]);
-        const cff w1 = pack(ar, ai);
-        *wk = w1;
+    for (int i = 0; i < nv; ++i) {
+        const CFactor h = hs[i];
+#pragma unroll
+        for (int u = 0; u < kAxpyPer; ++u) cff_mac2(p[u], h, *(const float4 *)(Vb + (int64_t)i * a.n2 + k[u]));
+    }
+    ffloat q(0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < kAxpyPer; ++u) {
+        if (!on[u]) continue;
+        // w - h v: (a.x - b.y, a.y + b.x)
+        const cff w1 = pack(ff_norm(ffloat(p[u].a.hi.x, p[u].a.lo.x)) - ff_norm(ffloat(p[u].b.hi.y, p[u].b.lo.y)),
+                            ff_norm(ffloat(p[u].a.hi.y, p[u].a.lo.y)) + ff_norm(ffloat(p[u].b.hi.x, p[u].b.lo.x)));
+        wb[k[u]] = w1;
         cff_abs2_mac(q, re_of(w1), im_of(w1));
     }
     const double t = block_sum_ff(q, sh);
     if (threadIdx.x == 0) a.npart[(int64_t)b * a.nblk + blockIdx.x] = t;
-    if (last_block(a.tick + a.B + b, a.nblk)) norm_final(a, b, sh, pass == 0);
+    if (last_block(a.tick + a.B + b, gridDim.x)) norm_final(a, b, gridDim.x, sh, pass == 0);
 }
 
-// shared memory of the rotation kernel per warp: column (m+1), sines (m), cosines (m)
-inline size_t tail_smem_per_warp(int m) { return (size_t)(3 * m + 1) * sizeof(double2); }
+// shared memory of the rotation kernel: column (m+1), sines (m), cosines (m)
+inline size_t tail_smem(int m) { return (size_t)(3 * m + 1) * sizeof(double2); }
 
-// End of an Arnoldi step, one warp per system: the new Hessenberg column (hcol, ||w||)
+// End of an Arnoldi step, one warp (and block) per system: the new Hessenberg column (hcol, ||w||)
 // is rotated by the previous Givens rotations, a new rotation zeroes its subdiagonal,
 // g is rotated, |g_{j+1}| is the residual estimate and decides whether the system keeps
-// running.  The block then advances j and sets the loop condition (the graph's, or the flag
+// running.  The last block then advances j and sets the loop condition (the graph's, or the flag
 // the host reads): another step runs while a system is running and j < m.
-__global__ void arn_tail_kernel(Arn a) {
+// An FP64 instruction of a single lane holds the SM's FP64 pipe as long as one of 32, so the systems'
+// warps are spread over SMs and the rotations composed by a scan.  16 systems, 30 rotations: 31 us with
+// the systems on 16 warps of one block, 18 spread, less with the scan.
+__global__ void __launch_bounds__(32) arn_tail_kernel(Arn a) {
     extern __shared__ double2 dsm[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x, b = blockIdx.x;
     const int m = a.m, j = *a.jdev;
-    double2 *col = dsm + (size_t)warp * (3 * m + 1);
-    double2 *snw = col + m + 1;
-    double2 *csw = snw + m;
-    const double tol = a.par[0];
-    const int maxit = (int)a.par[1];
-    int any = 0;
-    for (int b = warp; b < a.B; b += nw) {
-        if (!a.active[b]) continue;   // warp-uniform
+    if (__ldcg(a.active + b)) {
+        double2 *col = dsm, *snw = col + m + 1, *csw = snw + m;
         const double2 *hc = a.hcol + (int64_t)b * (m + 1);
         for (int i = lane; i <= j; i += 32) col[i] = hc[i];
         for (int i = lane; i < j; i += 32) {
@@ -435,16 +522,33 @@ __global__ void arn_tail_kernel(Arn a) {
             csw[i] = make_double2(a.cs[(int64_t)b * m + i], 0.0);
         }
         __syncwarp();
-        int act = 0;
-        if (lane == 0) {
-            double2 *Hb = a.H + (int64_t)b * (m + 1) * m;
-            double2 a0 = col[0];
-            for (int i = 0; i < j; ++i) {   // previous rotations, carrying row i+1
-                const double c = csw[i].x;
-                const double2 sg = snw[i], d0 = col[i + 1];
-                Hb[(int64_t)i * m + j] = cadd(cscale(a0, c), cmul(sg, d0));
-                a0 = csub(cscale(d0, c), cmul(cconj(sg), a0));
+        // The previous rotations carry row i + 1: a_0 = col_0, row i gets c a_i + s d, d = col_(i+1), and
+        // a_(i+1) = c d - conj(s) a_i.  Each is an affine map of a_i, so a scan over the lanes composes 32
+        // of them in five steps (the factors conj(s) are at most 1 in magnitude).
+        double2 *Hb = a.H + (int64_t)b * (m + 1) * m;
+        double2 a0 = col[0];
+        for (int i0 = 0; i0 < j; i0 += 32) {
+            const int i = i0 + lane;
+            const bool on = i < j;
+            const double c = on ? csw[i].x : 0.0;
+            const double2 sg = on ? snw[i] : make_double2(0.0, 0.0), d0 = on ? col[i + 1] : make_double2(0.0, 0.0);
+            double2 A = on ? make_double2(-sg.x, sg.y) : make_double2(1.0, 0.0), Bc = cscale(d0, c);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {   // maps composed with those of the lanes before
+                const double2 pA = make_double2(__shfl_up_sync(0xffffffffu, A.x, o), __shfl_up_sync(0xffffffffu, A.y, o));
+                const double2 pB = make_double2(__shfl_up_sync(0xffffffffu, Bc.x, o), __shfl_up_sync(0xffffffffu, Bc.y, o));
+                if (lane >= o) {
+                    Bc = cadd(Bc, cmul(A, pB));
+                    A = cmul(A, pA);
+                }
             }
+            const double2 nx = cadd(Bc, cmul(A, a0));   // a_(i+1)
+            double2 ai = make_double2(__shfl_up_sync(0xffffffffu, nx.x, 1), __shfl_up_sync(0xffffffffu, nx.y, 1));
+            if (lane == 0) ai = a0;
+            if (on) Hb[(int64_t)i * m + j] = cadd(cscale(ai, c), cmul(sg, d0));
+            a0 = make_double2(__shfl_sync(0xffffffffu, nx.x, 31), __shfl_sync(0xffffffffu, nx.y, 31));
+        }
+        if (lane == 0) {
             const double hn = a.nrm[b];   // subdiagonal entry ||w||, real
             const double aa = sqrt(cabs2(a0)), t = sqrt(aa * aa + hn * hn);
             double c;
@@ -473,17 +577,15 @@ __global__ void arn_tail_kernel(Arn a) {
                 atomicAdd(a.stats + 3, 1ull);
             }
             const int it = ++a.iters[b];
-            act = (r / a.bn[b] > tol) && it < maxit && isfinite(r);
-            a.active[b] = act;
+            a.active[b] = (r / a.bn[b] > a.par[0]) && it < (int)a.par[1] && isfinite(r);
         }
-        any |= __shfl_sync(0xffffffffu, act, 0);
-        __syncwarp();
     }
-    const int go = __syncthreads_or(any);
-    if (threadIdx.x == 0) {
-        pack_running(a);
+    if (!last_block(a.tick + 2 * a.B, gridDim.x)) return;
+    const int n = pack_running(a);
+    if (lane == 0) {
+        a.tick[2 * a.B] = 0;
         *a.jdev = j + 1;
-        const unsigned more = (go && j + 1 < m) ? 1u : 0u;
+        const unsigned more = (n && j + 1 < m) ? 1u : 0u;
         if (a.go)
             *a.go = (int)more;
         else
@@ -491,27 +593,22 @@ __global__ void arn_tail_kernel(Arn a) {
     }
 }
 
-// R y = g by back substitution (one warp per system), y into a.y (FP64) and a.yff
-__global__ void arn_backsub_kernel(Arn a) {
-    extern __shared__ double2 ysm[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int m = a.m;
-    double2 *ys = ysm + (size_t)warp * m;
-    for (int b = warp; b < a.B; b += nw) {
-        const int n = a.jb[b];
-        const double2 *Hb = a.H + (int64_t)b * (m + 1) * m, *gb = a.g + (int64_t)b * (m + 1);
-        for (int i = n - 1; i >= 0; --i) {
-            double2 s = make_double2(0.0, 0.0);
-            for (int k = i + 1 + lane; k < n; k += 32) s = cadd(s, cmul(Hb[(int64_t)i * m + k], ys[k]));
-            s = warp_sum2(s);
-            if (lane == 0) ys[i] = cdiv(csub(gb[i], s), Hb[(int64_t)i * m + i]);
-            __syncwarp();
-        }
-        for (int i = lane; i < n; i += 32) {
-            a.y[(int64_t)b * m + i] = ys[i];
-            a.yff[(int64_t)b * m + i] = to_cff(ys[i]);
-        }
+// R y = g by back substitution (one warp and block per system), y into a.y (FP64) and a.yff
+__global__ void __launch_bounds__(32) arn_backsub_kernel(Arn a) {
+    extern __shared__ double2 ys[];
+    const int lane = threadIdx.x, b = blockIdx.x;
+    const int m = a.m, n = a.jb[b];
+    const double2 *Hb = a.H + (int64_t)b * (m + 1) * m, *gb = a.g + (int64_t)b * (m + 1);
+    for (int i = n - 1; i >= 0; --i) {
+        double2 s = make_double2(0.0, 0.0);
+        for (int k = i + 1 + lane; k < n; k += 32) s = cadd(s, cmul(Hb[(int64_t)i * m + k], ys[k]));
+        s = warp_sum2(s);
+        if (lane == 0) ys[i] = cdiv(csub(gb[i], s), Hb[(int64_t)i * m + i]);
         __syncwarp();
+    }
+    for (int i = lane; i < n; i += 32) {
+        a.y[(int64_t)b * m + i] = ys[i];
+        a.yff[(int64_t)b * m + i] = to_cff(ys[i]);
     }
 }
 
@@ -526,8 +623,8 @@ __global__ void __launch_bounds__(kT) arn_update_kernel(Arn a) {
     ffloat r0(0.f, 0.f), i0(0.f, 0.f), r1(0.f, 0.f), i1(0.f, 0.f);
     for (int i = 0; i < n; ++i) {
         const cff yi = yb[i];
-        cff_mac<false>(r0, i0, Vb[(int64_t)i * a.n2 + t], yi);
-        cff_mac<false>(r1, i1, Vb[(int64_t)i * a.n2 + a.N + t], yi);
+        cff_mac(r0, i0, Vb[(int64_t)i * a.n2 + t], yi);
+        cff_mac(r1, i1, Vb[(int64_t)i * a.n2 + a.N + t], yi);
     }
     const double2 u0 = make_double2((double)r0, (double)i0), u1 = make_double2((double)r1, (double)i1);
     double2 o0, o1;
@@ -557,9 +654,20 @@ uint64_t tc_scales(const Tree &tr) {
     return k;
 }
 
-int small_kernel_warps(int B, int m) {
-    const int by_smem = (int)(45000 / tail_smem_per_warp(m));
-    return std::max(1, std::min({B, kMaxWarpsSmall, by_smem}));
+// the two Gram-Schmidt passes and the end of an Arnoldi step
+int launch_orthogonalise(lspr_ctx *ctx, const Arn &a, cudaStream_t st) {
+    static int smem_set[kSmemDevices] = {};
+    LSPR_TRY(ctx, allow_smem(arn_dot_kernel, (int)dot_smem(a.m), ctx->device, smem_set));
+    const dim3 ga(grid_for(a.n2, kT * kAxpyPer), a.B);
+    for (int pass = 0; pass < 2; ++pass) {
+        arn_dot_kernel<<<dim3(a.nch, a.B), kT, dot_smem(a.m), st>>>(a, pass);
+        arn_axpy_kernel<<<ga, kT, 0, st>>>(a, pass);
+        ctx->n_launches += 2;
+    }
+    arn_tail_kernel<<<a.B, 32, tail_smem(a.m), st>>>(a);
+    ++ctx->n_launches;
+    LSPR_TRY(ctx, cudaGetLastError());
+    return LSPR_OK;
 }
 
 // Records one Arnoldi cycle into gc: [init] -> while{step} -> [back substitution, update].
@@ -570,7 +678,6 @@ int capture_cycle(lspr_ctx *ctx, int mode, const Arn &a0, GraphCache &gc) {
     gc.reset();
     cudaStream_t cs = ctx->gstream, saved = ctx->stream;
     const int64_t l0 = ctx->n_launches, mv0 = ctx->matvec_count;
-    const int nw = small_kernel_warps(a0.B, a0.m);
     const dim3 gv(grid_for(a0.n2, kT), a0.B), gN(grid_for(a0.N, kT), a0.B);
     cudaGraph_t g = nullptr;
     bool capturing = false;
@@ -630,21 +737,15 @@ int capture_cycle(lspr_ctx *ctx, int mode, const Arn &a0, GraphCache &gc) {
     const int rc = apply_operator(ctx, mode, a.z, a.w, a.s, a.B);
     ctx->rhs_map = ctx->rhs_inv = ctx->rhs_nact = nullptr;
     if (rc != LSPR_OK) return fail(rc);
-    for (int pass = 0; pass < 2; ++pass) {
-        arn_dot_kernel<<<dim3(a.nch, a.B), kT, 0, cs>>>(a, pass);
-        arn_axpy_kernel<<<gv, kT, 0, cs>>>(a, pass);
-        ctx->n_launches += 2;
-    }
-    arn_tail_kernel<<<1, 32 * nw, nw * tail_smem_per_warp(a.m), cs>>>(a);
-    ++ctx->n_launches;
-    CAP_TRY(cudaGetLastError());
+    const int rt = launch_orthogonalise(ctx, a, cs);
+    if (rt != LSPR_OK) return fail(rt);
     CAP_TRY(cudaStreamEndCapture(cs, &body));
     capturing = false;
     const int64_t l2 = ctx->n_launches;
     // tail: x += M^-1 V y
     CAP_TRY(cudaStreamBeginCaptureToGraph(cs, g, &loop, nullptr, 1, cudaStreamCaptureModeRelaxed));
     capturing = true;
-    arn_backsub_kernel<<<1, 32 * nw, nw * a.m * sizeof(double2), cs>>>(a);
+    arn_backsub_kernel<<<a.B, 32, a.m * sizeof(double2), cs>>>(a);
     arn_update_kernel<<<gN, kT, 0, cs>>>(a);
     CAP_TRY(cudaGetLastError());
     CAP_TRY(cudaStreamEndCapture(cs, &g));
@@ -673,7 +774,6 @@ int host_cycle(lspr_ctx *ctx, int mode, const Arn &a0, int *go_d) {
     a.go = go_d;
     a.cond = 0;
     const int64_t mv0 = ctx->matvec_count;
-    const int nw = small_kernel_warps(a.B, a.m);
     const dim3 gv(grid_for(a.n2, kT), a.B), gN(grid_for(a.N, kT), a.B);
     cudaEvent_t ev;
     timer_begin(ctx, T_GMRES, &ev);
@@ -700,22 +800,15 @@ int host_cycle(lspr_ctx *ctx, int mode, const Arn &a0, int *go_d) {
         ctx->timing_sets = -1;
         LSPR_TRY_ST(rc);
         timer_begin(ctx, T_GMRES, &ev);
-        for (int pass = 0; pass < 2; ++pass) {
-            arn_dot_kernel<<<dim3(a.nch, a.B), kT, 0, st>>>(a, pass);
-            arn_axpy_kernel<<<gv, kT, 0, st>>>(a, pass);
-            ctx->n_launches += 2;
-        }
-        arn_tail_kernel<<<1, 32 * nw, nw * tail_smem_per_warp(a.m), st>>>(a);
-        ++ctx->n_launches;
+        LSPR_TRY_ST(launch_orthogonalise(ctx, a, st));
         timer_end(ctx, T_GMRES, ev);
-        LSPR_TRY(ctx, cudaGetLastError());
         LSPR_TRY(ctx, cudaMemcpyAsync(&more, go_d, sizeof(int), cudaMemcpyDeviceToHost, st));
         if (count)
             LSPR_TRY(ctx, cudaMemcpyAsync(&sets, a.rmap + 2 * a.B + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
         LSPR_TRY(ctx, cudaStreamSynchronize(st));
     }
     timer_begin(ctx, T_GMRES, &ev);
-    arn_backsub_kernel<<<1, 32 * nw, nw * a.m * sizeof(double2), st>>>(a);
+    arn_backsub_kernel<<<a.B, 32, a.m * sizeof(double2), st>>>(a);
     arn_update_kernel<<<gN, kT, 0, st>>>(a);
     ctx->n_launches += 2;
     timer_end(ctx, T_GMRES, ev);
@@ -760,7 +853,7 @@ int gmres_graph_solve(lspr_ctx *ctx, int mode, int B, int m, int maxiter, double
     LSPR_TRY(ctx, ab.res.ensure(B));
     LSPR_TRY(ctx, ab.bn.ensure(B));
     LSPR_TRY(ctx, ab.par.ensure(2));
-    LSPR_TRY(ctx, ab.tick.ensure(2 * (size_t)B));
+    LSPR_TRY(ctx, ab.tick.ensure(2 * (size_t)B + 1));
     LSPR_TRY(ctx, ab.ctl.ensure(1 + 3 * (size_t)B));
     LSPR_TRY(ctx, ab.rmap.ensure(2 * (size_t)B + 2));
     LSPR_TRY(ctx, ab.hff.ensure((size_t)B * (m + 1)));
@@ -824,7 +917,7 @@ int gmres_graph_solve(lspr_ctx *ctx, int mode, int B, int m, int maxiter, double
     LSPR_TRY(ctx, cudaMemcpyAsync(ab.bn.p, bnorm.data(), sizeof(double) * B, cudaMemcpyHostToDevice, st));
     LSPR_TRY(ctx, cudaMemcpyAsync(ab.par.p, par, sizeof(par), cudaMemcpyHostToDevice, st));
     LSPR_TRY(ctx, cudaMemsetAsync(ab.ctl.p, 0, sizeof(int) * (1 + 3 * (size_t)B), st));
-    LSPR_TRY(ctx, cudaMemsetAsync(ab.tick.p, 0, sizeof(unsigned) * 2 * (size_t)B, st));
+    LSPR_TRY(ctx, cudaMemsetAsync(ab.tick.p, 0, sizeof(unsigned) * (2 * (size_t)B + 1), st));
     ++ctx->n_launches;
     arn_precond_setup_kernel<<<grid_for(std::max<int64_t>(N, (int64_t)B * me.S), kT), kT, 0, st>>>(
         N, B * me.S, me.Vself.p, s_d, ab.vinv.p, ab.pq.p);

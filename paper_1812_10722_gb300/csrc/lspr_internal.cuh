@@ -245,7 +245,7 @@ struct ArnoldiBufs {
     DArr<double> res;       // [B] residual estimate |g_{j+1}|
     DArr<double> bn;        // [B] reference norm of the relative residual
     DArr<double> par;       // [2] tolerance, iteration limit
-    DArr<unsigned> tick;    // [2B] last-block tickets
+    DArr<unsigned> tick;    // [2B + 1] last-block tickets
     DArr<int> ctl;          // [1 + 3B] current column j, active[B], jb[B], iters[B]
     DArr<int> rmap;         // [2B + 2] running systems packed first: slot -> b, b -> slot, count, sets
     DArr<float4> hff;       // [B][m+1]  h in float-float (re.hi, im.hi, re.lo, im.lo)
