@@ -113,6 +113,9 @@ struct Arn {
     const double2 *b, *s;
     const double *vinv;  // [N] 1 / V_ii (preconditioner)
     const double2 *pq;   // [B][S] 1 / (1 + s) (preconditioner)
+    const ffloat *vinvf; // [N] the same three in float-float: 1 / V_ii,
+    const cff *pqf, *sf; // [B] 1 / (1 + s), s (one surface)
+    float2 *xtf;         // [2N][B] preconditioned vectors in FP32 (null: z)
     const int *surf;     // surface of each panel; s is [B][S]
     int S;
     double2 *h, *hcol, *part, *H, *sn, *g, *y;
@@ -290,6 +293,52 @@ __global__ void __launch_bounds__(kT) arn_precond_kernel(Arn a) {
     precond(a.vinv[t], a.pq[b * a.S + a.surf[t]], a.s[b * a.S + a.surf[t]], to_d2(v0), to_d2(v1), o0, o1);
     a.z[(int64_t)b * a.n2 + t] = o0;
     a.z[(int64_t)b * a.n2 + a.N + t] = o1;
+}
+
+// The same for FP32 products of several right-hand sides (one surface), which read their vectors
+// transposed and in FP32: formed in float-float (the FP64 form above is bound by the FP64 pipe,
+// some 34 operations per panel) and written transposed, 32 panels x 32 systems per block, instead of
+// going through z and a transposing kernel.  20480 panels, 16 systems: solve 64.6 -> 63.4 ms; 81920
+// panels, 64: 976 -> 948.
+__global__ void __launch_bounds__(256) arn_precond_t_kernel(Arn a) {
+    __shared__ float2 tile[2][32][33];
+    const int64_t t0 = (int64_t)blockIdx.x * 32;
+    const int b0 = blockIdx.y * 32, tx = threadIdx.x;
+    const int j = *a.jdev;
+    const int64_t t = t0 + tx;
+    const ffloat vi = t < a.N ? a.vinvf[t] : ffloat(0.f, 0.f);
+    for (int r = threadIdx.y; r < 32; r += 8) {
+        const int b = b0 + r;
+        if (b >= a.B || t >= a.N || !a.active[b]) continue;
+        cff *Vj = a.V + (int64_t)b * a.vstride + (int64_t)j * a.n2;
+        cff v0, v1;
+        if (j == 0) {
+            v0 = Vj[t];
+            v1 = Vj[a.N + t];
+        } else {
+            const ffloat inv = a.ninv[b];
+            const cff *wb = wff(a, b);
+            const cff w0 = wb[t], w1 = wb[a.N + t];
+            v0 = pack(re_of(w0) * inv, im_of(w0) * inv);
+            v1 = pack(re_of(w1) * inv, im_of(w1) * inv);
+            Vj[t] = v0;
+            Vj[a.N + t] = v1;
+        }
+        const cff s = a.sf[b], q = a.pqf[b];
+        ffloat cr = re_of(v1), ci = im_of(v1), r0(0.f, 0.f), i0(0.f, 0.f), r1(0.f, 0.f), i1(0.f, 0.f);
+        cff_mac(cr, ci, v0, s);   // s u0 + u1
+        cff_mac(r0, i0, pack(cr, ci), q);
+        cff_mac(r1, i1, pack(re_of(v1) - re_of(v0), im_of(v1) - im_of(v0)), q);
+        tile[0][r][tx] = make_float2(2.f * ff_norm(r0).hi, 2.f * ff_norm(i0).hi);
+        tile[1][r][tx] = make_float2((ff_norm(r1) * vi).hi, (ff_norm(i1) * vi).hi);
+    }
+    __syncthreads();
+    const int b = b0 + tx;
+    if (b >= a.B || !a.active[b]) return;
+    for (int r = threadIdx.y; r < 32 && t0 + r < a.N; r += 8) {
+        a.xtf[(t0 + r) * a.B + b] = tile[0][tx][r];
+        a.xtf[(a.N + t0 + r) * a.B + b] = tile[1][tx][r];
+    }
 }
 
 // One classical Gram-Schmidt pass, first half: h_i = <v_i, w> for i <= j.  A block takes a
@@ -637,10 +686,17 @@ __global__ void __launch_bounds__(kT) arn_update_kernel(Arn a) {
 
 // preconditioner constants of a solve: vinv = 1 / V_ii, pq = 1 / (1 + s)
 __global__ void arn_precond_setup_kernel(int64_t N, int BS, const double *Vself, const double2 *s, double *vinv,
-                                         double2 *pq) {
+                                         double2 *pq, ffloat *vinvf, cff *pqf, cff *sf) {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t < N) vinv[t] = 1.0 / Vself[t];
-    if (t < BS) pq[t] = cdiv(make_double2(1.0, 0.0), make_double2(1.0 + s[t].x, s[t].y));
+    if (t < N) {
+        vinv[t] = 1.0 / Vself[t];
+        vinvf[t] = ffloat(vinv[t]);
+    }
+    if (t < BS) {
+        pq[t] = cdiv(make_double2(1.0, 0.0), make_double2(1.0 + s[t].x, s[t].y));
+        pqf[t] = to_cff(pq[t]);
+        sf[t] = to_cff(s[t]);
+    }
 }
 
 // the scales that the tensor-core launches carry by value (powers of two) and their operand parts
@@ -652,6 +708,17 @@ uint64_t tc_scales(const Tree &tr) {
         k = k << 9 | b >> 23;
     }
     return k;
+}
+
+// the start of an Arnoldi step: v_j and M^-1 v_j, which the product takes from z or (null) xtf
+int launch_precond(lspr_ctx *ctx, const Arn &a, cudaStream_t st) {
+    ++ctx->n_launches;
+    if (a.xtf)
+        arn_precond_t_kernel<<<dim3(grid_for(a.N, 32), grid_for(a.B, 32)), dim3(32, 8), 0, st>>>(a);
+    else
+        arn_precond_kernel<<<dim3(grid_for(a.N, kT), a.B), kT, 0, st>>>(a);
+    LSPR_TRY(ctx, cudaGetLastError());
+    return LSPR_OK;
 }
 
 // the two Gram-Schmidt passes and the end of an Arnoldi step
@@ -727,14 +794,14 @@ int capture_cycle(lspr_ctx *ctx, int mode, const Arn &a0, GraphCache &gc) {
     const int64_t l1 = ctx->n_launches;
     CAP_TRY(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
     capturing = true;
-    arn_precond_kernel<<<gN, kT, 0, cs>>>(a);
-    ++ctx->n_launches;
+    const int rp = launch_precond(ctx, a, cs);
+    if (rp != LSPR_OK) return fail(rp);
     // the product works on the running systems only, packed into the first slots (with
     // several surfaces, the S channel sets of a system follow each other)
     ctx->rhs_map = a.rmap;
     ctx->rhs_inv = a.rmap + a.B;
     ctx->rhs_nact = a.rmap + 2 * a.B + 1;
-    const int rc = apply_operator(ctx, mode, a.z, a.w, a.s, a.B);
+    const int rc = apply_operator(ctx, mode, a.xtf ? nullptr : a.z, a.w, a.s, a.B);
     ctx->rhs_map = ctx->rhs_inv = ctx->rhs_nact = nullptr;
     if (rc != LSPR_OK) return fail(rc);
     const int rt = launch_orthogonalise(ctx, a, cs);
@@ -788,14 +855,13 @@ int host_cycle(lspr_ctx *ctx, int mode, const Arn &a0, int *go_d) {
     }
     while (more) {
         timer_begin(ctx, T_GMRES, &ev);
-        arn_precond_kernel<<<gN, kT, 0, st>>>(a);
-        ++ctx->n_launches;
+        LSPR_TRY_ST(launch_precond(ctx, a, st));
         timer_end(ctx, T_GMRES, ev);
         ctx->rhs_map = a.rmap;
         ctx->rhs_inv = a.rmap + a.B;
         ctx->rhs_nact = a.rmap + 2 * a.B + 1;
         ctx->timing_sets = count ? sets : -1;
-        const int rc = apply_operator(ctx, mode, a.z, a.w, a.s, a.B);
+        const int rc = apply_operator(ctx, mode, a.xtf ? nullptr : a.z, a.w, a.s, a.B);
         ctx->rhs_map = ctx->rhs_inv = ctx->rhs_nact = nullptr;
         ctx->timing_sets = -1;
         LSPR_TRY_ST(rc);
@@ -861,6 +927,10 @@ int gmres_graph_solve(lspr_ctx *ctx, int mode, int B, int m, int maxiter, double
     LSPR_TRY(ctx, ab.ninv.ensure(B));
     LSPR_TRY(ctx, ab.vinv.ensure(N));
     LSPR_TRY(ctx, ab.pq.ensure((size_t)B * me.S));
+    LSPR_TRY(ctx, ab.vinvf.ensure(N));
+    LSPR_TRY(ctx, ab.pqf.ensure(2 * (size_t)B * me.S));
+    const bool transposed = mode_prec(mode) == PREC_F32 && B > 1 && me.S == 1;
+    if (transposed) LSPR_TRY(ctx, ctx->xtf.ensure((size_t)B * n2));
     LSPR_TRY(ctx, ab.go.ensure(1));
     if (!ab.stats.p) {
         LSPR_TRY(ctx, ab.stats.ensure(4));
@@ -882,6 +952,10 @@ int gmres_graph_solve(lspr_ctx *ctx, int mode, int B, int m, int maxiter, double
     a.s = s_d;
     a.vinv = ab.vinv.p;
     a.pq = ab.pq.p;
+    a.vinvf = (const ffloat *)ab.vinvf.p;
+    a.pqf = (const cff *)ab.pqf.p;
+    a.sf = a.pqf + (size_t)B * me.S;
+    a.xtf = transposed ? ctx->xtf.p : nullptr;
     a.surf = me.surf.p;
     a.S = me.S;
     a.h = ab.h.p;
@@ -920,7 +994,8 @@ int gmres_graph_solve(lspr_ctx *ctx, int mode, int B, int m, int maxiter, double
     LSPR_TRY(ctx, cudaMemsetAsync(ab.tick.p, 0, sizeof(unsigned) * (2 * (size_t)B + 1), st));
     ++ctx->n_launches;
     arn_precond_setup_kernel<<<grid_for(std::max<int64_t>(N, (int64_t)B * me.S), kT), kT, 0, st>>>(
-        N, B * me.S, me.Vself.p, s_d, ab.vinv.p, ab.pq.p);
+        N, B * me.S, me.Vself.p, s_d, ab.vinv.p, ab.pq.p, (ffloat *)ab.vinvf.p, (cff *)ab.pqf.p,
+        (cff *)ab.pqf.p + (size_t)B * me.S);
     for (int b = 0; b < B; ++b) {
         iters[b] = 0;
         relres[b] = 1.0;

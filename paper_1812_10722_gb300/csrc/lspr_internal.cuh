@@ -253,6 +253,8 @@ struct ArnoldiBufs {
     DArr<float2> ninv;      // [B] 1 / ||w|| in float-float
     DArr<double> vinv;      // [N] 1 / V_ii (preconditioner)
     DArr<double2> pq;       // [B][S] 1 / (1 + s) (preconditioner)
+    DArr<float2> vinvf;     // [N] vinv in float-float
+    DArr<float4> pqf;       // [2][B][S] pq and s in float-float
     DArr<int> go;           // host-driven cycles: the loop condition
     DArr<unsigned long long> stats;   // [4] work counters (lspr_get_arnoldi_stats)
 };
@@ -456,7 +458,8 @@ int launch_p2p_fp32_raw(cudaStream_t st, const int4 *items, int64_t nitems, cons
                         const float4 *spos, const float4 *snrm, const float4 *w, double *acc);
 
 // ------------------------------------------------------------ solve.cu
-// y = A(s) x for one right-hand side, x and y device [2N] complex
+// y = A(s) x for B right-hand sides, x and y device [B][2N] complex; x null: an FP32 product of several
+// right-hand sides on one surface whose transposed vectors are in xtf already
 int apply_operator(lspr_ctx *ctx, int mode, const double2 *x, double2 *y, const double2 *s, int B);
 // layer potentials without the block assembly: out[i] = (V dphi)_i, (K phi)_i
 // per source surface t (S of them): Vd[t * N + i] = (V dphi)_t, Kp[t * N + i] = (K phi)_t

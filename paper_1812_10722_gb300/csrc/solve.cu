@@ -371,8 +371,10 @@ static int far_part(lspr_ctx *ctx, int mode, const double2 *x, int B, bool near)
     if (B > 1 && prec == PREC_F32) {
         LSPR_TRY(ctx, ctx->xtf.ensure((size_t)B * 2 * N));
         if (S > 1) LSPR_TRY(ctx, ctx->xt.ensure((size_t)B * 2 * N));   // the FP64 assembly reads it
-        ++ctx->n_launches;
-        transpose_kernel<float2><<<tg, tb, 0, ctx->stream>>>(B, 2 * N, x, ctx->xtf.p, S > 1 ? ctx->xt.p : nullptr);
+        if (x) {
+            ++ctx->n_launches;
+            transpose_kernel<float2><<<tg, tb, 0, ctx->stream>>>(B, 2 * N, x, ctx->xtf.p, S > 1 ? ctx->xt.p : nullptr);
+        }
         xtf = ctx->xtf.p;
     } else if (B > 1) {
         LSPR_TRY(ctx, ctx->xt.ensure((size_t)B * 2 * N));
