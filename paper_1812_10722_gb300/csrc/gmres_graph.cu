@@ -40,9 +40,9 @@ namespace {
 
 constexpr int kT = 256;                 // threads per block of the vector kernels
 constexpr double kReorthEta = 0.70710678118654752;   // second pass when ||w_1|| < eta ||w_0||
-constexpr int kDotChunk = 1024;         // entries per inner-product block
-constexpr int kDotSub = 4;              // parts of a chunk: a warp's task is four basis vectors on one part
+constexpr int kDotPart = 256;           // entries of a part of a chunk: a warp's task is four vectors on one part
 constexpr int kAxpyPer = 2;             // entries per thread of the update
+constexpr int kUpdChunk = 512;          // entries per block of the update with the second inner products
 
 // one complex entry in float-float: re = rh + rl, im = ih + il
 struct __align__(16) cff {
@@ -104,7 +104,7 @@ __device__ __forceinline__ void cff_abs2_mac(ffloat &s, const ffloat &re, const 
 }
 
 struct Arn {
-    int B, m, nch, nblk;
+    int B, m, nch, nblk, chunk;   // chunk: entries per inner-product block, nch of them
     int64_t N, n2, vstride;
     cff *V;              // [B][m+1][2N] Krylov basis
     double2 *w;          // [B][2N] A z (FP64 from the operator; float-float in place once the
@@ -121,7 +121,7 @@ struct Arn {
     double2 *h, *hcol, *part, *H, *sn, *g, *y;
     cff *hff, *yff;      // [B][m+1] Gram-Schmidt coefficients, [B][m] update coefficients
     ffloat *ninv;        // [B] 1 / ||w||
-    double *npart, *nrm, *cs, *res, *npart0, *nrm0;
+    double *npart, *nrm, *cs, *res, *npart0;
     int *reorth;
     const double *bn, *par;
     unsigned *tick;      // [2B + 1] last-block tickets
@@ -206,7 +206,7 @@ __device__ __forceinline__ bool last_block(unsigned *t, unsigned count) {
 
 // final sum of the squared-norm partials of system b into nrm[b] and 1/nrm[b] (last block
 // only); decide: the first Gram-Schmidt pass decides whether the second runs
-__device__ __forceinline__ void norm_final(const Arn &a, int b, int nblk, double *sh, bool decide = false) {
+__device__ __forceinline__ void norm_final(const Arn &a, int b, int nblk, double *sh) {
     double t = 0.0;
     for (int c = threadIdx.x; c < nblk; c += kT) t += __ldcg(a.npart + (int64_t)b * a.nblk + c);
     t = block_sum(t, sh);
@@ -214,7 +214,6 @@ __device__ __forceinline__ void norm_final(const Arn &a, int b, int nblk, double
         const double r = sqrt(t);
         a.nrm[b] = r;
         a.ninv[b] = ffloat(r > 0 ? 1.0 / r : 0.0);
-        if (decide) a.reorth[b] = !(r >= kReorthEta * __ldcg(a.nrm0 + b));
         a.tick[a.B + b] = 0;
     }
 }
@@ -341,21 +340,33 @@ __global__ void __launch_bounds__(256) arn_precond_t_kernel(Arn a) {
     }
 }
 
-// One classical Gram-Schmidt pass, first half: h_i = <v_i, w> for i <= j.  A block takes a
-// chunk of kDotChunk entries of one system: its threads stage the chunk of w in shared memory
-// (pass 0 converts w to float-float in place and forms ||w||^2 of the chunk), then a warp takes
-// tasks of four basis vectors on a kDotSub-th of the chunk, so that an entry of w read from shared
-// memory serves four products and eight loads per lane are in flight.  The 8 sums of a task are
-// reduced over the warp by halves (9 exchanges instead of 40).  The last block of the system sums
-// the chunks into h (FP64 and float-float) and into the Hessenberg column (hcol = h on pass 0,
-// hcol += h on pass 1).
-// 20480 panels, 16 systems, mid-cycle, cold caches: 51 us (81 with one vector per warp, chunks of 2048 and
-// unpacked products, whose 320 blocks left SMs idle).
+// Inner products of a Gram-Schmidt pass, h_i = <v_i, w> for i <= j.  A block takes a chunk of CH
+// entries of one system: its threads stage the chunk of w in shared memory, then a warp takes
+// tasks of four basis vectors on a part of the chunk, so that an entry of w read from shared
+// memory serves four products and eight or sixteen loads per lane are in flight.  The 8 sums of a
+// task are reduced over the warp by halves (9 exchanges instead of 40).  The last block of the
+// system sums the chunks into h (FP64 and float-float) and into the Hessenberg column (hcol = h on
+// pass 0, hcol += h on pass 1).
+//   pass 0 converts w to float-float in place and forms ||w||^2; its last block decides from
+//     ||w||^2 - ||h||^2, the squared norm left, whether the second pass runs (reorth[b]).
+//   pass 1 (UPDATE) first does the update w -= sum_i v_i h_i of pass 0 on its chunk, for every
+//     system; the second inner products then find the chunk of the basis in the L2 (512 entries:
+//     some 50 MB over the blocks in flight at 20 vectors), so that the basis is read three times
+//     from memory per step instead of four (vector kernels of a solve, 81920 panels, 64 systems: 194 ->
+//     175 ms; 20480, 16: 14.1 -> 12.3).  A system without a second pass stops at its norm.
+// 20480 panels, 16 systems, mid-cycle, cold caches: 51 us for pass 0 (81 with one vector per warp,
+// chunks of 2048 and unpacked products, whose 320 blocks left SMs idle).
 constexpr int kDotVec = 4;
-inline size_t dot_smem(int m) {   // w and the sums of the parts
-    return kDotChunk * sizeof(cff) + (size_t)kDotSub * (m + 1) * sizeof(double2);
+// 2048 entries per block (one reduction over the warp per 16 entries of a lane) where that gives every SM
+// eight blocks, else 1024.  81920 panels, 64 systems: vector kernels of a solve 195 ms, 201 with 1024
+// throughout; 20480 panels, 16 systems: 14.3 ms with 1024, 14.7 with 2048.
+inline int dot_chunk(int64_t n2, int B, int num_sms) {
+    return (n2 + 2047) / 2048 * B >= 8 * (int64_t)num_sms ? 2048 : 1024;
 }
-template <int NV>
+inline size_t dot_smem(int chunk, int m, bool update) {   // w, the sums of the parts, the update's coefficients
+    return chunk * sizeof(cff) + (size_t)(m + 1) * (chunk / kDotPart * sizeof(double2) + (update ? sizeof(CFactor) : 0));
+}
+template <int NV, int U>
 __device__ __forceinline__ void dot_task(const cff *__restrict__ v, int64_t stride, const cff *ws, int e0, int len,
                                          double2 *red) {
     const int lane = threadIdx.x & 31;
@@ -363,18 +374,17 @@ __device__ __forceinline__ void dot_task(const cff *__restrict__ v, int64_t stri
 #pragma unroll
     for (int k = 0; k < NV; ++k)
         p[k].a.hi = p[k].a.lo = p[k].b.hi = p[k].b.lo = make_float2(0.f, 0.f);
-    constexpr int kU = 2;   // entries loaded together
 #pragma unroll 1
-    for (int e = e0 + lane; e < e0 + kDotChunk / kDotSub; e += 32 * kU) {
-        float4 x[kU][NV];
+    for (int e = e0 + lane; e < e0 + kDotPart; e += 32 * U) {
+        float4 x[U][NV];   // entries loaded together
 #pragma unroll
-        for (int u = 0; u < kU; ++u)
+        for (int u = 0; u < U; ++u)
 #pragma unroll
             for (int k = 0; k < NV; ++k)
                 x[u][k] = e + 32 * u < len ? __ldg((const float4 *)(v + k * stride + e + 32 * u))
                                            : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
+        for (int u = 0; u < U; ++u) {
             const CFactor f = factor(ws[e + 32 * u]);
 #pragma unroll
             for (int k = 0; k < NV; ++k) cff_mac2(p[k], f, x[u][k]);
@@ -412,65 +422,122 @@ __device__ __forceinline__ void dot_task(const cff *__restrict__ v, int64_t stri
     }
 }
 
-__global__ void __launch_bounds__(kT, 2) arn_dot_kernel(Arn a, int pass) {
+// this thread's entries k0 + u kT of w -= sum_{i < nv} v_i h_i (hs: -h), those below n; f(u, entry) takes
+// the results (an entry past the end reads the basis at the last one, and is dropped by f)
+template <class F>
+__device__ __forceinline__ void update_w(const cff *__restrict__ Vb, const cff *wb, int64_t n2, int nv,
+                                         const CFactor *hs, int64_t k0, int64_t n, F &&f) {
+    CPair p[kAxpyPer];
+    int64_t k[kAxpyPer];
+#pragma unroll
+    for (int u = 0; u < kAxpyPer; ++u) {
+        const bool on = k0 + u * kT < n;
+        k[u] = on ? k0 + u * kT : n - 1;
+        const cff w0 = on ? wb[k[u]] : cff{0.f, 0.f, 0.f, 0.f};
+        p[u].a.hi = make_float2(w0.rh, w0.ih);
+        p[u].a.lo = make_float2(w0.rl, w0.il);
+        p[u].b.hi = p[u].b.lo = make_float2(0.f, 0.f);
+    }
+#pragma unroll 4
+    for (int i = 0; i < nv; ++i) {
+        const CFactor h = hs[i];
+#pragma unroll
+        for (int u = 0; u < kAxpyPer; ++u) cff_mac2(p[u], h, *(const float4 *)(Vb + (int64_t)i * n2 + k[u]));
+    }
+    // w - h v: (a.x - b.y, a.y + b.x)
+#pragma unroll
+    for (int u = 0; u < kAxpyPer; ++u)
+        f(u, pack(ff_norm(ffloat(p[u].a.hi.x, p[u].a.lo.x)) - ff_norm(ffloat(p[u].b.hi.y, p[u].b.lo.y)),
+                  ff_norm(ffloat(p[u].a.hi.y, p[u].a.lo.y)) + ff_norm(ffloat(p[u].b.hi.x, p[u].b.lo.x))));
+}
+__device__ __forceinline__ void load_factors(const Arn &a, int b, int nv, CFactor *hs) {
+    for (int i = threadIdx.x; i < nv; i += kT) {
+        const cff h = a.hff[(int64_t)b * (a.m + 1) + i];
+        hs[i] = factor({-h.rh, -h.ih, -h.rl, -h.il});
+    }
+}
+
+template <int CH, bool UPDATE>
+__global__ void __launch_bounds__(kT, 2) arn_dot_kernel(Arn a) {
+    static_assert(CH % (kT * kAxpyPer) == 0 && CH % kDotPart == 0, "whole tasks");
+    constexpr int kSub = CH / kDotPart;
     extern __shared__ double2 dsm[];
     cff *ws = (cff *)dsm;
-    double2 *red = dsm + kDotChunk;   // [kDotSub][m + 1]
+    double2 *red = dsm + CH;   // [kSub][m + 1]
+    CFactor *hs = (CFactor *)(red + kSub * (a.m + 1));
     __shared__ double shn[kT / 32];
-    const int b = blockIdx.y, chunk = blockIdx.x;
-    if (!a.active[b] || (pass && !a.reorth[b])) return;
+    const int b = blockIdx.y, chunk = blockIdx.x, nch = gridDim.x;
+    if (!a.active[b]) return;
     const int nv = *a.jdev + 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t c0 = (int64_t)chunk * kDotChunk;
-    const int len = (int)min((int64_t)kDotChunk, a.n2 - c0);
+    const int64_t c0 = (int64_t)chunk * CH;
+    const int len = (int)min((int64_t)CH, a.n2 - c0);
     cff *wb = wff(a, b) + c0;
+    const cff *Vb = a.V + (int64_t)b * a.vstride + c0;
     ffloat w2(0.f, 0.f);
-    for (int e = threadIdx.x; e < kDotChunk; e += kT) {
-        cff v = {0.f, 0.f, 0.f, 0.f};
-        if (e < len) {
-            if (pass == 0) {
+    if (UPDATE) {
+        load_factors(a, b, nv, hs);
+        __syncthreads();
+        for (int e0 = threadIdx.x; e0 < CH; e0 += kT * kAxpyPer) {
+            update_w(Vb, wb, a.n2, nv, hs, e0, len, [&](int u, cff v) {
+                const int e = e0 + u * kT;
+                if (e < len) {
+                    wb[e] = v;
+                    cff_abs2_mac(w2, re_of(v), im_of(v));
+                } else {
+                    v = {0.f, 0.f, 0.f, 0.f};
+                }
+                ws[e] = v;
+            });
+        }
+        __syncthreads();
+        if (!a.reorth[b]) {   // one pass is enough: its norm
+            const double t = block_sum_ff(w2, shn);
+            if (threadIdx.x == 0) a.npart[(int64_t)b * a.nblk + chunk] = t;
+            if (last_block(a.tick + a.B + b, nch)) norm_final(a, b, nch, shn);
+            return;
+        }
+    } else {
+        for (int e = threadIdx.x; e < CH; e += kT) {
+            cff v = {0.f, 0.f, 0.f, 0.f};
+            if (e < len) {
                 v = to_cff(a.w[(int64_t)b * a.n2 + c0 + e]);
                 wb[e] = v;
-            } else {
-                v = wb[e];
             }
+            ws[e] = v;
+            cff_abs2_mac(w2, re_of(v), im_of(v));
         }
-        ws[e] = v;
-        if (pass == 0) cff_abs2_mac(w2, re_of(v), im_of(v));
-    }
-    if (pass == 0) {   // ||A z||^2 of this chunk, for the second-pass criterion
+        // ||A z||^2 of this chunk, for the second-pass criterion
         const double t = block_sum_ff(w2, shn);
-        if (threadIdx.x == 0) a.npart0[(int64_t)b * a.nch + chunk] = t;
+        if (threadIdx.x == 0) a.npart0[(int64_t)b * nch + chunk] = t;
+        __syncthreads();
     }
-    __syncthreads();
-    const cff *Vb = a.V + (int64_t)b * a.vstride + c0;
-    const int tasks = kDotSub * ((nv + kDotVec - 1) / kDotVec);
+    constexpr int kU = CH == 2048 ? 4 : 2;
+    const int tasks = kSub * ((nv + kDotVec - 1) / kDotVec);
     for (int q = warp; q < tasks; q += kT / 32) {
-        const int sub = q % kDotSub, i = q / kDotSub * kDotVec;
+        const int sub = q % kSub, i = q / kSub * kDotVec;
         const cff *v = Vb + (int64_t)i * a.n2;
         double2 *r = red + sub * (a.m + 1) + i;
-        const int e0 = sub * (kDotChunk / kDotSub);
         switch (min(kDotVec, nv - i)) {
-            case 4: dot_task<4>(v, a.n2, ws, e0, len, r); break;
-            case 3: dot_task<3>(v, a.n2, ws, e0, len, r); break;
-            case 2: dot_task<2>(v, a.n2, ws, e0, len, r); break;
-            default: dot_task<1>(v, a.n2, ws, e0, len, r); break;
+            case 4: dot_task<4, kU>(v, a.n2, ws, sub * kDotPart, len, r); break;
+            case 3: dot_task<3, kU>(v, a.n2, ws, sub * kDotPart, len, r); break;
+            case 2: dot_task<2, kU>(v, a.n2, ws, sub * kDotPart, len, r); break;
+            default: dot_task<1, kU>(v, a.n2, ws, sub * kDotPart, len, r); break;
         }
     }
     __syncthreads();
-    double2 *pb = a.part + (int64_t)b * (a.m + 1) * a.nch;
+    double2 *pb = a.part + (int64_t)b * (a.m + 1) * nch;
     for (int i = threadIdx.x; i < nv; i += kT) {
         double2 t = red[i];
 #pragma unroll
-        for (int s = 1; s < kDotSub; ++s) t = cadd(t, red[s * (a.m + 1) + i]);
-        pb[(int64_t)i * a.nch + chunk] = t;
+        for (int s = 1; s < kSub; ++s) t = cadd(t, red[s * (a.m + 1) + i]);
+        pb[(int64_t)i * nch + chunk] = t;
     }
-    if (!last_block(a.tick + b, a.nch)) return;
-    if (pass == 0) {
-        double t = 0.0;
-        for (int c = threadIdx.x; c < a.nch; c += kT) t += __ldcg(a.npart0 + (int64_t)b * a.nch + c);
-        t = block_sum(t, shn);
-        if (threadIdx.x == 0) a.nrm0[b] = sqrt(t);
+    if (!last_block(a.tick + b, nch)) return;
+    double n0 = 0.0, hh = 0.0;   // ||A z||^2 (thread 0), this warp's share of ||h||^2 (lane 0)
+    if (!UPDATE) {
+        for (int c = threadIdx.x; c < nch; c += kT) n0 += __ldcg(a.npart0 + (int64_t)b * nch + c);
+        n0 = block_sum(n0, shn);
     }
     // rows i = warp + 8 u: lanes stride over the chunks
     for (int i0 = warp; i0 < nv; i0 += 4 * (kT / 32)) {
@@ -480,7 +547,7 @@ __global__ void __launch_bounds__(kT, 2) arn_dot_kernel(Arn a, int pass) {
             t[u] = make_double2(0.0, 0.0);
             const int i = i0 + u * (kT / 32);
             if (i < nv)
-                for (int c = lane; c < a.nch; c += 32) t[u] = cadd(t[u], __ldcg(pb + (int64_t)i * a.nch + c));
+                for (int c = lane; c < nch; c += 32) t[u] = cadd(t[u], __ldcg(pb + (int64_t)i * nch + c));
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -490,61 +557,44 @@ __global__ void __launch_bounds__(kT, 2) arn_dot_kernel(Arn a, int pass) {
                 a.h[(int64_t)b * (a.m + 1) + i] = sum;
                 a.hff[(int64_t)b * (a.m + 1) + i] = to_cff(sum);
                 double2 &e = a.hcol[(int64_t)b * (a.m + 1) + i];
-                e = pass ? cadd(e, sum) : sum;
+                e = UPDATE ? cadd(e, sum) : sum;
+                hh += cabs2(sum);
             }
+        }
+    }
+    if (!UPDATE) {
+        __syncthreads();   // shn has been read
+        if (lane == 0) shn[warp] = hh;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int q = 1; q < kT / 32; ++q) hh += shn[q];
+            a.reorth[b] = !(n0 - hh >= kReorthEta * kReorthEta * n0);
         }
     }
     if (threadIdx.x == 0) a.tick[b] = 0;
 }
 
-// Second half of a pass: w -= sum_{i <= j} v_i h_i (float-float), then ||w|| into nrm[b]
-// (partials per block, the last block sums them); after the first pass the last block also
-// decides whether the second runs (reorth[b])
-__global__ void __launch_bounds__(kT) arn_axpy_kernel(Arn a, int pass) {
+// The second pass's update w -= sum_{i <= j} v_i h_i, then ||w|| into nrm[b] (partials per block, the
+// last block sums them)
+__global__ void __launch_bounds__(kT) arn_axpy_kernel(Arn a) {
     __shared__ double sh[kT / 32];
     __shared__ CFactor hs[kMaxRestart + 1];
     const int b = blockIdx.y;
-    if (!a.active[b] || (pass && !a.reorth[b])) return;
+    if (!a.active[b] || !a.reorth[b]) return;
     const int nv = *a.jdev + 1;
-    for (int i = threadIdx.x; i < nv; i += kT) {
-        const cff h = a.hff[(int64_t)b * (a.m + 1) + i];
-        hs[i] = factor({-h.rh, -h.ih, -h.rl, -h.il});
-    }
+    load_factors(a, b, nv, hs);
     __syncthreads();
     const int64_t k0 = blockIdx.x * (int64_t)(kT * kAxpyPer) + threadIdx.x;
-    const cff *Vb = a.V + (int64_t)b * a.vstride;
     cff *wb = wff(a, b);
-    CPair p[kAxpyPer];
-    bool on[kAxpyPer];
-    int64_t k[kAxpyPer];
-#pragma unroll
-    for (int u = 0; u < kAxpyPer; ++u) {
-        on[u] = k0 + u * kT < a.n2;
-        k[u] = on[u] ? k0 + u * kT : a.n2 - 1;   // the entry of a thread past the end is read and dropped
-        const cff w0 = wb[k[u]];
-        p[u].a.hi = make_float2(w0.rh, w0.ih);
-        p[u].a.lo = make_float2(w0.rl, w0.il);
-        p[u].b.hi = p[u].b.lo = make_float2(0.f, 0.f);
-    }
-#pragma unroll 4
-    for (int i = 0; i < nv; ++i) {
-        const CFactor h = hs[i];
-#pragma unroll
-        for (int u = 0; u < kAxpyPer; ++u) cff_mac2(p[u], h, *(const float4 *)(Vb + (int64_t)i * a.n2 + k[u]));
-    }
     ffloat q(0.f, 0.f);
-#pragma unroll
-    for (int u = 0; u < kAxpyPer; ++u) {
-        if (!on[u]) continue;
-        // w - h v: (a.x - b.y, a.y + b.x)
-        const cff w1 = pack(ff_norm(ffloat(p[u].a.hi.x, p[u].a.lo.x)) - ff_norm(ffloat(p[u].b.hi.y, p[u].b.lo.y)),
-                            ff_norm(ffloat(p[u].a.hi.y, p[u].a.lo.y)) + ff_norm(ffloat(p[u].b.hi.x, p[u].b.lo.x)));
-        wb[k[u]] = w1;
+    update_w(a.V + (int64_t)b * a.vstride, wb, a.n2, nv, hs, k0, a.n2, [&](int u, const cff &w1) {
+        if (k0 + u * kT >= a.n2) return;
+        wb[k0 + u * kT] = w1;
         cff_abs2_mac(q, re_of(w1), im_of(w1));
-    }
+    });
     const double t = block_sum_ff(q, sh);
     if (threadIdx.x == 0) a.npart[(int64_t)b * a.nblk + blockIdx.x] = t;
-    if (last_block(a.tick + a.B + b, gridDim.x)) norm_final(a, b, gridDim.x, sh, pass == 0);
+    if (last_block(a.tick + a.B + b, gridDim.x)) norm_final(a, b, gridDim.x, sh);
 }
 
 // shared memory of the rotation kernel: column (m+1), sines (m), cosines (m)
@@ -723,14 +773,18 @@ int launch_precond(lspr_ctx *ctx, const Arn &a, cudaStream_t st) {
 
 // the two Gram-Schmidt passes and the end of an Arnoldi step
 int launch_orthogonalise(lspr_ctx *ctx, const Arn &a, cudaStream_t st) {
-    static int smem_set[kSmemDevices] = {};
-    LSPR_TRY(ctx, allow_smem(arn_dot_kernel, (int)dot_smem(a.m), ctx->device, smem_set));
-    const dim3 ga(grid_for(a.n2, kT * kAxpyPer), a.B);
-    for (int pass = 0; pass < 2; ++pass) {
-        arn_dot_kernel<<<dim3(a.nch, a.B), kT, dot_smem(a.m), st>>>(a, pass);
-        arn_axpy_kernel<<<ga, kT, 0, st>>>(a, pass);
-        ctx->n_launches += 2;
-    }
+    static int set0[kSmemDevices] = {}, set1[kSmemDevices] = {}, setu[kSmemDevices] = {};
+    const bool wide = a.chunk == 2048;
+    const size_t smem = dot_smem(a.chunk, a.m, false), smem_u = dot_smem(kUpdChunk, a.m, true);
+    LSPR_TRY(ctx, wide ? allow_smem(arn_dot_kernel<2048, false>, (int)smem, ctx->device, set1)
+                       : allow_smem(arn_dot_kernel<1024, false>, (int)smem, ctx->device, set0));
+    LSPR_TRY(ctx, allow_smem(arn_dot_kernel<kUpdChunk, true>, (int)smem_u, ctx->device, setu));
+    const dim3 g0(a.nch, a.B);
+    if (wide) arn_dot_kernel<2048, false><<<g0, kT, smem, st>>>(a);
+    else arn_dot_kernel<1024, false><<<g0, kT, smem, st>>>(a);
+    arn_dot_kernel<kUpdChunk, true><<<dim3(grid_for(a.n2, kUpdChunk), a.B), kT, smem_u, st>>>(a);
+    arn_axpy_kernel<<<dim3(grid_for(a.n2, kT * kAxpyPer), a.B), kT, 0, st>>>(a);
+    ctx->n_launches += 3;
     arn_tail_kernel<<<a.B, 32, tail_smem(a.m), st>>>(a);
     ++ctx->n_launches;
     LSPR_TRY(ctx, cudaGetLastError());
@@ -898,18 +952,18 @@ int gmres_graph_solve(lspr_ctx *ctx, int mode, int B, int m, int maxiter, double
         LSPR_TRY(ctx, cudaEventCreateWithFlags(&ctx->ev_g1, cudaEventDisableTiming));
     }
     ArnoldiBufs &ab = ctx->arn;
-    const int nch = (int)((n2 + kDotChunk - 1) / kDotChunk), nblk = (int)grid_for(n2, kT);
+    const int chunk = dot_chunk(n2, B, std::max(1, ctx->num_sms));
+    const int nch = (int)((n2 + chunk - 1) / chunk), nblk = (int)grid_for(n2, kT);
     const int64_t vstride = (int64_t)(m + 1) * n2;
     LSPR_TRY(ctx, ctx->gm_V.ensure((size_t)B * vstride));
     LSPR_TRY(ctx, ctx->gm_w.ensure((size_t)B * n2));
     LSPR_TRY(ctx, ctx->gm_z.ensure((size_t)B * n2));
     LSPR_TRY(ctx, ab.h.ensure((size_t)B * (m + 1)));
     LSPR_TRY(ctx, ab.hcol.ensure((size_t)B * (m + 1)));
-    LSPR_TRY(ctx, ab.part.ensure((size_t)B * (m + 1) * nch));
+    LSPR_TRY(ctx, ab.part.ensure((size_t)B * (m + 1) * std::max<int64_t>(nch, grid_for(n2, kUpdChunk))));
     LSPR_TRY(ctx, ab.npart.ensure((size_t)B * nblk));
     LSPR_TRY(ctx, ab.nrm.ensure(B));
     LSPR_TRY(ctx, ab.npart0.ensure((size_t)B * nch));
-    LSPR_TRY(ctx, ab.nrm0.ensure(B));
     LSPR_TRY(ctx, ab.reorth.ensure(B));
     LSPR_TRY(ctx, ab.H.ensure((size_t)B * (m + 1) * m));
     LSPR_TRY(ctx, ab.cs.ensure((size_t)B * m));
@@ -940,6 +994,7 @@ int gmres_graph_solve(lspr_ctx *ctx, int mode, int B, int m, int maxiter, double
     a.B = B;
     a.m = m;
     a.nch = nch;
+    a.chunk = chunk;
     a.nblk = nblk;
     a.N = N;
     a.n2 = n2;
@@ -968,7 +1023,6 @@ int gmres_graph_solve(lspr_ctx *ctx, int mode, int B, int m, int maxiter, double
     a.npart = ab.npart.p;
     a.nrm = ab.nrm.p;
     a.npart0 = ab.npart0.p;
-    a.nrm0 = ab.nrm0.p;
     a.reorth = ab.reorth.p;
     a.cs = ab.cs.p;
     a.res = ab.res.p;
