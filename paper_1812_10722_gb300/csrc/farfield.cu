@@ -242,17 +242,26 @@ int launch_ff_boxes(lspr_ctx *ctx) {
 // with the tile's weights as two small matrix products, V += G W_V and K += dG/dn W_K: a thread holds
 // 8 targets x RB/2 channels of one layer (RB right-hand sides per chunk: 16, or 8 or 4 where no more are
 // left, as in a solve whose number in use falls), so four shared-memory reads feed 64 multiply-adds.
-// The FP32 pipe's share is 12 + 4 RB operations per pair.  20480 panels (86 M pairs), 16 right-hand
-// sides: 381 us, 476 with two targets per lane and the weights read by broadcast (bound by the
-// shared-memory reads, ten 16-byte reads per 32 packed multiply-adds); four targets per lane and 8
-// right-hand sides took 453 (217 registers, two warps per scheduler).
+// The FP32 pipe's share is 12 + 4 RB operations per pair.  A tile's weights are copied asynchronously
+// while its kernel values are formed, the next tile's geometry behind the products.  20480 panels (86 M pairs), 16 right-hand sides: 326 us; 377 with
+// both loaded through registers when the tile begins (FP32 pipe 52 % busy), 476 with two targets per lane
+// and the weights read by broadcast (bound by the shared-memory reads, ten 16-byte reads per 32 packed
+// multiply-adds); four targets per lane and 8 right-hand sides took 453 (217 registers, two warps per
+// scheduler).  81920 panels, P 7: 12 right-hand sides 2.47 -> 2.19 ms, 20: 3.92 -> 3.43.
 constexpr int kPgTile = 32, kPgThreads = 64, kPgRB = 16;
 struct PgSmem {
     float G[kPgTile][kTargetBlock], T[kPgTile][kTargetBlock];
-    float wv[kPgTile][2 * kPgRB], wk[kPgTile][2 * kPgRB];   // (re, im) per right-hand side
+    float4 w[kPgTile][kPgRB];                               // weights, (re, im) of both layers per right-hand side
     float src[6][kPgTile];                                  // -x, -y, -z, normal
+    float4 raw[2][kPgTile];                                 // the next tile's positions and normals
     int pid[kPgTile], tpid[kTargetBlock];
 };
+// 16 bytes into shared memory without a register; zeros where !on
+__device__ __forceinline__ void copy16(float4 *dst, const float4 *src, bool on) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(on ? 16 : 0)
+                 : "memory");
+}
 
 template <int RB, bool CHECK>
 __device__ __forceinline__ void pg_unit(const int4 &item, int B, int b0, int nb, PgSmem &sm, const float4 &q, int64_t t0,
@@ -268,22 +277,30 @@ __device__ __forceinline__ void pg_unit(const int4 &item, int B, int b0, int nb,
     for (int i = 0; i < 8; ++i)
 #pragma unroll
         for (int p = 0; p < NP; ++p) a[i][p] = make_float2(0.f, 0.f);
+    auto fetch = [&](int base) {   // a tile's geometry; past the end: the first source again, with zero weights
+        if (tid < kPgTile && base < item.z) {
+            const int s = base + (tid < item.z - base ? tid : 0);
+            copy16(&sm.raw[0][tid], spos + s, true);
+            copy16(&sm.raw[1][tid], snrm + s, true);
+        }
+    };
+    fetch(item.y);
     for (int base = item.y; base < item.z; base += kPgTile) {
         const int cnt = min(kPgTile, item.z - base);
+        asm volatile("cp.async.wait_all;" ::: "memory");   // the geometry, behind the previous tile's products
         __syncthreads();   // the previous tile has been read
-        if (tid < kPgTile) {   // past the end: the first source again, with zero weights
-            const int s = base + (tid < cnt ? tid : 0);
-            const float4 p = spos[s], n = snrm[s];
-            sm.src[0][tid] = -p.x; sm.src[1][tid] = -p.y; sm.src[2][tid] = -p.z;
-            sm.src[3][tid] = n.x; sm.src[4][tid] = n.y; sm.src[5][tid] = n.z;
-            sm.pid[tid] = panel_of(n.w);
-        }
+        // the weights arrive while G and dG/dn are formed
 #pragma unroll 4
         for (int e = tid; e < kPgTile * RB; e += kPgThreads) {
             const int s = e / RB, j = e - s * RB;
-            const float4 w = s < cnt && j < nb ? sw[(int64_t)(base + s) * B + b0 + j] : zero4<float4>();
-            *(float2 *)&sm.wv[s][2 * j] = make_float2(w.x, w.y);
-            *(float2 *)&sm.wk[s][2 * j] = make_float2(w.z, w.w);
+            const bool on = s < cnt && j < nb;
+            copy16(&sm.w[s][j], sw + (on ? (int64_t)(base + s) * B + b0 + j : 0), on);
+        }
+        if (tid < kPgTile) {
+            const float4 gp = sm.raw[0][tid], gn = sm.raw[1][tid];   // this thread's own copies
+            sm.src[0][tid] = -gp.x; sm.src[1][tid] = -gp.y; sm.src[2][tid] = -gp.z;
+            sm.src[3][tid] = gn.x; sm.src[4][tid] = gn.y; sm.src[5][tid] = gn.z;
+            sm.pid[tid] = panel_of(gn.w);
         }
         __syncthreads();
 #pragma unroll 4
@@ -306,22 +323,23 @@ __device__ __forceinline__ void pg_unit(const int4 &item, int B, int b0, int nb,
             sm.T[s][tid] = t.x;
             sm.T[s + 1][tid] = t.y;
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
+        fetch(base + kPgTile);
         const float (*m)[kTargetBlock] = layer ? sm.T : sm.G;
-        const float (*w)[2 * kPgRB] = layer ? sm.wk : sm.wv;
 #pragma unroll 4
         for (int s = 0; s < kPgTile; ++s) {
             const float4 g0 = *(const float4 *)&m[s][4 * tx], g1 = *(const float4 *)&m[s][32 + 4 * tx];
             const float g[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
-                const float2 wp = *(const float2 *)&w[s][2 * (NP * cg + p)];
+                const float2 wp = *((const float2 *)&sm.w[s][cg + 4 * p] + layer);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) a[i][p] = __ffma2_rn(make_float2(g[i], g[i]), wp, a[i][p]);
             }
         }
     }
-    // target (i < 4: 4 tx + i, else 28 + 4 tx + i), right-hand side NP cg + p, components 2 layer, + 1
+    // target (i < 4: 4 tx + i, else 28 + 4 tx + i), right-hand side cg + 4 p, components 2 layer, + 1
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int t = (i < 4 ? 0 : 28) + 4 * tx + i;
@@ -329,7 +347,7 @@ __device__ __forceinline__ void pg_unit(const int4 &item, int B, int b0, int nb,
         double *o = acc + 4 * ((int64_t)sm.tpid[t] * B + b0) + 2 * layer;
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-            const int j = NP * cg + p;
+            const int j = cg + 4 * p;
             if (j < nb) {
                 atomicAdd(o + 4 * j, (double)a[i][p].x);
                 atomicAdd(o + 4 * j + 1, (double)a[i][p].y);
@@ -346,7 +364,7 @@ __device__ __forceinline__ void pg_check(const int4 &item, A &&...a) {
 
 // Work units (item, chunk of kPgRB right-hand sides) from an atomic counter; nothing is done when at
 // least skip_from right-hand sides are in use (the tensor-core P2P then takes the product)
-__global__ void __launch_bounds__(kPgThreads, 8)
+__global__ void __launch_bounds__(kPgThreads, 7)
     p2p_multi_kernel(const int4 *__restrict__ items, int64_t nitems, int B, const float4 *__restrict__ tgt, int64_t ntgt,
                      const float4 *__restrict__ spos, const float4 *__restrict__ snrm, const float4 *__restrict__ sw,
                      double *__restrict__ acc, int *counter, const int *nact, int skip_from, int S) {
