@@ -113,16 +113,16 @@ TF32_PER_BF16 = 1.1 / 2.25  # nominal dense tensor rates, TF32 over BF16
 # DRAM bytes (read + write) per launch of the current kernels, from the ncu captures summarised in
 # profiles/ (dram__bytes_read.sum + dram__bytes_write.sum of one launch), keyed by workload, kernel and
 # treecode parameters (theta, P, Ncrit); None where no capture of the current kernel matches
-NCU_TRAFFIC = {("sphere20480", "m2p", 0.4, 5, 256): 2.410e6,          # m2p_fp32_sphere20480.md
-               ("sphere20480", "p2p", 0.4, 5, 256): 5.045e6,          # p2p1_fp32_sphere20480.md
-               ("sphere81920_sweep64", "m2p", 0.4, 7, 512): 8.883e9,  # m2p_tc_sphere81920_sweep64.md
-               ("sphere81920_sweep64", "p2p", 0.4, 7, 512): 9.805e8}  # p2p_tc_sphere81920_sweep64.md
+NCU_TRAFFIC = {("sphere81920_sweep64", "m2p", 0.4, 7, 512): 6.391e8,  # kernels_current.md
+               ("sphere81920_sweep64", "p2p", 0.4, 7, 512): 1.4684e9}
 
 
-def m2p_flops(P: int, B: int = 1) -> int:
-    """Flops per (target, box) M2P evaluation: the coefficient recurrence (once, whatever B)
+def m2p_flops(P: int, B: int = 1, harmonic: bool = False) -> int:
+    """harmonic: over the (P + 1)^2 terms with k_3 <= 1 that the kernels sum; else all Cartesian ones.
+    Flops per (target, box) M2P evaluation: the coefficient recurrence (once, whatever B)
     plus the 4-channel dot with the moments of each of the B right-hand sides (FMA = 2)."""
-    terms = [(a, b, n - a - b) for n in range(P + 1) for a in range(n, -1, -1) for b in range(n - a, -1, -1)]
+    terms = [(a, b, n - a - b) for n in range(P + 1) for a in range(n, -1, -1) for b in range(n - a, -1, -1)
+             if not harmonic or n - a - b <= 1]
     f = 3 + 5 + 1   # R components, r^2, 1/r^2
     for k in terms[1:]:
         m1 = sum(1 for d in range(3) if k[d] >= 1)
@@ -131,19 +131,19 @@ def m2p_flops(P: int, B: int = 1) -> int:
     return f + 8 * len(terms) * B
 
 
-def p2p_tc_bound(B: int, pairs: int, stages: int, peaks: dict, mhz: float) -> dict:
+def p2p_tc_bound(B: int, pairs: int, stages: int, peaks: dict, mhz: float, f16: bool = False) -> dict:
     """Time bound of one tensor-core P2P launch: the largest of its G and dG/dn generation on the
     FP32 pipe (the blocks' own pairs, once per unit of 64 right-hand sides), its rsqrt on the SFU,
     and its issued MMAs on the tensor pipe (per stage of 8 sources: M = 128 channels x N = 256
     targets x K = 8, for the single and the double layer, 3 products each above 32 right-hand
-    sides in the unit, 2 at 32 or fewer)."""
+    sides in the unit, 2 at 32 or fewer).  f16: FP16 parts, stages of 16 sources at the bf16 rate."""
     units = [min(64, B - b0) for b0 in range(0, B, 64)]
     gen = pairs * P2P_GEN_FLOPS * len(units)
     mufu = pairs * len(units)
-    mma = sum(stages * 2 * (3 if nb > 32 else 2) * 2 * 128 * 256 * 8 for nb in units)
+    mma = sum(stages * 2 * (3 if nb > 32 else 2) * 2 * 128 * 256 * (16 if f16 else 8) for nb in units)
     fp32_peak = fp32_peak_tflops(mhz) * 1e12
     sfu_peak = SFU_PER_CLK_SM * 152 * mhz * 1e6
-    tf32_peak = peaks.get("bf16_tflops_sustained", 1741.2) * TF32_PER_BF16 * 1e12
+    tf32_peak = peaks.get("bf16_tflops_sustained", 1741.2) * (1.0 if f16 else TF32_PER_BF16) * 1e12
     t = {"fp32_generation": gen / fp32_peak, "sfu": mufu / sfu_peak, "tensor_mma": mma / tf32_peak}
     return {"terms_s": t, "bound_s": max(t.values()), "limiter": max(t, key=t.get), "mma_flops": mma,
             "generation_flops": gen, "mufu_ops": mufu, "tf32_peak_tflops": tf32_peak / 1e12,
@@ -163,8 +163,8 @@ def tc_roofline(bnd: dict, t: float, kernel: str, traffic) -> dict:
             "frac": round(bnd["bound_s"] / t, 4), "traffic": traffic,
             "bound_terms_ms": {x: round(1e3 * y, 4) for x, y in bnd["terms_s"].items()},
             "peak_note": "frac = max(generation flops / FP32 peak (152 SM x 128 x 2 x 2070 MHz, derived), rsqrt / "
-                         "SFU peak (16 per clock per SM), issued TF32 MMA flops / TF32 peak (measured sustained "
-                         "bf16 x nominal 1.1/2.25)) / the launch time; achieved and peak are the limiting term's"}
+                         "SFU peak (16 per clock per SM), issued FP16 MMA flops / measured sustained bf16 peak) "
+                         "/ the launch time; achieved and peak are the limiting term's"}
 
 
 def max_over_ranks(x: float, world: int, device=None) -> float:
@@ -191,8 +191,10 @@ def arnoldi_gb(n_panels: int, c: dict) -> float:
                   + 3 * c["system_steps_second_pass"]) / 1e9
 
 
-def m2p_terms(P: int) -> int:
+def m2p_terms(P: int, harmonic: bool = False) -> int:
     """Taylor terms with |k| <= P."""
+    if harmonic:
+        return (P + 1) ** 2
     return (P + 1) * (P + 2) * (P + 3) // 6
 
 
@@ -202,24 +204,25 @@ def p2p_flops(B: int = 1) -> int:
     return P2P_GEN_FLOPS + 8 * B
 
 
-def m2p_tc_bound(P: int, B: int, group_box_pairs: int, peaks: dict, mhz: float) -> dict:
+def m2p_tc_bound(P: int, B: int, group_box_pairs: int, peaks: dict, mhz: float, f16: bool = False) -> dict:
     """Time bound of one tensor-core M2P launch: the largest of its coefficient generation on the
     FP32 pipe (the recurrence for 256 targets per (group, box) and unit of 16, 32 or 64 right-hand
     sides), its reciprocal square roots on the SFU, and its issued MMAs on the tensor pipe
     (M = 128 channels x N = 256 targets x K = 8 per step; 3 MMAs per step for each A part of 32
     right-hand sides, 2 for units of 16; above 32 right-hand sides a unit carries two A parts
-    against one set of coefficients)."""
-    nt = (P + 1) * (P + 2) * (P + 3) // 6
+    against one set of coefficients).  f16: FP16 parts of the harmonic terms, K = 16 per step at the bf16 rate."""
+    nt = m2p_terms(P, f16)
     rc = 16 if B <= 16 else (32 if B <= 32 else 64)
     units = (B + rc - 1) // rc                      # coefficient generations per (group, box)
     parts = (B + min(rc, 32) - 1) // min(rc, 32)    # A parts of 32 (or 16) right-hand sides
-    ksteps = sum((min(16, nt - kc) + 7) // 8 for kc in range(0, nt, 16))
-    gen = group_box_pairs * units * 256 * (m2p_flops(P, 0))
+    k = 16 if f16 else 8
+    ksteps = sum((min(2 * k, nt - kc) + k - 1) // k for kc in range(0, nt, 2 * k))
+    gen = group_box_pairs * units * 256 * m2p_flops(P, 0, f16)
     mufu = group_box_pairs * units * 256
-    mma = group_box_pairs * parts * (2 if rc == 16 else 3) * 2 * 128 * 256 * 8 * ksteps
+    mma = group_box_pairs * parts * (2 if rc == 16 else 3) * 2 * 128 * 256 * k * ksteps
     fp32_peak = fp32_peak_tflops(mhz) * 1e12
     sfu_peak = SFU_PER_CLK_SM * 152 * mhz * 1e6
-    tf32_peak = peaks.get("bf16_tflops_sustained", 1741.2) * TF32_PER_BF16 * 1e12
+    tf32_peak = peaks.get("bf16_tflops_sustained", 1741.2) * (1.0 if f16 else TF32_PER_BF16) * 1e12
     t = {"fp32_generation": gen / fp32_peak, "sfu": mufu / sfu_peak, "tensor_mma": mma / tf32_peak}
     return {"terms_s": t, "bound_s": max(t.values()), "limiter": max(t, key=t.get), "mma_flops": mma,
             "generation_flops": gen, "mufu_ops": mufu, "tf32_peak_tflops": tf32_peak / 1e12,
@@ -525,7 +528,7 @@ def run_ours(args, wl, rank, world, local_rank):
         if name.startswith("p2p"):
             return pairs * (P2P_GEN_FLOPS * n + 8 * r)
         if name.startswith("m2p"):
-            return tgt_box * (m2p_flops(wl["P"], 0) * n + 8 * m2p_terms(wl["P"]) * r)
+            return tgt_box * (m2p_flops(wl["P"], 0, True) * n + 8 * m2p_terms(wl["P"], True) * r)
         return None
 
     for name in ("p2p", "m2p", "p2p_fp64", "m2p_fp64", "p2p_ff", "m2p_ff"):
@@ -534,9 +537,9 @@ def run_ours(args, wl, rank, world, local_rank):
             k["algorithmic_tflops"] = work(name) / (k["ms_total"] * 1e-3) / 1e12
     if "p2p" in kernels:
         kernels["p2p"]["pairs_per_launch"] = pairs
-        kernels["p2p"]["path"] = "tcgen05 (TF32 hi/lo split, FP32 accumulation)" if p2p_tc else "FP32 pipe"
+        kernels["p2p"]["path"] = "tcgen05 (FP16 hi/lo split, FP32 accumulation)" if p2p_tc else "FP32 pipe"
     if "m2p" in kernels:
-        kernels["m2p"]["path"] = "tcgen05 (TF32 hi/lo split, FP32 accumulation)" if m2p_tc else "FP32 pipe"
+        kernels["m2p"]["path"] = "tcgen05 (FP16 hi/lo split, FP32 accumulation)" if m2p_tc else "FP32 pipe"
     if "gmres" in kernels and arn["system_steps"]:
         # basis traffic of the Arnoldi vector kernels (16 bytes per complex entry of 2N): per
         # system-step 3 vectors (v_j, z, w read) + 2 (j + 3) for the first Gram-Schmidt pass
@@ -556,7 +559,7 @@ def run_ours(args, wl, rank, world, local_rank):
     for name in ("p2p", "m2p"):
         if name in full:
             n = full[name]["launches"]
-            w = (pairs * p2p_flops(B) if name == "p2p" else tgt_box * m2p_flops(wl["P"], B))
+            w = (pairs * p2p_flops(B) if name == "p2p" else tgt_box * m2p_flops(wl["P"], B, True))
             full[name]["algorithmic_tflops"] = round(w / (full[name]["ms_per_launch"] * 1e-3) / 1e12, 3)
     roof = None
     dom = max((k for k in kernels if k in ("p2p", "m2p", "p2p_fp64", "m2p_fp64", "p2p_ff", "m2p_ff")),
@@ -568,12 +571,12 @@ def run_ours(args, wl, rank, world, local_rank):
                 "frac": round(a / FP64_PEAK_TFLOPS, 4), "traffic": traffic,
                 "peak_note": "FP64 nominal 1.25 TFLOP/s (no measured FP64 peak)"}
     elif dom == "m2p" and m2p_tc and "m2p" in full:
-        # max(generation / FP32 peak, rsqrt / SFU peak, issued MMA flops / TF32 peak) per launch of
+        # max(generation / FP32 peak, rsqrt / SFU peak, issued MMA flops / bf16 peak) per launch of
         # all B right-hand sides
-        bnd = m2p_tc_bound(wl["P"], B, ctx_tc["m2p_group_boxes"], peaks, mhz)
+        bnd = m2p_tc_bound(wl["P"], B, ctx_tc["m2p_group_boxes"], peaks, mhz, f16=True)
         roof = tc_roofline(bnd, full["m2p"]["ms_per_launch"] * 1e-3, dom, traffic)
     elif dom == "p2p" and p2p_tc and "p2p" in full:
-        bnd = p2p_tc_bound(B, pairs, ctx_tc["p2p_stages"], peaks, mhz)
+        bnd = p2p_tc_bound(B, pairs, ctx_tc["p2p_stages"], peaks, mhz, f16=True)
         roof = tc_roofline(bnd, full["p2p"]["ms_per_launch"] * 1e-3, dom, traffic)
     elif dom in ("p2p", "m2p") and fp32 and dom in full:
         a = full[dom]["algorithmic_tflops"]
@@ -588,7 +591,7 @@ def run_ours(args, wl, rank, world, local_rank):
     # the other tensor-core kernel at the full batch, on the same max-of-three bound
     roof2 = None
     if roof is not None and roof.get("kernel") == "m2p" and p2p_tc and "p2p" in full:
-        roof2 = tc_roofline(p2p_tc_bound(B, pairs, ctx_tc["p2p_stages"], peaks, mhz),
+        roof2 = tc_roofline(p2p_tc_bound(B, pairs, ctx_tc["p2p_stages"], peaks, mhz, f16=True),
                             full["p2p"]["ms_per_launch"] * 1e-3, "p2p",
                             NCU_TRAFFIC.get((args.workload, "p2p", wl["theta"], wl["P"], wl["Ncrit"])))
         del roof2["peak_note"]

@@ -258,7 +258,7 @@ LSPR_API int lspr_get_info(lspr_ctx *ctx, int64_t *n_panels, int64_t *n_sources,
  * several right-hand sides forms them; any pointer may be null): M2P work units (a group of
  * four consecutive 64-target blocks and a stretch of its box list), (group, box) entries of
  * the groups' united box lists, source entries of the P2P groups' united source ranges, and
- * the P2P pipeline stages (8 sources of one range each) that one unit of right-hand sides
+ * the P2P pipeline stages (16 sources of one range each, 8 with TF32 parts) that one unit of right-hand sides
  * takes.  LSPR_E_ARG: null context. */
 LSPR_API int lspr_get_tc_info(lspr_ctx *ctx, int64_t *m2p_units, int64_t *m2p_group_boxes,
                               int64_t *p2p_group_sources, int64_t *p2p_stages);
@@ -301,10 +301,10 @@ LSPR_API int lspr_get_arnoldi_stats(lspr_ctx *ctx, int64_t *out);
  * cycles. */
 LSPR_API int lspr_set_graphs(lspr_ctx *ctx, int32_t enable);
 /* Tensor cores for the FP32 far field of several right-hand sides (B >= 2), as a mask:
- * bit 0 (default on): the M2P contraction on tcgen05 (TF32 operands split into high and low
- * parts, FP32 accumulation in tensor memory; about 2x the FP32-pipe kernel at 16 right-hand
- * sides, 4x at 64); bit 1 (default off; lspr_tune_solver sets it where it pays): the tree P2P
- * on tcgen05 (same split; 2.3x the FP32-pipe kernel at 64 right-hand sides) for products with
+ * bit 0 (default on): the M2P contraction on tcgen05 (operands split into FP16 high and low
+ * parts that hold 22 bits, FP32 accumulation in tensor memory); bit 1 (default off;
+ * lspr_tune_solver sets it where it pays): the tree P2P on tcgen05 (same split, TF32 parts where
+ * the distances span too much; 3x the FP32-pipe kernel at 32 right-hand sides) for products with
  * at least 24 right-hand sides (channel sets) in use, the FP32-pipe P2P below that (inside a
  * solve the count falls as wavelengths converge, and the choice is then made on the device).
  * 0 selects the FP32-pipe kernels of the same sums.  Bits above 1 are ignored.
