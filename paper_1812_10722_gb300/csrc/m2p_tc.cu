@@ -117,6 +117,7 @@ __device__ __forceinline__ int core_off(int r, int k) {
 __device__ __forceinline__ float box_scale(const float4 &c, float rho_min) {
     return __int_as_float(__float_as_int(fmaxf(c.w, rho_min)) & 0x7f800000);
 }
+__device__ __forceinline__ int exponent_of(float p) { return (__float_as_int(p) >> 23) - 127; }
 __device__ __forceinline__ float inv_pow2(float p) { return __int_as_float((254 << 23) - __float_as_int(p)); }
 
 // largest |M_k| / rho^(n+1) per layer and right-hand side over the accepted boxes: mx[2 j] single layer,
@@ -133,16 +134,15 @@ __global__ void __launch_bounds__(256)
     __syncthreads();
     for (int64_t box = blockIdx.x; box < nbox; box += gridDim.x) {
         if (!used[box]) continue;
-        const float ir = inv_pow2(box_scale(box_c[box], rho_min));
+        const int ie = -exponent_of(box_scale(box_c[box], rho_min));
         const float4 *m = mom + box * NT * B;
         for (int q = threadIdx.x; q < NT * nj; q += blockDim.x) {
             const int t = q / nj, j = q - t * nj;
             if (NS > 1 && !(box_surf[box] & set_surfaces(j0 + j, 1, Bact, NS))) continue;
-            float f = ir;
-            for (int n = c_deg[t]; n > 0; --n) f *= ir;
+            const int k = (c_deg[t] + 1) * ie;
             const float4 v = __ldg(m + (int64_t)t * B + j0 + j);
-            const int a = __float_as_int(fmaxf(fabsf(v.x), fabsf(v.y)) * f);
-            const int b = __float_as_int(fmaxf(fabsf(v.z), fabsf(v.w)) * f);
+            const int a = __float_as_int(times_pow2(fmaxf(fabsf(v.x), fabsf(v.y)), k));
+            const int b = __float_as_int(times_pow2(fmaxf(fabsf(v.z), fabsf(v.w)), k));
             // (a NaN loses against the other component in fmaxf; its rows are NaN whatever the scale)
             if (a > smax[2 * j]) atomicMax(&smax[2 * j], a);
             if (b > smax[2 * j + 1]) atomicMax(&smax[2 * j + 1], b);
@@ -179,15 +179,14 @@ __global__ void tc_image_kernel(int64_t nbox, int B, int nrc, const float4 *__re
         const int j = rc * RC + (r >> 2), cpt = r & 3, t0 = kc * kKC + 8 * k8;
         float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         if (t0 < S::NT && j < Bact) {
-            const float ir = inv_pow2(box_scale(__ldg(box_c + box), rho_min));
-            float f = f16_scale(__ldg(mx + 2 * j + (cpt >> 1))) * ir;
-            int n = 0;
+            // 2^e rho^-(n+1) is not formed: small boxes under a small or zero layer take it out of FP32
+            const int ie = -exponent_of(box_scale(__ldg(box_c + box), rho_min));
+            const int e16 = f16_exponent(__ldg(mx + 2 * j + (cpt >> 1)));
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-                if (t0 + u < S::NT) {
-                    for (const int d = c_deg[t0 + u]; n < d; ++n) f *= ir;
-                    v[u] = __ldg((const float *)(mom + (box * S::NT + t0 + u) * B + j) + cpt) * f;
-                }
+                if (t0 + u < S::NT)
+                    v[u] = times_pow2(__ldg((const float *)(mom + (box * S::NT + t0 + u) * B + j) + cpt),
+                                      e16 + (c_deg[t0 + u] + 1) * ie);
         }
         const HalfPair sp = f16_split(v);
         unsigned char *dst = img + c * (2 * S::A_CH) + 16 * e;

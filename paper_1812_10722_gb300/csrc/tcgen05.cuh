@@ -60,12 +60,21 @@ __device__ __forceinline__ HalfPair f16_split(const float (&v)[8]) {
     }
     return p;
 }
-// the power of two that brings a largest magnitude (the bits of a non-negative float) into
-// [2^14, 2^15), at most 2^126 so that its reciprocal is normal; 1 for infinities and NaN
-__device__ __forceinline__ float f16_scale(int bits) {
-    const int e = bits >> 23;
-    return e >= 255 ? 1.f : __int_as_float(min(253, 268 - e) << 23);
+// 2^k, -126 <= k <= 127
+__device__ __forceinline__ float pow2(int k) { return __int_as_float((k + 127) << 23); }
+// v 2^k in two exact factors: where neither v nor the result leaves the FP32 range nothing between them
+// does, although 2^k itself may (and a zero stays zero)
+__device__ __forceinline__ float times_pow2(float v, int k) {
+    k = max(-252, min(252, k));   // beyond, the result of any finite v is below the last place of FP16 or v is 0
+    return v * pow2(k >> 1) * pow2(k - (k >> 1));
 }
+// the exponent of the power of two that brings a largest magnitude (the bits of a non-negative float)
+// into [2^14, 2^15), at most 126 so that the power's reciprocal is normal; 0 for zero, infinities and NaN
+__device__ __forceinline__ int f16_exponent(int bits) {
+    const int e = bits >> 23;
+    return bits == 0 || e >= 255 ? 0 : min(126, 141 - e);
+}
+__device__ __forceinline__ float f16_scale(int bits) { return pow2(f16_exponent(bits)); }
 
 __device__ __forceinline__ uint64_t now_ns() {
     uint64_t t;
