@@ -432,10 +432,10 @@ int launch_p2p(lspr_ctx *ctx, int prec, const int4 *items, int64_t nitems, doubl
                int *counter, int B);
 // the moments are zero on entry (launch_weights clears them)
 int launch_p2m(lspr_ctx *ctx, int prec, int B);
-// behind the accumulators of a product, cleared with them: the work-item counters, then per layer and
-// channel set the largest magnitudes that scale the tensor-core operands
+// behind the accumulators of a product, cleared with them: the work-item counters, then per channel set
+// and component (re and im of both layers) the largest magnitudes that scale the tensor-core operands
 constexpr int kCounters = 8;
-inline int64_t acc_tail_ints(int64_t BS) { return kCounters + 4 * BS; }   // M2P's, then P2P's
+inline int64_t acc_tail_ints(int64_t BS) { return kCounters + 8 * BS; }   // M2P's, then P2P's
 int launch_m2p(lspr_ctx *ctx, int prec, double *acc, int *counter, int B);
 // float-float copies of the work-order geometry / box centres
 int launch_ff_geometry(lspr_ctx *ctx);

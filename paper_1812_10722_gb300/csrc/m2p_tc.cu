@@ -16,8 +16,9 @@
 //   - lengths of a box are measured in rho_b (box_scale): with rho_b / r < theta the coefficients
 //     A_k rho_b^(n+1) stay below 1.2 (the largest |A_k| r^(n+1) of any degree up to 8 and direction),
 //     and are carried times 2^15;
-//   - the moments M_k / rho_b^(n+1) of one right-hand side and layer are scaled by their largest
-//     magnitude over all boxes (m2p_max_kernel) into [2^14, 2^15).
+//   - the moments M_k / rho_b^(n+1) of one right-hand side, layer and part (re, im: the channels are
+//     sums of their own, and one may be far smaller) are scaled by their largest magnitude over all
+//     boxes (m2p_max_kernel) into [2^14, 2^15).
 // What falls below full precision is then at most 2^-25 absolute in both: 2^-40 of the largest.
 // Against TF32 parts the MMAs take half the K steps and the operands half the bytes: 81920 panels, P 7,
 // 64 right-hand sides 2.57 -> 1.58 ms with both preparing kernels; sensor of 145920 panels 6.12 -> 4.38.
@@ -120,17 +121,18 @@ __device__ __forceinline__ float box_scale(const float4 &c, float rho_min) {
 __device__ __forceinline__ int exponent_of(float p) { return (__float_as_int(p) >> 23) - 127; }
 __device__ __forceinline__ float inv_pow2(float p) { return __int_as_float((254 << 23) - __float_as_int(p)); }
 
-// largest |M_k| / rho^(n+1) per layer and right-hand side over the accepted boxes: mx[2 j] single layer,
-// mx[2 j + 1] double layer, as the bits of non-negative floats.  One block per box (grid stride).
+// largest |M_k| / rho^(n+1) per channel over the accepted boxes: mx[4 j + c] of right-hand side j, c = re
+// and im of the single layer, then of the double layer, as the bits of non-negative floats (of a NaN
+// where there is one: its rows are NaN whatever the scale).  One block per box (grid stride).
 constexpr int kMaxSets = 512;   // channel sets per block column of m2p_max_kernel
 __global__ void __launch_bounds__(256)
     m2p_max_kernel(int64_t nbox, int NT, int B, const float4 *__restrict__ mom, const float4 *__restrict__ box_c,
                    float rho_min, const int *__restrict__ used, int *mx, const int *nact,
                    const int *__restrict__ box_surf, int NS) {
-    __shared__ int smax[2 * kMaxSets];
+    __shared__ int smax[4 * kMaxSets];
     const int Bact = nact ? *nact : B, j0 = blockIdx.y * kMaxSets, nj = min(kMaxSets, Bact - j0);
     if (nj <= 0) return;
-    for (int j = threadIdx.x; j < 2 * nj; j += blockDim.x) smax[j] = 0;
+    for (int j = threadIdx.x; j < 4 * nj; j += blockDim.x) smax[j] = 0;
     __syncthreads();
     for (int64_t box = blockIdx.x; box < nbox; box += gridDim.x) {
         if (!used[box]) continue;
@@ -141,16 +143,17 @@ __global__ void __launch_bounds__(256)
             if (NS > 1 && !(box_surf[box] & set_surfaces(j0 + j, 1, Bact, NS))) continue;
             const int k = (c_deg[t] + 1) * ie;
             const float4 v = __ldg(m + (int64_t)t * B + j0 + j);
-            const int a = __float_as_int(times_pow2(fmaxf(fabsf(v.x), fabsf(v.y)), k));
-            const int b = __float_as_int(times_pow2(fmaxf(fabsf(v.z), fabsf(v.w)), k));
-            // (a NaN loses against the other component in fmaxf; its rows are NaN whatever the scale)
-            if (a > smax[2 * j]) atomicMax(&smax[2 * j], a);
-            if (b > smax[2 * j + 1]) atomicMax(&smax[2 * j + 1], b);
+            const float w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int a = __float_as_int(fabsf(times_pow2(w[c], k)));
+                if (a > smax[4 * j + c]) atomicMax(&smax[4 * j + c], a);
+            }
         }
     }
     __syncthreads();
-    for (int j = threadIdx.x; j < 2 * nj; j += blockDim.x)
-        if (smax[j] > 0) atomicMax(&mx[2 * j0 + j], smax[j]);
+    for (int j = threadIdx.x; j < 4 * nj; j += blockDim.x)
+        if (smax[j] > 0) atomicMax(&mx[4 * j0 + j], smax[j]);
 }
 
 // The split moments of every box in stage layout: image[((box * nrc + rc) * NKC + kc)] holds
@@ -181,7 +184,7 @@ __global__ void tc_image_kernel(int64_t nbox, int B, int nrc, const float4 *__re
         if (t0 < S::NT && j < Bact) {
             // 2^e rho^-(n+1) is not formed: small boxes under a small or zero layer take it out of FP32
             const int ie = -exponent_of(box_scale(__ldg(box_c + box), rho_min));
-            const int e16 = f16_exponent(__ldg(mx + 2 * j + (cpt >> 1)));
+            const int e16 = f16_exponent(__ldg(mx + 4 * j + cpt));
 #pragma unroll
             for (int u = 0; u < 8; ++u)
                 if (t0 + u < S::NT)
@@ -407,7 +410,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 const int m = (32 * qd + lane) % S::ROWS, j = m >> 2, cpt = m & 3;
                 const int jb = p_b0 + hh * S::HRC + j;   // the right-hand side of row m
                 // both operands' scales undone: 2^-15 for the coefficients, 1 / f16_scale for the moments
-                const float undo = j < hnb ? inv_pow2(f16_scale(__ldg(mx + 2 * jb + (cpt >> 1)))) * 0x1p-15f : 0.f;
+                const float undo = j < hnb ? inv_pow2(f16_scale(__ldg(mx + 4 * jb + cpt))) * 0x1p-15f : 0.f;
 #pragma unroll 1
                 for (int c0 = 0; c0 < kTcN / 2; c0 += 32) {
                     const int64_t tc = p_tbase + half * (kTcN / 2) + c0 + lane;   // this lane's column's target

@@ -26,7 +26,7 @@
 // nothing; dG/dn falls to 2^-9 at the largest distances, where its parts keep 2^-25 absolute: summed
 // over the sources of a P2P region of area a that is below 2^-40 a / r_min^2 of a potential of order 2 pi
 // (2^-27 at a = 10 nm^2, r_min = 0.04 nm), less than the accumulation rounds off.  The weights of one
-// right-hand side and layer are scaled by a bound of their largest magnitude.  All scales are powers of
+// right-hand side, layer and part (re, im) are scaled by a bound of their largest magnitude.  All scales are powers of
 // two: those of G and dG/dn are folded into the positions and normals, all are undone as the
 // accumulators are drained.
 //
@@ -126,34 +126,36 @@ static_assert(kRC * 2 == 128, "re and im of the unit's right-hand sides fill the
 // 16-byte core matrices, no swizzle)
 __device__ __forceinline__ int core_off(int r, int c) { return (r >> 3) * kSBO + c * 128 + (r & 7) * 16; }
 
-// largest magnitude per layer and system of the right-hand sides xt [2N][B], times the largest source
-// weight: a bound of the weights of the system's sets, as the bits of a non-negative float in mx[2 set]
-// (single layer) and mx[2 set + 1]
+// largest magnitude per layer, part (re, im) and system of the right-hand sides xt [2N][B], times the
+// largest source weight: a bound of the weights of the system's sets, as the bits of non-negative floats
+// in mx[4 set + c], c = re and im of the single layer, then of the double layer
 constexpr int kMaxSets = 512;   // right-hand sides per block column
 __global__ void __launch_bounds__(256)
     p2p_max_kernel(int64_t N, int B, int S, const float2 *__restrict__ xt, const int *__restrict__ stat, int *mx,
                    const int *inv, const int *nact, int min_rhs) {
-    __shared__ int smax[2 * kMaxSets];
+    __shared__ int smax[4 * kMaxSets];
     const int sets = nact ? *nact : B * S;
     if (sets < min_rhs) return;
     const int j0 = blockIdx.y * kMaxSets, nj = min(kMaxSets, B - j0), K = sets / S;
-    for (int j = threadIdx.x; j < 2 * nj; j += blockDim.x) smax[j] = 0;
+    for (int j = threadIdx.x; j < 4 * nj; j += blockDim.x) smax[j] = 0;
     __syncthreads();
     const float wa = __int_as_float(stat[2]);
     const int64_t rows = (2 * N + gridDim.x - 1) / gridDim.x;
     const int64_t r0 = blockIdx.x * rows, r1 = min(2 * N, r0 + rows);
     for (int64_t q = threadIdx.x; q < (r1 - r0) * nj; q += blockDim.x) {
         const int64_t r = r0 + q / nj;
-        const int j = (int)(q % nj), layer = r < N ? 1 : 0;
+        const int j = (int)(q % nj);
+        int *const s = smax + 4 * j + (r < N ? 2 : 0);
         const float2 v = __ldg(xt + r * B + j0 + j);
-        const int a = __float_as_int(fmaxf(fabsf(v.x), fabsf(v.y)) * wa);
-        if (a > smax[2 * j + layer]) atomicMax(&smax[2 * j + layer], a);
+        const int re = __float_as_int(fabsf(v.x) * wa), im = __float_as_int(fabsf(v.y) * wa);
+        if (re > s[0]) atomicMax(s, re);
+        if (im > s[1]) atomicMax(s + 1, im);
     }
     __syncthreads();
-    for (int j = threadIdx.x; j < 2 * nj; j += blockDim.x) {
-        const int b = j0 + (j >> 1), k = inv ? inv[b] : b;
+    for (int j = threadIdx.x; j < 4 * nj; j += blockDim.x) {
+        const int b = j0 + (j >> 2), k = inv ? inv[b] : b;
         if (k < 0 || smax[j] == 0) continue;
-        for (int t = 0; t < S; ++t) atomicMax(&mx[2 * (t * K + k) + (j & 1)], smax[j]);
+        for (int t = 0; t < S; ++t) atomicMax(&mx[4 * (t * K + k) + (j & 3)], smax[j]);
     }
 }
 
@@ -176,16 +178,17 @@ __global__ void __launch_bounds__(128)
     // no range that holds these sources has one of the chunk's surfaces: no unit reads the block
     if (nsurf > 1 && !(mask[g] & set_surfaces(b0, nb, Bact, nsurf))) return;
     if (j >= nb) return;
-    const float fv = F16 ? f16_scale(__ldg(mx + 2 * (b0 + j))) : 1.f;
-    const float fk = F16 ? f16_scale(__ldg(mx + 2 * (b0 + j) + 1)) : 1.f;
+    float f[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) f[c] = F16 ? f16_scale(__ldg(mx + 4 * (b0 + j) + c)) : 1.f;
     float w[4][H::PART];
 #pragma unroll
     for (int i = 0; i < H::PART; ++i) {
         const float4 v = s0 + i < Ns ? __ldg(sw + (s0 + i) * B + b0 + j) : make_float4(0.f, 0.f, 0.f, 0.f);
-        w[0][i] = v.x * fv;
-        w[1][i] = v.y * fv;
-        w[2][i] = v.z * fk;
-        w[3][i] = v.w * fk;
+        w[0][i] = v.x * f[0];
+        w[1][i] = v.y * f[1];
+        w[2][i] = v.z * f[2];
+        w[3][i] = v.w * f[3];
     }
     const bool stacked = nb <= kRC / 2;
     // rows: 2 j + (0: re, 1: im), the high part, then the low part; stacked: the low rows are 64 + 2 j + ..
@@ -405,8 +408,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             // the scales undone: of the kernel values and of the weights
             float undo_v = 1.f, undo_k = 1.f;
             if (F16 && j < p_nb) {
-                undo_v = 1.f / gs * (1.f / f16_scale(__ldg(mx + 2 * (p_b0 + j))));
-                undo_k = 1.f / ts * (1.f / f16_scale(__ldg(mx + 2 * (p_b0 + j) + 1)));
+                undo_v = 1.f / gs * (1.f / f16_scale(__ldg(mx + 4 * (p_b0 + j) + (m & 1))));
+                undo_k = 1.f / ts * (1.f / f16_scale(__ldg(mx + 4 * (p_b0 + j) + 2 + (m & 1))));
             }
             if (!warp_wait(smem_addr(&acc_full), (uint32_t)((nu - 1) & 1), &abort_s)) return false;
             asm volatile("tcgen05.fence::after_thread_sync;");
@@ -564,7 +567,7 @@ int launch_parts(lspr_ctx *ctx, double *acc, cudaStream_t st, int *counter, int 
     const int nrc = (B + kRC - 1) / kRC;
     const int64_t Ns = ctx->mesh.Ns, N = ctx->mesh.N, ng = (Ns + H::SRC - 1) / H::SRC;
     LSPR_TRY(ctx, ctx->tcp_img.ensure((size_t)(ng * nrc) * kImgBlock));
-    int *mx = (int *)(acc + 4 * N * B) + kCounters + 2 * B;   // cleared with the accumulators
+    int *mx = (int *)(acc + 4 * N * B) + kCounters + 4 * B;   // cleared with the accumulators
     if (F16) {
         const int S = ctx->mesh.S, nsys = B / S;
         ++ctx->n_launches;
