@@ -304,12 +304,17 @@ __device__ __forceinline__ bool near_decide(const float4 &fi, const float4 &fj, 
     return near_exact(xi, yi, zi, cx[j], cy[j], cz[j], L[j], thr);
 }
 
-// One warp per occupied cell: lane c < 27 searches neighbour cell c once for all the cell's targets;
-// the neighbours' panels, in cell order, are the candidates.  Each lane holds one candidate of a
-// chunk of 32 and tests it against the targets in turn, a ballot counts the hits.  A row is laid out
-// as the self entry, then the hits of cell 0, 1, ... in sorted order.  Bound by the searches'
-// latency: 140 us for both passes at 81920 panels, 317 with a warp (and its searches) per target.
-constexpr int kCellTargets = 64;   // targets of a cell taken together
+// One warp per slice of up to kCellTargets panels of an occupied cell: lane c < 27 searches neighbour
+// cell c once for all the slice's targets; the neighbours' panels, in cell order, are the candidates.
+// Each lane holds one candidate of a chunk of 32 and tests it against the targets in turn, a ballot
+// counts the hits.  A row is laid out as the self entry, then the hits of cell 0, 1, ... in sorted order.
+// Bound by the searches' latency where cells hold few panels: 140 us for both passes at 81920 panels,
+// 317 with a warp (and its searches) per target.  Cells are sized by the largest panel, so beside a few
+// large panels, or at a small threshold, thousands of panels share a cell and a slice's chain of tests
+// sets the time.  Whole uploads of 20480 panels beside 20 large ones: 5.7 ms in slices of 16, 8.2 of
+// 32, 15.4 of 64, 3630 with a warp per cell, 58.7 with a warp per target; 5120 panels at threshold 0.1:
+// 3.6, 4.2, 5.4, 12.0, 4.6; a uniform mesh of 81920 2.40 in all three.
+constexpr int kCellTargets = 16;   // targets of a slice
 constexpr int kCellWarps = 4;
 template <bool FILL>
 __global__ void __launch_bounds__(kCellWarps * 32)
@@ -323,7 +328,13 @@ __global__ void __launch_bounds__(kCellWarps * 32)
     int *hit = hits[threadIdx.x >> 5];
     if (k >= N) return;
     const unsigned mykey = skeys[k];
-    if (k > 0 && skeys[k - 1] == mykey) return;   // not the first panel of its cell
+    // the first panel of a slice of its cell?
+    int t0 = 0;
+    if (k > 0 && skeys[k - 1] == mykey) {
+        if (k < kCellTargets || skeys[k - kCellTargets] != mykey) return;
+        t0 = (int)k - lower_bound_u(skeys, (int)k, mykey);
+        if (t0 % kCellTargets) return;
+    }
     const float cmax = (float)grid[4];
     const int i0 = sidx[k];
     const int ix = cell_coord(cx[i0], grid[0], grid[3]), iy = cell_coord(cy[i0], grid[1], grid[3]),
@@ -344,55 +355,51 @@ __global__ void __launch_bounds__(kCellWarps * 32)
     }
     const int total = __shfl_sync(0xffffffffu, pre, 31);
     const int mine = __shfl_sync(0xffffffffu, len, 13);   // the cell itself (offsets 0, 0, 0)
-    for (int t0 = 0; t0 < mine; t0 += kCellTargets) {
-        const int nt = min(kCellTargets, mine - t0);
-        for (int t = lane; t < nt; t += 32) hit[t] = 0;
-        __syncwarp();
-        for (int c0 = 0; c0 < total; c0 += 32) {
-            const int c = c0 + lane;
-            // the cell that holds candidate c: the first lane whose inclusive count exceeds it
-            int lo = 0;
+    const int nt = min(kCellTargets, mine - t0);
+    for (int t = lane; t < nt; t += 32) hit[t] = 0;
+    __syncwarp();
+    for (int c0 = 0; c0 < total; c0 += 32) {
+        const int c = c0 + lane;
+        // the cell that holds candidate c: the first lane whose inclusive count exceeds it
+        int lo = 0;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const int v = __shfl_sync(0xffffffffu, pre, lo + o - 1);
-                if (v <= c) lo += o;
-            }
-            lo = min(lo, 31);
-            const int cb = __shfl_sync(0xffffffffu, k0, lo), cp = __shfl_sync(0xffffffffu, pre - len, lo);
-            int j = -1;
-            float4 fj = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (c < total) {
-                j = sidx[cb + (c - cp)];
-                fj = cf[j];
-            }
-            for (int t = 0; t < nt; ++t) {
-                const int i = sidx[k + t0 + t];
-                bool near = false;
-                if (j >= 0 && j != i)
-                    near = near_decide(cf[i], fj, 1e-6f * fj.w + 5e-7f * cmax, cx[i], cy[i], cz[i], j, cx, cy, cz, L,
-                                       thr);
-                const unsigned m = __ballot_sync(0xffffffffu, near);
-                const int run = hit[t];
-                if (FILL && near) {
-                    const int64_t out = ptr[i] + 1 + run + __popc(m & ((1u << lane) - 1u));
-                    col[out] = j;
-                    row[out] = i;
-                }
-                __syncwarp();
-                if (lane == 0) hit[t] = run + __popc(m);
-                __syncwarp();
-            }
+        for (int o = 16; o > 0; o >>= 1) {
+            const int v = __shfl_sync(0xffffffffu, pre, lo + o - 1);
+            if (v <= c) lo += o;
         }
-        for (int t = lane; t < nt; t += 32) {
-            const int i = sidx[k + t0 + t];
-            if (FILL) {
-                col[ptr[i]] = i;   // self entry first
-                row[ptr[i]] = i;
-            } else {
-                count[i] = hit[t] + 1;
-            }
+        lo = min(lo, 31);
+        const int cb = __shfl_sync(0xffffffffu, k0, lo), cp = __shfl_sync(0xffffffffu, pre - len, lo);
+        int j = -1;
+        float4 fj = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (c < total) {
+            j = sidx[cb + (c - cp)];
+            fj = cf[j];
         }
-        __syncwarp();
+        for (int t = 0; t < nt; ++t) {
+            const int i = sidx[k + t];
+            bool near = false;
+            if (j >= 0 && j != i)
+                near = near_decide(cf[i], fj, 1e-6f * fj.w + 5e-7f * cmax, cx[i], cy[i], cz[i], j, cx, cy, cz, L, thr);
+            const unsigned m = __ballot_sync(0xffffffffu, near);
+            const int run = hit[t];
+            if (FILL && near) {
+                const int64_t out = ptr[i] + 1 + run + __popc(m & ((1u << lane) - 1u));
+                col[out] = j;
+                row[out] = i;
+            }
+            __syncwarp();
+            if (lane == 0) hit[t] = run + __popc(m);
+            __syncwarp();
+        }
+    }
+    for (int t = lane; t < nt; t += 32) {
+        const int i = sidx[k + t];
+        if (FILL) {
+            col[ptr[i]] = i;   // self entry first
+            row[ptr[i]] = i;
+        } else {
+            count[i] = hit[t] + 1;
+        }
     }
 }
 
