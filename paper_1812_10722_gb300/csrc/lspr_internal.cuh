@@ -42,12 +42,15 @@ inline bool mode_tree(int mode) { return mode == LSPR_TREE_FP64 || mode == LSPR_
 constexpr double kInv4Pi = 0.079577471545947667884;   // 1 / (4 pi)
 constexpr int kTargetBlock = 64;                       // targets per interaction block (2 per lane)
 constexpr int kTcGroup = 4;        // target blocks per tensor-core M2P group (256 targets)
-// Boxes per tensor-core M2P work unit and sources per P2P unit (stages of 16, of 8 with TF32 parts), at most
-// (tc_unit).  A unit ends with its accumulators added in FP64, which no MMA overlaps; the upper limits bound
-// the steps added in FP32 (at most 672 K steps of boxes, 256 stages of sources).
-constexpr int kTcSegMin = 32;
-constexpr int tc_seg_max(int P) { return P < 7 ? 64 : 112; }
-constexpr int kTcSrcMin = 1024, kTcSrcMax = 4096;
+// Boxes per tensor-core M2P work unit and sources per P2P unit, at most (tc_unit).  A unit ends with its
+// accumulators added in FP64, which no MMA overlaps, so units are long; but a sum of one sign loses a part
+// of its last place at every step added in FP32, and the upper limits keep the error of products of smooth
+// vectors below that of TF32 parts in units of 32 boxes and 2048 sources (256 stages of 8, still the limit
+// with TF32 parts).  81920 panels, P 7, 64 right-hand sides, smooth vectors, M2P on the tensor cores / P2P
+// / both: 3.3e-6, 1.7e-6, 4.8e-6 in 4.14 ms; 5.7e-6, 2.6e-6, 8.1e-6 in 4.01 ms with limits of 112 and 4096;
+// 4.7e-6, 2.1e-6, 6.6e-6 with TF32 parts.  3072 sources: above TF32 parts at P 8 (1.01 times); 2048: 4.22 ms.
+constexpr int kTcSegMin = 32, kTcSegMax = 64;
+constexpr int kTcSrcMin = 1024, kTcSrcMax = 2560, kTcSrcMaxTf32 = 2048;
 constexpr int kTcSrcRows = 8;      // tensor-core P2P source geometry per stage: rows -x, -y, -z, normal, panel, -
 constexpr float kTcP2PRange = 4096.f;   // largest ratio of P2P distances for FP16 parts
 constexpr int kTcSurf = 8;         // tensor-core M2P list entry.y: block mask, from this bit the box's surfaces

@@ -1000,7 +1000,7 @@ int tree_tc_lists(lspr_ctx *ctx, bool p2p) {
         std::vector<TcItem> gitems;
         tc_union_m2p(ntb, kTcGroup, hlist.data(), (const int *)hitems.data(), tr.n_m2p_items, glist, gitems);
         tr.n_tc_pairs = (int64_t)glist.size();
-        tc_cut_m2p(tc_unit(tr.n_tc_pairs, ctx->num_sms, kTcSegMin, tc_seg_max(tr.P)), gitems);
+        tc_cut_m2p(tc_unit(tr.n_tc_pairs, ctx->num_sms, kTcSegMin, kTcSegMax), gitems);
         tr.n_tc_items = (int64_t)gitems.size();
         LSPR_TRY(ctx, tr.tc_list.ensure(std::max<size_t>(1, glist.size())));
         LSPR_TRY(ctx, tr.tc_items.ensure(std::max<size_t>(1, gitems.size())));
@@ -1052,7 +1052,7 @@ int tree_tc_lists(lspr_ctx *ctx, bool p2p) {
         tr.tcp_gs = tr.tcp_f16 ? std::exp2(std::floor(std::log2(32768.f * std::sqrt(r2lo)))) : 1.f;
         tr.tcp_ts = tr.tcp_f16 ? std::exp2(std::floor(std::log2(32768.f * r2lo))) : 1.f;
         const int per = tr.tcp_f16 ? 16 : 8;   // sources per stage
-        tc_cut_p2p(tc_unit(psrc, ctx->num_sms, kTcSrcMin, kTcSrcMax / 16 * per), pivl, pitems);
+        tc_cut_p2p(tc_unit(psrc, ctx->num_sms, kTcSrcMin, tr.tcp_f16 ? kTcSrcMax : kTcSrcMaxTf32), pivl, pitems);
         tr.n_tcp_items = (int64_t)pitems.size();
         tr.n_tcp_ivl = (int64_t)pivl.size();
         for (const TcRange &r : pivl) tr.n_tcp_stages += (r.s1 + per - 1) / per - r.s0 / per;
