@@ -423,10 +423,10 @@ int launch_p2p(lspr_ctx *ctx, int prec, const int4 *items, int64_t nitems, doubl
         if (B == 1) p2p_launch<ffloat, 1>(ctx, items, nitems, B, acc, st, counter);
         else LSPR_TRY_ST(p2p_ff_multi(ctx, items, nitems, B, acc, st, counter));
     } else if (B > 1 && (ctx->tensor_cores & 2) && items == ctx->tree.p2p_items.p) {
-        // the tensor-core P2P for products of at least tc_p2p_min_rhs right-hand sides in use, the
+        // the tensor-core P2P for products of at least kTcP2PMinSets right-hand sides in use, the
         // FP32 pipe below: decided on the host when every slot is in use, else on the device from
         // the count of running systems (both kernels are launched; the one not chosen returns at once)
-        const int mn = std::max(2, ctx->tc_p2p_min_rhs);
+        const int mn = kTcP2PMinSets;
         if (!ctx->rhs_nact) {
             if (B >= mn) LSPR_TRY_ST(p2p_tc_launch(ctx, acc, st, counter, B, 0));
             else LSPR_TRY_ST(p2p_multi_launch(ctx, items, nitems, B, acc, st, counter));

@@ -58,6 +58,11 @@ constexpr int kMaxP = 8;                               // highest Taylor order c
 constexpr int kMaxDepth = 10;                          // octree levels below the root (10 bits per axis)
 constexpr int kMaxNk = 32;
 constexpr int kMaxSurfaces = 16;                       // particle + analyte surfaces
+// The tensor-core P2P takes products of at least this many right-hand sides (channel sets) in use; fewer
+// take the FP32-pipe P2P.  It bounds the weights from the transposed FP32 vectors, which products of one
+// system do not form, so it must never take one system's surfaces.
+constexpr int kTcP2PMinSets = 24;
+static_assert(kTcP2PMinSets > kMaxSurfaces, "the tensor-core P2P needs two systems or more");
 
 // terms of an expansion of order P in the harmonic basis: the multi-indices |k| <= P with k_3 <= 1
 __host__ __device__ constexpr int n_terms(int P) { return (P + 1) * (P + 1); }
@@ -315,8 +320,6 @@ struct lspr_ctx {
     // device-driven Arnoldi cycles (a CUDA graph per configuration, gmres_graph.cu)
     bool use_graphs = true;
     int tensor_cores = 1;              // tcgen05 for B >= 2 in FP32: bit 0 M2P, bit 1 P2P
-    int tc_p2p_min_rhs = 24;           // the tensor-core P2P takes products of at least this many
-                                       // right-hand sides in use; fewer take the FP32-pipe P2P
     lspr::DArr<unsigned char> tc_img;  // split moments in tensor-core operand layout
     lspr::DArr<unsigned char> tcp_img; // split source weights in tensor-core operand layout
     lspr::DArr<int> dev_err;           // [0] bounded device waits that ran out (never reset);
