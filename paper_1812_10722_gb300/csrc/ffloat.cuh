@@ -116,8 +116,8 @@ __device__ __forceinline__ ffloat &operator+=(ffloat &x, const ffloat &y) { retu
 __device__ __forceinline__ ffloat &operator-=(ffloat &x, const ffloat &y) { return x = x - y; }
 __device__ __forceinline__ ffloat &operator*=(ffloat &x, const ffloat &y) { return x = x * y; }
 
-// 1/sqrt(x): FP32 seed y0, then one third-order step y0 (1 + h/2 + 3 h^2/8), h = 1 - x y0^2
-// formed in float-float (1 - leading part is exact since x y0^2 is close to 1).
+// 1/sqrt(x): FP32 seed y0, then one third-order (Householder) step, the binomial series of
+// y0 (1 - h)^(-1/2) up to h^2: y0 (1 + h/2 + 3 h^2/8), h = 1 - x y0^2 formed in float-float (1 - leading part is exact since x y0^2 is close to 1).
 __device__ __forceinline__ ffloat rsq(const ffloat &x) {
     const float y0 = rsqrtf(x.hi);
     const ffloat xy2 = x * (ffloat(y0) * ffloat(y0));
