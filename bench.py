@@ -131,6 +131,13 @@ def m2p_flops(P: int, B: int = 1, harmonic: bool = False) -> int:
     return f + 8 * len(terms) * B
 
 
+def p2p_f16_parts(tc: dict) -> bool:
+    """Whether the tree's tensor-core P2P takes FP16 parts (stages of 16 sources) rather than TF32 parts
+    (8), from Context.tc_info(): stages of 8 are at least an eighth of the sources, and stages of 16 fewer
+    as long as a range holds some 16 sources or more (leaves of the benched trees hold hundreds)."""
+    return 8 * tc["p2p_stages"] < tc["p2p_group_sources"]
+
+
 def p2p_tc_bound(B: int, pairs: int, stages: int, peaks: dict, mhz: float, f16: bool = False) -> dict:
     """Time bound of one tensor-core P2P launch: the largest of its G and dG/dn generation on the
     FP32 pipe (the blocks' own pairs, once per unit of 64 right-hand sides), its rsqrt on the SFU,
@@ -163,7 +170,8 @@ def tc_roofline(bnd: dict, t: float, kernel: str, traffic) -> dict:
             "frac": round(bnd["bound_s"] / t, 4), "traffic": traffic,
             "bound_terms_ms": {x: round(1e3 * y, 4) for x, y in bnd["terms_s"].items()},
             "peak_note": "frac = max(generation flops / FP32 peak (152 SM x 128 x 2 x 2070 MHz, derived), rsqrt / "
-                         "SFU peak (16 per clock per SM), issued FP16 MMA flops / measured sustained bf16 peak) "
+                         "SFU peak (16 per clock per SM), issued MMA flops / measured sustained bf16 peak, "
+                         "half of it for TF32 parts) "
                          "/ the launch time; achieved and peak are the limiting term's"}
 
 
@@ -521,6 +529,7 @@ def run_ours(args, wl, rank, world, local_rank):
     peak_fp32 = fp32_peak_tflops(mhz)
     m2p_tc = B > 1 and fp32 and not args.no_tc and (args.tc is None or args.tc & 1)   # M2P of several RHS on tcgen05
     p2p_tc = B > 1 and fp32 and not args.no_tc and ctx_tc["p2p_stages"] > 0           # P2P of several RHS on tcgen05
+    p2p_f16 = p2p_f16_parts(ctx_tc)
 
     def work(name):
         """Algorithmic flops of all timed launches of a far-field slot."""
@@ -537,7 +546,8 @@ def run_ours(args, wl, rank, world, local_rank):
             k["algorithmic_tflops"] = work(name) / (k["ms_total"] * 1e-3) / 1e12
     if "p2p" in kernels:
         kernels["p2p"]["pairs_per_launch"] = pairs
-        kernels["p2p"]["path"] = "tcgen05 (FP16 hi/lo split, FP32 accumulation)" if p2p_tc else "FP32 pipe"
+        kernels["p2p"]["path"] = (f"tcgen05 ({'FP16' if p2p_f16 else 'TF32'} hi/lo split, FP32 accumulation)" if p2p_tc
+                                  else "FP32 pipe")
     if "m2p" in kernels:
         kernels["m2p"]["path"] = "tcgen05 (FP16 hi/lo split, FP32 accumulation)" if m2p_tc else "FP32 pipe"
     if "gmres" in kernels and arn["system_steps"]:
@@ -576,7 +586,7 @@ def run_ours(args, wl, rank, world, local_rank):
         bnd = m2p_tc_bound(wl["P"], B, ctx_tc["m2p_group_boxes"], peaks, mhz, f16=True)
         roof = tc_roofline(bnd, full["m2p"]["ms_per_launch"] * 1e-3, dom, traffic)
     elif dom == "p2p" and p2p_tc and "p2p" in full:
-        bnd = p2p_tc_bound(B, pairs, ctx_tc["p2p_stages"], peaks, mhz, f16=True)
+        bnd = p2p_tc_bound(B, pairs, ctx_tc["p2p_stages"], peaks, mhz, f16=p2p_f16)
         roof = tc_roofline(bnd, full["p2p"]["ms_per_launch"] * 1e-3, dom, traffic)
     elif dom in ("p2p", "m2p") and fp32 and dom in full:
         a = full[dom]["algorithmic_tflops"]
@@ -591,7 +601,7 @@ def run_ours(args, wl, rank, world, local_rank):
     # the other tensor-core kernel at the full batch, on the same max-of-three bound
     roof2 = None
     if roof is not None and roof.get("kernel") == "m2p" and p2p_tc and "p2p" in full:
-        roof2 = tc_roofline(p2p_tc_bound(B, pairs, ctx_tc["p2p_stages"], peaks, mhz, f16=True),
+        roof2 = tc_roofline(p2p_tc_bound(B, pairs, ctx_tc["p2p_stages"], peaks, mhz, f16=p2p_f16),
                             full["p2p"]["ms_per_launch"] * 1e-3, "p2p",
                             NCU_TRAFFIC.get((args.workload, "p2p", wl["theta"], wl["P"], wl["Ncrit"])))
         del roof2["peak_note"]
