@@ -113,8 +113,8 @@ TF32_PER_BF16 = 1.1 / 2.25  # nominal dense tensor rates, TF32 over BF16
 # DRAM bytes (read + write) per launch of the current kernels, from the ncu captures summarised in
 # profiles/ (dram__bytes_read.sum + dram__bytes_write.sum of one launch), keyed by workload, kernel and
 # treecode parameters (theta, P, Ncrit); None where no capture of the current kernel matches
-NCU_TRAFFIC = {("sphere81920_sweep64", "m2p", 0.4, 7, 512): 6.391e8,  # kernels_current.md
-               ("sphere81920_sweep64", "p2p", 0.4, 7, 512): 1.4684e9}
+NCU_TRAFFIC = {("sphere81920_sweep64", "m2p", 0.4, 7, 512): 6.274e8,  # kernels_current.md
+               ("sphere81920_sweep64", "p2p", 0.4, 7, 512): 1.0815e9}
 
 
 def m2p_flops(P: int, B: int = 1, harmonic: bool = False) -> int:

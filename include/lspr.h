@@ -302,7 +302,8 @@ LSPR_API int lspr_get_arnoldi_stats(lspr_ctx *ctx, int64_t *out);
 LSPR_API int lspr_set_graphs(lspr_ctx *ctx, int32_t enable);
 /* Tensor cores for the FP32 far field of several right-hand sides (B >= 2), as a mask:
  * bit 0 (default on): the M2P contraction on tcgen05 (operands split into FP16 high and low
- * parts that hold 22 bits, FP32 accumulation in tensor memory); bit 1 (default off;
+ * parts that hold 22 bits down to 2^-16 of the largest of a channel and 2^-40 of it below, FP32
+ * accumulation in tensor memory); bit 1 (default off;
  * lspr_tune_solver sets it where it pays): the tree P2P on tcgen05 (same split, TF32 parts where
  * the distances span too much; 3x the FP32-pipe kernel at 32 right-hand sides) for products with
  * at least 24 right-hand sides (channel sets) in use, the FP32-pipe P2P below that (inside a

@@ -68,9 +68,10 @@ void timer_collect(lspr_ctx *ctx) {
 
 namespace lspr {
 
+static int judge_count(lspr_ctx *c, int count, int rc);
+
 // LSPR_E_TIMEOUT if a bounded device wait ran out since the last status that reported one
 // (the stream is synchronised by the caller); otherwise rc
-static int judge_count(lspr_ctx *c, int count, int rc);
 int timeout_status(lspr_ctx *c, int rc) {
     int count = 0;
     if (cudaMemcpy(&count, c->dev_err.p, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
@@ -79,6 +80,7 @@ int timeout_status(lspr_ctx *c, int rc) {
     return judge_count(c, count, rc);
 }
 
+// the same for a stream that is not synchronised yet
 int finish_status(lspr_ctx *c) {
     const bool read = c->tc_launched;   // only the tensor-core kernels hold bounded waits
     if (read) LSPR_TRY(c, cudaMemcpyAsync(c->host_err, c->dev_err.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
@@ -87,6 +89,7 @@ int finish_status(lspr_ctx *c) {
     return read ? judge_count(c, *c->host_err, LSPR_OK) : LSPR_OK;
 }
 
+// the status for an error count just read
 static int judge_count(lspr_ctx *c, int count, int rc) {
     if (count == c->dev_err_seen) return rc;
     c->dev_err_seen = count;

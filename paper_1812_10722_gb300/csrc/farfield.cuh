@@ -1158,9 +1158,9 @@ int p2m_orders_f32(lspr_ctx *ctx, int B);
 int p2m_orders_f64(lspr_ctx *ctx, int B);
 int p2m_orders_ff(lspr_ctx *ctx, int B);
 int m2p_orders_f32(lspr_ctx *ctx, double *acc, int *counter, int B);
-// tensor-core M2P (m2p_tc.cu): FP32 operands as 3xTF32, B >= 2; LSPR_E_STATE otherwise
+// tensor-core M2P (m2p_tc.cu): FP32 operands as FP16 high/low parts, B >= 2; LSPR_E_STATE otherwise
 int m2p_tc_launch(lspr_ctx *ctx, double *acc, int *counter, int B);
-// tensor-core P2P of the tree mode (p2p_tc.cu): FP32 weights as TF32 high/low parts, B >= 2
+// tensor-core P2P of the tree mode (p2p_tc.cu): FP32 operands as FP16 (or TF32) high/low parts, B >= 2
 // min_rhs: the kernel does nothing when fewer right-hand sides are in use (the FP32-pipe P2P
 // then takes the product)
 int p2p_tc_launch(lspr_ctx *ctx, double *acc, cudaStream_t st, int *counter, int B, int min_rhs);

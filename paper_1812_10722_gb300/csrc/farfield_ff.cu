@@ -217,8 +217,8 @@ int m2p_ff_launch(lspr_ctx *ctx, double *acc, int *counter, int B) {
     const int NT = n_terms(tr.P), W = ff_ring(tr.P);
     LSPR_TRY(ctx, allow_smem(m2p_ff_kernel<NB>, (int)ff_m2p_smem(NT, W, NB), ctx->device, smem_set));
     if (occ_nt != NT) {
-        // the fewest parts (1 to 3) of a box's moments that give the most resident blocks per SM
-        // (P 7, 8 right-hand sides: three parts of 40 terms, 53.8 KB, four blocks instead of three)
+        // the fewest parts (1 to 3) of a box's moments that give the most resident blocks per SM (P 7,
+        // 8 right-hand sides: whole, 36 KB, which leaves room for the six blocks that the registers allow)
         occ = 0;
         tp_sel = NT;
         for (int parts = 1; parts <= 3; ++parts) {

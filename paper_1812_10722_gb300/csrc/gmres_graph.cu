@@ -851,7 +851,7 @@ int capture_cycle(lspr_ctx *ctx, int mode, const Arn &a0, GraphCache &gc) {
     const int rp = launch_precond(ctx, a, cs);
     if (rp != LSPR_OK) return fail(rp);
     // the product works on the running systems only, packed into the first slots (with
-    // several surfaces, the S channel sets of a system follow each other)
+    // several surfaces, set t K + k is surface t of the k-th of the K running systems)
     ctx->rhs_map = a.rmap;
     ctx->rhs_inv = a.rmap + a.B;
     ctx->rhs_nact = a.rmap + 2 * a.B + 1;

@@ -201,7 +201,7 @@ struct Tree {
     DArr<int> tcp_stat;      // bits of the smallest and largest squared P2P distance, the largest source weight
     bool tcp_f16 = false;    // FP16 parts (16 sources per stage) rather than TF32 (8)
     float tcp_gs = 1.f, tcp_ts = 1.f;   // scales of G and dG/dn
-    int64_t n_tcp_items = 0, n_tcp_ivl = 0, n_tcp_sources = 0, n_tcp_stages = 0;   // stages of 8 sources
+    int64_t n_tcp_items = 0, n_tcp_ivl = 0, n_tcp_sources = 0, n_tcp_stages = 0;   // stages of 16 (TF32: 8) sources
     bool tc_built = false, tcp_built = false;   // the group lists above match the tree
     DArr<int4> p2m_items;    // (leaf, source begin, source end, 0): leaves under an accepted box
     DArr<int> box_parent;    // parent box (-1 for the root)

@@ -22,8 +22,9 @@
 // What falls below full precision is then at most 2^-25 absolute in both: 2^-40 of the largest.
 // Against TF32 parts the MMAs take half the K steps and the operands half the bytes: 81920 panels, P 7,
 // 64 right-hand sides 2.57 -> 1.58 ms with both preparing kernels; sensor of 145920 panels 6.12 -> 4.38.
-// Error of the product against the float-float operator of the same tree, over batches of 2 to 28 on
-// spheres and sensors: 0.4 to 0.9 of the TF32 form's (half as many accumulation steps).
+// Error of the product against the float-float operator of the same tree, with the unit lengths of
+// lspr_internal.cuh: 0.4 to 0.97 of that with TF32 parts in units of 32 boxes, over random and smooth vectors,
+// orders 4 to 8, batches of 2 to 64, spheres of 5120 to 81920 panels and sensors.
 // Three kernels per product:
 //   - m2p_max_kernel finds the scales;
 //   - tc_image_kernel writes, once per product, the split moments of every box in the

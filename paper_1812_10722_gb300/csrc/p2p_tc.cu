@@ -20,7 +20,7 @@
 // (the epilogue adds both halves).
 //
 // The parts are FP16 (16 sources per stage) where the kernel values' range allows it, else TF32 (8
-// sources; FP16 parts hold the same 22 bits at twice the rate).  The smallest and the largest distance
+// sources; FP16 parts hold the same 22 bits at twice the rate, but for the smallest values, see below).  The smallest and the largest distance
 // of a P2P pair (pair_range_kernel, once per tree) set powers of two that bring G and dG/dn (at most
 // 1/r and 1/r^2) below 2^15.  With their ratio at most kTcP2PRange = 4096, G stays above 2^3 and loses
 // nothing; dG/dn falls to 2^-9 at the largest distances, where its parts keep 2^-25 absolute: summed
@@ -48,9 +48,10 @@
 // While a unit's accumulators are drained no MMA runs, so units are long (tc_unit) and the drain adds
 // whole 32-byte sectors: rows 2 j and 2 j + 1 of an operand are re and im of right-hand side j, and a
 // warp exchanges halves of D_V and D_K so that one instruction adds all four components of eight.
-// 81920 panels, 64 right-hand sides, with the preparing kernels: 1.77 ms; 1.92 with the sectors
+// 81920 panels, 64 right-hand sides, with the preparing kernels: 1.84 ms; 1.76 with units of 4096 sources,
+// whose error was too large (lspr_internal.cuh); at that length 1.92 with the sectors
 // touched by two instructions each and every range's bounds loaded when it begins instead of one range
-// ahead, 2.19 with units of 2048 sources besides; 3.44 with TF32 parts (a stage
+// ahead, and 2.19 in that form with units of 2048 sources; 3.44 with TF32 parts (a stage
 // of 8 sources took 0.86 us, 0.48 of it the MMAs and as much its 121 KB of shared-memory traffic; FP16
 // halves both per source); 4.24 with the weights split by four of the generating warps (which every
 // stage waited for) and a barrier arrival per thread.  Error of the product of 28 right-hand sides

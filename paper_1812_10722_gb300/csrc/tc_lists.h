@@ -24,7 +24,7 @@ struct TcRange {   // layout of int4
 // The size of the units when `total` boxes or sources are spread over `sms` persistent blocks: as
 // long as some 2.5 units per block remain, between lo and hi.  M2P of 20480 panels, 16 right-hand sides
 // (23979 boxes, 152 blocks): 268, 240, 279 us with units of 32, 64, 128 boxes; 81920 panels, 64 (80757
-// boxes): 1574, 1470, 1419 us.
+// boxes): 1574, 1470, 1419 us, where the error sets the limit (lspr_internal.cuh).
 inline int tc_unit(int64_t total, int sms, int lo, int hi) {
     const int64_t n = 2 * total / (5 * (int64_t)std::max(1, sms));
     return (int)std::min<int64_t>(hi, std::max<int64_t>(lo, n));

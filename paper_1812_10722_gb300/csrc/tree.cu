@@ -4,7 +4,7 @@
 // expansion, M2P) and of leaves summed directly (P2P).
 //
 // Device pipeline: bounding cube -> 30-bit Morton keys (10 bits per axis) ->
-// LSD radix sort (4-bit digits, stable) of sources and targets -> permuted
+// LSD radix sort (8-bit digits, stable) of sources and targets -> permuted
 // work-order arrays -> octree, level by level in one CTA (deterministic box
 // numbering) -> box centres (centre of the sources' bounding box) and radii
 // r_b = max |y - c| -> target-block bounding boxes -> interaction lists (count,
